@@ -59,12 +59,16 @@ extern "C" sste_status sste_create(sste_ctx **out, int device, void *workspace, 
     ctx->partials_dev = reinterpret_cast<double *>(ws + SSTE_WS_PARTIALS_OFF);
     ctx->cu_tensor_map_encode = encode;
     ctx->splitk_partials = nullptr;
+    ctx->splitk_tickets = nullptr;
     ctx->splitk_partial_bytes = 0;
     if (workspace_bytes > SSTE_WS_SPLITK_PARTIALS_OFF + (size_t(1) << 20)) {
         ctx->splitk_partials = reinterpret_cast<float *>(ws + SSTE_WS_SPLITK_PARTIALS_OFF);
         ctx->splitk_partial_bytes = workspace_bytes - SSTE_WS_SPLITK_PARTIALS_OFF;
     }
-    if (cudaMemset(ws, 0, SSTE_WS_PARTIALS_OFF) != cudaSuccess) {
+    if (ctx->splitk_partials) ctx->splitk_tickets = reinterpret_cast<unsigned int *>(ws + SSTE_WS_SPLITK_TICKETS_OFF);
+    if (cudaMemset(ws, 0, SSTE_WS_PARTIALS_OFF) != cudaSuccess ||
+        (ctx->splitk_tickets &&
+         cudaMemset(ctx->splitk_tickets, 0, SSTE_SPLITK_TICKETS * sizeof(unsigned int)) != cudaSuccess)) {
         delete ctx;
         return SSTE_ERR_CUDA;
     }
@@ -89,6 +93,9 @@ extern "C" sste_status sste_poll_device_status(sste_ctx *ctx, void *stream)
     SSTE_CUDA_TRY(cudaMemcpyAsync(&word, ctx->status_dev, sizeof word, cudaMemcpyDeviceToHost, s));
     SSTE_CUDA_TRY(cudaMemsetAsync(ctx->status_dev, 0, sizeof word, s));
     SSTE_CUDA_TRY(cudaStreamSynchronize(s));
+    // a product that gave up on a wait may have left split tiles half counted
+    if (word == SSTE_ERR_TIMEOUT && ctx->splitk_tickets)
+        SSTE_CUDA_TRY(cudaMemsetAsync(ctx->splitk_tickets, 0, SSTE_SPLITK_TICKETS * sizeof(unsigned int), s));
     if (word > SSTE_ERR_TIMEOUT) return SSTE_ERR_CUDA;
     return static_cast<sste_status>(word);
 }

@@ -18,6 +18,7 @@ struct sste_ctx {
     double *partials_dev;       // 2 doubles per reduction block
     void *cu_tensor_map_encode; // cuTensorMapEncodeTiled, resolved through the runtime
     float *splitk_partials;         // fp32 partial tiles of split-K products; null if the workspace is minimal
+    unsigned int *splitk_tickets;   // arrival counters of the split tiles, zero between launches
     size_t splitk_partial_bytes;
 };
 
@@ -26,8 +27,10 @@ constexpr size_t SSTE_WS_STATUS_OFF = 0;
 constexpr size_t SSTE_WS_COUNTER_OFF = 64;
 constexpr size_t SSTE_WS_PARTIALS_OFF = 256;
 constexpr size_t SSTE_WS_BYTES = SSTE_WS_PARTIALS_OFF + 2 * sizeof(double) * SSTE_MAX_REDUCE_BLOCKS;
-// optional tail of the workspace, used by split-K products
-constexpr size_t SSTE_WS_SPLITK_PARTIALS_OFF = (SSTE_WS_BYTES + 1023) / 1024 * 1024;
+// optional tail of the workspace, used by split-K products: arrival counters, then partial tiles
+constexpr int SSTE_SPLITK_TICKETS = 2048;
+constexpr size_t SSTE_WS_SPLITK_TICKETS_OFF = (SSTE_WS_BYTES + 1023) / 1024 * 1024;
+constexpr size_t SSTE_WS_SPLITK_PARTIALS_OFF = SSTE_WS_SPLITK_TICKETS_OFF + SSTE_SPLITK_TICKETS * sizeof(unsigned int);
 constexpr size_t SSTE_WS_RECOMMENDED_BYTES = SSTE_WS_SPLITK_PARTIALS_OFF + (size_t(192) << 20);
 
 static inline bool sste_mult128(int v) { return v > 0 && (v % 128) == 0; }

@@ -9,12 +9,11 @@
 // at half the rate per SM -- with one CTA per tile the sparse instruction is bound by that
 // stream and runs no faster than the dense one -- and L2 -> SM traffic per flop drops.
 //   warp 0    TMA producer (both CTAs; all transaction bytes land on the leader's barrier)
-//   warp 1    leader CTA: tcgen05.mma[.sp] issue; both CTAs: tensor-memory allocation
-//   warps 2-5 epilogue: TMEM -> registers -> bf16 -> shared memory -> TMA store
-//   warps 6-9 sparse A: metadata HBM -> registers -> tensor memory (tcgen05.st), so that no
-//             metadata copy sits between two MMAs in the tensor pipe (a tcgen05.cp there drains it);
-//             compressed B (grad_X from the forward's operand): expansion of values + metadata
-//             into the dense shared-memory stage
+//   warp 1    leader CTA: tcgen05.cp of the stage's metadata, tcgen05.mma[.sp] issue; both CTAs: tensor-memory allocation
+//   warps 2-9 epilogue, each on its own 32 accumulator rows and half of the columns: TMEM -> registers -> bf16 ->
+//             shared memory -> TMA store
+//   compressed B only (grad_X from the forward's operand): warps 2-5 epilogue on all columns, warps 6-9 expand values +
+//             metadata into the dense shared-memory stage
 // Output tiles are handed out band by band (tile_coords) so that operands are read from HBM about
 // once; tile width, split-K plan and band height come from cost models on the host (make_plan).
 // Every wait is bounded: on expiry the CTA records SSTE_ERR_TIMEOUT and leaves.
@@ -29,7 +28,8 @@ namespace {
 
 constexpr int BM = 128;            // rows of A per CTA (a pair covers 256)
 constexpr int TMEM_COLS = 512;
-constexpr int STAGING_BYTES = 32768;   // two epilogue panels of 128 x 64 bf16
+constexpr int MAX_SPLITS = 4;      // split-K factor limit
+constexpr int PANEL_BYTES = 2048;  // epilogue panel: 32 x 32 bf16
 constexpr unsigned long long WAIT_LIMIT_NS = 2000000000ull;   // two seconds of wall time (%globaltimer)
 
 enum class BMajor { K, MN };
@@ -143,24 +143,6 @@ __device__ __forceinline__ void prefetch_tensormap(const CUtensorMap *map)
 {
     asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
 }
-__device__ __forceinline__ void epilogue_barrier() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
-// Barrier of the 128 epilogue threads that also combines a flag: true only if every thread passed true.
-// The four epilogue warps wait for an accumulator separately; they must leave TOGETHER when one wait
-// expired, or the others would park at the next epilogue barrier for good.
-__device__ __forceinline__ bool epilogue_all(bool ok)
-{
-    uint32_t r;
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t"
-        "setp.ne.b32 p, %1, 0;\n\t"
-        "bar.red.and.pred q, 1, 128, p;\n\t"
-        "selp.b32 %0, 1, 0, q;\n\t}"
-        : "=r"(r)
-        : "r"(ok ? 1u : 0u)
-        : "memory");
-    return r != 0;
-}
-
 __device__ __forceinline__ void tmem_alloc(uint32_t dst_smem, uint32_t cols)
 {
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst_smem), "r"(cols) : "memory");
@@ -223,6 +205,46 @@ __device__ __forceinline__ void tmem_ld_32x32(uint32_t taddr, uint32_t r[32])
           "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
         : "r"(taddr));
 }
+// 16 lanes x 32 consecutive 32-bit columns in the fragment layout of the 8 x 8 matrix stores: for the 8-column block b
+// thread t holds r[4b], r[4b + 1] = row t / 4, columns 2 (t % 4), + 1 and r[4b + 2], r[4b + 3] = the same of row t / 4 + 8
+__device__ __forceinline__ void tmem_ld_16x256_x4(uint32_t taddr, uint32_t r[16])
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.16x256b.x4.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr));
+}
+// 32 accumulator columns of a warp's 32 rows -> 32 registers.  TRANSPOSED = false: r[c] = column c of row `lane`;
+// true: r[16 h + i] = fragment i (above) of rows 16 h .. 16 h + 15.
+template <bool TRANSPOSED>
+__device__ __forceinline__ void tmem_ld_32cols(uint32_t taddr, uint32_t *r)
+{
+    if (TRANSPOSED) {
+        tmem_ld_16x256_x4(taddr, r);
+        tmem_ld_16x256_x4(taddr + (16u << 16), r + 16);
+    } else {
+        tmem_ld_32x32(taddr, r);
+    }
+}
+// four 8 x 8 matrices of 16-bit elements, stored transposed: thread t gives the address of row t % 8 of matrix t / 8
+__device__ __forceinline__ void stmatrix_x4_trans(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
+{
+    asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1, %2, %3, %4};"
+                 ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+__device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
+{
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+// One metadata atom (128 lanes x 16 bytes, contiguous in shared memory) -> four tensor-memory columns, in both CTAs of
+// the pair from their own shared memory at the same offset.  Issued by the thread that issues the MMAs: it executes in
+// order with the MMAs that follow.
+__device__ __forceinline__ void tc_cp_meta_atom(uint32_t taddr, uint64_t sdesc)
+{
+    asm volatile("tcgen05.cp.cta_group::2.128x128b [%0], %1;" ::"r"(taddr), "l"(sdesc) : "memory");
+}
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // ------------------------------------------------------------------ descriptors
@@ -278,91 +300,77 @@ struct GemmParams {
     int group_m;            // tile rows per band of the tile order (see tile_coords)
     int splits;             // split-K factor of the tiles from `split_from` on (1 = none)
     int split_from;         // first split tile: tiles below it are computed whole
-    float *partials;        // split-K: fp32 partial tiles [tile][cta][split][128][BN], summed by splitk_reduce_kernel
+    float *partials;        // split-K: fp32 partial tiles [split tile][cta][split][row quarter][BN / 4][32 lanes][4]
+    unsigned int *tickets;  // split-K: arrivals per [split tile][cta][epilogue warp]; zero between launches
 };
 
-// 32 lanes x 16 consecutive 32-bit columns <- 16 registers per thread (four metadata atoms in one instruction)
-__device__ __forceinline__ void tmem_st_32x16(uint32_t taddr, const uint4 (&v)[4])
-{
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
-        "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
-        ::"r"(taddr), "r"(v[0].x), "r"(v[0].y), "r"(v[0].z), "r"(v[0].w), "r"(v[1].x), "r"(v[1].y), "r"(v[1].z),
-          "r"(v[1].w), "r"(v[2].x), "r"(v[2].y), "r"(v[2].z), "r"(v[2].w), "r"(v[3].x), "r"(v[3].y), "r"(v[3].z),
-          "r"(v[3].w)
-        : "memory");
-}
-__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 // Shared-memory / tensor-memory plan of one CTA for a tile of 256 x BN.  A stage holds 128 bytes of K per
 // A row and, for the sparse kernels, two B sub-tiles of 128 bytes of K each (the compressed A row covers
-// twice the K of one B row); the dense kernel pairs it with one B sub-tile.  A sparse tile of BN = 256
-// leaves room for one accumulator buffer beside the metadata regions in the 512 tensor-memory columns;
-// BN <= 192, and every dense tile, has two, so the epilogue of a tile overlaps the next tile's main loop.
-template <bool SPARSE, int BN, bool BCOMP = false>
+// twice the K of one B row) and the metadata atoms of that K; the dense kernel pairs it with one B sub-tile.
+// Tensor memory: the accumulators, then the stages' metadata (four columns per atom, one region per stage, so a region
+// is free again exactly when its stage is).  A sparse tile of BN = 256 leaves room for one accumulator buffer; BN <= 224,
+// and every dense tile, has two, so the epilogue of a tile overlaps the next tile's main loop.
+template <bool SPARSE, int ELT, int BN, bool BCOMP = false>
 struct Cfg {
     static constexpr int A_STAGE = 16384;                        // 128 rows x 128 bytes
     static constexpr int B_SUB = (BN / 2) * 128;                 // this CTA's half of one B sub-tile
     static constexpr int B_STAGE = SPARSE ? 2 * B_SUB : B_SUB;
-    static constexpr int STAGE = A_STAGE + B_STAGE;
-    static constexpr int FIT = (232448 - 1024 - 512 - STAGING_BYTES) / STAGE;   // 227 KB of shared memory per CTA
+    static constexpr int ATOMS = SPARSE ? 256 / ELT / 128 : 0;   // metadata atoms (128 logical K, 2 KB) per stage
+    static constexpr int STAGE = A_STAGE + B_STAGE + 2048 * ATOMS;
+    static constexpr int EPI_WARPS = BCOMP ? 4 : 8;              // compressed B: the other four expand
+    static constexpr int ROOM = 232448 - 1024 - 512;             // 227 KB of shared memory per CTA, slack, barriers
+    static constexpr int FIT = (ROOM - EPI_WARPS * PANEL_BYTES) / STAGE;
     static constexpr int STAGES = FIT > 8 ? 8 : FIT;
-    static constexpr int ACC_BUFS = (!SPARSE || BN <= 224) ? 2 : 1;   // the dense kernel keeps no metadata in TMEM
+    // epilogue panels per warp: two (a panel is filled while the other is stored) where they fit
+    static constexpr int PANELS = (ROOM - STAGES * STAGE >= 2 * EPI_WARPS * PANEL_BYTES) ? 2 : 1;
+    static constexpr int STAGING_BYTES = EPI_WARPS * PANELS * PANEL_BYTES;
+    static constexpr int ACC_BUFS = (!SPARSE || BN <= 224) ? 2 : 1;
     static constexpr int META_COL0 = ACC_BUFS * BN;              // metadata regions follow the accumulators
-    static constexpr int META_FIT = (TMEM_COLS - META_COL0) / 16;
-    static constexpr int META_REGIONS = !SPARSE ? 1 : (META_FIT > 8 ? 8 : META_FIT);   // regions of 16 columns (four atoms)
-    static constexpr int THREADS = (SPARSE || BCOMP) ? 320 : 192;     // + 4 metadata (sparse A) or expander (compressed B) warps
-    static constexpr int PANEL = (BN % 64 == 0) ? 64 : 32;       // columns per epilogue panel (one TMA store)
+    static constexpr int META_COLS = 4 * ATOMS;                  // tensor-memory columns of one stage's metadata
+    static constexpr int THREADS = 320;
     static constexpr int SMEM_BYTES = STAGES * STAGE + STAGING_BYTES + 1024 /* alignment slack */ + 512 /* barriers */;
-    static_assert(META_COL0 + (SPARSE ? META_REGIONS * 16 : 0) <= TMEM_COLS, "tensor memory budget");
-    static_assert(!SPARSE || META_REGIONS >= 4, "metadata regions");
+    static_assert(META_COL0 + STAGES * META_COLS <= TMEM_COLS, "tensor memory budget");
     static_assert(STAGES >= 3, "pipeline depth");
+    static_assert(STAGE % 1024 == 0 && BN % 32 == 0, "swizzle alignment, epilogue panels");
 };
 
 // ELT: operand element size in bytes (2 = bf16 via kind::f16, 1 = fp8 via kind::f8f6f4).
 // OUT_T: store D transposed (out[n, m]); OUT_F32: fp32 output (direct stores) instead of bf16 (TMA stores).
 // BCOMP: the (dense-product) B operand is given in compressed 2:4 form and expanded in shared memory.
 template <bool SPARSE, BMajor BMAJ, int ELT, int BN, bool OUT_T, bool OUT_F32, bool BCOMP = false>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Cfg<SPARSE, BN, BCOMP>::THREADS, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Cfg<SPARSE, ELT, BN, BCOMP>::THREADS, 1)
 gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
-            const __grid_constant__ CUtensorMap map_d, const __grid_constant__ CUtensorMap map_p,
+            const __grid_constant__ CUtensorMap map_d, const __grid_constant__ CUtensorMap map_m,
             const uint8_t *__restrict__ meta, const GemmParams p)
 {
     sste_pdl_trigger();
-    using C = Cfg<SPARSE, BN, BCOMP>;
-    constexpr int META_REGIONS = C::META_REGIONS;
+    using C = Cfg<SPARSE, ELT, BN, BCOMP>;
     constexpr int NS = C::STAGES;
     constexpr int NB = C::ACC_BUFS;
     constexpr bool F8 = (ELT == 1);
     constexpr int BK = (SPARSE ? 256 : 128) / ELT;    // logical K per stage
     constexpr int B_SUBS = SPARSE ? 2 : 1;
     constexpr int SUB_K = 128 / ELT;                  // logical K of one B sub-tile
-    constexpr int ATOMS_PER_STAGE = SPARSE ? BK / 128 : 1;   // metadata atoms (128 logical K) per stage
     constexpr int B_CHUNK_N = 128 / ELT;              // MN-major: N elements per 128-byte row
     constexpr int B_CHUNKS_HALF = (BN / 2) / B_CHUNK_N;
     constexpr uint32_t STAGE_TX = 2u * (BCOMP ? C::A_STAGE : C::STAGE);   // both CTAs' bytes that arrive by TMA
-    constexpr int PANEL = C::PANEL;                   // the epilogue works in panels of 64 (or 32) columns
-    constexpr int DIRECT_PANELS = (BN - 128) / PANEL; // the last 128 columns go through registers (early release)
     static_assert(BMAJ == BMajor::K || (BN / 2) % B_CHUNK_N == 0, "MN-major B needs whole 128-byte chunks per CTA");
-    static_assert(PANEL == 64 || (OUT_T && !OUT_F32), "32-column panels exist for the transposed bf16 store only");
     static_assert(!BCOMP || (!SPARSE && BMAJ == BMajor::MN), "compressed B: dense A, MN-major B");
 
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t staging = smem_base + NS * C::STAGE;
-    const uint32_t bars = staging + STAGING_BYTES;
+    const uint32_t bars = staging + C::STAGING_BYTES;
     auto full_bar = [&](int s) { return bars + 8u * s; };              // used in the leader only
     auto empty_bar = [&](int s) { return bars + 8u * (NS + s); };      // one per CTA
     auto acc_full_bar = [&](int b) { return bars + 8u * (2 * NS + b); };           // one per CTA
-    auto acc_empty_bar = [&](int b) { return bars + 8u * (2 * NS + 2 + b); };      // leader only, 2 arrivals
-    auto meta_full_bar = [&](int r) { return bars + 8u * (2 * NS + 4 + r); };             // leader only, 8 arrivals
-    auto meta_empty_bar = [&](int r) { return bars + 8u * (2 * NS + 4 + META_REGIONS + r); };   // one per CTA
-    constexpr int MISC = 2 * NS + 4 + 2 * META_REGIONS;
+    auto acc_empty_bar = [&](int b) { return bars + 8u * (2 * NS + 2 + b); };      // leader only, one arrival per epilogue warp of the pair
+    constexpr int MISC = 2 * NS + 4;
     const uint32_t tmem_slot = bars + 8u * MISC;
     uint8_t *bars_generic = smem_raw + (bars - smem_u32(smem_raw));
     volatile uint32_t *tmem_slot_ptr = reinterpret_cast<volatile uint32_t *>(bars_generic + 8u * MISC);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(bars_generic + 8u * (MISC + 1));
-    uint8_t *staging_generic = smem_raw + (staging - smem_u32(smem_raw));
     static_assert(8 * (MISC + 2) + 64 <= 512, "barrier block (+ the expander's 16-entry selector table)");
     const WaitCtx wc{p.status, abort_flag, p.wait_limit_ns};
 
@@ -374,33 +382,32 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     const int n_tiles = (p.N + BN - 1) / BN;
     const int num_tiles = m_tiles * n_tiles;
     const int k_blocks_total = (p.K + BK - 1) / BK;   // a ragged last stage reads zero-filled K
-    // Work units: tiles [0, split_from) are whole; every later tile is cut into `splits` K ranges (the
-    // host makes the division exact).  Whole tiles fill complete waves, the split ones spread the
-    // last, partial wave over all pairs.
+    // Work units: tiles [0, split_from) are whole; every later tile is cut into `splits` K ranges that differ by
+    // at most one stage.  Whole tiles fill complete waves, the split ones spread the last, partial wave over all pairs.
     const int num_units = p.split_from + (num_tiles - p.split_from) * p.splits;
-    struct Unit { int tile, split, k_blocks; };
+    struct Unit { int tile, split, kb0, kb1; };
     auto decode = [&](int unit) {
         Unit u;
-        if (unit < p.split_from) { u.tile = unit; u.split = 0; u.k_blocks = k_blocks_total; }
+        if (unit < p.split_from) { u.tile = unit; u.split = 0; u.kb0 = 0; u.kb1 = k_blocks_total; }
         else {
             const int v = unit - p.split_from;
             u.tile = p.split_from + v / p.splits;
             u.split = v % p.splits;
-            u.k_blocks = k_blocks_total / p.splits;
+            u.kb0 = u.split * k_blocks_total / p.splits;
+            u.kb1 = (u.split + 1) * k_blocks_total / p.splits;
         }
         return u;
     };
-    const int k_atoms = p.K / 128;
 
     if (threadIdx.x == 0) {
         // full: the producer's arrival with the TMA byte count (+ the eight expander warps of the pair)
         for (int s = 0; s < NS; ++s) { mbar_init(full_bar(s), BCOMP ? 9 : 1); mbar_init(empty_bar(s), 1); }
-        for (int b = 0; b < 2; ++b) { mbar_init(acc_full_bar(b), 1); mbar_init(acc_empty_bar(b), 2); }
-        for (int r = 0; r < META_REGIONS; ++r) { mbar_init(meta_full_bar(r), 8); mbar_init(meta_empty_bar(r), 1); }
+        for (int b = 0; b < 2; ++b) { mbar_init(acc_full_bar(b), 1); mbar_init(acc_empty_bar(b), 2 * C::EPI_WARPS); }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         prefetch_tensormap(&map_a);
         if (!BCOMP) prefetch_tensormap(&map_b);
+        if (SPARSE) prefetch_tensormap(&map_m);
         if (!OUT_F32) prefetch_tensormap(&map_d);
     }
     if (warp == 1) {
@@ -417,20 +424,18 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer (both CTAs)
         if (lane == 0) {
-            uint32_t it = 0;
+            const int k_atoms = p.K / 128;
+            uint32_t s = 0, ph = 0;          // stage of the ring and the parity of its round
             bool ok = true;
             for (int unit = pair; unit < num_units && ok; unit += num_pairs) {
                 const Unit u = decode(unit);
-                const int tile = u.tile, k_blocks = u.k_blocks, kb0 = u.split * u.k_blocks;
                 int mt, nt;
-                tile_coords(tile, m_tiles, n_tiles, p.group_m, mt, nt);
+                tile_coords(u.tile, m_tiles, n_tiles, p.group_m, mt, nt);
                 const int m0 = mt * 2 * BM + static_cast<int>(rank) * BM;      // this CTA's rows of A
                 const int n0 = nt * BN + static_cast<int>(rank) * (BN / 2);    // this CTA's half of B
-                for (int kb = kb0; kb < kb0 + k_blocks; ++kb, ++it) {
-                    const int s = it % NS;
-                    const uint32_t ph = (it / NS) & 1u;
+                for (int kb = u.kb0; kb < u.kb1; ++kb) {
                     // test hook: the stage is never loaded nor announced, so the MMA warp's wait for it runs out
-                    if (p.skip_last_stage && unit + num_pairs >= num_units && kb == kb0 + k_blocks - 1) break;
+                    if (p.skip_last_stage && unit + num_pairs >= num_units && kb == u.kb1 - 1) break;
                     if (!mbar_wait(empty_bar(s), ph ^ 1u, wc)) { ok = false; break; }
                     const uint32_t lead_full = map_to_cta(full_bar(s), 0);
                     if (leader) mbar_arrive_expect_tx(full_bar(s), STAGE_TX);
@@ -438,6 +443,10 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                     const uint32_t b_dst = a_dst + C::A_STAGE;
                     // A: 128 bytes per row = BK/2 compressed (sparse) or BK dense elements
                     tma_load_2d(a_dst, &map_a, lead_full, kb * (SPARSE ? BK / 2 : BK), m0);
+                    // metadata: the atoms of this K, 2 KB each, as rows of 512 bytes.  (With an odd number of atoms the
+                    // last 8-bit stage also fetches the first atom of the next row block: it meets zero-filled K.)
+                    if (SPARSE)
+                        tma_load_2d(b_dst + C::B_STAGE, &map_m, lead_full, 0, ((m0 / BM) * k_atoms + kb * C::ATOMS) * 4);
                     if (BCOMP) {
                         // B is written into the stage by the expander warps
                     } else if (BMAJ == BMajor::K) {
@@ -450,6 +459,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                         for (int c = 0; c < B_CHUNKS_HALF; ++c)
                             tma_load_2d(b_dst + c * (BK * 128), &map_b, lead_full, n0 + c * B_CHUNK_N, kb * BK);
                     }
+                    if (++s == NS) { s = 0; ph ^= 1u; }
                 }
             }
         }
@@ -457,34 +467,30 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         // ------------------------------------------------------------ MMA issuer (leader CTA only)
         if (leader && lane == 0) {
             const uint32_t idesc = instr_desc(SPARSE, p.afmt, p.bfmt, BMAJ == BMajor::MN, BN);
-            uint32_t it = 0, local_tile = 0, group_it = 0;
+            uint32_t s = 0, ph = 0, local_tile = 0;
             bool ok = true;
             for (int unit = pair; unit < num_units && ok; unit += num_pairs, ++local_tile) {
-                const int k_blocks = decode(unit).k_blocks;
+                const Unit u = decode(unit);
                 const uint32_t buf = local_tile % NB, use = local_tile / NB;
                 if (!mbar_wait(acc_empty_bar(buf), (use & 1u) ^ 1u, wc)) { ok = false; break; }
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + buf * BN;
-                for (int kb = 0; kb < k_blocks; ++kb, ++it) {     // stage index inside the unit's K range
-                    const int s = it % NS;
-                    const uint32_t ph = (it / NS) & 1u;
-                    uint32_t meta_cols = 0;
-                    if (SPARSE) {
-                        // metadata groups of four atoms rotate over META_REGIONS tensor-memory regions,
-                        // written by the metadata warps of both CTAs
-                        const int atom0 = kb * ATOMS_PER_STAGE;
-                        const uint32_t region = group_it % META_REGIONS;
-                        if ((atom0 & 3) == 0 &&
-                            !mbar_wait(meta_full_bar(region), (group_it / META_REGIONS) & 1u, wc)) {
-                            ok = false;
-                            break;
-                        }
-                        meta_cols = tmem_base + C::META_COL0 + 16 * region + 4 * (atom0 & 3);
-                    }
+                uint32_t acc = 0;
+                for (int kb = u.kb0; kb < u.kb1; ++kb) {
                     if (!mbar_wait(full_bar(s), ph, wc)) { ok = false; break; }
                     tc_fence_after();
                     const uint32_t a_src = smem_base + s * C::STAGE;
                     const uint32_t b_src = a_src + C::A_STAGE;
+                    const uint32_t meta_cols = tmem_base + C::META_COL0 + s * C::META_COLS;
+                    // Metadata rides in the stage and is copied to tensor memory in front of the stage's MMAs.  (It used
+                    // to go through the registers of four extra warps, tcgen05.st and a handshake per four atoms: their
+                    // round trip paced the loop.  4096 x 8192 x 4096, clk per stage, bf16 / FP8: 783 / 1186 before,
+                    // 639 / 612 now, against 594 / 562 with no metadata refreshed at all.)
+                    if (SPARSE) {
+#pragma unroll
+                        for (int i = 0; i < C::ATOMS; ++i)
+                            tc_cp_meta_atom(meta_cols + 4 * i, smem_desc(b_src + C::B_STAGE + 2048 * i, 128, 128, 0));
+                    }
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
                         const uint64_t adesc = smem_desc(a_src + 32 * j, 16, 1024, 2);
@@ -496,7 +502,6 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                             constexpr int ROWS_PER_MMA = BK / 4;     // K rows of 128 bytes per instruction
                             bdesc = smem_desc(b_src + ROWS_PER_MMA * 128 * j, BK * 128, 1024, 2);
                         }
-                        const uint32_t acc = (kb > 0 || j > 0) ? 1u : 0u;
                         if (SPARSE) {
                             // bf16: one 32-bit metadata column per instruction, the column pair is addressed and
                             // the descriptor's sparse selector picks the column; fp8: two columns per instruction
@@ -506,51 +511,88 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                         } else {
                             tc_mma_dense<F8>(d_tmem, adesc, bdesc, idesc, acc);
                         }
+                        acc = 1u;
                     }
                     tc_commit_pair(empty_bar(s));     // frees the stage in both CTAs once these MMAs have read it
-                    if (SPARSE) {
-                        const int atom_end = (kb + 1) * ATOMS_PER_STAGE;
-                        if ((atom_end & 3) == 0 || kb == k_blocks - 1) {
-                            tc_commit_pair(meta_empty_bar(group_it % META_REGIONS));
-                            ++group_it;
-                        }
-                    }
+                    if (++s == NS) { s = 0; ph ^= 1u; }
                 }
                 if (ok) tc_commit_pair(acc_full_bar(buf));
             }
         }
-    } else if (warp < 6) {
-        // ------------------------------------------------------------ epilogue (warps 2..5, both CTAs)
+    } else if (warp < 2 + C::EPI_WARPS) {
+        // ------------------------------------------------------------ epilogue (warps 2.., both CTAs)
+        // A warp owns 32 rows and a range of columns (half of them with eight warps) of the accumulator from tensor memory
+        // to the output and waits for no other warp.  Its part is pulled into registers (packed bf16) and the accumulator
+        // released before the first store, so that the next main loop waits for the tensor-memory reads only.  The chain of
+        // each panel (wait for the buffer, fill, proxy fence, store) is latency, hence eight warps and not four.
         const int quarter = warp & 3;                  // tensor-memory lanes [32*quarter, 32*quarter + 32)
-        const int row = quarter * 32 + lane;           // row of this CTA's 128 x BN accumulator
+        constexpr int PANELS_MAX = C::EPI_WARPS == 8 ? (BN / 32 + 1) / 2 : BN / 32;   // 32-column panels per warp
+        const int pnl0 = ((warp - 2) >> 2) * PANELS_MAX;                              // first panel of this warp
+        const int n_pnl = (C::EPI_WARPS == 8 && pnl0 > 0) ? BN / 32 - PANELS_MAX : PANELS_MAX;
         const float scale = sste_out_scale(p.a_amax, p.a_fp8_max, p.b_amax, p.b_fp8_max);
         const bool want_amax = (p.out_amax != nullptr);
-        const bool plain = !want_amax && scale == 1.0f;
+        const int kind = want_amax ? 2 : scale != 1.0f ? 1 : 0;      // what a stored value needs besides the rounding
         uint32_t amax2 = 0;                            // bf16 output: running max of the magnitude bits, two lanes of 16
         float amaxf = 0.0f;                            // fp32 output
-        const bool store_thread = (threadIdx.x == 64);
         const uint32_t lane_base = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
+        const uint32_t my_staging = staging + (warp - 2) * (C::PANELS * PANEL_BYTES);
         uint32_t local_tile = 0, panel_it = 0;
-        bool ok = true;
-        for (int unit = pair; unit < num_units && ok; unit += num_pairs, ++local_tile) {
+        // Two accumulator values -> one word of two bf16 (packed conversion).  KIND 0: unit scale and no amax wanted
+        // (every bf16 product of the path); 1: scale; 2: scale and running maximum.
+        auto pack2 = [&](float lo, float hi, auto kind_tag) -> uint32_t {
+            constexpr int KIND = decltype(kind_tag)::value;
+            if (KIND >= 1) {
+                lo = __fmul_rn(lo, scale);
+                hi = __fmul_rn(hi, scale);
+            }
+            const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+            const uint32_t w = *reinterpret_cast<const uint32_t *>(&v);
+            if (KIND == 2) amax2 = __vmaxu2(amax2, w & 0x7fff7fffu);
+            return w;
+        };
+        // 32 columns (as tmem_ld_32cols leaves them) -> 16 packed words, ordered as store_panel takes them
+        auto pack_impl = [&](const uint32_t *r, uint32_t *w, auto kind_tag) {
+            if (OUT_T) {
+#pragma unroll
+                for (int b = 0; b < 4; ++b)            // 8-column blocks
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {      // 8-row blocks
+                        const int i = 16 * (k >> 1) + 4 * b + 2 * (k & 1);
+                        w[4 * b + k] = pack2(__uint_as_float(r[i]), __uint_as_float(r[i + 1]), kind_tag);
+                    }
+            } else {
+#pragma unroll
+                for (int i = 0; i < 16; ++i)
+                    w[i] = pack2(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1]), kind_tag);
+            }
+        };
+        auto pack_chunk = [&](const uint32_t *r, uint32_t *w) {
+            if (kind == 0) pack_impl(r, w, std::integral_constant<int, 0>{});
+            else if (kind == 1) pack_impl(r, w, std::integral_constant<int, 1>{});
+            else pack_impl(r, w, std::integral_constant<int, 2>{});
+        };
+        for (int unit = pair; unit < num_units; unit += num_pairs, ++local_tile) {
             const Unit u = decode(unit);
-            const int tile = u.tile, split = u.split;
             int mt, nt;
-            tile_coords(tile, m_tiles, n_tiles, p.group_m, mt, nt);
+            tile_coords(u.tile, m_tiles, n_tiles, p.group_m, mt, nt);
             const int m0 = mt * 2 * BM + static_cast<int>(rank) * BM;
             const int n0 = nt * BN;
             const uint32_t buf = local_tile % NB, use = local_tile / NB;
             const uint32_t acc_base = lane_base + buf * BN;
-            const uint32_t lead_acc_empty = map_to_cta(acc_empty_bar(buf), 0);
-            if (!epilogue_all(mbar_wait_warp(acc_full_bar(buf), use & 1u, wc))) { ok = false; break; }
+            auto release_acc = [&] {       // this warp has read its rows: count towards the buffer's release
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_cluster(map_to_cta(acc_empty_bar(buf), 0));
+            };
+            if (!mbar_wait_warp(acc_full_bar(buf), use & 1u, wc)) break;
             tc_fence_after();
             if (OUT_F32) {
+                const int m = m0 + quarter * 32 + lane;
 #pragma unroll 1
-                for (int c0 = 0; c0 < BN; c0 += 32) {
+                for (int c0 = 32 * pnl0; c0 < 32 * (pnl0 + n_pnl); c0 += 32) {
                     uint32_t r[32];
                     tmem_ld_32x32(acc_base + c0, r);
                     tmem_ld_wait();
-                    const int m = m0 + row;
                     if (m < p.M && n0 + c0 < p.N) {
                         float v[32];
 #pragma unroll
@@ -571,142 +613,128 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                         }
                     }
                 }
-                tc_fence_before();
-                epilogue_barrier();
-                if (store_thread) mbar_arrive_cluster(lead_acc_empty);
+                release_acc();
                 continue;
             }
-            if (unit >= p.split_from && p.splits > 1) {
-                // Split-K: the unit stores its fp32 partial tile [128][BN]; a second kernel adds the
-                // partials of a tile in split order (bit-reproducible) and writes the bf16 result.
-                // Panels of 32 fp32 columns (128-byte rows, swizzled) go out through the staging buffers and
-                // TMA stores: whole lines instead of 16-byte pieces of 32 different rows per instruction.
-                const int part_row0 =
-                    static_cast<int>(((static_cast<size_t>(tile - p.split_from) * 2 + rank) * p.splits + split) * BM);
-#pragma unroll 1
-                for (int c0 = 0; c0 < BN; c0 += 32) {
-                    if (store_thread) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
-                    epilogue_barrier();
-                    const uint32_t off = (panel_it & 1u) * 16384u;
-                    uint32_t r[32];
-                    tmem_ld_32x32(acc_base + c0, r);
-                    tmem_ld_wait();
-                    uint8_t *dst = staging_generic + off + row * 128;
-#pragma unroll
-                    for (int c = 0; c < 8; ++c)
-                        *reinterpret_cast<uint4 *>(dst + ((c ^ (row & 7)) << 4)) = make_uint4(r[4 * c], r[4 * c + 1], r[4 * c + 2], r[4 * c + 3]);
-                    fence_proxy_async();
-                    epilogue_barrier();
-                    if (store_thread) {
-                        tma_store_2d(&map_p, staging + off, c0, part_row0);
-                        tma_store_commit();
-                    }
-                    ++panel_it;
-                }
-                tc_fence_before();
-                epilogue_barrier();
-                if (store_thread) mbar_arrive_cluster(lead_acc_empty);
-                continue;
-            }
-            // bf16 output in panels of PANEL columns through two 16 KB staging buffers and TMA stores.
-            // 32 accumulator columns -> bf16 -> staging buffer `sb`, columns [c0, c0 + 32) of the panel
-            // Two accumulator values -> one word of two bf16 (packed conversion).  PLAIN: unit scale and no amax
-            // wanted (every bf16 product of the path): no multiply, no maximum.
-            auto pack2 = [&](uint32_t a, uint32_t b, auto plain_tag) -> uint32_t {
-                float lo = __uint_as_float(a), hi = __uint_as_float(b);
-                if (!decltype(plain_tag)::value) {
-                    lo = __fmul_rn(lo, scale);
-                    hi = __fmul_rn(hi, scale);
-                }
-                const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-                const uint32_t w = *reinterpret_cast<const uint32_t *>(&v);
-                if (!decltype(plain_tag)::value) amax2 = __vmaxu2(amax2, w & 0x7fff7fffu);
-                return w;
-            };
-            auto stage_impl = [&](const uint32_t (&r)[32], uint8_t *sb, int c0, auto plain_tag) {
+            // A panel of 32 columns x this warp's 32 rows through one of two 2 KB buffers: 64-byte rows with the 64-byte
+            // swizzle of the TMA store (16-byte chunk index ^= (row >> 1) & 3), which keeps both kinds of store
+            // conflict-free.
+            auto store_panel = [&](int pnl, const uint32_t *w) {
+                const uint32_t sb = my_staging + (C::PANELS == 2 ? (panel_it & 1u) * PANEL_BYTES : 0u);
+                ++panel_it;
+                // the buffer is writable once the store issued from it last has read it
+                if (lane == 0) asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(C::PANELS - 1) : "memory");
+                __syncwarp();
                 if (OUT_T) {
-                    // staging[n][m]: PANEL rows of 128 bf16; a warp writes 32 consecutive m per n
-                    uint16_t *st = reinterpret_cast<uint16_t *>(sb);
+                    // staging row = column n of the accumulator, 32 m; matrix k = rows m 8k .. 8k + 7
 #pragma unroll
-                    for (int c = 0; c < 32; c += 2) {
-                        const uint32_t w = pack2(r[c], r[c + 1], plain_tag);
-                        st[(c0 + c) * BM + row] = static_cast<uint16_t>(w);
-                        st[(c0 + c + 1) * BM + row] = static_cast<uint16_t>(w >> 16);
+                    for (int b = 0; b < 4; ++b) {
+                        const uint32_t n = 8u * b + (lane & 7);
+                        stmatrix_x4_trans(sb + n * 64 + (((lane >> 3) ^ ((n >> 1) & 3)) << 4), w[4 * b], w[4 * b + 1],
+                                          w[4 * b + 2], w[4 * b + 3]);
                     }
                 } else {
-                    // [128 rows][64 bf16] with the 128-byte swizzle of the TMA store: 16-byte chunk index ^= row & 7
-                    uint8_t *dst = sb + row * 128;
-                    const int chunk0 = c0 >> 3;
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        uint32_t w[4];
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) w[e] = pack2(r[8 * c + 2 * e], r[8 * c + 2 * e + 1], plain_tag);
-                        *reinterpret_cast<uint4 *>(dst + (((chunk0 + c) ^ (row & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
-                    }
+                    for (int c = 0; c < 4; ++c)
+                        st_shared_v4(sb + lane * 64 + ((c ^ ((lane >> 1) & 3)) << 4), w[4 * c], w[4 * c + 1], w[4 * c + 2],
+                                     w[4 * c + 3]);
                 }
-            };
-            auto stage_chunk = [&](const uint32_t (&r)[32], uint8_t *sb, int c0) {
-                if (plain) stage_impl(r, sb, c0, std::true_type{});
-                else stage_impl(r, sb, c0, std::false_type{});
-            };
-            // staging buffer of the next panel becomes writable once the store issued two panels ago has read it
-            auto acquire_staging = [&]() -> uint32_t {
-                if (store_thread) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
-                epilogue_barrier();
-                return (panel_it & 1u) * 16384u;
-            };
-            auto store_panel = [&](uint32_t off, int panel) {
                 fence_proxy_async();
-                epilogue_barrier();
-                if (store_thread) {
-                    if (OUT_T) tma_store_2d(&map_d, staging + off, m0, n0 + PANEL * panel);
-                    else tma_store_2d(&map_d, staging + off, n0 + PANEL * panel, m0);
+                __syncwarp();
+                if (lane == 0) {
+                    if (OUT_T) tma_store_2d(&map_d, sb, m0 + 32 * quarter, n0 + 32 * pnl);
+                    else tma_store_2d(&map_d, sb, n0 + 32 * pnl, m0 + 32 * quarter);
                     tma_store_commit();
                 }
-                ++panel_it;
             };
+            if (unit >= p.split_from && p.splits > 1) {
+                // Split-K: every unit of the tile leaves its fp32 partial in the workspace, in the order of its own
+                // registers (512 contiguous bytes per warp and store); the warp whose ticket is the last one adds the
+                // partials of its rows in split order (bit-reproducible) and stores them.  No unit waits for another.
+                constexpr size_t PART = static_cast<size_t>(BN / 4) * 32;          // float4 per 32 rows and split
+                const size_t slot = (static_cast<size_t>(u.tile - p.split_from) * 2 + rank) * p.splits;
+                float4 *part0 = reinterpret_cast<float4 *>(p.partials) + (slot * 4 + quarter) * PART + lane;
+                float4 *mine = part0 + static_cast<size_t>(u.split) * 4 * PART;
 #pragma unroll 1
-            for (int pnl = 0; pnl < DIRECT_PANELS; ++pnl) {
-                const uint32_t off = acquire_staging();
-                uint32_t ra[32], rb[32];
-                tmem_ld_32x32(acc_base + PANEL * pnl, ra);
-                if (PANEL == 64) tmem_ld_32x32(acc_base + PANEL * pnl + 32, rb);
-                tmem_ld_wait();
-                stage_chunk(ra, staging_generic + off, 0);
-                if (PANEL == 64) stage_chunk(rb, staging_generic + off, 32);
-                store_panel(off, pnl);
-            }
-            // last 128 columns -> registers, then the accumulator buffer is free for the next tile
-            uint32_t r0[32], r1[32], r2[32], r3[32];
-            tmem_ld_32x32(acc_base + BN - 128, r0);
-            tmem_ld_32x32(acc_base + BN - 96, r1);
-            tmem_ld_32x32(acc_base + BN - 64, r2);
-            tmem_ld_32x32(acc_base + BN - 32, r3);
-            tmem_ld_wait();
-            tc_fence_before();
-            {
-                const uint32_t off = acquire_staging();      // includes the barrier after everyone's loads
-                if (store_thread) mbar_arrive_cluster(lead_acc_empty);
-                stage_chunk(r0, staging_generic + off, 0);
-                if (PANEL == 64) stage_chunk(r1, staging_generic + off, 32);
-                store_panel(off, DIRECT_PANELS);
-            }
-            if (PANEL == 32) {
-                const uint32_t off = acquire_staging();
-                stage_chunk(r1, staging_generic + off, 0);
-                store_panel(off, DIRECT_PANELS + 1);
-            }
-            {
-                const uint32_t off = acquire_staging();
-                stage_chunk(r2, staging_generic + off, 0);
-                if (PANEL == 64) stage_chunk(r3, staging_generic + off, 32);
-                store_panel(off, DIRECT_PANELS + (PANEL == 64 ? 1 : 2));
-            }
-            if (PANEL == 32) {
-                const uint32_t off = acquire_staging();
-                stage_chunk(r3, staging_generic + off, 0);
-                store_panel(off, DIRECT_PANELS + 3);
+                for (int c0 = 32 * pnl0; c0 < 32 * (pnl0 + n_pnl); c0 += 32) {
+                    uint32_t r[32];
+                    tmem_ld_32cols<OUT_T>(acc_base + c0, r);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int i = 0; i < 8; ++i)
+                        __stcg(mine + (c0 / 4 + i) * 32, make_float4(__uint_as_float(r[4 * i]), __uint_as_float(r[4 * i + 1]),
+                                                                     __uint_as_float(r[4 * i + 2]), __uint_as_float(r[4 * i + 3])));
+                }
+                release_acc();
+                unsigned int last = 0;
+                if (lane == 0) {
+                    unsigned int *ticket = p.tickets + (static_cast<size_t>(u.tile - p.split_from) * 2 + rank) * C::EPI_WARPS + (warp - 2);
+                    __threadfence();                   // the warp's partial before the ticket (ordered by __syncwarp above)
+                    last = (atomicAdd(ticket, 1u) == static_cast<unsigned int>(p.splits) - 1u) ? 1u : 0u;
+                    if (last) *ticket = 0u;            // zero again for the next launch
+                    __threadfence();                   // the ticket before the others' partials
+                }
+                if (!__shfl_sync(0xffffffffu, last, 0)) continue;
+                __syncwarp();
+#pragma unroll 1
+                for (int pnl = pnl0; pnl < pnl0 + n_pnl; ++pnl) {
+                    const float4 *src = part0 + pnl * 8 * 32;
+                    uint32_t v[32], w[16];
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        float4 q[MAX_SPLITS][4];       // all partials of half a panel in flight at once
+#pragma unroll
+                        for (int sp = 0; sp < MAX_SPLITS; ++sp) {
+                            if (sp >= p.splits) break;
+#pragma unroll
+                            for (int i = 0; i < 4; ++i)
+                                q[sp][i] = __ldcg(src + static_cast<size_t>(sp) * 4 * PART + (4 * h + i) * 32);
+                        }
+#pragma unroll
+                        for (int sp = 1; sp < MAX_SPLITS; ++sp) {
+                            if (sp >= p.splits) break;
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) {
+                                q[0][i].x = __fadd_rn(q[0][i].x, q[sp][i].x);
+                                q[0][i].y = __fadd_rn(q[0][i].y, q[sp][i].y);
+                                q[0][i].z = __fadd_rn(q[0][i].z, q[sp][i].z);
+                                q[0][i].w = __fadd_rn(q[0][i].w, q[sp][i].w);
+                            }
+                        }
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            v[16 * h + 4 * i] = __float_as_uint(q[0][i].x);
+                            v[16 * h + 4 * i + 1] = __float_as_uint(q[0][i].y);
+                            v[16 * h + 4 * i + 2] = __float_as_uint(q[0][i].z);
+                            v[16 * h + 4 * i + 3] = __float_as_uint(q[0][i].w);
+                        }
+                    }
+                    pack_chunk(v, w);
+                    store_panel(pnl, w);
+                }
+            } else {
+                // at most four panels are held packed in registers at a time
+                constexpr int HOLD = PANELS_MAX < 4 ? PANELS_MAX : 4;
+                static_assert(PANELS_MAX % HOLD == 0, "whole rounds of panels");
+#pragma unroll
+                for (int h0 = 0; h0 < PANELS_MAX; h0 += HOLD) {
+                    uint32_t pk[16 * HOLD];
+                    const uint32_t cols = acc_base + 32 * (pnl0 + h0);
+#pragma unroll
+                    for (int i = 0; i < HOLD; i += 2) {
+                        uint32_t r[64];
+                        const bool first = h0 + i < n_pnl, second = i + 1 < HOLD && h0 + i + 1 < n_pnl;
+                        if (first) tmem_ld_32cols<OUT_T>(cols + 32 * i, r);
+                        if (second) tmem_ld_32cols<OUT_T>(cols + 32 * i + 32, r + 32);
+                        tmem_ld_wait();
+                        if (first) pack_chunk(r, pk + 16 * i);
+                        if (second) pack_chunk(r + 32, pk + 16 * i + 16);
+                    }
+                    if (h0 + HOLD == PANELS_MAX) release_acc();
+#pragma unroll
+                    for (int i = 0; i < HOLD; ++i)
+                        if (h0 + i < n_pnl) store_panel(pnl0 + h0 + i, pk + 16 * i);
+                }
             }
         }
         if (want_amax) {
@@ -716,72 +744,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             for (int off = 16; off > 0; off >>= 1) best = max(best, __shfl_xor_sync(0xffffffffu, best, off));
             if (lane == 0 && best != 0) atomicMax(p.out_amax, best);
         }
-        if (store_thread && !OUT_F32) tma_store_wait_all();
-    } else if (SPARSE) {
-        // ------------------------------------------------------------ metadata warps (6..9, both CTAs)
-        // HBM -> registers -> tensor memory: lane L of an atom's image is exactly the 16 bytes the
-        // instruction expects in tensor-memory lane L, four 32-bit columns per atom.
-        // The loads run six groups (of four atoms) ahead of the stores, in registers: a group's round trip
-        // to L2 / HBM is then off the path that feeds the MMA warp (with load -> store -> signal in sequence
-        // per group, that latency, not the tensor pipe, set the pace of every sparse product; with three groups
-        // in flight the 8-bit kinds, which consume two atoms per stage, were still paced by it).
-        const int quarter = warp & 3;
-        const uint32_t lane_base = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + C::META_COL0;
-        // loader cursor: (unit, first atom of the next group)
-        int l_unit = pair, l_a0 = 0, l_end = 0;
-        const uint4 *l_src = nullptr;
-        bool l_rows = false;
-        auto l_setup = [&]() {
-            if (l_unit >= num_units) return;
-            const Unit u = decode(l_unit);
-            int mt, nt;
-            tile_coords(u.tile, m_tiles, n_tiles, p.group_m, mt, nt);
-            const int m0 = mt * 2 * BM + static_cast<int>(rank) * BM;
-            l_rows = m0 < p.M;
-            l_src = reinterpret_cast<const uint4 *>(meta + static_cast<size_t>(m0 / BM) * k_atoms * 2048) + quarter * 32 + lane;
-            l_a0 = u.split * u.k_blocks * ATOMS_PER_STAGE;
-            l_end = l_a0 + u.k_blocks * ATOMS_PER_STAGE;
-        };
-        auto l_issue = [&](uint4 (&v)[4]) -> bool {
-            if (l_unit >= num_units) return false;
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-                v[i] = (l_rows && l_a0 + i < k_atoms) ? __ldg(l_src + static_cast<size_t>(l_a0 + i) * 128)
-                                                      : make_uint4(0, 0, 0, 0);
-            l_a0 += 4;
-            if (l_a0 >= l_end) {
-                l_unit += num_pairs;
-                l_setup();
-            }
-            return true;
-        };
-        l_setup();
-        // META_DEPTH groups of loads are in flight per lane (a ring of registers; the loop is unrolled over it):
-        // a group must be on its way for several stages before its turn, or the round trip to L2 paces the warp
-        constexpr int META_DEPTH = 6;
-        uint4 q[META_DEPTH][4];
-        bool have[META_DEPTH];
-#pragma unroll
-        for (int d = 0; d < META_DEPTH; ++d) have[d] = l_issue(q[d]);
-        uint32_t group_it = 0;
-        bool running = true;
-        while (running) {
-#pragma unroll
-            for (int d = 0; d < META_DEPTH; ++d) {
-                if (!running) break;
-                if (!have[d]) { running = false; break; }
-                const uint32_t region = group_it % META_REGIONS;
-                if (!mbar_wait_warp(meta_empty_bar(region), ((group_it / META_REGIONS) & 1u) ^ 1u, wc)) { running = false; break; }
-                tc_fence_after();
-                tmem_st_32x16(lane_base + 16 * region, q[d]);      // one store for the group's four atoms
-                tmem_st_wait();
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive_cluster(map_to_cta(meta_full_bar(region), 0));
-                ++group_it;
-                have[d] = l_issue(q[d]);
-            }
-        }
+        if (lane == 0 && !OUT_F32) tma_store_wait_all();
     } else if (BCOMP) {
         // ------------------------------------------------------------ expander warps (6..9, both CTAs)
         // grad_X = grad_Z S(W) reads S(W) [O, I] as its MN-major B operand.  Here S(W) is given as the forward's
@@ -833,8 +796,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             e_cols = n0 < p.N;
             e_vals = p.b_vals + (static_cast<size_t>(n0 / 2) + seg * (EPU / 2)) * ELT + r0 * row_bytes;
             e_meta = meta + static_cast<size_t>(n0 >> 7) * 2048;
-            e_kb = u.split * u.k_blocks;
-            e_kend = e_kb + u.k_blocks;
+            e_kb = u.kb0;
+            e_kend = u.kb1;
         };
         auto e_issue = [&](uint4 (&v)[UNITS], uint32_t (&m)[UNITS]) -> bool {
             if (e_unit >= num_units) return false;
@@ -938,57 +901,6 @@ bool make_map(const sste_ctx *ctx, CUtensorMap *map, const void *base, int elt, 
               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Split-K second pass over the split tiles: out[m, n] = bf16(scale * sum over splits, in split order, of
-// the fp32 partial tiles [split tile][cta][split][128][bn]).  One thread per 8 consecutive n.
-__global__ void __launch_bounds__(256)
-splitk_reduce_kernel(const float *__restrict__ partials, int M, int N, int bn, int splits, int m_tiles, int n_tiles,
-                     int group_m, int split_from,
-                     int n_split_tiles, const float *__restrict__ a_amax, float a_fp8_max,
-                     const float *__restrict__ b_amax, float b_fp8_max, unsigned int *__restrict__ out_amax,
-                     uint4 *__restrict__ out)
-{
-    sste_pdl_trigger();
-    const int vec_per_row = bn / 8;
-    const size_t vecs = static_cast<size_t>(n_split_tiles) * 2 * BM * vec_per_row;
-    sste_pdl_wait();
-    const float scale = sste_out_scale(a_amax, a_fp8_max, b_amax, b_fp8_max);
-    uint32_t amax2 = 0;
-    for (size_t v = static_cast<size_t>(blockIdx.x) * 256 + threadIdx.x; v < vecs; v += static_cast<size_t>(gridDim.x) * 256) {
-        const int col = static_cast<int>(v % vec_per_row) * 8;
-        const int row = static_cast<int>((v / vec_per_row) % BM);
-        const size_t slot = v / (static_cast<size_t>(vec_per_row) * BM);        // (split tile, cta)
-        const int tile = split_from + static_cast<int>(slot >> 1);
-        int mt, nt;
-        tile_coords(tile, m_tiles, n_tiles, group_m, mt, nt);
-        const int m = mt * 2 * BM + static_cast<int>(slot & 1) * BM + row;
-        const int n = nt * bn + col;
-        if (m >= M || n >= N) continue;
-        const float *src = partials + (slot * splits * BM + row) * bn + col;
-        float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        for (int s = 0; s < splits; ++s) {
-            const float4 a = __ldcg(reinterpret_cast<const float4 *>(src + static_cast<size_t>(s) * BM * bn));
-            const float4 b = __ldcg(reinterpret_cast<const float4 *>(src + static_cast<size_t>(s) * BM * bn) + 1);
-            acc[0] = __fadd_rn(acc[0], a.x); acc[1] = __fadd_rn(acc[1], a.y); acc[2] = __fadd_rn(acc[2], a.z); acc[3] = __fadd_rn(acc[3], a.w);
-            acc[4] = __fadd_rn(acc[4], b.x); acc[5] = __fadd_rn(acc[5], b.y); acc[6] = __fadd_rn(acc[6], b.z); acc[7] = __fadd_rn(acc[7], b.w);
-        }
-        uint32_t w[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-            w[e] = sste_f32_to_bf16_bits(__fmul_rn(acc[2 * e], scale)) | (sste_f32_to_bf16_bits(__fmul_rn(acc[2 * e + 1], scale)) << 16);
-        if (out_amax) {
-#pragma unroll
-            for (int e = 0; e < 4; ++e) amax2 = __vmaxu2(amax2, w[e] & 0x7fff7fffu);
-        }
-        out[(static_cast<size_t>(m) * N + n) / 8] = make_uint4(w[0], w[1], w[2], w[3]);
-    }
-    if (out_amax) {
-        uint32_t best = max(amax2 & 0xffffu, amax2 >> 16) << 16;
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) best = max(best, __shfl_xor_sync(0xffffffffu, best, off));
-        if ((threadIdx.x & 31) == 0 && best != 0) atomicMax(out_amax, best);
-    }
-}
-
 // Runs `fn` once per device ordinal (and again after a failure); thread-safe.
 struct DeviceOnce {
     static constexpr int MAX_DEVICES = 64;
@@ -1025,36 +937,92 @@ int pick_group_m(int m_tiles, int n_tiles, int pairs, double a_tile, double b_ti
     return gm;
 }
 
-struct SplitPlan { int splits, split_from; };
-SplitPlan pick_split_plan(int sm_count, size_t partial_bytes, int tiles, int k_blocks, int align, int bn, double stage_us);
+int g_force_splits = 0;   // test hook: 0 = automatic split-K factor
+int g_force_bn = 0;       // test hook: 0 = automatic tile width
 
-// Everything the host decides about one product launch of a given tile width (the width itself: pick_bn).
-struct LaunchPlan { int splits, split_from, group_m; };
-LaunchPlan make_plan(bool sparse, int elt, int bn, bool out_t, bool out_f32, bool bcomp, int sm_count,
-                     size_t partial_bytes, int M, int N, int K)
+enum Product { FORWARD = 0, GRAD_WEIGHT = 1, GRAD_INPUT = 2 };
+
+// Tile widths a product supports (0 ends the list).  The MN-major B of the two gradient products needs whole 128-byte
+// chunks of N per CTA: 128 columns wide only with 2-byte operands.
+struct Widths { int bn[4]; };
+constexpr Widths widths_of(Product pr, int elt)
 {
-    const int bk = (sparse ? 256 : 128) / elt;
-    const int m_tiles = (M + 2 * BM - 1) / (2 * BM), n_tiles = (N + bn - 1) / bn, tiles = m_tiles * n_tiles;
-    LaunchPlan plan{1, tiles, m_tiles};
-    plan.group_m = pick_group_m(m_tiles, n_tiles, sm_count / 2,
-                                static_cast<double>(K) * (sparse ? 0.5 * elt + 0.125 : 1.0 * elt) * 2 * BM,
-                                static_cast<double>(K) * ((bcomp ? 0.5 : 1.0) * elt) * bn);
-    if (!out_f32 && !out_t) {   // a stage takes about 790 clk (sparse) / 512 clk (dense) at 1.9 GHz
-        const SplitPlan sp = pick_split_plan(sm_count, partial_bytes, tiles, (K + bk - 1) / bk, sparse ? 4 / (bk / 128) : 1,
-                                             bn, sparse ? 0.42 : 0.27);
-        plan.splits = sp.splits;
-        plan.split_from = sp.split_from;
+    return pr == FORWARD ? Widths{{256, 224, 192, 128}} : elt == 2 ? Widths{{256, 128, 0, 0}} : Widths{{256, 0, 0, 0}};
+}
+
+// Microseconds of one stage of the main loop and what a tile costs besides (tensor-memory reads that the next main loop
+// waits for, the output's share of the L2 traffic), all CTA pairs busy; fitted to timings of every width on B200 at
+// K = 768 ... 16384.  A narrower tile moves more operand bytes per flop, a wider one quantises worse into waves.
+struct TileCost { double stage_us, tile_us; };
+constexpr TileCost tile_cost(Product pr, int elt, int bn)
+{
+    if (pr == FORWARD && elt == 2)
+        return bn == 256 ? TileCost{0.50, 1.6} : bn == 224 ? TileCost{0.385, 1.4} : bn == 192 ? TileCost{0.34, 1.25} : TileCost{0.24, 1.3};
+    if (pr == FORWARD)
+        return bn == 256 ? TileCost{0.45, 2.2} : bn == 224 ? TileCost{0.48, 1.4} : bn == 192 ? TileCost{0.43, 0.95} : TileCost{0.34, 0.9};
+    if (pr == GRAD_WEIGHT) return bn == 256 ? TileCost{elt == 2 ? 0.42 : 0.49, 0.5} : TileCost{0.40, 0.5};
+    return bn == 256 ? TileCost{0.33, 0.6} : TileCost{0.28, 0.6};
+}
+
+// Everything the host decides about one product launch.
+struct LaunchPlan { int bn, splits, split_from, group_m; };
+
+// Tile width and split-K factor by the model's time.  Tiles that fill complete waves of CTA pairs are computed whole; the
+// tiles of the last, partial wave (all of them when there are fewer tiles than pairs, as for the weight gradient of a
+// GPT-2-sized layer: 36 tiles, 74 pairs) may be cut into `splits` K ranges of at least eight stages, so that the wave
+// takes 1/splits of a tile time and the partials' round trip through L2 on top: measured 5-17 us, close to
+// bn/256 (5.5 + splits) us of latency + the bytes written and read at 8 MB/us.  Among widths within 3 % the first wins.
+LaunchPlan make_plan(Product pr, int elt, int only_bn, bool out_f32, bool bcomp, int sm_count, size_t partial_bytes, int M,
+                     int N, int K)
+{
+    const bool sparse = (pr != GRAD_INPUT);
+    const int bk = (sparse ? 256 : 128) / elt, k_blocks = (K + bk - 1) / bk, pairs = sm_count / 2;
+    const int m_tiles = (M + 2 * BM - 1) / (2 * BM);
+    const Widths widths = widths_of(pr, elt);
+    int forced = only_bn;
+    for (int bn : widths.bn)
+        if (!forced && bn && bn == g_force_bn) forced = bn;
+    LaunchPlan best{0, 1, 0, m_tiles};
+    double best_us = 0.0;
+    for (int bn : widths.bn) {
+        if (!bn || (forced && bn != forced)) continue;
+        const int tiles = m_tiles * ((N + bn - 1) / bn);
+        const int whole = tiles / pairs * pairs, tail = tiles - whole;
+        const TileCost c = tile_cost(pr, elt, bn);
+        const double whole_us = (whole / pairs) * (k_blocks * c.stage_us + c.tile_us);
+        for (int s = 1; s <= MAX_SPLITS; ++s) {
+            double us = whole_us;
+            if (s > 1) {
+                // behind whole waves equal ranges only (an uneven split gains less than the exchange costs there)
+                if (out_f32 || tail == 0 || k_blocks / s < 8 || (whole > 0 && k_blocks % s != 0)) continue;
+                if (tail * 16 > SSTE_SPLITK_TICKETS) continue;
+                const size_t bytes = static_cast<size_t>(tail) * s * 2 * BM * bn * sizeof(float);
+                if (bytes > partial_bytes) continue;
+                us += bn / 256.0 * (5.5 + s) + 2.0 * bytes / 8e6;
+            }
+            if (tail) us += ((tail * s + pairs - 1) / pairs) * ((k_blocks + s - 1) / s * c.stage_us + c.tile_us);
+            const bool wanted = (g_force_splits == s && best.bn == bn);      // the hook applies where the shape allows it
+            if (!best.bn || us < best_us * (best.bn == bn ? 1.0 : 0.97) || wanted) {
+                if (g_force_splits && best.bn == bn && best.splits == g_force_splits) continue;
+                best = LaunchPlan{bn, s, s > 1 ? whole : tiles, m_tiles};
+                best_us = us;
+            }
+            if (g_force_splits == 1) break;
+        }
     }
-    return plan;
+    const int n_tiles = (N + best.bn - 1) / best.bn;
+    best.group_m = pick_group_m(m_tiles, n_tiles, pairs, static_cast<double>(K) * (sparse ? 0.5 * elt + 0.125 : 1.0 * elt) * 2 * BM,
+                                static_cast<double>(K) * ((bcomp ? 0.5 : 1.0) * elt) * best.bn);
+    return best;
 }
 
 template <bool SPARSE, BMajor BMAJ, int ELT, int BN, bool OUT_T, bool OUT_F32, bool BCOMP = false>
 sste_status launch(const sste_ctx *ctx, const void *A, const void *B, const void *meta, const GemmParams &p,
-                   cudaStream_t stream)
+                   const LaunchPlan &plan, cudaStream_t stream)
 {
-    using C = Cfg<SPARSE, BN, BCOMP>;
+    using C = Cfg<SPARSE, ELT, BN, BCOMP>;
     constexpr int BK = (SPARSE ? 256 : 128) / ELT;
-    CUtensorMap map_a, map_b, map_d, map_p;
+    CUtensorMap map_a, map_b, map_d, map_m;
     bool ok;
     if (SPARSE)   // compressed values [M, K/2]: 128 bytes per row per stage
         ok = make_map(ctx, &map_a, A, ELT, p.M, p.K / 2, BK / 2, BM, CU_TENSOR_MAP_SWIZZLE_128B);
@@ -1068,11 +1036,16 @@ sste_status launch(const sste_ctx *ctx, const void *A, const void *B, const void
         ok = ok && make_map(ctx, &map_b, B, ELT, p.K, p.N, 128 / ELT, BK, CU_TENSOR_MAP_SWIZZLE_128B);
     if (OUT_F32) {
         map_d = map_a;       // unused: the fp32 epilogue stores directly
-    } else if (OUT_T) {      // out[N, M] bf16: panels of 128 m x 64 (or 32) n
-        ok = ok && make_map(ctx, &map_d, p.D, 2, p.N, p.M, BM, C::PANEL, CU_TENSOR_MAP_SWIZZLE_NONE);
-    } else {                 // out[M, N] bf16: panels of 64 n x 128 m, 128-byte swizzle
-        ok = ok && make_map(ctx, &map_d, p.D, 2, p.M, p.N, 64, BM, CU_TENSOR_MAP_SWIZZLE_128B);
+    } else if (OUT_T) {      // out[N, M] bf16: panels of 32 m x 32 n, 64-byte swizzle
+        ok = ok && make_map(ctx, &map_d, p.D, 2, p.N, p.M, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B);
+    } else {                 // out[M, N] bf16: panels of 32 n x 32 m, 64-byte swizzle
+        ok = ok && make_map(ctx, &map_d, p.D, 2, p.M, p.N, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B);
     }
+    if (SPARSE)              // metadata image as rows of 512 bytes, four per atom
+        ok = ok && make_map(ctx, &map_m, meta, 4, static_cast<uint64_t>(p.M / 128) * (p.K / 128) * 4, 128, 128, 4 * C::ATOMS,
+                            CU_TENSOR_MAP_SWIZZLE_NONE);
+    else
+        map_m = map_a;       // unused
     if (!ok) return SSTE_ERR_CUDA;
     auto kern = gemm_kernel<SPARSE, BMAJ, ELT, BN, OUT_T, OUT_F32, BCOMP>;
     // The opt-in to more than 48 KB of dynamic shared memory is a per-DEVICE attribute of the kernel:
@@ -1096,94 +1069,20 @@ sste_status launch(const sste_ctx *ctx, const void *A, const void *B, const void
     if (BCOMP) pp.b_vals = static_cast<const uint8_t *>(B);
     if (pp.out_amax && cudaMemsetAsync(pp.out_amax, 0, sizeof(unsigned int), stream) != cudaSuccess) return SSTE_ERR_CUDA;
     const int tiles = m_tiles * n_tiles;
-    const LaunchPlan plan = make_plan(SPARSE, ELT, BN, OUT_T, OUT_F32, BCOMP, ctx->sm_count,
-                                      ctx->splitk_partials ? ctx->splitk_partial_bytes : 0, p.M, p.N, p.K);
     pp.group_m = plan.group_m;
     pp.splits = plan.splits;
     pp.split_from = plan.split_from;
     pp.partials = ctx->splitk_partials;
+    pp.tickets = ctx->splitk_tickets;
     const int n_split_tiles = tiles - pp.split_from;
     int pairs = pp.split_from + n_split_tiles * pp.splits;
     if (pairs > ctx->sm_count / 2) pairs = ctx->sm_count / 2;
-    map_p = map_a;   // unused without split-K
-    if (pp.splits > 1 &&
-        !make_map(ctx, &map_p, pp.partials, 4, static_cast<uint64_t>(n_split_tiles) * 2 * pp.splits * BM, BN, 32, BM,
-                  CU_TENSOR_MAP_SWIZZLE_128B))
-        return SSTE_ERR_CUDA;
-    if (sste_launch(kern, dim3(2 * pairs), dim3(C::THREADS), C::SMEM_BYTES, stream, map_a, map_b, map_d, map_p,
+    if (sste_launch(kern, dim3(2 * pairs), dim3(C::THREADS), C::SMEM_BYTES, stream, map_a, map_b, map_d, map_m,
                     static_cast<const uint8_t *>(meta), pp) != cudaSuccess)
         return SSTE_ERR_CUDA;
-    if (pp.splits > 1) {
-        const size_t vecs = static_cast<size_t>(n_split_tiles) * 2 * BM * (BN / 8);
-        size_t blocks = (vecs + 255) / 256;
-        if (blocks > static_cast<size_t>(ctx->sm_count) * 16) blocks = static_cast<size_t>(ctx->sm_count) * 16;
-        if (sste_launch(splitk_reduce_kernel, dim3(static_cast<unsigned int>(blocks)), dim3(256), 0, stream,
-                        pp.partials, p.M, p.N, BN, pp.splits, m_tiles, n_tiles, pp.group_m, pp.split_from, n_split_tiles, p.a_amax,
-                        p.a_fp8_max, p.b_amax, p.b_fp8_max, pp.out_amax, static_cast<uint4 *>(p.D)) != cudaSuccess)
-            return SSTE_ERR_CUDA;
-    }
     if (cudaGetLastError() != cudaSuccess) return SSTE_ERR_CUDA;
-    sste_count_launches(pp.splits > 1 ? 2 : 1);
+    sste_count_launches(1);
     return SSTE_OK;
-}
-
-int g_force_splits = 0;   // test hook: 0 = automatic split-K factor
-
-
-// Split-K plan.  Tiles that fill complete waves of CTA pairs are computed whole; the tiles of the last,
-// partial wave (all of them when there are fewer tiles than pairs, as for the weight gradient of a
-// GPT-2-sized layer: 36 tiles, 74 pairs) are cut into `splits` K ranges so that the wave takes 1/splits
-// of a tile time.  `align` = stages per metadata group (K ranges must start on a group boundary).
-SplitPlan pick_split_plan(int sm_count, size_t partial_bytes, int tiles, int k_blocks, int align, int bn, double stage_us)
-{
-    SplitPlan none{1, tiles};
-    if (partial_bytes == 0) return none;
-    const int pairs = sm_count / 2;
-    const int whole = (tiles / pairs) * pairs;
-    const int tail = tiles - whole;
-    if (tail == 0) return none;
-    int best = 1;
-    const double tile_us = k_blocks * stage_us;
-    double best_cost = tile_us;        // time of the last wave, microseconds
-    for (int s = 2; s <= 4; ++s) {
-        if (k_blocks % (s * align) != 0 || k_blocks / s < 8) continue;
-        if (static_cast<size_t>(tail) * 2 * s * BM * bn * sizeof(float) > partial_bytes) continue;
-        if (g_force_splits == s) return SplitPlan{s, whole};
-        const int waves = (tail * s + pairs - 1) / pairs;
-        // + the second pass (a launch of its own) and the partial tiles' round trip through L2
-        const double cost = tile_us * waves / s + 4.0 + 0.3 * s;
-        if (cost < best_cost - 1e-9) { best = s; best_cost = cost; }
-    }
-    if (g_force_splits == 1 || best == 1) return none;
-    return SplitPlan{best, whole};
-}
-
-// Tile width of the forward (K-major B), from timings on B200 over the GPT-2- and 7B-shaped layers.
-// bf16: the time of a tile is close to  K * bn * k(bn) + f(bn)  microseconds with
-//   bn = 192: k = 1.93e-5, f = 0.4;   224: k = 1.83e-5, f = 0.5;   256: k = 1.52e-5, f = 1.7
-// (wider tiles stream less B per flop; the 256-wide tile has one accumulator, so its epilogue is exposed), and
-// the launch takes ceil(tiles / pairs) such tile times: the width with the smallest product wins, which is
-// mostly a matter of how the tile count quantises into waves.  FP8: 256 columns unless they quantise badly.
-int pick_bn(bool b_k_major, int elt, int M, int N, int K, int pairs)
-{
-    if (!b_k_major) return 256;
-    const long m_tiles = (M + 2 * BM - 1) / (2 * BM);
-    auto waves = [&](int bn) { return (m_tiles * ((N + bn - 1) / bn) + pairs - 1) / pairs; };
-    if (elt == 2) {
-        const int widths[3] = {224, 192, 256};
-        const double k[3] = {1.83e-5, 1.93e-5, 1.52e-5}, f[3] = {0.5, 0.4, 1.7};
-        int best = 0;
-        double best_cost = 0.0;
-        for (int i = 0; i < 3; ++i) {
-            const double cost = static_cast<double>(waves(widths[i])) * (static_cast<double>(K) * widths[i] * k[i] + f[i]);
-            if (i == 0 || cost < best_cost * 0.995) { best = i; best_cost = cost; }
-        }
-        return widths[best];
-    }
-    if (K <= 1024) return 192;
-    // Longer reductions: 256 columns unless the tile count quantises badly; a 192-wide tile costs about 8 %
-    // more per flop (measured at many waves).
-    return (waves(192) * 192 * 108 < waves(256) * 256 * 100) ? 192 : 256;
 }
 
 bool fmt_code(sste_dtype dt, int *elt, uint32_t *code)
@@ -1196,34 +1095,25 @@ bool fmt_code(sste_dtype dt, int *elt, uint32_t *code)
     }
 }
 
-int g_force_bn = 0;   // test hook: 0 = automatic tile width
-
 // Dispatch on tile width and output dtype.  fp32 output (a test / debug path) always uses 256-wide tiles.
-template <bool SPARSE, BMajor BMAJ, int ELT, bool OUT_T>
+template <Product PR, int ELT>
 sste_status launch_out(const sste_ctx *ctx, const void *A, const void *B, const void *meta, const GemmParams &p,
                        sste_dtype odt, cudaStream_t s)
 {
-    if (odt == SSTE_F32) return launch<SPARSE, BMAJ, ELT, 256, OUT_T, true>(ctx, A, B, meta, p, s);
-    if (odt != SSTE_BF16) return SSTE_ERR_DTYPE;
-    constexpr bool MN = (BMAJ == BMajor::MN);
-    int cands[4], n = 0;
-    cands[n++] = 256;
-    if (!(MN && ELT == 1)) cands[n++] = 128;   // MN-major B: each CTA needs whole 128-byte chunks of N
-    if (!MN) cands[n++] = 192;
-    if (!MN && SPARSE && OUT_T) cands[n++] = 224;
-    int bn = pick_bn(!MN, ELT, p.M, p.N, p.K, ctx->sm_count / 2);
-    for (int i = 0; i < n; ++i)
-        if (cands[i] == g_force_bn) bn = g_force_bn;
-    if constexpr (!MN && SPARSE && OUT_T) {
-        if (bn == 224) return launch<SPARSE, BMAJ, ELT, 224, OUT_T, false>(ctx, A, B, meta, p, s);
+    constexpr bool SPARSE = (PR != GRAD_INPUT), OUT_T = (PR == FORWARD);
+    constexpr BMajor BMAJ = (PR == FORWARD) ? BMajor::K : BMajor::MN;
+    if (odt != SSTE_F32 && odt != SSTE_BF16) return SSTE_ERR_DTYPE;
+    const LaunchPlan plan = make_plan(PR, ELT, odt == SSTE_F32 ? 256 : 0, odt == SSTE_F32, false, ctx->sm_count,
+                                      ctx->splitk_partials ? ctx->splitk_partial_bytes : 0, p.M, p.N, p.K);
+    if (odt == SSTE_F32) return launch<SPARSE, BMAJ, ELT, 256, OUT_T, true>(ctx, A, B, meta, p, plan, s);
+    if constexpr (PR == FORWARD) {
+        if (plan.bn == 224) return launch<SPARSE, BMAJ, ELT, 224, OUT_T, false>(ctx, A, B, meta, p, plan, s);
+        if (plan.bn == 192) return launch<SPARSE, BMAJ, ELT, 192, OUT_T, false>(ctx, A, B, meta, p, plan, s);
     }
-    if constexpr (!MN) {
-        if (bn == 192) return launch<SPARSE, BMAJ, ELT, 192, OUT_T, false>(ctx, A, B, meta, p, s);
+    if constexpr (PR == FORWARD || ELT == 2) {
+        if (plan.bn == 128) return launch<SPARSE, BMAJ, ELT, 128, OUT_T, false>(ctx, A, B, meta, p, plan, s);
     }
-    if constexpr (!(MN && ELT == 1)) {
-        if (bn == 128) return launch<SPARSE, BMAJ, ELT, 128, OUT_T, false>(ctx, A, B, meta, p, s);
-    }
-    return launch<SPARSE, BMAJ, ELT, 256, OUT_T, false>(ctx, A, B, meta, p, s);
+    return launch<SPARSE, BMAJ, ELT, 256, OUT_T, false>(ctx, A, B, meta, p, plan, s);
 }
 
 // FP8 operands come with the amax of the tensors they were quantised from (both or neither); bf16 with none.
@@ -1250,15 +1140,10 @@ extern "C" sste_status sste_debug_plan(int product, sste_dtype opdt, int O, int 
     if (!sste_mult128(T) || !sste_mult128(O) || !sste_mult128(I)) return SSTE_ERR_SHAPE;
     // the (M, N, K) of the launch, as in the three entry points below
     const int M = product == 2 ? T : O, N = product == 0 ? T : I, K = product == 0 ? I : product == 1 ? T : O;
-    const bool sparse = product != 2, mn = product != 0, out_t = product == 0;
-    int bn = pick_bn(!mn, elt, M, N, K, sm_count / 2);
-    const int cands[4] = {256, (mn && elt == 1) ? 0 : 128, mn ? 0 : 192, (!mn && sparse) ? 224 : 0};
-    for (int c : cands)
-        if (c && c == g_force_bn) bn = c;
     const size_t partial_bytes =
         workspace_bytes > SSTE_WS_SPLITK_PARTIALS_OFF + (size_t(1) << 20) ? workspace_bytes - SSTE_WS_SPLITK_PARTIALS_OFF : 0;
-    const LaunchPlan plan = make_plan(sparse, elt, bn, out_t, false, false, sm_count, partial_bytes, M, N, K);
-    if (tile_width) *tile_width = bn;
+    const LaunchPlan plan = make_plan(static_cast<Product>(product), elt, 0, false, false, sm_count, partial_bytes, M, N, K);
+    if (tile_width) *tile_width = plan.bn;
     if (splits) *splits = plan.splits;
     if (split_from) *split_from = plan.split_from;
     if (group_m) *group_m = plan.group_m;
@@ -1327,8 +1212,8 @@ extern "C" sste_status sste_linear_fwd(sste_ctx *ctx, const void *X, int T, cons
     GemmParams p{O, T, I, Y, w_amax_dev, x_amax_dev, sste_fp8_max(opdt), sste_fp8_max(opdt),
                  reinterpret_cast<unsigned int *>(y_amax_out_dev), ctx->status_dev, code, code, nullptr};
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (elt == 2) return launch_out<true, BMajor::K, 2, true>(ctx, vals, X, meta, p, ydt, s);
-    return launch_out<true, BMajor::K, 1, true>(ctx, vals, X, meta, p, ydt, s);
+    if (elt == 2) return launch_out<FORWARD, 2>(ctx, vals, X, meta, p, ydt, s);
+    return launch_out<FORWARD, 1>(ctx, vals, X, meta, p, ydt, s);
 }
 
 extern "C" sste_status sste_linear_bwd_weight(sste_ctx *ctx, const void *gvals, const void *gmeta, int O, int T,
@@ -1352,8 +1237,8 @@ extern "C" sste_status sste_linear_bwd_weight(sste_ctx *ctx, const void *gvals, 
     GemmParams p{O, I, T, dW, g_amax_dev, x_amax_dev, sste_fp8_max(gdt), sste_fp8_max(xdt), nullptr,
                  ctx->status_dev, ca, cb, nullptr};
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (ea == 2) return launch_out<true, BMajor::MN, 2, false>(ctx, gvals, X, gmeta, p, dwdt, s);
-    return launch_out<true, BMajor::MN, 1, false>(ctx, gvals, X, gmeta, p, dwdt, s);
+    if (ea == 2) return launch_out<GRAD_WEIGHT, 2>(ctx, gvals, X, gmeta, p, dwdt, s);
+    return launch_out<GRAD_WEIGHT, 1>(ctx, gvals, X, gmeta, p, dwdt, s);
 }
 
 extern "C" sste_status sste_linear_bwd_input(sste_ctx *ctx, const void *dY, int T, int O, sste_dtype gdt,
@@ -1382,12 +1267,14 @@ extern "C" sste_status sste_linear_bwd_input(sste_ctx *ctx, const void *dY, int 
     if (!Wt_dense) {
         // S(W) from the forward's compressed operand, expanded in shared memory (256-wide tiles)
         const bool f32 = (xdt == SSTE_F32);
+        const LaunchPlan plan = make_plan(GRAD_INPUT, ea, 256, f32, true, ctx->sm_count,
+                                          ctx->splitk_partials ? ctx->splitk_partial_bytes : 0, p.M, p.N, p.K);
         if (ea == 2)
-            return f32 ? launch<false, BMajor::MN, 2, 256, false, true, true>(ctx, dY, vals, meta, p, s)
-                       : launch<false, BMajor::MN, 2, 256, false, false, true>(ctx, dY, vals, meta, p, s);
-        return f32 ? launch<false, BMajor::MN, 1, 256, false, true, true>(ctx, dY, vals, meta, p, s)
-                   : launch<false, BMajor::MN, 1, 256, false, false, true>(ctx, dY, vals, meta, p, s);
+            return f32 ? launch<false, BMajor::MN, 2, 256, false, true, true>(ctx, dY, vals, meta, p, plan, s)
+                       : launch<false, BMajor::MN, 2, 256, false, false, true>(ctx, dY, vals, meta, p, plan, s);
+        return f32 ? launch<false, BMajor::MN, 1, 256, false, true, true>(ctx, dY, vals, meta, p, plan, s)
+                   : launch<false, BMajor::MN, 1, 256, false, false, true>(ctx, dY, vals, meta, p, plan, s);
     }
-    if (ea == 2) return launch_out<false, BMajor::MN, 2, false>(ctx, dY, Wt_dense, nullptr, p, xdt, s);
-    return launch_out<false, BMajor::MN, 1, false>(ctx, dY, Wt_dense, nullptr, p, xdt, s);
+    if (ea == 2) return launch_out<GRAD_INPUT, 2>(ctx, dY, Wt_dense, nullptr, p, xdt, s);
+    return launch_out<GRAD_INPUT, 1>(ctx, dY, Wt_dense, nullptr, p, xdt, s);
 }
