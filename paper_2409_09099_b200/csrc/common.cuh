@@ -7,6 +7,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <mutex>
+
 #include "sste.h"
 
 // The context owns nothing but views into the caller's workspace.
@@ -55,6 +57,21 @@ struct sste_device_guard {
     ~sste_device_guard()
     {
         if (prev >= 0) cudaSetDevice(prev);
+    }
+};
+
+// Runs `fn` once per device ordinal (and again after a failure); thread-safe.
+struct DeviceOnce {
+    static constexpr int MAX_DEVICES = 64;
+    std::mutex mu;
+    bool done[MAX_DEVICES] = {};
+    template <typename F>
+    bool run(int device, F fn)
+    {
+        if (device < 0 || device >= MAX_DEVICES) return fn();
+        std::lock_guard<std::mutex> lock(mu);
+        if (!done[device]) done[device] = fn();
+        return done[device];
     }
 };
 

@@ -255,19 +255,111 @@ __device__ __forceinline__ void philox4x32_10(uint32_t c0, uint32_t c1, uint32_t
     out[0] = c0; out[1] = c1; out[2] = c2; out[3] = c3;
 }
 
-// ---------------------------------------------------------------- MVUE of one group
+// ---------------------------------------------------------------- MVUE of two groups
 
-// a <= b as an integer mask (all ones / zero) in one instruction
-__device__ __forceinline__ int fset_le(float a, float b)
+// Two fp32 values in one register pair: one instruction per operation for both (sm_100 f32x2), each lane a single
+// rounded operation, subnormals included.
+using f32x2 = unsigned long long;
+// byte permute with the selector as the instruction takes it (four nibbles in the low half)
+__device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel)
 {
-    int r;
-    asm("set.le.s32.f32 %0, %1, %2;" : "=r"(r) : "f"(a), "f"(b));
+    uint32_t r;
+    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(sel));
     return r;
 }
+__device__ __forceinline__ f32x2 pack2(float lo, float hi)
+{
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float &lo, float &hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
+{
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f32x2 both(float v) { return pack2(v, v); }
+// a <= b, a >= b as 1.0f / 0.0f (0 if either is a NaN), one instruction
+__device__ __forceinline__ float one_if_le(float a, float b)
+{
+    float r;
+    asm("set.le.f32.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 one_if_le2(f32x2 a, f32x2 b)
+{
+    float a0, a1, b0, b1;
+    unpack2(a, a0, a1);
+    unpack2(b, b0, b1);
+    return pack2(one_if_le(a0, b0), one_if_le(a1, b1));
+}
 
-struct MvueGroup {
-    uint32_t q0, q1;  // kept positions q0 < q1
-    float v0, v1;     // their values before the cast
+// What a group's draw comes to, by table: the kept positions q0 < q1 and how to pick their bits.
+//   x: byte-permute selector over (a0 a1 | a2 a3) for the two kept elements | (q0 | q1 << 2) << 16
+//      (bf16: both halfwords; FP8: the two upper bytes, which carry the signs)
+//   y: bf16: which bits of the kept halfwords stay (the rest comes from bf16(h)); FP8: selector of the two result bytes
+//      among (e5m2(h), e5m2(max)) | mask of the sign bits to keep << 16
+// Entry numbers: unclipped j1 + 4 n2 (counts of cumulative sums at or below the two points); clipped
+// MVUE_CLIP + j + 4 x with x the maximum's position and j the other's; clipped with no other nonzero element
+// MVUE_CLIP + 4 (x - 3).  (j = x never happens, so the two clipped ranges share one unused number.)
+constexpr int MVUE_CLIP = 28, MVUE_ENTRIES = MVUE_CLIP + 16;
+struct MvueTable { uint2 e[MVUE_ENTRIES]; };
+constexpr uint2 mvue_entry(bool FP8, int n)
+{
+    int q0 = 0, q1 = 0, x = -1;    // x: the kept position that keeps its own value
+    bool zero = false;             // the other kept value is +0
+    if (n < 16) {
+        const int j1 = n & 3, n2 = n >> 2;
+        q0 = j1 < 2 ? j1 : 2;
+        q1 = j1 + 1 > n2 ? j1 + 1 : n2;
+        q1 = q1 < 3 ? q1 : 3;
+    } else {
+        zero = n < MVUE_CLIP || n == MVUE_CLIP;
+        x = zero ? (n - MVUE_CLIP) / 4 + 3 : (n - MVUE_CLIP) >> 2;
+        const int j = zero ? (x == 0 ? 1 : 0) : (n - MVUE_CLIP) & 3;
+        q0 = x < j ? x : j;
+        q1 = x < j ? j : x;
+    }
+    uint2 e{0, 0};
+    const uint32_t nib = static_cast<uint32_t>(q0 | (q1 << 2)) << 16;
+    if (FP8) {
+        e.x = static_cast<uint32_t>((2 * q0 + 1) | ((2 * q1 + 1) << 4)) | nib;
+        const uint32_t s0 = (zero && q0 != x) ? 0u : 0x80u, s1 = (zero && q1 != x) ? 0u : 0x8000u;
+        e.y = (q0 == x ? 0x01u : 0u) | (q1 == x ? 0x10u : 0u) | ((s0 | s1) << 16);
+    } else {
+        e.x = 0x1010u + 0x22u * q0 + 0x2200u * q1 + nib;
+        const uint32_t s0 = q0 == x ? 0xffffu : zero ? 0u : 0x8000u, s1 = q1 == x ? 0xffffu : zero ? 0u : 0x8000u;
+        e.y = s0 | (s1 << 16);
+    }
+    return e;
+}
+constexpr MvueTable mvue_table(bool FP8)
+{
+    MvueTable t{};
+    for (int n = 16; n < MVUE_ENTRIES; ++n) t.e[n] = (n < MVUE_CLIP && n % 4) ? uint2{0, 0} : mvue_entry(FP8, n);   // 17..27: multiples of 4 only
+    for (int n = 0; n < 16; ++n) t.e[n] = mvue_entry(FP8, n);
+    return t;
+}
+__device__ const MvueTable mvue_table_bf16 = mvue_table(false), mvue_table_fp8 = mvue_table(true);
+
+struct MvuePair {
+    uint2 e0, e1;     // table entries of the two groups
+    f32x2 h;          // magnitude of a kept value other than a clipped maximum
+    f32x2 mx;         // largest magnitude
 };
 
 // Inclusion probabilities p_i = min(1, c |a_i|) with sum 2, kept values a_i / p_i, systematic sampling
@@ -277,63 +369,72 @@ struct MvueGroup {
 //                            sign(a_j)*rest;
 //   unclipped (m_x <  rest): the points u*S/2 and u*S/2 + S/2 on the cumulative sums pick two elements,
 //                            both carry sign(a_j)*S/2.
-// The kernel is bound by instruction issue, not by HBM, so this is written for instruction count: no
-// branches, one-hot predicates, compares counted as 0 / -1 masks, and the two kept inputs picked by a byte
-// permute of the packed bf16 pairs p01 = a0 | a1 << 16, p23 = a2 | a3 << 16 (only their sign, or for the
-// clipped maximum their 16 bits, is needed).  Every fp32 step is a single rounded operation.
-__device__ __forceinline__ MvueGroup mvue_group(uint32_t p01, uint32_t p23, float u)
+// Two groups at a time: w[i] holds token i's bf16 values of the columns in its halves.  The kernel is bound by instruction
+// issue (half-rate integer / compare pipe first), not by HBM, so the rule is written for that: sums and selections are
+// f32x2 arithmetic on the FMA pipe (a selection is a multiply by an exact 0 or 1), comparisons give 1.0 / 0.0, their
+// counts are added up as subnormal floats whose bit pattern IS the byte offset of the table entry that holds the kept
+// pair.  118 -> about 70 issued instructions per group, of them about 31 (from 78) on the half-rate pipe.  No branches;
+// every fp32 step is a single rounded operation in the oracle's order.
+__device__ __forceinline__ MvuePair mvue_pair(const uint32_t (&w)[4], uint32_t k_lo, uint32_t k_hi, const uint8_t *lut)
 {
-    const float a0 = __uint_as_float(p01 << 16), a1 = __uint_as_float(p01 & 0xffff0000u);
-    const float a2 = __uint_as_float(p23 << 16), a3 = __uint_as_float(p23 & 0xffff0000u);
-    const float m0 = fabsf(a0), m1 = fabsf(a1), m2 = fabsf(a2), m3 = fabsf(a3);
-    const float mx = fmaxf(fmaxf(m0, m1), fmaxf(m2, m3));
-    const bool e0 = (m0 == mx);
-    const bool e1 = !e0 && (m1 == mx);
-    const bool e2 = !e0 && !e1 && (m2 == mx);
-    const bool e3 = !e0 && !e1 && !e2;
-    const uint32_t xi = e0 ? 0u : e1 ? 1u : e2 ? 2u : 3u;
-    // cumulative sums without x (adding +0 is exact) and with it
-    const float z0 = e0 ? 0.0f : m0;
-    const float z1 = __fadd_rn(z0, e1 ? 0.0f : m1);
-    const float z2 = __fadd_rn(z1, e2 ? 0.0f : m2);
-    const float rest = __fadd_rn(z2, e3 ? 0.0f : m3);
-    const float s1 = __fadd_rn(m0, m1);
-    const float s2 = __fadd_rn(s1, m2);
-    const float s3 = __fadd_rn(s2, m3);
-    const bool clipped = (mx >= rest);
-    const float h = clipped ? rest : __fmul_rn(0.5f, s3);
-    const float c0 = clipped ? z0 : m0, c1 = clipped ? z1 : s1, c2 = clipped ? z2 : s2;
-    const float r1 = __fmul_rn(u, h);
-    const float r2 = __fadd_rn(r1, h);
-    // Clipped: a point that rounding put AT rest (possible only when u * rest is subnormal) counts as just below
-    // it, which selects the last other element of nonzero magnitude.  (rest == 0: the second operand is a NaN and
-    // fminf returns r1; that case is decided below.)
-    const float r1c = clipped ? fminf(r1, __uint_as_float(__float_as_uint(rest) - 1u)) : r1;
-    // number of cumulative sums at or below each point: compares as 0 / -1, one three-input add each
-    const int j1 = -(fset_le(c0, r1c) + fset_le(c1, r1c) + fset_le(c2, r1c));
-    const int n2 = -(fset_le(c0, r2) + fset_le(c1, r2) + fset_le(c2, r2));
-    // index pair before ordering: (other, x) when clipped; (j1, j2) otherwise, where a first point in the
-    // last element (j1 = 3) gives the pair (2, 3)
-    const int ia_c = (rest == 0.0f) ? (e0 ? 1 : 0) : j1;
-    const int ia_u = min(j1, 2);
-    const int ib_u = min(max(j1 + 1, n2), 3);
-    const uint32_t ia = static_cast<uint32_t>(clipped ? ia_c : ia_u);
-    const uint32_t ib = clipped ? xi : static_cast<uint32_t>(ib_u);
-    // bf16 bits of a_ia and a_ib in the upper half (lower half: don't care)
-    const uint32_t sa = __byte_perm(p01, p23, ia * 0x2200u + 0x1000u);
-    const uint32_t sb = __byte_perm(p01, p23, ib * 0x2200u + 0x1000u);
-    // kept values sign(a_i) * h; a zero h yields +0; the clipped maximum keeps its own value
-    const uint32_t hb = __float_as_uint(h);
-    const uint32_t sgn = (hb == 0u) ? 0u : 0x80000000u;
-    const float va = __uint_as_float((sa & sgn) | hb);
-    const float vb = __uint_as_float(clipped ? (sb & 0xffff0000u) : ((sb & sgn) | hb));
-    MvueGroup r;
-    const bool swap = ia > ib;
-    r.q0 = min(ia, ib);
-    r.q1 = max(ia, ib);
-    r.v0 = swap ? vb : va;
-    r.v1 = swap ? va : vb;
-    return r;
+    float lo[4], hi[4];
+    f32x2 m[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const uint32_t mm = w[i] & 0x7fff7fffu;
+        lo[i] = __uint_as_float(mm << 16);
+        hi[i] = __uint_as_float(mm & 0xffff0000u);
+        m[i] = pack2(lo[i], hi[i]);
+    }
+    // running maxima; X_i = 1 where the first largest magnitude is at or before position i
+    const float l1 = fmaxf(lo[0], lo[1]), h1 = fmaxf(hi[0], hi[1]);
+    const float l2 = fmaxf(l1, lo[2]), h2 = fmaxf(h1, hi[2]);
+    const float lx = fmaxf(l2, lo[3]), hx = fmaxf(h2, hi[3]);
+    const f32x2 mx = pack2(lx, hx);
+    const f32x2 X0 = pack2(one_if_le(lx, lo[0]), one_if_le(hx, hi[0]));
+    const f32x2 X1 = pack2(one_if_le(lx, l1), one_if_le(hx, h1));
+    const f32x2 X2 = pack2(one_if_le(lx, l2), one_if_le(hx, h2));
+    const f32x2 minus1 = both(-1.0f);
+    // -1 at the maximum's position, 0 elsewhere
+    const f32x2 E0 = mul2(X0, minus1), E1 = fma2(X1, minus1, X0), E2 = fma2(X2, minus1, X1), E3 = add2(X2, minus1);
+    // sums without the maximum and with it
+    const f32x2 rest = add2(add2(add2(fma2(E0, mx, m[0]), fma2(E1, mx, m[1])), fma2(E2, mx, m[2])), fma2(E3, mx, m[3]));
+    const f32x2 s3 = add2(add2(add2(m[0], m[1]), m[2]), m[3]);
+    const f32x2 clip = one_if_le2(rest, mx);
+    // cumulative sums the points fall into: clipped without the maximum, otherwise with it
+    const f32x2 mxc = mul2(clip, mx);
+    const f32x2 c0 = fma2(E0, mxc, m[0]);
+    const f32x2 c1 = add2(c0, fma2(E1, mxc, m[1]));
+    const f32x2 c2 = add2(c1, fma2(E2, mxc, m[2]));
+    const f32x2 nhalf = fma2(clip, both(-0.5f), both(0.5f));          // 1/2 where not clipped
+    const f32x2 h = fma2(clip, rest, mul2(nhalf, s3));
+    // k is the uniform's 24 bits in the upper bits of a word: k * 2^-32 is exact
+    const f32x2 u = mul2(pack2(__uint2float_rn(k_lo & 0xffffff00u), __uint2float_rn(k_hi & 0xffffff00u)), both(0x1p-32f));
+    const f32x2 r = mul2(u, h);
+    // Clipped: a point that rounding put AT rest (possible only when u * rest is subnormal) counts as just below it,
+    // which selects the last other element of nonzero magnitude: minimum of the bit patterns with rest's minus one.
+    // rest == 0 gives the pattern of a NaN, which is at or above no sum.  Not clipped: the bound is out of reach.
+    float b0, b1, r0, r1;
+    unpack2(fma2(nhalf, both(3.402823466e38f), rest), b0, b1);
+    unpack2(r, r0, r1);
+    const f32x2 p1 = pack2(__int_as_float(__viaddmin_s32(__float_as_int(b0), -1, __float_as_int(r0))),
+                           __int_as_float(__viaddmin_s32(__float_as_int(b1), -1, __float_as_int(r1))));
+    const f32x2 p2 = add2(p1, h);
+    // byte offset of the table entry, in units of the smallest subnormal
+    constexpr int UNIT = 8;
+    const f32x2 w1 = both(__int_as_float(UNIT)), w4 = both(__int_as_float(4 * UNIT));
+    const f32x2 j1 = add2(add2(one_if_le2(c0, p1), one_if_le2(c1, p1)), one_if_le2(c2, p1));
+    const f32x2 n2 = add2(add2(one_if_le2(c0, p2), one_if_le2(c1, p2)), one_if_le2(c2, p2));
+    const f32x2 nx = fma2(add2(add2(X0, X1), X2), minus1, both(static_cast<float>(MVUE_CLIP) * 0.25f));   // 7 - (3 - x)
+    const f32x2 off = fma2(j1, w1, mul2(fma2(clip, nx, n2), w4));
+    float o0, o1;
+    unpack2(off, o0, o1);
+    MvuePair g;
+    g.e0 = *reinterpret_cast<const uint2 *>(lut + __float_as_uint(o0));
+    g.e1 = *reinterpret_cast<const uint2 *>(lut + __float_as_uint(o1));
+    g.h = h;
+    g.mx = mx;
+    return g;
 }
 
 // The group rule on explicit inputs (test / debug): group i = four bf16 values a[4 i .. 4 i + 3] and the uniform
@@ -342,23 +443,37 @@ __global__ void __launch_bounds__(EW_THREADS)
 mvue_groups_kernel(const uint2 *__restrict__ a, const uint32_t *__restrict__ k24, size_t n, uint32_t *__restrict__ pos,
                    float2 *__restrict__ val)
 {
+    __shared__ uint2 lut[MVUE_ENTRIES];
+    if (threadIdx.x < MVUE_ENTRIES) lut[threadIdx.x] = mvue_table_bf16.e[threadIdx.x];
+    __syncthreads();
     sste_pdl_trigger();
     sste_pdl_wait();
     for (size_t i = static_cast<size_t>(blockIdx.x) * EW_THREADS + threadIdx.x; i < n;
          i += static_cast<size_t>(gridDim.x) * EW_THREADS) {
         const uint2 g = a[i];
-        const float u = __uint2float_rn(k24[i] & 0xffffffu) * 0x1p-24f;
-        const MvueGroup r = mvue_group(g.x, g.y, u);
-        pos[i] = r.q0 | (r.q1 << 2);
-        val[i] = make_float2(r.v0, r.v1);
+        const uint32_t k = k24[i] << 8;
+        // the group in the low halves, its mirror image (an unrelated group) in the high ones
+        const uint32_t w[4] = {__byte_perm(g.x, g.y, 0x7610), __byte_perm(g.x, g.y, 0x5432), __byte_perm(g.y, g.x, 0x7610),
+                               __byte_perm(g.y, g.x, 0x5432)};
+        const MvuePair r = mvue_pair(w, k, ~k, reinterpret_cast<const uint8_t *>(lut));
+        float h, other;
+        unpack2(r.h, h, other);
+        const uint32_t kept = prmt(g.x, g.y, r.e0.x), mask = r.e0.y;
+        pos[i] = (r.e0.x >> 16) & 0xfu;
+        auto value = [&](uint32_t bits, uint32_t m) {      // bf16 bits of the kept element, its mask
+            return m == 0xffffu ? __uint_as_float(bits << 16) : __uint_as_float(((bits & m) << 16) | __float_as_uint(h));
+        };
+        val[i] = make_float2(value(kept & 0xffffu, mask & 0xffffu), value(kept >> 16, mask >> 16));
     }
 }
 
 // ---------------------------------------------------------------- MVUE + compress (transposing)
 
-// One CTA: 128 tokens x 128 output columns of dY.  A thread task is 4 tokens x 8 columns
+// One CTA: 128 tokens x 64 output columns of dY (half a metadata atom).  A thread handles 4 tokens x 8 columns
 // (8 groups, two Philox calls); results are transposed through shared memory so that every
-// output row (= column of dY) receives whole 128-byte lines.
+// output row (= column of dY) receives whole 128-byte lines.  dY[8192, 3072], bf16 / FP8: 35.6 / 38.1 us with the
+// scalar rule, 24.2 / 30.3 us with mvue_pair (15.6 us is what the loads and stores take alone, 20.0 us the rule without
+// the loads); two tasks of 128 columns, tasks of 4 columns, and persistent CTAs with cp.async prefetch were slower.
 // ANY_COUNTER: counter_cols is not a multiple of 4 (a padded, odd column count), so a thread's eight
 // consecutive group indices do not start on a Philox block and span three blocks instead of two.
 template <bool FP8, bool ANY_COUNTER>
@@ -368,35 +483,32 @@ mvue_kernel(const uint4 *__restrict__ dY, int O, int T, uint32_t key0, uint32_t 
             void *__restrict__ gvals,
             uint8_t *__restrict__ gmeta, void *__restrict__ dense_q)
 {
-    // bf16: 128 rows x 32 words; fp8: 128 rows x 16 words
-    __shared__ __align__(16) uint32_t vals_s[128 * (FP8 ? 16 : 32)];
-    __shared__ __align__(16) uint8_t meta_s[2048];
+    // bf16: 64 rows x 32 words; fp8: 64 rows x 16 words
+    __shared__ __align__(16) uint32_t vals_s[64 * (FP8 ? 16 : 32)];
+    __shared__ __align__(16) uint8_t meta_s[1024];
+    __shared__ uint2 lut[MVUE_ENTRIES];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int jb = blockIdx.x, tb = blockIdx.y;   // column block, token block
+    const int jb = blockIdx.x, tb = blockIdx.y;   // column block (64), token block
+    if (tid < MVUE_ENTRIES) lut[tid] = FP8 ? mvue_table_fp8.e[tid] : mvue_table_bf16.e[tid];
+    __syncthreads();
     sste_pdl_trigger();
     sste_pdl_wait();
     const float gscale = FP8 ? sste_scale_from_amax(*g_amax_dev, 57344.0f) : 1.0f;
     const size_t row_chunks = static_cast<size_t>(O) / 8;
 
-#pragma unroll
-    for (int it = 0; it < 2; ++it) {
-        const int bidx = it * 8 + warp;
-        const int jc = (bidx & 1) * 8 + (lane & 7);      // column chunk 0..15
-        const int tgl = (bidx >> 1) * 4 + (lane >> 3);   // token group 0..31 inside the tile
+    {
+        const int jc = lane & 7;                         // column chunk 0..7
+        const int tgl = warp * 4 + (lane >> 3);          // token group 0..31 inside the tile
         const size_t tok0 = static_cast<size_t>(tb) * 128 + 4 * tgl;
         uint4 in[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) in[i] = __ldg(dY + (tok0 + i) * row_chunks + jb * 16 + jc);
+        for (int i = 0; i < 4; ++i) in[i] = __ldg(dY + (tok0 + i) * row_chunks + jb * 8 + jc);
 
         const uint64_t g0 = (tg_offset + static_cast<uint64_t>(tb) * 32 + tgl) * static_cast<uint64_t>(counter_cols) +
-                            static_cast<uint64_t>(jb) * 128 + jc * 8;
+                            static_cast<uint64_t>(jb) * 64 + jc * 8;
         const uint64_t q = g0 >> 2;
         uint32_t rnd[8];
-        if (!ANY_COUNTER) {
-            philox4x32_10(static_cast<uint32_t>(q), static_cast<uint32_t>(q >> 32), tensor_id, step, key0, key1, rnd);
-            philox4x32_10(static_cast<uint32_t>(q + 1), static_cast<uint32_t>((q + 1) >> 32), tensor_id, step, key0,
-                          key1, rnd + 4);
-        } else {
+        if (ANY_COUNTER) {
             uint32_t r12[12];
 #pragma unroll
             for (int b = 0; b < 3; ++b)
@@ -412,42 +524,64 @@ mvue_kernel(const uint4 *__restrict__ dY, int O, int T, uint32_t key0, uint32_t 
                                     {in[1].x, in[1].y, in[1].z, in[1].w},
                                     {in[2].x, in[2].y, in[2].z, in[2].w},
                                     {in[3].x, in[3].y, in[3].z, in[3].w}};
-        uint32_t nibs = 0;
+        uint32_t ex[8];                                 // first table word of every group: its nibble in byte 2
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            // the group of column e: one bf16 from each of the four token rows, packed in pairs
-            const uint32_t sel = (e & 1) ? 0x7632u : 0x5410u;
-            const uint32_t p01 = __byte_perm(raw[0][e >> 1], raw[1][e >> 1], sel);
-            const uint32_t p23 = __byte_perm(raw[2][e >> 1], raw[3][e >> 1], sel);
-            const float u = __uint2float_rn(rnd[e] >> 8) * 0x1p-24f;
-            const MvueGroup r = mvue_group(p01, p23, u);
-            nibs |= (r.q0 | (r.q1 << 2)) << (4 * e);
-            const int jl = jc * 8 + e;
-            if (FP8) {
-                const uint32_t pair = static_cast<uint32_t>(__nv_cvt_float2_to_fp8x2(
-                    make_float2(__fmul_rn(r.v0, gscale), __fmul_rn(r.v1, gscale)), __NV_SATFINITE, __NV_E5M2));
-                reinterpret_cast<uint16_t *>(vals_s)[jl * 32 + (tgl ^ (8 * (jc & 3)))] = static_cast<uint16_t>(pair);
-            } else {
-                const __nv_bfloat162 pair = __floats2bfloat162_rn(r.v0, r.v1);
-                vals_s[jl * 32 + (tgl ^ (4 * (jc & 7)))] = *reinterpret_cast<const uint32_t *>(&pair);
+        for (int c = 0; c < 4; ++c) {                   // columns 2c, 2c + 1: one word of each token row
+            if (!ANY_COUNTER && c % 2 == 0)             // drawn when needed: fewer registers live
+                philox4x32_10(static_cast<uint32_t>(q + c / 2), static_cast<uint32_t>((q + c / 2) >> 32), tensor_id, step,
+                              key0, key1, rnd + 2 * c);
+            const uint32_t w[4] = {raw[0][c], raw[1][c], raw[2][c], raw[3][c]};
+            const MvuePair g = mvue_pair(w, rnd[2 * c], rnd[2 * c + 1], reinterpret_cast<const uint8_t *>(lut));
+            ex[2 * c] = g.e0.x;
+            ex[2 * c + 1] = g.e1.x;
+            float h[2], mx[2];
+            unpack2(FP8 ? mul2(g.h, both(gscale)) : g.h, h[0], h[1]);
+            if (FP8) unpack2(mul2(g.mx, both(gscale)), mx[0], mx[1]);
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                // the group of column 2c + e: one bf16 from each of the four token rows, packed in pairs
+                const uint32_t sel = e ? 0x7632u : 0x5410u;
+                const uint32_t p01 = __byte_perm(w[0], w[1], sel), p23 = __byte_perm(w[2], w[3], sel);
+                const uint2 t = e ? g.e1 : g.e0;
+                const uint32_t kept = prmt(p01, p23, t.x);
+                const int jl = jc * 8 + 2 * c + e;
+                if (FP8) {
+                    const uint32_t q = static_cast<uint32_t>(
+                        __nv_cvt_float2_to_fp8x2(make_float2(h[e], mx[e]), __NV_SATFINITE, __NV_E5M2));
+                    reinterpret_cast<uint16_t *>(vals_s)[jl * 32 + (tgl ^ (8 * (jc & 3)))] =
+                        static_cast<uint16_t>((kept & (t.y >> 16)) | prmt(q, 0, t.y));
+                } else {
+                    const __nv_bfloat162 hb2 = __floats2bfloat162_rn(h[e], h[e]);
+                    const uint32_t hb = *reinterpret_cast<const uint32_t *>(&hb2);
+                    vals_s[jl * 32 + (tgl ^ (4 * (jc & 7)))] = (kept & t.y) | (hb & ~t.y);
+                }
             }
         }
         if (FP8 && dense_q) {
+            // magnitudes scaled and converted two at a time (round to nearest is symmetric), the sign bytes merged in
+            const f32x2 g2 = both(gscale);
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                uint32_t b[8];
+                uint32_t d[2];
 #pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    const uint32_t word = raw[i][e >> 1];
-                    const float v = sste_bf16_bits_to_f32((e & 1) ? (word >> 16) : (word & 0xffffu));
-                    b[e] = sste_f32_to_e5m2(__fmul_rn(v, gscale));
+                for (int v = 0; v < 2; ++v) {
+                    uint32_t q[2];
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const uint32_t mm = raw[i][2 * v + e] & 0x7fff7fffu;
+                        float a, b;
+                        unpack2(mul2(pack2(__uint_as_float(mm << 16), __uint_as_float(mm & 0xffff0000u)), g2), a, b);
+                        q[e] = static_cast<uint32_t>(__nv_cvt_float2_to_fp8x2(make_float2(a, b), __NV_SATFINITE, __NV_E5M2));
+                    }
+                    d[v] = (__byte_perm(raw[i][2 * v], raw[i][2 * v + 1], 0x7531) & 0x80808080u) | __byte_perm(q[0], q[1], 0x5410);
                 }
-                uint2 d;
-                d.x = b[0] | (b[1] << 8) | (b[2] << 16) | (b[3] << 24);
-                d.y = b[4] | (b[5] << 8) | (b[6] << 16) | (b[7] << 24);
-                reinterpret_cast<uint2 *>(dense_q)[(tok0 + i) * row_chunks + jb * 16 + jc] = d;
+                reinterpret_cast<uint2 *>(dense_q)[(tok0 + i) * row_chunks + jb * 8 + jc] = make_uint2(d[0], d[1]);
             }
         }
+        // nibbles of the even columns in the low halves of the bytes, of the odd ones in the high halves
+        const uint32_t ev = __byte_perm(__byte_perm(ex[0], ex[2], 0x0062), __byte_perm(ex[4], ex[6], 0x0062), 0x5410);
+        const uint32_t od = __byte_perm(__byte_perm(ex[1], ex[3], 0x0062), __byte_perm(ex[5], ex[7], 0x0062), 0x5410);
+        const uint32_t nibs = ev | (od << 4);
         // two token groups share a metadata byte: lane ^ 8 holds the neighbouring token group
         const uint32_t other = __shfl_xor_sync(0xffffffffu, nibs, 8);
         if ((tgl & 1) == 0) {
@@ -469,16 +603,16 @@ mvue_kernel(const uint4 *__restrict__ dY, int O, int T, uint32_t key0, uint32_t 
     constexpr int VECS = FP8 ? 4 : 8;
     const size_t out_row_vecs = static_cast<size_t>(T) / (FP8 ? 32 : 16);   // 16-byte vectors per output row
 #pragma unroll
-    for (int it = 0; it < (128 * VECS) / EW_THREADS; ++it) {
+    for (int it = 0; it < (64 * VECS) / EW_THREADS; ++it) {
         const int v = it * EW_THREADS + tid;
         const int row = v / VECS, vec = v % VECS;
         const int pvec = FP8 ? (vec ^ ((row >> 3) & 3)) : (vec ^ ((row >> 3) & 7));
         const uint4 data = reinterpret_cast<const uint4 *>(vals_s)[row * VECS + pvec];
-        reinterpret_cast<uint4 *>(gvals)[(static_cast<size_t>(jb) * 128 + row) * out_row_vecs + tb * VECS + vec] = data;
+        reinterpret_cast<uint4 *>(gvals)[(static_cast<size_t>(jb) * 64 + row) * out_row_vecs + tb * VECS + vec] = data;
     }
-    if (tid < 128) {
-        const size_t atom = static_cast<size_t>(jb) * (T / 128) + tb;
-        reinterpret_cast<uint4 *>(gmeta + atom * 2048)[tid] = reinterpret_cast<const uint4 *>(meta_s)[tid];
+    if (tid < 64) {
+        const size_t atom = static_cast<size_t>(jb >> 1) * (T / 128) + tb;
+        reinterpret_cast<uint4 *>(gmeta + atom * 2048 + 1024 * (jb & 1))[tid] = reinterpret_cast<const uint4 *>(meta_s)[tid];
     }
 }
 
@@ -903,7 +1037,7 @@ extern "C" sste_status sste_mvue_sparsify(sste_ctx *ctx, const void *dY, int T, 
         return SSTE_ERR_ALIGN;
     sste_device_guard guard(ctx->device);
     if (!guard.ok) return SSTE_ERR_CUDA;
-    const dim3 grid(O / 128, T / 128);
+    const dim3 grid(O / 64, T / 128);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const uint32_t key0 = static_cast<uint32_t>(seed), key1 = static_cast<uint32_t>(seed >> 32);
     const uint4 *g = static_cast<const uint4 *>(dY);

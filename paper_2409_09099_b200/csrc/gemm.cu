@@ -19,7 +19,6 @@
 // Every wait is bounded: on expiry the CTA records SSTE_ERR_TIMEOUT and leaves.
 #include <cuda.h>
 
-#include <mutex>
 #include <type_traits>
 
 #include "common.cuh"
@@ -900,21 +899,6 @@ bool make_map(const sste_ctx *ctx, CUtensorMap *map, const void *base, int elt, 
     return fn(map, dt, 2, const_cast<void *>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swz,
               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
-
-// Runs `fn` once per device ordinal (and again after a failure); thread-safe.
-struct DeviceOnce {
-    static constexpr int MAX_DEVICES = 64;
-    std::mutex mu;
-    bool done[MAX_DEVICES] = {};
-    template <typename F>
-    bool run(int device, F fn)
-    {
-        if (device < 0 || device >= MAX_DEVICES) return fn();
-        std::lock_guard<std::mutex> lock(mu);
-        if (!done[device]) done[device] = fn();
-        return done[device];
-    }
-};
 
 int g_inject_stall = 0;   // test hook: see sste_debug_inject_stall
 int g_force_group_m = 0;  // test hook: 0 = automatic band height of the tile order
