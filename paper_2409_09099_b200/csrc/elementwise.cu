@@ -618,6 +618,22 @@ mvue_kernel(const uint4 *__restrict__ dY, int O, int T, uint32_t key0, uint32_t 
 
 // ---------------------------------------------------------------- FP8 helpers
 
+// *amax_dev = max(*amax_dev, every thread's `bits`), the bit patterns of non-negative fp32 values, which order like
+// unsigned integers.  One atomic per block: with one per warp the 9472 of a full grid queued up at the one address for
+// 9 us, whatever the tensor's size (amax of 12.6 MB: 10.3 -> 4 us).
+__device__ __forceinline__ void block_max_to(uint32_t bits, float *amax_dev)
+{
+    __shared__ unsigned int best_s[EW_THREADS / 32];
+    bits = __reduce_max_sync(0xffffffffu, bits);
+    if ((threadIdx.x & 31) == 0) best_s[threadIdx.x >> 5] = bits;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int w = 1; w < EW_THREADS / 32; ++w) bits = max(bits, best_s[w]);
+        if (bits != 0) atomicMax(reinterpret_cast<unsigned int *>(amax_dev), bits);
+    }
+}
+
 __global__ void __launch_bounds__(EW_THREADS)
 amax_kernel(const uint4 *__restrict__ x, size_t n_chunks, float *__restrict__ amax_dev)
 {
@@ -638,11 +654,7 @@ amax_kernel(const uint4 *__restrict__ x, size_t n_chunks, float *__restrict__ am
             best2 = __vmaxu2(best2, v[j].w & 0x7fff7fffu);
         }
     }
-    uint32_t best = max(best2 & 0xffffu, best2 >> 16);
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) best = max(best, __shfl_xor_sync(0xffffffffu, best, off));
-    if ((threadIdx.x & 31) == 0 && best != 0)
-        atomicMax(reinterpret_cast<unsigned int *>(amax_dev), best << 16);   // non-negative floats order as uints
+    block_max_to(max(best2 & 0xffffu, best2 >> 16) << 16, amax_dev);
 }
 
 // amax of the bf16 projection w~ = bf16(beta * S_soft(W)) without writing it: rounding to bf16 is monotone,
@@ -675,11 +687,7 @@ project_amax_kernel(const uint4 *__restrict__ W, size_t n_chunks, const float *_
             }
         }
     }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, off));
-    const uint32_t bits = sste_f32_to_bf16_bits(best);
-    if ((threadIdx.x & 31) == 0 && bits != 0)
-        atomicMax(reinterpret_cast<unsigned int *>(amax_dev), bits << 16);   // non-negative floats order as uints
+    block_max_to(sste_f32_to_bf16_bits(best) << 16, amax_dev);
 }
 
 __global__ void fp8_scale_kernel(const float *amax_dev, float fp8_max, float *scale_dev, float *inv_scale_dev)
