@@ -242,6 +242,42 @@ sste_status sste_fp8_scale(sste_ctx *ctx, const float *amax_dev, sste_dtype odt,
 sste_status sste_quantize_fp8(sste_ctx *ctx, const void *x, size_t n, const float *amax_dev,
                               sste_dtype odt, void *q, void *stream);
 
+/* ---- one layer, one call per phase of the iteration ---- */
+
+/*
+ * The buffers of one S-STE linear, as the calls above take them; the caller fills it in once and keeps it.  All pointers
+ * are device memory.  op_dtype SSTE_BF16: amax, Xq, dYq and scratch are NULL.  SSTE_E4M3 (the FP8 variant, gradients
+ * E5M2): amax is three floats, max|X|, max|w~|, max|dY|; Xq [T, I] E4M3 and dYq [T, O] E5M2 receive the quantised tensors;
+ * scratch is 8 bytes of the caller's, zero before the first call and left zero by every call (calls on one layer are
+ * stream-ordered).  w_dense NULL: grad_X works from the compressed operand.
+ */
+typedef struct sste_layer {
+    int O, I, T;
+    int op_dtype;               /* SSTE_BF16 or SSTE_E4M3 */
+    int out_dtype;              /* of Y, dX and dW: SSTE_BF16 or SSTE_F32 */
+    int counter_cols;           /* see sste_mvue_sparsify */
+    unsigned int tensor_id;
+    unsigned int reserved;      /* 0 */
+    unsigned long long seed;
+    const void *W;              /* bf16 [O, I] */
+    const float *beta;
+    float *amax;
+    void *vals, *meta, *w_dense;
+    void *gvals, *gmeta;
+    void *Xq, *dYq;
+    void *Y, *dX, *dW;
+    void *scratch;
+} sste_layer;
+
+/* sste_project_compress of the layer's weight (FP8: after sste_project_amax). */
+sste_status sste_layer_prune(sste_ctx *ctx, const sste_layer *layer, void *stream);
+/* sste_linear_fwd of X (FP8: after sste_amax and sste_quantize_fp8 of it).  X bf16 [T, I]. */
+sste_status sste_layer_forward(sste_ctx *ctx, const sste_layer *layer, const void *X, float *y_amax_out_dev, void *stream);
+/* sste_mvue_sparsify of dY (FP8: after sste_amax of it), sste_linear_bwd_weight with X (FP8: with the layer's Xq; X may
+ * be NULL), sste_linear_bwd_input.  dY bf16 [T, O]. */
+sste_status sste_layer_backward(sste_ctx *ctx, const sste_layer *layer, const void *X, const void *dY, uint32_t step,
+                                uint64_t token_offset, void *stream);
+
 /* ---- ablation variants of the pruning step (the axes of the paper's ablations; not on the default path) ---- */
 
 typedef enum { SSTE_PRUNE_SOFT = 0, SSTE_PRUNE_HARD = 1 } sste_pruning;

@@ -32,8 +32,38 @@ EXPORTS = [
     "sste_project_compress_variant", "sste_beta_init_l1", "sste_srste_decay", "sste_project_amax",
     "sste_decompress", "sste_padded_dim", "sste_pad_2d", "sste_crop_2d", "sste_debug_inject_stall",
     "sste_debug_force_tile_order", "sste_debug_plan", "sste_debug_tile_coords",
-    "sste_debug_mvue_groups", "sste_debug_selftest_device_once",
+    "sste_debug_mvue_groups", "sste_debug_selftest_device_once", "sste_layer_prune", "sste_layer_forward",
+    "sste_layer_backward",
 ]
+
+_P, _I, _Z, _U32, _U64, _F = (ctypes.c_void_p, ctypes.c_int, ctypes.c_size_t, ctypes.c_uint32, ctypes.c_uint64,
+                              ctypes.c_float)
+# Argument types of the calls of an iteration: plain Python ints then convert without a ctypes object for each of them.
+_ARGTYPES = {
+    "sste_beta_init": [_P, _P, _I, _I, _I, _P, _P],
+    "sste_project_compress": [_P, _P, _I, _I, _I, _P, _P, _I, _P, _P, _P, _P],
+    "sste_linear_fwd": [_P, _P, _I, _P, _P, _I, _I, _I, _P, _P, _P, _I, _P, _P],
+    "sste_mvue_sparsify": [_P, _P, _I, _I, _I, _U64, _U32, _U32, _U64, _I, _P, _I, _P, _P, _P, _P],
+    "sste_linear_bwd_input": [_P, _P, _I, _I, _I, _P, _P, _P, _I, _I, _P, _P, _P, _I, _P, _P],
+    "sste_linear_bwd_weight": [_P, _P, _P, _I, _I, _I, _P, _I, _I, _P, _P, _P, _I, _P],
+    "sste_amax": [_P, _P, _Z, _I, _P, _P],
+    "sste_project_amax": [_P, _P, _I, _I, _I, _P, _P, _P],
+    "sste_quantize_fp8": [_P, _P, _Z, _P, _I, _P, _P],
+    "sste_flip_count": [_P, _P, _P, _I, _I, _P, _P],
+    "sste_pad_2d": [_P, _P, _I, _I, _P, _I, _I, _P],
+    "sste_crop_2d": [_P, _P, _I, _I, _P, _I, _I, _P],
+    "sste_layer_prune": [_P, _P, _P],
+    "sste_layer_forward": [_P, _P, _P, _P, _P],
+    "sste_layer_backward": [_P, _P, _P, _P, _U32, _U64, _P],
+}
+
+
+class LayerBuffers(ctypes.Structure):
+    """sste_layer: the buffers of one layer, filled in once (layer.py)."""
+    _fields_ = [("O", _I), ("I", _I), ("T", _I), ("op_dtype", _I), ("out_dtype", _I), ("counter_cols", _I),
+                ("tensor_id", _U32), ("reserved", _U32), ("seed", _U64), ("W", _P), ("beta", _P), ("amax", _P),
+                ("vals", _P), ("meta", _P), ("w_dense", _P), ("gvals", _P), ("gmeta", _P), ("Xq", _P), ("dYq", _P),
+                ("Y", _P), ("dX", _P), ("dW", _P), ("scratch", _P)]
 
 
 class SsteError(RuntimeError):
@@ -57,19 +87,31 @@ def load() -> ctypes.CDLL:
         lib.sste_vals_bytes.restype = ctypes.c_size_t
         lib.sste_meta_bytes.restype = ctypes.c_size_t
         lib.sste_status_string.restype = ctypes.c_char_p
+        for name, types in _ARGTYPES.items():
+            getattr(lib, name).argtypes = types
         _lib = lib
     return _lib
 
 
 def _ptr(t):
+    """Device address of a tensor (None: a null pointer), an int; _vp wraps it for calls without argument types."""
     if t is None:
-        return ctypes.c_void_p(0)
+        return None
     assert t.is_cuda and t.is_contiguous(), "device, contiguous tensors only"
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
+
+
+def _vp(t):
+    return ctypes.c_void_p(_ptr(t))
 
 
 def _stream():
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    """Handle of torch's current stream of the current device."""
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+
+
+def _vstream():
+    return ctypes.c_void_p(_stream())
 
 
 def padded_dim(n: int) -> int:
@@ -104,7 +146,7 @@ def beta_init_static(W, beta_dev):
     """
     lib = load()
     O, I = W.shape
-    st = lib.sste_beta_init_static(W.device.index or 0, _ptr(W), O, I, _CODE_OF[W.dtype], _ptr(beta_dev), _stream())
+    st = lib.sste_beta_init_static(W.device.index or 0, _vp(W), O, I, _CODE_OF[W.dtype], _vp(beta_dev), _vstream())
     if st != OK:
         raise SsteError(st, lib.sste_status_string(st).decode())
 
@@ -118,7 +160,7 @@ class Context:
         n = self.lib.sste_workspace_bytes() if minimal_workspace else self.lib.sste_workspace_bytes_recommended()
         self.workspace = torch.zeros(n, dtype=torch.uint8, device=f"cuda:{device}")
         handle = ctypes.c_void_p()
-        st = self.lib.sste_create(ctypes.byref(handle), device, _ptr(self.workspace), ctypes.c_size_t(n))
+        st = self.lib.sste_create(ctypes.byref(handle), device, _vp(self.workspace), ctypes.c_size_t(n))
         self._check(st)
         self.handle = handle
 
@@ -160,8 +202,8 @@ class Context:
                       token_offset=0, counter_cols=0):
         T, O = dY.shape
         self._check(self.lib.sste_mvue_sparsify(
-            self.handle, _ptr(dY), T, O, _CODE_OF[dY.dtype], ctypes.c_uint64(seed), ctypes.c_uint32(tensor_id),
-            ctypes.c_uint32(step), ctypes.c_uint64(token_offset), ctypes.c_int(counter_cols), _ptr(g_amax_dev),
+            self.handle, _ptr(dY), T, O, _CODE_OF[dY.dtype], seed, tensor_id, step, token_offset, counter_cols,
+            _ptr(g_amax_dev),
             _CODE_OF[gvals.dtype], _ptr(gvals), _ptr(gmeta), _ptr(dense_q_out), _stream()))
 
     def linear_bwd_input(self, dY, Wt_dense, dX, g_amax_dev=None, w_amax_dev=None, vals=None, meta=None,
@@ -186,7 +228,7 @@ class Context:
     # ---- FP8 helpers ----------------------------------------------------------------------------
 
     def amax(self, x, amax_dev):
-        self._check(self.lib.sste_amax(self.handle, _ptr(x), ctypes.c_size_t(x.numel()), _CODE_OF[x.dtype],
+        self._check(self.lib.sste_amax(self.handle, _ptr(x), x.numel(), _CODE_OF[x.dtype],
                                        _ptr(amax_dev), _stream()))
 
     def project_amax(self, W, beta_dev, amax_dev):
@@ -195,11 +237,11 @@ class Context:
                                                _ptr(amax_dev), _stream()))
 
     def fp8_scale(self, amax_dev, odt, scale_dev, inv_scale_dev=None):
-        self._check(self.lib.sste_fp8_scale(self.handle, _ptr(amax_dev), odt, _ptr(scale_dev), _ptr(inv_scale_dev),
-                                            _stream()))
+        self._check(self.lib.sste_fp8_scale(self.handle, _vp(amax_dev), odt, _vp(scale_dev), _vp(inv_scale_dev),
+                                            _vstream()))
 
     def quantize_fp8(self, x, amax_dev, q):
-        self._check(self.lib.sste_quantize_fp8(self.handle, _ptr(x), ctypes.c_size_t(x.numel()), _ptr(amax_dev),
+        self._check(self.lib.sste_quantize_fp8(self.handle, _ptr(x), x.numel(), _ptr(amax_dev),
                                                _CODE_OF[q.dtype], _ptr(q), _stream()))
 
     # ---- ablation variants of the pruning step ---------------------------------------------------
@@ -208,19 +250,19 @@ class Context:
                                  gamma=0.0):
         O, I = W.shape
         self._check(self.lib.sste_project_compress_variant(
-            self.handle, _ptr(W), O, I, _CODE_OF[W.dtype], _ptr(beta_dev), _ptr(w_amax_dev), _CODE_OF[vals.dtype],
-            PRUNE_HARD if hard else PRUNE_SOFT, ctypes.c_float(gamma), _ptr(vals), _ptr(meta), _ptr(dense_out),
-            _stream()))
+            self.handle, _vp(W), O, I, _CODE_OF[W.dtype], _vp(beta_dev), _vp(w_amax_dev), _CODE_OF[vals.dtype],
+            PRUNE_HARD if hard else PRUNE_SOFT, ctypes.c_float(gamma), _vp(vals), _vp(meta), _vp(dense_out),
+            _vstream()))
 
     def beta_init_l1(self, W, beta_dev):
         O, I = W.shape
-        self._check(self.lib.sste_beta_init_l1(self.handle, _ptr(W), O, I, _CODE_OF[W.dtype], _ptr(beta_dev),
-                                               _stream()))
+        self._check(self.lib.sste_beta_init_l1(self.handle, _vp(W), O, I, _CODE_OF[W.dtype], _vp(beta_dev),
+                                               _vstream()))
 
     def srste_decay(self, W, meta, meta_dt, lam, dW):
         O, I = W.shape
-        self._check(self.lib.sste_srste_decay(self.handle, _ptr(W), _ptr(meta), O, I, meta_dt, ctypes.c_float(lam),
-                                              _ptr(dW), _stream()))
+        self._check(self.lib.sste_srste_decay(self.handle, _vp(W), _vp(meta), O, I, meta_dt, ctypes.c_float(lam),
+                                              _vp(dW), _vstream()))
 
     # ---- diagnostics ----------------------------------------------------------------------------
 
@@ -233,8 +275,8 @@ class Context:
 
     def decompress(self, vals, meta, dense_out):
         rows, k = dense_out.shape
-        self._check(self.lib.sste_decompress(self.handle, _ptr(vals), _ptr(meta), rows, k, _CODE_OF[vals.dtype],
-                                             _ptr(dense_out), _stream()))
+        self._check(self.lib.sste_decompress(self.handle, _vp(vals), _vp(meta), rows, k, _CODE_OF[vals.dtype],
+                                             _vp(dense_out), _vstream()))
 
     def pad_2d(self, src, dst):
         """dst[:rows, :cols] = src, zeros elsewhere (2-byte elements)."""
@@ -247,12 +289,12 @@ class Context:
                                           dst.shape[1], _stream()))
 
     def meta_to_canonical(self, meta, rows, k, dt, out):
-        self._check(self.lib.sste_meta_to_canonical(self.handle, _ptr(meta), rows, k, dt, _ptr(out), _stream()))
+        self._check(self.lib.sste_meta_to_canonical(self.handle, _vp(meta), rows, k, dt, _vp(out), _vstream()))
 
     def debug_mvue_groups(self, a, k24, pos_out, val_out):
         """sste_debug_mvue_groups: the MVUE group rule on explicit groups a [n, 4] (bf16) and 24-bit uniforms k24 [n]."""
-        self._check(self.lib.sste_debug_mvue_groups(self.handle, _ptr(a), _ptr(k24), ctypes.c_size_t(a.shape[0]),
-                                                    _ptr(pos_out), _ptr(val_out), _stream()))
+        self._check(self.lib.sste_debug_mvue_groups(self.handle, _vp(a), _vp(k24), ctypes.c_size_t(a.shape[0]),
+                                                    _vp(pos_out), _vp(val_out), _vstream()))
 
     def debug_force_splits(self, splits: int):
         self._check(self.lib.sste_debug_force_splits(splits))
@@ -267,7 +309,7 @@ class Context:
         self._check(self.lib.sste_debug_force_tile_width(bn))
 
     def poll_device_status(self) -> int:
-        return self.lib.sste_poll_device_status(self.handle, _stream())
+        return self.lib.sste_poll_device_status(self.handle, _vstream())
 
     # ---- allocation helpers (torch as the allocator) ---------------------------------------------
 

@@ -148,3 +148,9 @@ inline cudaError_t sste_launch(void (*kern)(KArgs...), dim3 grid, dim3 block, si
 
 // Process-wide count of kernels this library has launched (read by sste_debug_launch_count).
 void sste_count_launches(int n);
+
+// sste_amax / sste_project_amax without a memset in front: the running maximum and the arrival counter live in 8 bytes of
+// the caller's (zero before and after every call) and the block that arrives last stores the result.
+sste_status sste_amax_scratch(sste_ctx *ctx, const void *x, size_t n, float *amax_dev, void *scratch, void *stream);
+sste_status sste_project_amax_scratch(sste_ctx *ctx, const void *W, int O, int I, const float *beta_dev, float *amax_dev,
+                                      void *scratch, void *stream);

@@ -618,24 +618,33 @@ mvue_kernel(const uint4 *__restrict__ dY, int O, int T, uint32_t key0, uint32_t 
 
 // ---------------------------------------------------------------- FP8 helpers
 
-// *amax_dev = max(*amax_dev, every thread's `bits`), the bit patterns of non-negative fp32 values, which order like
+// *amax_dev = max over the grid of every thread's `bits`, the bit patterns of non-negative fp32 values, which order like
 // unsigned integers.  One atomic per block: with one per warp the 9472 of a full grid queued up at the one address for
-// 9 us, whatever the tensor's size (amax of 12.6 MB: 10.3 -> 4 us).
-__device__ __forceinline__ void block_max_to(uint32_t bits, float *amax_dev)
+// 9 us, whatever the tensor's size (amax of 12.6 MB: 10.3 -> 6.1 us).  scratch NULL: *amax_dev was zeroed by a memset in
+// front of the kernel.  Otherwise scratch[0] takes the running maximum and scratch[1] counts the blocks; the last one
+// stores the result and leaves both zero: no memset, which would also keep this kernel from starting early (-2 us).
+__device__ __forceinline__ void grid_max_to(uint32_t bits, float *amax_dev, unsigned int *scratch)
 {
     __shared__ unsigned int best_s[EW_THREADS / 32];
     bits = __reduce_max_sync(0xffffffffu, bits);
     if ((threadIdx.x & 31) == 0) best_s[threadIdx.x >> 5] = bits;
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (threadIdx.x != 0) return;
 #pragma unroll
-        for (int w = 1; w < EW_THREADS / 32; ++w) bits = max(bits, best_s[w]);
-        if (bits != 0) atomicMax(reinterpret_cast<unsigned int *>(amax_dev), bits);
+    for (int w = 1; w < EW_THREADS / 32; ++w) bits = max(bits, best_s[w]);
+    unsigned int *acc = scratch ? scratch : reinterpret_cast<unsigned int *>(amax_dev);
+    if (bits != 0) atomicMax(acc, bits);
+    if (!scratch) return;
+    __threadfence();
+    if (atomicAdd(scratch + 1, 1u) == gridDim.x - 1) {
+        __threadfence();
+        *reinterpret_cast<unsigned int *>(amax_dev) = atomicExch(scratch, 0u);
+        scratch[1] = 0u;
     }
 }
 
 __global__ void __launch_bounds__(EW_THREADS)
-amax_kernel(const uint4 *__restrict__ x, size_t n_chunks, float *__restrict__ amax_dev)
+amax_kernel(const uint4 *__restrict__ x, size_t n_chunks, float *__restrict__ amax_dev, unsigned int *__restrict__ scratch)
 {
     uint32_t best2 = 0;   // magnitude bits of bf16 compare like unsigned integers: running maximum in both halves
     sste_pdl_trigger();
@@ -654,14 +663,14 @@ amax_kernel(const uint4 *__restrict__ x, size_t n_chunks, float *__restrict__ am
             best2 = __vmaxu2(best2, v[j].w & 0x7fff7fffu);
         }
     }
-    block_max_to(max(best2 & 0xffffu, best2 >> 16) << 16, amax_dev);
+    grid_max_to(max(best2 & 0xffffu, best2 >> 16) << 16, amax_dev, scratch);
 }
 
 // amax of the bf16 projection w~ = bf16(beta * S_soft(W)) without writing it: rounding to bf16 is monotone,
 // so the maximum of the rounded magnitudes is the rounded maximum of the fp32 ones.
 __global__ void __launch_bounds__(EW_THREADS)
 project_amax_kernel(const uint4 *__restrict__ W, size_t n_chunks, const float *__restrict__ beta_dev,
-                    float *__restrict__ amax_dev)
+                    float *__restrict__ amax_dev, unsigned int *__restrict__ scratch)
 {
     sste_pdl_trigger();
     sste_pdl_wait();
@@ -687,7 +696,7 @@ project_amax_kernel(const uint4 *__restrict__ W, size_t n_chunks, const float *_
             }
         }
     }
-    block_max_to(sste_f32_to_bf16_bits(best) << 16, amax_dev);
+    grid_max_to(sste_f32_to_bf16_bits(best) << 16, amax_dev, scratch);
 }
 
 __global__ void fp8_scale_kernel(const float *amax_dev, float fp8_max, float *scale_dev, float *inv_scale_dev)
@@ -1061,19 +1070,51 @@ extern "C" sste_status sste_mvue_sparsify(sste_ctx *ctx, const void *dY, int T, 
     return launch_result();
 }
 
+namespace {
+
+sste_status amax_launch(sste_ctx *ctx, const void *x, size_t n, float *amax_dev, void *scratch, void *stream)
+{
+    if (!ctx || !x || !amax_dev) return SSTE_ERR_INVALID_ARG;
+    if (n == 0 || n % 8 != 0) return SSTE_ERR_SHAPE;
+    if (!sste_aligned(x, 16) || !sste_aligned(amax_dev, 4) || !sste_aligned(scratch, 8)) return SSTE_ERR_ALIGN;
+    sste_device_guard guard(ctx->device);
+    if (!guard.ok) return SSTE_ERR_CUDA;
+    const size_t n_chunks = n / 8;
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    if (!scratch) SSTE_CUDA_TRY(cudaMemsetAsync(amax_dev, 0, sizeof(float), s));
+    sste_launch(amax_kernel, dim3(grid_for(n_chunks, ctx->sm_count)), dim3(EW_THREADS), 0, s, static_cast<const uint4 *>(x),
+                n_chunks, amax_dev, static_cast<unsigned int *>(scratch));
+    return launch_result();
+}
+
+sste_status project_amax_launch(sste_ctx *ctx, const void *W, int O, int I, const float *beta_dev, float *amax_dev,
+                                void *scratch, void *stream)
+{
+    if (!ctx || !W || !beta_dev || !amax_dev) return SSTE_ERR_INVALID_ARG;
+    if (!sste_mult128(O) || !sste_mult128(I)) return SSTE_ERR_SHAPE;
+    if (!sste_aligned(W, 16) || !sste_aligned(amax_dev, 4) || !sste_aligned(scratch, 8)) return SSTE_ERR_ALIGN;
+    sste_device_guard guard(ctx->device);
+    if (!guard.ok) return SSTE_ERR_CUDA;
+    const size_t n_chunks = static_cast<size_t>(O) * I / 8;
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    if (!scratch) SSTE_CUDA_TRY(cudaMemsetAsync(amax_dev, 0, sizeof(float), s));
+    sste_launch(project_amax_kernel, dim3(grid_for(n_chunks, ctx->sm_count)), dim3(EW_THREADS), 0, s,
+                static_cast<const uint4 *>(W), n_chunks, beta_dev, amax_dev, static_cast<unsigned int *>(scratch));
+    return launch_result();
+}
+
+}  // namespace
+
 extern "C" sste_status sste_amax(sste_ctx *ctx, const void *x, size_t n, sste_dtype dt, float *amax_dev, void *stream)
 {
     if (!ctx || !x || !amax_dev) return SSTE_ERR_INVALID_ARG;
     if (dt != SSTE_BF16) return SSTE_ERR_DTYPE;
-    if (n == 0 || n % 8 != 0) return SSTE_ERR_SHAPE;
-    if (!sste_aligned(x, 16) || !sste_aligned(amax_dev, 4)) return SSTE_ERR_ALIGN;
-    sste_device_guard guard(ctx->device);
-    if (!guard.ok) return SSTE_ERR_CUDA;
-    const size_t n_chunks = n / 8;
-    SSTE_CUDA_TRY(cudaMemsetAsync(amax_dev, 0, sizeof(float), static_cast<cudaStream_t>(stream)));
-    sste_launch(amax_kernel, dim3(grid_for(n_chunks, ctx->sm_count)), dim3(EW_THREADS), 0,
-                static_cast<cudaStream_t>(stream), static_cast<const uint4 *>(x), n_chunks, amax_dev);
-    return launch_result();
+    return amax_launch(ctx, x, n, amax_dev, nullptr, stream);
+}
+
+sste_status sste_amax_scratch(sste_ctx *ctx, const void *x, size_t n, float *amax_dev, void *scratch, void *stream)
+{
+    return amax_launch(ctx, x, n, amax_dev, scratch, stream);
 }
 
 extern "C" sste_status sste_project_amax(sste_ctx *ctx, const void *W, int O, int I, sste_dtype wdt,
@@ -1081,16 +1122,13 @@ extern "C" sste_status sste_project_amax(sste_ctx *ctx, const void *W, int O, in
 {
     if (!ctx || !W || !beta_dev || !amax_dev) return SSTE_ERR_INVALID_ARG;
     if (wdt != SSTE_BF16) return SSTE_ERR_DTYPE;
-    if (!sste_mult128(O) || !sste_mult128(I)) return SSTE_ERR_SHAPE;
-    if (!sste_aligned(W, 16) || !sste_aligned(amax_dev, 4)) return SSTE_ERR_ALIGN;
-    sste_device_guard guard(ctx->device);
-    if (!guard.ok) return SSTE_ERR_CUDA;
-    const size_t n_chunks = static_cast<size_t>(O) * I / 8;
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
-    SSTE_CUDA_TRY(cudaMemsetAsync(amax_dev, 0, sizeof(float), s));
-    sste_launch(project_amax_kernel, dim3(grid_for(n_chunks, ctx->sm_count)), dim3(EW_THREADS), 0, s,
-                static_cast<const uint4 *>(W), n_chunks, beta_dev, amax_dev);
-    return launch_result();
+    return project_amax_launch(ctx, W, O, I, beta_dev, amax_dev, nullptr, stream);
+}
+
+sste_status sste_project_amax_scratch(sste_ctx *ctx, const void *W, int O, int I, const float *beta_dev, float *amax_dev,
+                                      void *scratch, void *stream)
+{
+    return project_amax_launch(ctx, W, O, I, beta_dev, amax_dev, scratch, stream);
 }
 
 extern "C" sste_status sste_fp8_scale(sste_ctx *ctx, const float *amax_dev, sste_dtype odt, float *scale_dev,

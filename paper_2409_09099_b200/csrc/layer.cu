@@ -1,0 +1,68 @@
+// One call per phase of a layer's iteration (prune, forward, backward): the calls of the path in order, on the buffers of an
+// sste_layer.  A caller in an interpreted language pays for one call instead of two to four, each with a dozen arguments
+// to convert: on a 256 x 256 layer that conversion, not the GPU, set the pace.
+#include "common.cuh"
+
+namespace {
+
+bool fp8_of(const sste_layer *l) { return l->op_dtype == SSTE_E4M3; }
+
+// bf16 with none of the FP8 buffers, or E4M3 with all of them
+bool layer_ok(const sste_layer *l)
+{
+    if (!l || (l->op_dtype != SSTE_BF16 && l->op_dtype != SSTE_E4M3)) return false;
+    return !fp8_of(l) || (l->amax && l->Xq && l->dYq && l->scratch);
+}
+
+}  // namespace
+
+extern "C" sste_status sste_layer_prune(sste_ctx *ctx, const sste_layer *l, void *stream)
+{
+    if (!ctx || !layer_ok(l)) return SSTE_ERR_INVALID_ARG;
+    float *w_amax = fp8_of(l) ? l->amax + 1 : nullptr;
+    if (fp8_of(l)) {
+        const sste_status st = sste_project_amax_scratch(ctx, l->W, l->O, l->I, l->beta, w_amax, l->scratch, stream);
+        if (st != SSTE_OK) return st;
+    }
+    return sste_project_compress(ctx, l->W, l->O, l->I, SSTE_BF16, l->beta, w_amax, static_cast<sste_dtype>(l->op_dtype),
+                                 l->vals, l->meta, l->w_dense, stream);
+}
+
+extern "C" sste_status sste_layer_forward(sste_ctx *ctx, const sste_layer *l, const void *X, float *y_amax_out_dev, void *stream)
+{
+    if (!ctx || !layer_ok(l) || !X) return SSTE_ERR_INVALID_ARG;
+    float *x_amax = nullptr, *w_amax = nullptr;
+    if (fp8_of(l)) {
+        x_amax = l->amax;
+        w_amax = l->amax + 1;
+        const size_t n = static_cast<size_t>(l->T) * l->I;
+        sste_status st = sste_amax_scratch(ctx, X, n, x_amax, l->scratch, stream);
+        if (st == SSTE_OK) st = sste_quantize_fp8(ctx, X, n, x_amax, SSTE_E4M3, l->Xq, stream);
+        if (st != SSTE_OK) return st;
+        X = l->Xq;
+    }
+    return sste_linear_fwd(ctx, X, l->T, l->vals, l->meta, l->O, l->I, static_cast<sste_dtype>(l->op_dtype), x_amax, w_amax,
+                           l->Y, static_cast<sste_dtype>(l->out_dtype), y_amax_out_dev, stream);
+}
+
+extern "C" sste_status sste_layer_backward(sste_ctx *ctx, const sste_layer *l, const void *X, const void *dY, uint32_t step,
+                                           uint64_t token_offset, void *stream)
+{
+    if (!ctx || !layer_ok(l) || !dY) return SSTE_ERR_INVALID_ARG;
+    const bool fp8 = fp8_of(l);
+    const sste_dtype gdt = fp8 ? SSTE_E5M2 : SSTE_BF16, wdt = static_cast<sste_dtype>(l->op_dtype);
+    const sste_dtype odt = static_cast<sste_dtype>(l->out_dtype);
+    float *x_amax = fp8 ? l->amax : nullptr, *w_amax = fp8 ? l->amax + 1 : nullptr, *g_amax = fp8 ? l->amax + 2 : nullptr;
+    if (fp8) {
+        const sste_status st = sste_amax_scratch(ctx, dY, static_cast<size_t>(l->T) * l->O, g_amax, l->scratch, stream);
+        if (st != SSTE_OK) return st;
+    }
+    sste_status st = sste_mvue_sparsify(ctx, dY, l->T, l->O, SSTE_BF16, l->seed, l->tensor_id, step, token_offset,
+                                        l->counter_cols, g_amax, gdt, l->gvals, l->gmeta, fp8 ? l->dYq : nullptr, stream);
+    if (st != SSTE_OK) return st;
+    st = sste_linear_bwd_weight(ctx, l->gvals, l->gmeta, l->O, l->T, gdt, fp8 ? l->Xq : X, l->I, wdt, g_amax, x_amax, l->dW,
+                                odt, stream);
+    if (st != SSTE_OK) return st;
+    return sste_linear_bwd_input(ctx, fp8 ? l->dYq : dY, l->T, l->O, gdt, l->w_dense, l->w_dense ? nullptr : l->vals,
+                                 l->w_dense ? nullptr : l->meta, l->I, wdt, g_amax, w_amax, l->dX, odt, nullptr, stream);
+}

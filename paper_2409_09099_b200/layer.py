@@ -7,9 +7,16 @@ sparse weight and is meant to be applied to the dense weight unchanged.
 """
 from __future__ import annotations
 
+import ctypes
+
 import torch
 
 from . import binding as B
+
+# attributes the sste_layer descriptor is made of: setting one makes the next call build it anew
+_DESCRIBED = frozenset(("ctx", "W", "T", "tensor_id", "seed", "fp8", "counter_cols", "beta", "vals", "meta", "w_dense",
+                        "gvals", "gmeta", "Y", "dX", "dW", "amax", "Xq", "dYq", "_scratch"))
+_bf16, _raw_stream, _device = torch.bfloat16, torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
 
 
 class SsteLinear:
@@ -52,9 +59,40 @@ class SsteLinear:
             self.flips = torch.zeros(1, dtype=torch.int64, device=dev)   # mask entries changed by the last prune
             self._have_prev = False
         self.amax = torch.zeros(3, **f32) if fp8 else None     # max|X|, max|w~| (bf16 projection), max|dY|
+        self.Xq = self.dYq = self._scratch = None
         if fp8:
+            self._scratch = torch.zeros(2, dtype=torch.int32, device=dev)
             self.Xq = torch.empty((T, I), dtype=torch.float8_e4m3fn, device=dev)
             self.dYq = torch.empty((T, O), dtype=torch.float8_e5m2, device=dev)
+
+    def __setattr__(self, name, value):
+        if name in _DESCRIBED:
+            self.__dict__["_desc"] = None
+        self.__dict__[name] = value
+
+    # One C call per phase (prune, forward, backward) on buffers described once: what a small layer costs is host time.
+    # The per-call path below it runs when something wants to see the single calls or the tensors are of other sizes.
+    def _describe(self):
+        d = B.LayerBuffers(self.O, self.I, self.T, B.E4M3 if self.fp8 else B.BF16, B._CODE_OF[self.Y.dtype],
+                           self.counter_cols, self.tensor_id & 0xffffffff, 0, self.seed & 0xffffffffffffffff,
+                           *[B._ptr(t) for t in (self.W, self.beta, self.amax, self.vals, self.meta, self.w_dense,
+                                                 self.gvals, self.gmeta, self.Xq, self.dYq, self.Y, self.dX, self.dW,
+                                                 self._scratch)])
+        x_shape, g_shape = torch.Size((self.T, self.I)), torch.Size((self.T, self.O))
+        # a layer whose buffers were replaced by ones of other sizes or types is not described: the single calls check it
+        wdt, gdt = (B._TORCH_DT[B.E4M3], B._TORCH_DT[B.E5M2]) if self.fp8 else (_bf16, _bf16)
+        fits = (self.W.dtype is _bf16 and tuple(self.W.shape) == (self.O, self.I) and self.beta.dtype is torch.float32
+                and self.vals.dtype is wdt and tuple(self.vals.shape) == (self.O, self.I // 2)
+                and self.gvals.dtype is gdt and tuple(self.gvals.shape) == (self.O, self.T // 2)
+                and (self.w_dense is None or (self.w_dense.dtype is wdt and tuple(self.w_dense.shape) == (self.O, self.I)))
+                and self.Y.shape == g_shape and self.dX.shape == x_shape and tuple(self.dW.shape) == (self.O, self.I)
+                and self.dX.dtype is self.Y.dtype and self.dW.dtype is self.Y.dtype
+                and (not self.fp8 or (self.Xq.dtype is wdt and self.Xq.shape == x_shape
+                                      and self.dYq.dtype is gdt and self.dYq.shape == g_shape)))
+        lib = self.ctx.lib
+        self.__dict__["_desc"] = desc = (fits, ctypes.addressof(d), self.W.data_ptr(), lib.sste_layer_prune,
+                                         lib.sste_layer_forward, lib.sste_layer_backward, x_shape, g_shape, d)
+        return desc
 
     def _amax(self, k):
         return self.amax[k:k + 1] if self.fp8 else None
@@ -72,6 +110,14 @@ class SsteLinear:
     # (1) prune: w~ = beta * S_soft(W), compressed for the sparse products (and for grad_X)
     def prune(self):
         assert self.beta_ready, "call init_beta() in the first iteration"
+        if self.mark is None and not self.track_flips:
+            desc = self._desc or self._describe()
+            if desc[0] and self.W.data_ptr() == desc[2]:          # W is the caller's: its storage may have been exchanged
+                st = desc[3](self.ctx.handle, desc[1], _raw_stream(_device()))
+                if st:
+                    self.ctx._check(st)
+                self.__dict__["launches"] += 2 if self.fp8 else 1
+                return
         c = self.ctx
         if self.track_flips:
             self.meta, self.meta_prev = self.meta_prev, self.meta     # last iteration's image becomes "previous"
@@ -96,6 +142,19 @@ class SsteLinear:
 
     # (2a) forward with the sparse weight
     def forward(self, X, y_amax_out=None):
+        if self.mark is None:
+            desc = self._desc or self._describe()
+            if desc[0] and X.dtype is _bf16 and X.shape == desc[6] and X.is_cuda and X.is_contiguous():
+                st = desc[4](self.ctx.handle, desc[1], X.data_ptr(), B._ptr(y_amax_out), _raw_stream(_device()))
+                if st:
+                    self.ctx._check(st)
+                d = self.__dict__
+                if self.fp8:
+                    d["launches"] += 3
+                else:
+                    d["X"] = X
+                    d["launches"] += 1
+                return self.Y
         c = self.ctx
         if not self.fp8:
             self.X = X
@@ -115,6 +174,17 @@ class SsteLinear:
 
     # (2b) backward: MVUE on the output gradient for grad_W, dense product for grad_X
     def backward(self, dY, step: int = 0, token_offset: int = 0):
+        if self.mark is None:
+            desc = self._desc or self._describe()
+            X = None if self.fp8 else self.X
+            if (desc[0] and dY.dtype is _bf16 and dY.shape == desc[7] and dY.is_cuda and dY.is_contiguous()
+                    and (X is None or X.shape == desc[6])):
+                st = desc[5](self.ctx.handle, desc[1], None if X is None else X.data_ptr(), dY.data_ptr(), step, token_offset,
+                             _raw_stream(_device()))
+                if st:
+                    self.ctx._check(st)
+                self.__dict__["launches"] += 4 if self.fp8 else 3
+                return self.dX, self.dW
         self.sparsify_grad(dY, step, token_offset)
         self.grad_weight()
         self.grad_input(dY)
@@ -146,11 +216,7 @@ class SsteLinear:
         main = torch.cuda.current_stream()
         side_stream.wait_stream(main)
         with torch.cuda.stream(side_stream):
-            saved, self.ctx = self.ctx, side_ctx
-            try:
-                self.grad_weight()
-            finally:
-                self.ctx = saved
+            self.grad_weight(side_ctx)
         self.grad_input(dY)
         main.wait_stream(side_stream)
         return self.dX, self.dW
@@ -169,9 +235,9 @@ class SsteLinear:
         self.launches += 1
 
     # (2b.2) grad_W = MVUE(dY^T) X, sparse
-    def grad_weight(self):
+    def grad_weight(self, ctx: B.Context | None = None):
         self._m("linear_bwd_weight")
-        self.ctx.linear_bwd_weight(self.gvals, self.gmeta, self.Xq if self.fp8 else self.X, self.dW,
+        (ctx or self.ctx).linear_bwd_weight(self.gvals, self.gmeta, self.Xq if self.fp8 else self.X, self.dW,
                                    g_amax_dev=self._amax(2), x_amax_dev=self._amax(0))
         self.launches += 1
         return self.dW

@@ -1,0 +1,73 @@
+"""The one-call-per-phase path of a layer (sste_layer_prune / _forward / _backward) against the single calls.
+
+The layer takes the single calls when a `mark` callback wants to see them, so both paths run on the same buffers' shapes
+and must leave the same bits.  The FP8 maxima come without a memset there (a scratch word that every call leaves zero):
+checked over repeated iterations with maxima that shrink, and for a tensor of zeros.
+"""
+import pytest
+import torch
+
+from paper_2409_09099_b200 import synth
+from tests.gpu_util import DEV, dbf16
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    from paper_2409_09099_b200 import binding
+    c = binding.Context(0)
+    yield c
+    assert c.poll_device_status() == 0
+    c.close()
+
+
+def _bits(t):
+    return t.contiguous().view(torch.uint8)
+
+
+@pytest.mark.parametrize("fp8,dense_copy", [(False, True), (False, False), (True, True), (True, False)])
+@pytest.mark.parametrize("O,I,T", [(128, 128, 128), (384, 640, 256)])
+def test_layer_calls_equal_single_calls(ctx, O, I, T, fp8, dense_copy):
+    from paper_2409_09099_b200.layer import SsteLinear
+    W = dbf16(synth.gaussian_bf16(O + 11, (O, I), 0.02))
+    layers = [SsteLinear(ctx, W, T, tensor_id=4, seed=17, fp8=fp8, dense_copy=dense_copy) for _ in range(2)]
+    layers[1].mark = lambda label: None                     # the single calls
+    for step, scale in enumerate((1.0, 0.25, 0.0)):
+        X = dbf16(synth.gaussian_bf16(O + 12 + step, (T, I), 1.0)) * scale
+        dY = dbf16(synth.gaussian_bf16(O + 22 + step, (T, O), 1e-2)) * scale
+        for lin in layers:
+            if step == 0:
+                lin.init_beta()
+            lin.prune()
+            lin.forward(X)
+            lin.backward(dY, step=step, token_offset=4 * step)
+        a, b = layers
+        for name in ("vals", "meta", "gvals", "gmeta", "Y", "dX", "dW"):
+            assert torch.equal(_bits(getattr(a, name)), _bits(getattr(b, name))), (step, name)
+        if fp8:
+            assert torch.equal(a.amax, b.amax) and not a._scratch.any()
+        assert a.launches == b.launches
+
+
+def test_described_buffers_follow_the_attributes(ctx):
+    """A replaced buffer, exchanged weight storage or a shorter batch takes effect in the next call."""
+    from paper_2409_09099_b200.layer import SsteLinear
+    O, I, T = 256, 128, 256
+    W1, W2 = (dbf16(synth.gaussian_bf16(s, (O, I), 0.02)) for s in (31, 32))
+    X = dbf16(synth.gaussian_bf16(33, (T, I), 1.0))
+    lin = SsteLinear(ctx, W1.clone(), T)
+    lin.init_beta(); lin.prune()
+    Y1 = lin.forward(X).clone()
+    lin.W.data = W2                                          # same tensor object, other storage
+    lin.prune()
+    Y2 = lin.forward(X).clone()
+    ref = SsteLinear(ctx, W2, T)
+    ref.beta.copy_(lin.beta); ref.beta_ready = True
+    ref.prune()
+    assert torch.equal(Y2, ref.forward(X)) and not torch.equal(Y1, Y2)
+    lin.Y = torch.empty_like(lin.Y)
+    assert lin.forward(X) is lin.Y and torch.equal(lin.Y, Y2)
+    lin.Y.fill_(7.0)
+    lin.forward(X[:128])                                     # a shorter batch fills the first rows only
+    assert torch.equal(lin.Y[:128], Y2[:128]) and bool((lin.Y[128:] == 7.0).all())
