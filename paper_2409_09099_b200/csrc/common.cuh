@@ -33,6 +33,9 @@ constexpr size_t SSTE_WS_BYTES = SSTE_WS_PARTIALS_OFF + 2 * sizeof(double) * SST
 constexpr int SSTE_SPLITK_TICKETS = 2048;
 constexpr size_t SSTE_WS_SPLITK_TICKETS_OFF = (SSTE_WS_BYTES + 1023) / 1024 * 1024;
 constexpr size_t SSTE_WS_SPLITK_PARTIALS_OFF = SSTE_WS_SPLITK_TICKETS_OFF + SSTE_SPLITK_TICKETS * sizeof(unsigned int);
+// room that a dense copy of the weight in the workspace leaves to the partials: the most a plan asks for on 148 SMs
+// (73 split tiles x 4 ranges x 256 KB)
+constexpr size_t SSTE_DENSE_COPY_RESERVE = size_t(80) << 20;
 constexpr size_t SSTE_WS_RECOMMENDED_BYTES = SSTE_WS_SPLITK_PARTIALS_OFF + (size_t(192) << 20);
 
 static inline bool sste_mult128(int v) { return v > 0 && (v % 128) == 0; }
