@@ -168,6 +168,7 @@ class Context:
         if getattr(self, "handle", None):
             self.lib.sste_destroy(self.handle)
             self.handle = None
+            self.workspace = None      # 192 MB: not kept by whatever still refers to a closed context
 
     def __del__(self):
         try:

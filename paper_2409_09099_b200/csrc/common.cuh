@@ -30,7 +30,7 @@ constexpr size_t SSTE_WS_COUNTER_OFF = 64;
 constexpr size_t SSTE_WS_PARTIALS_OFF = 256;
 constexpr size_t SSTE_WS_BYTES = SSTE_WS_PARTIALS_OFF + 2 * sizeof(double) * SSTE_MAX_REDUCE_BLOCKS;
 // optional tail of the workspace, used by split-K products: arrival counters, then partial tiles
-constexpr int SSTE_SPLITK_TICKETS = 2048;
+constexpr int SSTE_SPLITK_TICKETS = 8192;
 constexpr size_t SSTE_WS_SPLITK_TICKETS_OFF = (SSTE_WS_BYTES + 1023) / 1024 * 1024;
 constexpr size_t SSTE_WS_SPLITK_PARTIALS_OFF = SSTE_WS_SPLITK_TICKETS_OFF + SSTE_SPLITK_TICKETS * sizeof(unsigned int);
 // room that a dense copy of the weight in the workspace leaves to the partials: the most a plan asks for on 148 SMs

@@ -27,8 +27,9 @@ namespace {
 
 constexpr int BM = 128;            // rows of A per CTA (a pair covers 256)
 constexpr int TMEM_COLS = 512;
-constexpr int MAX_SPLITS = 4;      // split-K factor limit
-constexpr int PANEL_BYTES = 2048;  // epilogue panel: 32 x 32 bf16
+constexpr int MAX_SPLITS = 16;     // split-K factor limit
+constexpr int MAX_PARTS = 2;       // parts that a warp's share of a split tile is exchanged in
+constexpr int PANEL_BYTES = 2048;  // epilogue panel: 32 rows x 32 columns of bf16
 constexpr unsigned long long WAIT_LIMIT_NS = 2000000000ull;   // two seconds of wall time (%globaltimer)
 
 enum class BMajor { K, MN };
@@ -204,6 +205,16 @@ __device__ __forceinline__ void tmem_ld_32x32(uint32_t taddr, uint32_t r[32])
           "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
         : "r"(taddr));
 }
+// 32 lanes x 16 consecutive 32-bit columns -> 16 registers per thread
+__device__ __forceinline__ void tmem_ld_32x16(uint32_t taddr, uint32_t r[16])
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr));
+}
 // 16 lanes x 32 consecutive 32-bit columns in the fragment layout of the 8 x 8 matrix stores: for the 8-column block b
 // thread t holds r[4b], r[4b + 1] = row t / 4, columns 2 (t % 4), + 1 and r[4b + 2], r[4b + 3] = the same of row t / 4 + 8
 __device__ __forceinline__ void tmem_ld_16x256_x4(uint32_t taddr, uint32_t r[16])
@@ -227,11 +238,39 @@ __device__ __forceinline__ void tmem_ld_32cols(uint32_t taddr, uint32_t *r)
         tmem_ld_32x32(taddr, r);
     }
 }
+// half h (registers 16 h .. 16 h + 15) of what tmem_ld_32cols loads
+template <bool TRANSPOSED>
+__device__ __forceinline__ void tmem_ld_half(uint32_t taddr, int h, uint32_t *r)
+{
+    if (TRANSPOSED) tmem_ld_16x256_x4(taddr + (static_cast<uint32_t>(16 * h) << 16), r);
+    else tmem_ld_32x16(taddr + 16 * h, r);
+}
 // four 8 x 8 matrices of 16-bit elements, stored transposed: thread t gives the address of row t % 8 of matrix t / 8
 __device__ __forceinline__ void stmatrix_x4_trans(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
 {
     asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1, %2, %3, %4};"
                  ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+__device__ __forceinline__ void pair_barrier(int id) { asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory"); }
+// Barrier of two warps that also combines a flag: true if all 64 threads passed true.
+__device__ __forceinline__ bool pair_barrier_and(int id, bool ok)
+{
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.b32 p, %1, 0;\n\t"
+        "bar.red.and.pred q, %2, 64, p;\n\t"
+        "selp.b32 %0, 1, 0, q;\n\t}"
+        : "=r"(r)
+        : "r"(ok ? 1u : 0u), "r"(id)
+        : "memory");
+    return r != 0;
+}
+__device__ __forceinline__ uint32_t ld_acquire_gpu(const unsigned int *a)
+{
+    uint32_t r;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(r) : "l"(a) : "memory");
+    return r;
 }
 __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
 {
@@ -300,7 +339,8 @@ struct GemmParams {
     int splits;             // split-K factor of the tiles from `split_from` on (1 = none)
     int split_from;         // first split tile: tiles below it are computed whole
     float *partials;        // split-K: fp32 partial tiles [split tile][cta][split][row quarter][BN / 4][32 lanes][4]
-    unsigned int *tickets;  // split-K: arrivals per [split tile][cta][epilogue warp]; zero between launches
+    unsigned int *tickets;  // split-K: claims (low half) and finished partials (high half) per [split tile][cta][epilogue
+                            // warp][part]; zero between launches
 };
 
 
@@ -321,7 +361,7 @@ struct Cfg {
     static constexpr int ROOM = 232448 - 1024 - 512;             // 227 KB of shared memory per CTA, slack, barriers
     static constexpr int FIT = (ROOM - EPI_WARPS * PANEL_BYTES) / STAGE;
     static constexpr int STAGES = FIT > 8 ? 8 : FIT;
-    // epilogue panels per warp: two (a panel is filled while the other is stored) where they fit
+    // staging: panels per epilogue warp, two where they fit
     static constexpr int PANELS = (ROOM - STAGES * STAGE >= 2 * EPI_WARPS * PANEL_BYTES) ? 2 : 1;
     static constexpr int STAGING_BYTES = EPI_WARPS * PANELS * PANEL_BYTES;
     static constexpr int ACC_BUFS = (!SPARSE || BN <= 224) ? 2 : 1;
@@ -521,21 +561,29 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     } else if (warp < 2 + C::EPI_WARPS) {
         // ------------------------------------------------------------ epilogue (warps 2.., both CTAs)
         // A warp owns 32 rows and a range of columns (half of them with eight warps) of the accumulator from tensor memory
-        // to the output and waits for no other warp.  Its part is pulled into registers (packed bf16) and the accumulator
-        // released before the first store, so that the next main loop waits for the tensor-memory reads only.  The chain of
-        // each panel (wait for the buffer, fill, proxy fence, store) is latency, hence eight warps and not four.
+        // to the output.  Its part is pulled into registers (packed bf16) and the accumulator released before the first
+        // store, so that the next main loop waits for the tensor-memory reads only.
+        // What leaves is whole 128-byte lines: a row-major output by boxes of 32 rows x 64 columns of one warp, a transposed
+        // one by boxes of 64 rows x 32 columns of a pair of warps (a warp alone has 64 bytes of each output row).  Half
+        // lines by TMA were 2-3 % slower (3840 x 1280, 16384 tokens, bf16 forward: 82 -> 80 us), by plain stores 25 %.
         const int quarter = warp & 3;                  // tensor-memory lanes [32*quarter, 32*quarter + 32)
         constexpr int PANELS_MAX = C::EPI_WARPS == 8 ? (BN / 32 + 1) / 2 : BN / 32;   // 32-column panels per warp
         const int pnl0 = ((warp - 2) >> 2) * PANELS_MAX;                              // first panel of this warp
         const int n_pnl = (C::EPI_WARPS == 8 && pnl0 > 0) ? BN / 32 - PANELS_MAX : PANELS_MAX;
+        constexpr int BOXP = (!OUT_T && C::PANELS == 2) ? 2 : 1;     // panels per box
+        constexpr int BOXES = OUT_T ? C::PANELS : 1;                 // boxes that the group's staging holds
+        const int group_bar = 1 + ((warp - 2) >> 1);                 // OUT_T: barrier of warps 2k, 2k + 1
+        const bool elect = lane == 0 && (!OUT_T || (warp & 1) == 0); // issues the group's stores
+        auto group_sync = [&] { if (OUT_T) pair_barrier(group_bar); else __syncwarp(); };
+        auto group_all = [&](bool ok) -> bool { return OUT_T ? pair_barrier_and(group_bar, ok) : __all_sync(0xffffffffu, ok); };
         const float scale = sste_out_scale(p.a_amax, p.a_fp8_max, p.b_amax, p.b_fp8_max);
         const bool want_amax = (p.out_amax != nullptr);
         const int kind = want_amax ? 2 : scale != 1.0f ? 1 : 0;      // what a stored value needs besides the rounding
         uint32_t amax2 = 0;                            // bf16 output: running max of the magnitude bits, two lanes of 16
         float amaxf = 0.0f;                            // fp32 output
         const uint32_t lane_base = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
-        const uint32_t my_staging = staging + (warp - 2) * (C::PANELS * PANEL_BYTES);
-        uint32_t local_tile = 0, panel_it = 0;
+        const uint32_t my_staging = staging + (OUT_T ? (warp - 2) & ~1 : warp - 2) * (C::PANELS * PANEL_BYTES);
+        uint32_t local_tile = 0, box_it = 0;
         // Two accumulator values -> one word of two bf16 (packed conversion).  KIND 0: unit scale and no amax wanted
         // (every bf16 product of the path); 1: scale; 2: scale and running maximum.
         auto pack2 = [&](float lo, float hi, auto kind_tag) -> uint32_t {
@@ -549,26 +597,28 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             if (KIND == 2) amax2 = __vmaxu2(amax2, w & 0x7fff7fffu);
             return w;
         };
-        // 32 columns (as tmem_ld_32cols leaves them) -> 16 packed words, ordered as store_panel takes them
-        auto pack_impl = [&](const uint32_t *r, uint32_t *w, auto kind_tag) {
+        // half h (tmem_ld_half) of 32 columns -> its 8 of the 16 packed words that store_box takes per panel
+        auto pack_impl = [&](const uint32_t *r, uint32_t *w, int h, auto kind_tag) {
             if (OUT_T) {
 #pragma unroll
                 for (int b = 0; b < 4; ++b)            // 8-column blocks
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) {      // 8-row blocks
-                        const int i = 16 * (k >> 1) + 4 * b + 2 * (k & 1);
-                        w[4 * b + k] = pack2(__uint_as_float(r[i]), __uint_as_float(r[i + 1]), kind_tag);
-                    }
+                    for (int k = 0; k < 2; ++k)        // 8-row blocks
+                        w[4 * b + 2 * h + k] = pack2(__uint_as_float(r[4 * b + 2 * k]), __uint_as_float(r[4 * b + 2 * k + 1]), kind_tag);
             } else {
 #pragma unroll
-                for (int i = 0; i < 16; ++i)
-                    w[i] = pack2(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1]), kind_tag);
+                for (int i = 0; i < 8; ++i)
+                    w[8 * h + i] = pack2(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1]), kind_tag);
             }
         };
+        auto pack_half = [&](const uint32_t *r, uint32_t *w, int h) {
+            if (kind == 0) pack_impl(r, w, h, std::integral_constant<int, 0>{});
+            else if (kind == 1) pack_impl(r, w, h, std::integral_constant<int, 1>{});
+            else pack_impl(r, w, h, std::integral_constant<int, 2>{});
+        };
         auto pack_chunk = [&](const uint32_t *r, uint32_t *w) {
-            if (kind == 0) pack_impl(r, w, std::integral_constant<int, 0>{});
-            else if (kind == 1) pack_impl(r, w, std::integral_constant<int, 1>{});
-            else pack_impl(r, w, std::integral_constant<int, 2>{});
+            pack_half(r, w, 0);
+            pack_half(r + 16, w, 1);
         };
         for (int unit = pair; unit < num_units; unit += num_pairs, ++local_tile) {
             const Unit u = decode(unit);
@@ -583,7 +633,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                 __syncwarp();
                 if (lane == 0) mbar_arrive_cluster(map_to_cta(acc_empty_bar(buf), 0));
             };
-            if (!mbar_wait_warp(acc_full_bar(buf), use & 1u, wc)) break;
+            // (a pair of warps leaves together when a wait expired: its barriers need both)
+            if (!group_all(mbar_wait_warp(acc_full_bar(buf), use & 1u, wc))) break;
             tc_fence_after();
             if (OUT_F32) {
                 const int m = m0 + quarter * 32 + lane;
@@ -615,106 +666,185 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                 release_acc();
                 continue;
             }
-            // A panel of 32 columns x this warp's 32 rows through one of two 2 KB buffers: 64-byte rows with the 64-byte
-            // swizzle of the TMA store (16-byte chunk index ^= (row >> 1) & 3), which keeps both kinds of store
-            // conflict-free.
-            auto store_panel = [&](int pnl, const uint32_t *w) {
-                const uint32_t sb = my_staging + (C::PANELS == 2 ? (panel_it & 1u) * PANEL_BYTES : 0u);
-                ++panel_it;
+            // BOXP packed panels of this warp -> staging (swizzled as the TMA store expects, conflict-free) -> output
+            auto store_box = [&](int pnl, const uint32_t *w) {
+                const uint32_t sb = my_staging + (BOXES == 2 ? (box_it & 1u) * (2 * PANEL_BYTES) : 0u);
+                ++box_it;
                 // the buffer is writable once the store issued from it last has read it
-                if (lane == 0) asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(C::PANELS - 1) : "memory");
-                __syncwarp();
+                if (elect) asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(BOXES - 1) : "memory");
+                group_sync();
                 if (OUT_T) {
-                    // staging row = column n of the accumulator, 32 m; matrix k = rows m 8k .. 8k + 7
+                    // staging row = column n of the accumulator, 64 m of the pair; matrix k = rows m 8k .. 8k + 7 of the warp
 #pragma unroll
                     for (int b = 0; b < 4; ++b) {
                         const uint32_t n = 8u * b + (lane & 7);
-                        stmatrix_x4_trans(sb + n * 64 + (((lane >> 3) ^ ((n >> 1) & 3)) << 4), w[4 * b], w[4 * b + 1],
-                                          w[4 * b + 2], w[4 * b + 3]);
+                        stmatrix_x4_trans(sb + n * 128 + (((4 * (quarter & 1) + (lane >> 3)) ^ (n & 7)) << 4), w[4 * b],
+                                          w[4 * b + 1], w[4 * b + 2], w[4 * b + 3]);
                     }
+                } else if (BOXP == 2) {
+#pragma unroll
+                    for (int c = 0; c < 8; ++c)
+                        st_shared_v4(sb + lane * 128 + ((c ^ (lane & 7)) << 4), w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
                 } else {
+                    // no room for whole lines (256-wide weight gradient): 64-byte rows, 64-byte swizzle
 #pragma unroll
                     for (int c = 0; c < 4; ++c)
                         st_shared_v4(sb + lane * 64 + ((c ^ ((lane >> 1) & 3)) << 4), w[4 * c], w[4 * c + 1], w[4 * c + 2],
                                      w[4 * c + 3]);
                 }
                 fence_proxy_async();
-                __syncwarp();
-                if (lane == 0) {
-                    if (OUT_T) tma_store_2d(&map_d, sb, m0 + 32 * quarter, n0 + 32 * pnl);
+                group_sync();
+                if (elect) {
+                    if (OUT_T) tma_store_2d(&map_d, sb, m0 + 64 * (quarter >> 1), n0 + 32 * pnl);
                     else tma_store_2d(&map_d, sb, n0 + 32 * pnl, m0 + 32 * quarter);
                     tma_store_commit();
                 }
             };
             if (unit >= p.split_from && p.splits > 1) {
-                // Split-K: every unit of the tile leaves its fp32 partial in the workspace, in the order of its own
-                // registers (512 contiguous bytes per warp and store); the warp whose ticket is the last one adds the
-                // partials of its rows in split order (bit-reproducible) and stores them.  No unit waits for another.
+                // Split-K.  The group's panels are exchanged in up to MAX_PARTS parts, which the units of a tile take in
+                // rotated order.  For each part a unit draws a number: all but the last to come leave their fp32 partial in
+                // the workspace (512 contiguous bytes per warp and store) and count it as finished; the last one keeps its
+                // own in tensor memory, waits for the others' (they are past their main loop and wait for nobody: the
+                // wait ends whatever else the GPU runs), adds all in split order (bit-reproducible) and stores the result.  With
+                // the rotation each unit ends up last for about its share of the parts.  (When the unit that came last
+                // read all partials, its own too, and added up the whole tile, an exchange took 10 us; now 5-6 us between two
+                // units, 8-10 between four.  3072 x 768, 8192 tokens, bf16 grad_W: 26.2 -> 22.5 us.)
                 constexpr size_t PART = static_cast<size_t>(BN / 4) * 32;          // float4 per 32 rows and split
-                const size_t slot = (static_cast<size_t>(u.tile - p.split_from) * 2 + rank) * p.splits;
-                float4 *part0 = reinterpret_cast<float4 *>(p.partials) + (slot * 4 + quarter) * PART + lane;
-                float4 *mine = part0 + static_cast<size_t>(u.split) * 4 * PART;
+                const size_t slot = static_cast<size_t>(u.tile - p.split_from) * 2 + rank;
+                float4 *part0 = reinterpret_cast<float4 *>(p.partials) + (slot * p.splits * 4 + quarter) * PART + lane;
+                unsigned int *tickets = p.tickets + (slot * C::EPI_WARPS + (OUT_T ? (warp - 2) & ~1 : warp - 2)) * MAX_PARTS;
+                const int n_box = n_pnl / BOXP;
+                const int parts = min(n_box, MAX_PARTS);
+                constexpr int AHEAD = 2;               // (three spill registers of the ordinary epilogue)
+                bool ok = true;
+                uint32_t drawn = 0;
+                if (elect) drawn = atomicAdd(tickets + u.split % parts, 1u);
 #pragma unroll 1
-                for (int c0 = 32 * pnl0; c0 < 32 * (pnl0 + n_pnl); c0 += 32) {
-                    uint32_t r[32];
-                    tmem_ld_32cols<OUT_T>(acc_base + c0, r);
-                    tmem_ld_wait();
-#pragma unroll
-                    for (int i = 0; i < 8; ++i)
-                        __stcg(mine + (c0 / 4 + i) * 32, make_float4(__uint_as_float(r[4 * i]), __uint_as_float(r[4 * i + 1]),
-                                                                     __uint_as_float(r[4 * i + 2]), __uint_as_float(r[4 * i + 3])));
-                }
-                release_acc();
-                unsigned int last = 0;
-                if (lane == 0) {
-                    unsigned int *ticket = p.tickets + (static_cast<size_t>(u.tile - p.split_from) * 2 + rank) * C::EPI_WARPS + (warp - 2);
-                    __threadfence();                   // the warp's partial before the ticket (ordered by __syncwarp above)
-                    last = (atomicAdd(ticket, 1u) == static_cast<unsigned int>(p.splits) - 1u) ? 1u : 0u;
-                    if (last) *ticket = 0u;            // zero again for the next launch
-                    __threadfence();                   // the ticket before the others' partials
-                }
-                if (!__shfl_sync(0xffffffffu, last, 0)) continue;
-                __syncwarp();
+                for (int k = 0; k < parts && ok; ++k) {
+                    const int part = (u.split + k) % parts;
+                    const int box_lo = part * n_box / parts, box_hi = (part + 1) * n_box / parts;
+                    const int lo = pnl0 + box_lo * BOXP, hi = pnl0 + box_hi * BOXP;
+                    unsigned int *ticket = tickets + part;
+                    if (group_all(!elect || (drawn & 0xffffu) != static_cast<unsigned int>(p.splits) - 1u)) {
+                        float4 *mine = part0 + static_cast<size_t>(u.split) * 4 * PART;
 #pragma unroll 1
-                for (int pnl = pnl0; pnl < pnl0 + n_pnl; ++pnl) {
-                    const float4 *src = part0 + pnl * 8 * 32;
-                    uint32_t v[32], w[16];
+                        for (int pnl = lo; pnl < hi; ++pnl) {
+                            uint32_t r[32];
+                            tmem_ld_32cols<OUT_T>(acc_base + 32 * pnl, r);
+                            tmem_ld_wait();
 #pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        float4 q[MAX_SPLITS][4];       // all partials of half a panel in flight at once
-#pragma unroll
-                        for (int sp = 0; sp < MAX_SPLITS; ++sp) {
-                            if (sp >= p.splits) break;
-#pragma unroll
-                            for (int i = 0; i < 4; ++i)
-                                q[sp][i] = __ldcg(src + static_cast<size_t>(sp) * 4 * PART + (4 * h + i) * 32);
+                            for (int i = 0; i < 8; ++i)
+                                __stcg(mine + (8 * pnl + i) * 32,
+                                       make_float4(__uint_as_float(r[4 * i]), __uint_as_float(r[4 * i + 1]),
+                                                   __uint_as_float(r[4 * i + 2]), __uint_as_float(r[4 * i + 3])));
                         }
-#pragma unroll
-                        for (int sp = 1; sp < MAX_SPLITS; ++sp) {
-                            if (sp >= p.splits) break;
-#pragma unroll
-                            for (int i = 0; i < 4; ++i) {
-                                q[0][i].x = __fadd_rn(q[0][i].x, q[sp][i].x);
-                                q[0][i].y = __fadd_rn(q[0][i].y, q[sp][i].y);
-                                q[0][i].z = __fadd_rn(q[0][i].z, q[sp][i].z);
-                                q[0][i].w = __fadd_rn(q[0][i].w, q[sp][i].w);
+                        group_sync();
+                        if (elect) {
+                            if (k + 1 < parts) drawn = atomicAdd(tickets + (u.split + k + 1) % parts, 1u);   // on its way meanwhile
+                            __threadfence();               // the group's partial (ordered by group_sync) before the count
+                            atomicAdd(ticket, 0x10000u);
+                        }
+                        continue;
+                    }
+                    if (elect) {
+                        const uint32_t all = (static_cast<uint32_t>(p.splits) << 16) - 0x10000u + static_cast<uint32_t>(p.splits);
+                        if (ld_acquire_gpu(ticket) != all) {
+                            const unsigned long long start = global_ns();
+                            while (ok && ld_acquire_gpu(ticket) != all) {
+                                if (*wc.abort_flag) ok = false;
+                                else if (global_ns() - start > wc.limit_ns) {
+                                    atomicCAS(wc.status, 0u, static_cast<unsigned int>(SSTE_ERR_TIMEOUT));
+                                    *wc.abort_flag = 1;
+                                    ok = false;
+                                }
                             }
                         }
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            v[16 * h + 4 * i] = __float_as_uint(q[0][i].x);
-                            v[16 * h + 4 * i + 1] = __float_as_uint(q[0][i].y);
-                            v[16 * h + 4 * i + 2] = __float_as_uint(q[0][i].z);
-                            v[16 * h + 4 * i + 3] = __float_as_uint(q[0][i].w);
-                        }
+                        if (ok) *ticket = 0u;              // zero again for the next launch
+                        if (k + 1 < parts) drawn = atomicAdd(tickets + (u.split + k + 1) % parts, 1u);
                     }
-                    pack_chunk(v, w);
-                    store_panel(pnl, w);
+                    ok = group_all(ok);
+                    if (!ok) break;
+                    if (p.splits == 2) {
+                        // one other partial, and a sum of two has no order: the next panel is on its way while one is stored
+                        const float4 *src = part0 + static_cast<size_t>(1 - u.split) * 4 * PART;
+                        float4 q[8];
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) q[i] = __ldcg(src + (8 * lo + i) * 32);
+                        uint32_t w[16 * BOXP];
+#pragma unroll 1
+                        for (int pnl = lo; pnl < hi; pnl += BOXP) {
+#pragma unroll
+                            for (int b = 0; b < BOXP; ++b) {
+                                uint32_t own[32];
+                                tmem_ld_32cols<OUT_T>(acc_base + 32 * (pnl + b), own);
+                                tmem_ld_wait();
+#pragma unroll
+                                for (int i = 0; i < 8; ++i) {
+                                    own[4 * i] = __float_as_uint(__fadd_rn(__uint_as_float(own[4 * i]), q[i].x));
+                                    own[4 * i + 1] = __float_as_uint(__fadd_rn(__uint_as_float(own[4 * i + 1]), q[i].y));
+                                    own[4 * i + 2] = __float_as_uint(__fadd_rn(__uint_as_float(own[4 * i + 2]), q[i].z));
+                                    own[4 * i + 3] = __float_as_uint(__fadd_rn(__uint_as_float(own[4 * i + 3]), q[i].w));
+                                }
+                                if (pnl + b + 1 < hi) {
+#pragma unroll
+                                    for (int i = 0; i < 8; ++i) q[i] = __ldcg(src + (8 * (pnl + b + 1) + i) * 32);
+                                }
+                                pack_chunk(own, w + 16 * b);
+                            }
+                            store_box(pnl, w);
+                        }
+                        continue;
+                    }
+#pragma unroll 1
+                    for (int pnl = lo; pnl < hi; pnl += BOXP) {
+                        uint32_t w[16 * BOXP];
+#pragma unroll
+                        for (int b = 0; b < BOXP; ++b) {
+                            const float4 *src = part0 + (pnl + b) * 8 * 32;
+#pragma unroll
+                            for (int h = 0; h < 2; ++h) {
+                                uint32_t v[16];
+#pragma unroll 1
+                                for (int sp = 0; sp < p.splits; sp += AHEAD) {
+                                    uint32_t q[AHEAD][16];     // half a panel of AHEAD splits in flight
+#pragma unroll
+                                    for (int d = 0; d < AHEAD; ++d) {
+                                        if (sp + d >= p.splits) break;
+                                        if (sp + d == u.split) {
+                                            tmem_ld_half<OUT_T>(acc_base + 32 * (pnl + b), h, q[d]);
+                                        } else {
+#pragma unroll
+                                            for (int i = 0; i < 4; ++i) {
+                                                const float4 x = __ldcg(src + static_cast<size_t>(sp + d) * 4 * PART + (4 * h + i) * 32);
+                                                q[d][4 * i] = __float_as_uint(x.x);
+                                                q[d][4 * i + 1] = __float_as_uint(x.y);
+                                                q[d][4 * i + 2] = __float_as_uint(x.z);
+                                                q[d][4 * i + 3] = __float_as_uint(x.w);
+                                            }
+                                        }
+                                    }
+                                    tmem_ld_wait();
+#pragma unroll
+                                    for (int d = 0; d < AHEAD; ++d) {
+                                        if (sp + d >= p.splits) break;
+#pragma unroll
+                                        for (int i = 0; i < 16; ++i)
+                                            v[i] = (d == 0 && sp == 0) ? q[0][i]
+                                                                       : __float_as_uint(__fadd_rn(__uint_as_float(v[i]), __uint_as_float(q[d][i])));
+                                    }
+                                }
+                                pack_half(v, w + 16 * b, h);
+                            }
+                        }
+                        store_box(pnl, w);
+                    }
                 }
+                release_acc();
+                if (!ok) break;
             } else {
                 // at most four panels are held packed in registers at a time
                 constexpr int HOLD = PANELS_MAX < 4 ? PANELS_MAX : 4;
-                static_assert(PANELS_MAX % HOLD == 0, "whole rounds of panels");
+                static_assert(PANELS_MAX % HOLD == 0 && HOLD % BOXP == 0, "whole rounds of panels");
 #pragma unroll
                 for (int h0 = 0; h0 < PANELS_MAX; h0 += HOLD) {
                     uint32_t pk[16 * HOLD];
@@ -731,8 +861,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                     }
                     if (h0 + HOLD == PANELS_MAX) release_acc();
 #pragma unroll
-                    for (int i = 0; i < HOLD; ++i)
-                        if (h0 + i < n_pnl) store_panel(pnl0 + h0 + i, pk + 16 * i);
+                    for (int i = 0; i < HOLD; i += BOXP)
+                        if (h0 + i < n_pnl) store_box(pnl0 + h0 + i, pk + 16 * i);
                 }
             }
         }
@@ -743,7 +873,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             for (int off = 16; off > 0; off >>= 1) best = max(best, __shfl_xor_sync(0xffffffffu, best, off));
             if (lane == 0 && best != 0) atomicMax(p.out_amax, best);
         }
-        if (lane == 0 && !OUT_F32) tma_store_wait_all();
+        if (elect && !OUT_F32) tma_store_wait_all();
     } else if (BCOMP) {
         // ------------------------------------------------------------ expander warps (6..9, both CTAs)
         // grad_X = grad_Z S(W) reads S(W) [O, I] as its MN-major B operand.  Here S(W) is given as the forward's
@@ -941,11 +1071,11 @@ struct TileCost { double stage_us, tile_us; };
 constexpr TileCost tile_cost(Product pr, int elt, int bn)
 {
     if (pr == FORWARD && elt == 2)
-        return bn == 256 ? TileCost{0.50, 1.6} : bn == 224 ? TileCost{0.385, 1.4} : bn == 192 ? TileCost{0.34, 1.25} : TileCost{0.24, 1.3};
+        return bn == 256 ? TileCost{0.46, 1.6} : bn == 224 ? TileCost{0.44, 0.9} : bn == 192 ? TileCost{0.40, 0.8} : TileCost{0.31, 0.75};
     if (pr == FORWARD)
-        return bn == 256 ? TileCost{0.45, 2.2} : bn == 224 ? TileCost{0.48, 1.4} : bn == 192 ? TileCost{0.43, 0.95} : TileCost{0.34, 0.9};
-    if (pr == GRAD_WEIGHT) return bn == 256 ? TileCost{elt == 2 ? 0.42 : 0.49, 0.5} : TileCost{0.40, 0.5};
-    return bn == 256 ? TileCost{0.33, 0.6} : TileCost{0.28, 0.6};
+        return bn == 256 ? TileCost{0.53, 2.0} : bn == 224 ? TileCost{0.46, 1.65} : bn == 192 ? TileCost{0.41, 1.55} : TileCost{0.33, 1.3};
+    if (pr == GRAD_WEIGHT) return bn == 256 ? TileCost{elt == 2 ? 0.405 : 0.47, 1.0} : TileCost{0.345, 0.9};
+    return bn == 256 ? TileCost{0.34, elt == 2 ? 1.1 : 1.4} : TileCost{0.27, 1.0};
 }
 
 // Everything the host decides about one product launch.
@@ -954,8 +1084,9 @@ struct LaunchPlan { int bn, splits, split_from, group_m; };
 // Tile width and split-K factor by the model's time.  Tiles that fill complete waves of CTA pairs are computed whole; the
 // tiles of the last, partial wave (all of them when there are fewer tiles than pairs, as for the weight gradient of a
 // GPT-2-sized layer: 36 tiles, 74 pairs) may be cut into `splits` K ranges of at least eight stages, so that the wave
-// takes 1/splits of a tile time and the partials' round trip through L2 on top: measured 5-17 us, close to
-// bn/256 (5.5 + splits) us of latency + the bytes written and read at 8 MB/us.  Among widths within 3 % the first wins.
+// takes 1/splits of a tile time and the exchange of the partials on top: 2.4 + 2.6 bn/256 us between two units,
+// 4.4 + 3.8 bn/256 between three and so on (measured at 9 ... 36 tiles), and their bytes.  Among widths within 3 % the
+// first wins.
 LaunchPlan make_plan(Product pr, int elt, int only_bn, bool out_f32, bool bcomp, int sm_count, size_t partial_bytes, int M,
                      int N, int K)
 {
@@ -979,10 +1110,12 @@ LaunchPlan make_plan(Product pr, int elt, int only_bn, bool out_f32, bool bcomp,
             if (s > 1) {
                 // behind whole waves equal ranges only (an uneven split gains less than the exchange costs there)
                 if (out_f32 || tail == 0 || k_blocks / s < 8 || (whole > 0 && k_blocks % s != 0)) continue;
-                if (tail * 16 > SSTE_SPLITK_TICKETS) continue;
+                if (s > 4 && (whole > 0 || tail * s > pairs)) continue;      // many ranges: for a few tiles of a long reduction
+                if (tail * 2 * 8 * MAX_PARTS > SSTE_SPLITK_TICKETS) continue;
                 const size_t bytes = static_cast<size_t>(tail) * s * 2 * BM * bn * sizeof(float);
                 if (bytes > partial_bytes) continue;
-                us += bn / 256.0 * (5.5 + s) + 2.0 * bytes / 8e6;
+                us += s == 2 ? 2.4 + 2.6 * bn / 256.0 : 2.5 + 0.65 * s + (2.6 + 0.4 * s) * bn / 256.0;
+                us += bytes / 15e6;
             }
             if (tail) us += ((tail * s + pairs - 1) / pairs) * ((k_blocks + s - 1) / s * c.stage_us + c.tile_us);
             const bool wanted = (g_force_splits == s && best.bn == bn);      // the hook applies where the shape allows it
@@ -1020,9 +1153,11 @@ sste_status launch(const sste_ctx *ctx, const void *A, const void *B, const void
         ok = ok && make_map(ctx, &map_b, B, ELT, p.K, p.N, 128 / ELT, BK, CU_TENSOR_MAP_SWIZZLE_128B);
     if (OUT_F32) {
         map_d = map_a;       // unused: the fp32 epilogue stores directly
-    } else if (OUT_T) {      // out[N, M] bf16: panels of 32 m x 32 n, 64-byte swizzle
-        ok = ok && make_map(ctx, &map_d, p.D, 2, p.N, p.M, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B);
-    } else {                 // out[M, N] bf16: panels of 32 n x 32 m, 64-byte swizzle
+    } else if (OUT_T) {      // out[N, M] bf16: boxes of 64 m x 32 n
+        ok = ok && make_map(ctx, &map_d, p.D, 2, p.N, p.M, 64, 32, CU_TENSOR_MAP_SWIZZLE_128B);
+    } else if (C::PANELS == 2) {   // out[M, N] bf16: boxes of 64 n x 32 m
+        ok = ok && make_map(ctx, &map_d, p.D, 2, p.M, p.N, 64, 32, CU_TENSOR_MAP_SWIZZLE_128B);
+    } else {                 // out[M, N] bf16: boxes of 32 n x 32 m
         ok = ok && make_map(ctx, &map_d, p.D, 2, p.M, p.N, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B);
     }
     if (SPARSE)              // metadata image as rows of 512 bytes, four per atom
@@ -1087,7 +1222,7 @@ sste_status launch_out(const sste_ctx *ctx, const void *A, const void *B, const 
     constexpr bool SPARSE = (PR != GRAD_INPUT), OUT_T = (PR == FORWARD);
     constexpr BMajor BMAJ = (PR == FORWARD) ? BMajor::K : BMajor::MN;
     if (odt != SSTE_F32 && odt != SSTE_BF16) return SSTE_ERR_DTYPE;
-    const LaunchPlan plan = make_plan(PR, ELT, odt == SSTE_F32 ? 256 : 0, odt == SSTE_F32, false, ctx->sm_count,
+    const LaunchPlan plan = make_plan(PR, ELT, odt == SSTE_F32 || g_inject_stall ? 256 : 0, odt == SSTE_F32, false, ctx->sm_count,
                                       ctx->splitk_partials ? ctx->splitk_partial_bytes : 0, p.M, p.N, p.K);
     if (odt == SSTE_F32) return launch<SPARSE, BMAJ, ELT, 256, OUT_T, true>(ctx, A, B, meta, p, plan, s);
     if constexpr (PR == FORWARD) {
@@ -1249,6 +1384,7 @@ extern "C" sste_status sste_linear_bwd_input(sste_ctx *ctx, const void *dY, int 
                  reinterpret_cast<unsigned int *>(dx_amax_out_dev), ctx->status_dev, ca, cb, nullptr};
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (!Wt_dense) {
+        if (g_inject_stall) return SSTE_ERR_INVALID_ARG;      // the hook is for the dense operand only
         // S(W) from the forward's compressed operand.  Where the workspace has room for the dense copy (in its last bytes;
         // split-K partials stay in front of it), it is expanded there first and the dense product runs on it: the same
         // bits, and one pass over the weight costs little (1280 x 5120, 16384 tokens, bf16: 511 -> 152 us for both).

@@ -2,6 +2,8 @@
 
 dst is compared whole, with elements in front of and behind it that must stay as they were.
 """
+import gc
+
 import pytest
 import torch
 
@@ -17,6 +19,7 @@ def ctx():
     yield c
     assert c.poll_device_status() == 0
     c.close()
+    gc.collect()      # models of earlier tests hold GPU memory through reference cycles: not left to chance
 
 
 def _at(offset, rows, cols, fill=None):
