@@ -273,10 +273,13 @@ typedef struct sste_layer {
 sste_status sste_layer_prune(sste_ctx *ctx, const sste_layer *layer, void *stream);
 /* sste_linear_fwd of X (FP8: after sste_amax and sste_quantize_fp8 of it).  X bf16 [T, I]. */
 sste_status sste_layer_forward(sste_ctx *ctx, const sste_layer *layer, const void *X, float *y_amax_out_dev, void *stream);
-/* sste_mvue_sparsify of dY (FP8: after sste_amax of it), sste_linear_bwd_weight with X (FP8: with the layer's Xq; X may
- * be NULL), sste_linear_bwd_input.  dY bf16 [T, O]. */
+/* sste_mvue_sparsify of dY (FP8: after sste_amax of it), then sste_layer_grads.  dY bf16 [T, O]. */
 sste_status sste_layer_backward(sste_ctx *ctx, const sste_layer *layer, const void *X, const void *dY, uint32_t step,
                                 uint64_t token_offset, void *stream);
+/* grad_W and grad_X after sste_mvue_sparsify: sste_linear_bwd_weight with X (FP8: with the layer's Xq; X may be NULL) and
+ * sste_linear_bwd_input.  With bf16 outputs both run in ONE launch: the pairs of SMs that grad_W's tiles leave idle start
+ * on grad_X's.  (The split of grad_W's reduction may then differ from the single call's: same sums, other rounding.) */
+sste_status sste_layer_grads(sste_ctx *ctx, const sste_layer *layer, const void *X, const void *dY, void *stream);
 
 /* ---- ablation variants of the pruning step (the axes of the paper's ablations; not on the default path) ---- */
 
@@ -387,6 +390,11 @@ sste_status sste_debug_mvue_groups(sste_ctx *ctx, const void *a, const void *k24
  * above apply.  sste_debug_tile_coords maps a tile number to its (row, column) of tiles under a band height. */
 sste_status sste_debug_plan(int product, sste_dtype opdt, int O, int I, int T, int sm_count, size_t workspace_bytes,
                             int *tile_width, int *splits, int *split_from, int *group_m);
+/* The plan of a one-launch grad_W + grad_X (sste_layer_grads), host only; out: grad_W's tile width, split factor, first
+ * split tile, band height; grad_X's tile width, band height; CTA pairs; how many of them have a grad_W unit more than the
+ * others; the rounds of grad_X tiles that the others take among themselves first; whether they also come first in the
+ * rounds after. */
+sste_status sste_debug_joint_plan(sste_dtype opdt, int O, int I, int T, int sm_count, size_t workspace_bytes, int out[10]);
 sste_status sste_debug_tile_coords(int tile, int m_tiles, int n_tiles, int group_m, int *mt, int *nt);
 
 /* Host-only self-check of the once-per-device bookkeeping behind per-device kernel attributes (a context may live on

@@ -33,7 +33,7 @@ EXPORTS = [
     "sste_decompress", "sste_padded_dim", "sste_pad_2d", "sste_crop_2d", "sste_debug_inject_stall",
     "sste_debug_force_tile_order", "sste_debug_plan", "sste_debug_tile_coords",
     "sste_debug_mvue_groups", "sste_debug_selftest_device_once", "sste_layer_prune", "sste_layer_forward",
-    "sste_layer_backward",
+    "sste_layer_backward", "sste_layer_grads", "sste_debug_joint_plan",
 ]
 
 _P, _I, _Z, _U32, _U64, _F = (ctypes.c_void_p, ctypes.c_int, ctypes.c_size_t, ctypes.c_uint32, ctypes.c_uint64,
@@ -55,6 +55,7 @@ _ARGTYPES = {
     "sste_layer_prune": [_P, _P, _P],
     "sste_layer_forward": [_P, _P, _P, _P, _P],
     "sste_layer_backward": [_P, _P, _P, _P, _U32, _U64, _P],
+    "sste_layer_grads": [_P, _P, _P, _P, _P],
 }
 
 
@@ -128,6 +129,17 @@ def plan(product: int, opdt: int, O: int, I: int, T: int, sm_count: int = 148, w
     if st != OK:
         raise SsteError(st, lib.sste_status_string(st).decode())
     return tuple(o.value for o in out)
+
+
+def joint_plan(opdt: int, O: int, I: int, T: int, sm_count: int = 148, workspace_bytes: int | None = None):
+    """sste_debug_joint_plan: the ten numbers of a one-launch grad_W + grad_X, in the order of the header; host only."""
+    lib = load()
+    ws = lib.sste_workspace_bytes_recommended() if workspace_bytes is None else workspace_bytes
+    out = (ctypes.c_int * 10)()
+    st = lib.sste_debug_joint_plan(opdt, O, I, T, sm_count, ctypes.c_size_t(ws), out)
+    if st != OK:
+        raise SsteError(st, lib.sste_status_string(st).decode())
+    return tuple(out)
 
 
 def launch_count() -> int:

@@ -157,3 +157,10 @@ void sste_count_launches(int n);
 sste_status sste_amax_scratch(sste_ctx *ctx, const void *x, size_t n, float *amax_dev, void *scratch, void *stream);
 sste_status sste_project_amax_scratch(sste_ctx *ctx, const void *W, int O, int I, const float *beta_dev, float *amax_dev,
                                       void *scratch, void *stream);
+
+// grad_W and grad_X of a layer (the two products behind sste_linear_bwd_weight and sste_linear_bwd_input, same arguments), in
+// one launch where that is possible.
+sste_status sste_bwd_products(sste_ctx *ctx, const void *gvals, const void *gmeta, const void *X, const void *dY, int O, int I,
+                              int T, sste_dtype gdt, sste_dtype wdt, const void *w_dense, const void *vals, const void *meta,
+                              const float *g_amax, const float *x_amax, const float *w_amax, void *dW, void *dX,
+                              sste_dtype odt, void *stream);

@@ -27,6 +27,9 @@ namespace {
 
 constexpr int BM = 128;            // rows of A per CTA (a pair covers 256)
 constexpr int TMEM_COLS = 512;
+// Shared memory starts with a control block: barriers of the kernel's first product at 0 and of its second at 512, the
+// expander's selector table at 256, the tensor-memory address at 1008 and the abort flag at 1016.
+constexpr int CTRL_BYTES = 1024, CTRL_SECOND = 512, CTRL_LUT = 256, CTRL_TMEM = 1008, CTRL_ABORT = 1016;
 constexpr int MAX_SPLITS = 16;     // split-K factor limit
 constexpr int MAX_PARTS = 2;       // parts that a warp's share of a split tile is exchanged in
 constexpr int PANEL_BYTES = 2048;  // epilogue panel: 32 rows x 32 columns of bf16
@@ -358,7 +361,7 @@ struct Cfg {
     static constexpr int ATOMS = SPARSE ? 256 / ELT / 128 : 0;   // metadata atoms (128 logical K, 2 KB) per stage
     static constexpr int STAGE = A_STAGE + B_STAGE + 2048 * ATOMS;
     static constexpr int EPI_WARPS = BCOMP ? 4 : 8;              // compressed B: the other four expand
-    static constexpr int ROOM = 232448 - 1024 - 512;             // 227 KB of shared memory per CTA, slack, barriers
+    static constexpr int ROOM = 232448 - 1024 - CTRL_BYTES;      // 227 KB of shared memory per CTA, alignment slack, control block
     static constexpr int FIT = (ROOM - EPI_WARPS * PANEL_BYTES) / STAGE;
     static constexpr int STAGES = FIT > 8 ? 8 : FIT;
     // staging: panels per epilogue warp, two where they fit
@@ -368,22 +371,45 @@ struct Cfg {
     static constexpr int META_COL0 = ACC_BUFS * BN;              // metadata regions follow the accumulators
     static constexpr int META_COLS = 4 * ATOMS;                  // tensor-memory columns of one stage's metadata
     static constexpr int THREADS = 320;
-    static constexpr int SMEM_BYTES = STAGES * STAGE + STAGING_BYTES + 1024 /* alignment slack */ + 512 /* barriers */;
+    static constexpr int SMEM_BYTES = 1024 /* alignment slack */ + CTRL_BYTES + STAGES * STAGE + STAGING_BYTES;
     static_assert(META_COL0 + STAGES * META_COLS <= TMEM_COLS, "tensor memory budget");
     static_assert(STAGES >= 3, "pipeline depth");
     static_assert(STAGE % 1024 == 0 && BN % 32 == 0, "swizzle alignment, epilogue panels");
 };
 
+// The units a pair works on, in order, until one is out of range: `early` rounds over `early_pairs` pairs only (those that
+// have nothing to do before), then rounds over all `pairs` from unit `base` on.
+struct UnitSeq {
+    int early, early_pairs, early_rank, base, pairs, rank;
+    __device__ __forceinline__ int first() const { return early > 0 ? early_rank : base + rank; }
+    // the unit after `unit`; j: its number in the pair's order
+    __device__ __forceinline__ int next(int unit, int j) const
+    {
+        return j < early ? unit + early_pairs : (early > 0 && j == early) ? base + rank : unit + pairs;
+    }
+};
+
+template <typename C, bool BCOMP>
+__device__ __forceinline__ void init_barriers(uint32_t bars)
+{
+    constexpr int NS = C::STAGES;
+    static_assert(8 * (2 * NS + 4) <= CTRL_LUT, "barrier block");
+    // full: the producer's arrival with the TMA byte count (+ the eight expander warps of the pair)
+    for (int s = 0; s < NS; ++s) { mbar_init(bars + 8u * s, BCOMP ? 9 : 1); mbar_init(bars + 8u * (NS + s), 1); }
+    for (int b = 0; b < 2; ++b) { mbar_init(bars + 8u * (2 * NS + b), 1); mbar_init(bars + 8u * (2 * NS + 2 + b), 2 * C::EPI_WARPS); }
+}
+
+// One product on a CTA pair: all warp roles, from the first unit of `seq` to the last.
 // ELT: operand element size in bytes (2 = bf16 via kind::f16, 1 = fp8 via kind::f8f6f4).
 // OUT_T: store D transposed (out[n, m]); OUT_F32: fp32 output (direct stores) instead of bf16 (TMA stores).
 // BCOMP: the (dense-product) B operand is given in compressed 2:4 form and expanded in shared memory.
-template <bool SPARSE, BMajor BMAJ, int ELT, int BN, bool OUT_T, bool OUT_F32, bool BCOMP = false>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Cfg<SPARSE, ELT, BN, BCOMP>::THREADS, 1)
-gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
-            const __grid_constant__ CUtensorMap map_d, const __grid_constant__ CUtensorMap map_m,
-            const uint8_t *__restrict__ meta, const GemmParams p)
+// FINAL: nothing follows in the kernel (else another product reuses the shared memory).
+template <bool SPARSE, BMajor BMAJ, int ELT, int BN, bool OUT_T, bool OUT_F32, bool BCOMP, bool FINAL>
+__device__ __forceinline__ void
+product(const CUtensorMap &map_a, const CUtensorMap &map_b, const CUtensorMap &map_d, const CUtensorMap &map_m,
+        const uint8_t *__restrict__ meta, const GemmParams &p, const UnitSeq &seq, uint8_t *ctrl_generic, uint32_t bars,
+        uint32_t smem_base, uint32_t tmem_base, const WaitCtx &wc)
 {
-    sste_pdl_trigger();
     using C = Cfg<SPARSE, ELT, BN, BCOMP>;
     constexpr int NS = C::STAGES;
     constexpr int NB = C::ACC_BUFS;
@@ -397,26 +423,15 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     static_assert(BMAJ == BMajor::K || (BN / 2) % B_CHUNK_N == 0, "MN-major B needs whole 128-byte chunks per CTA");
     static_assert(!BCOMP || (!SPARSE && BMAJ == BMajor::MN), "compressed B: dense A, MN-major B");
 
-    extern __shared__ uint8_t smem_raw[];
-    const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t staging = smem_base + NS * C::STAGE;
-    const uint32_t bars = staging + C::STAGING_BYTES;
     auto full_bar = [&](int s) { return bars + 8u * s; };              // used in the leader only
     auto empty_bar = [&](int s) { return bars + 8u * (NS + s); };      // one per CTA
     auto acc_full_bar = [&](int b) { return bars + 8u * (2 * NS + b); };           // one per CTA
     auto acc_empty_bar = [&](int b) { return bars + 8u * (2 * NS + 2 + b); };      // leader only, one arrival per epilogue warp of the pair
-    constexpr int MISC = 2 * NS + 4;
-    const uint32_t tmem_slot = bars + 8u * MISC;
-    uint8_t *bars_generic = smem_raw + (bars - smem_u32(smem_raw));
-    volatile uint32_t *tmem_slot_ptr = reinterpret_cast<volatile uint32_t *>(bars_generic + 8u * MISC);
-    volatile int *abort_flag = reinterpret_cast<volatile int *>(bars_generic + 8u * (MISC + 1));
-    static_assert(8 * (MISC + 2) + 64 <= 512, "barrier block (+ the expander's 16-entry selector table)");
-    const WaitCtx wc{p.status, abort_flag, p.wait_limit_ns};
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();
     const bool leader = (rank == 0);
-    const int pair = blockIdx.x >> 1, num_pairs = gridDim.x >> 1;
     const int m_tiles = (p.M + 2 * BM - 1) / (2 * BM);
     const int n_tiles = (p.N + BN - 1) / BN;
     const int num_tiles = m_tiles * n_tiles;
@@ -438,35 +453,13 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         return u;
     };
 
-    if (threadIdx.x == 0) {
-        // full: the producer's arrival with the TMA byte count (+ the eight expander warps of the pair)
-        for (int s = 0; s < NS; ++s) { mbar_init(full_bar(s), BCOMP ? 9 : 1); mbar_init(empty_bar(s), 1); }
-        for (int b = 0; b < 2; ++b) { mbar_init(acc_full_bar(b), 1); mbar_init(acc_empty_bar(b), 2 * C::EPI_WARPS); }
-        *abort_flag = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        prefetch_tensormap(&map_a);
-        if (!BCOMP) prefetch_tensormap(&map_b);
-        if (SPARSE) prefetch_tensormap(&map_m);
-        if (!OUT_F32) prefetch_tensormap(&map_d);
-    }
-    if (warp == 1) {
-        tmem_alloc(tmem_slot, TMEM_COLS);
-        tmem_relinquish();
-    }
-    tc_fence_before();
-    __syncthreads();
-    cluster_sync();          // the peer's barriers are initialised before anything signals them
-    tc_fence_after();
-    sste_pdl_wait();         // everything above overlapped the previous kernel; global memory from here on
-    const uint32_t tmem_base = *tmem_slot_ptr;
-
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer (both CTAs)
         if (lane == 0) {
             const int k_atoms = p.K / 128;
             uint32_t s = 0, ph = 0;          // stage of the ring and the parity of its round
             bool ok = true;
-            for (int unit = pair; unit < num_units && ok; unit += num_pairs) {
+            for (int j = 0, unit = seq.first(); unit < num_units && ok; ++j, unit = seq.next(unit, j)) {
                 const Unit u = decode(unit);
                 int mt, nt;
                 tile_coords(u.tile, m_tiles, n_tiles, p.group_m, mt, nt);
@@ -474,7 +467,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                 const int n0 = nt * BN + static_cast<int>(rank) * (BN / 2);    // this CTA's half of B
                 for (int kb = u.kb0; kb < u.kb1; ++kb) {
                     // test hook: the stage is never loaded nor announced, so the MMA warp's wait for it runs out
-                    if (p.skip_last_stage && unit + num_pairs >= num_units && kb == u.kb1 - 1) break;
+                    if (p.skip_last_stage && seq.next(unit, j + 1) >= num_units && kb == u.kb1 - 1) break;
                     if (!mbar_wait(empty_bar(s), ph ^ 1u, wc)) { ok = false; break; }
                     const uint32_t lead_full = map_to_cta(full_bar(s), 0);
                     if (leader) mbar_arrive_expect_tx(full_bar(s), STAGE_TX);
@@ -508,7 +501,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             const uint32_t idesc = instr_desc(SPARSE, p.afmt, p.bfmt, BMAJ == BMajor::MN, BN);
             uint32_t s = 0, ph = 0, local_tile = 0;
             bool ok = true;
-            for (int unit = pair; unit < num_units && ok; unit += num_pairs, ++local_tile) {
+            for (int unit = seq.first(); unit < num_units && ok; ++local_tile, unit = seq.next(unit, local_tile)) {
                 const Unit u = decode(unit);
                 const uint32_t buf = local_tile % NB, use = local_tile / NB;
                 if (!mbar_wait(acc_empty_bar(buf), (use & 1u) ^ 1u, wc)) { ok = false; break; }
@@ -620,7 +613,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             pack_half(r, w, 0);
             pack_half(r + 16, w, 1);
         };
-        for (int unit = pair; unit < num_units; unit += num_pairs, ++local_tile) {
+        for (int unit = seq.first(); unit < num_units; ++local_tile, unit = seq.next(unit, local_tile)) {
             const Unit u = decode(unit);
             int mt, nt;
             tile_coords(u.tile, m_tiles, n_tiles, p.group_m, mt, nt);
@@ -842,8 +835,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                 release_acc();
                 if (!ok) break;
             } else {
-                // at most four panels are held packed in registers at a time
-                constexpr int HOLD = PANELS_MAX < 4 ? PANELS_MAX : 4;
+                // panels held packed in registers at a time: two where another accumulator keeps the MMAs busy, else four
+                constexpr int HOLD = (NB == 2 && PANELS_MAX % 2 == 0) ? 2 : PANELS_MAX < 4 ? PANELS_MAX : 4;
                 static_assert(PANELS_MAX % HOLD == 0 && HOLD % BOXP == 0, "whole rounds of panels");
 #pragma unroll
                 for (int h0 = 0; h0 < PANELS_MAX; h0 += HOLD) {
@@ -873,7 +866,10 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             for (int off = 16; off > 0; off >>= 1) best = max(best, __shfl_xor_sync(0xffffffffu, best, off));
             if (lane == 0 && best != 0) atomicMax(p.out_amax, best);
         }
-        if (elect && !OUT_F32) tma_store_wait_all();
+        if (elect && !OUT_F32) {
+            if (FINAL) tma_store_wait_all();
+            else asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+        }
     } else if (BCOMP) {
         // ------------------------------------------------------------ expander warps (6..9, both CTAs)
         // grad_X = grad_Z S(W) reads S(W) [O, I] as its MN-major B operand.  Here S(W) is given as the forward's
@@ -889,7 +885,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         // byte-permute selectors per metadata nibble p0 | p1 << 2: which source byte feeds each output byte
         // (4 = a zero byte).  bf16: low / high 16 bits select the two output words of a group from the pair word;
         // fp8: 16 bits select the output word of a group from its two value bytes (0, 1).
-        uint32_t *lut = reinterpret_cast<uint32_t *>(bars_generic + 8u * (MISC + 2));
+        uint32_t *lut = reinterpret_cast<uint32_t *>(ctrl_generic + CTRL_LUT);
         if (t < 16) {
             const uint32_t p0 = t & 3, p1 = t >> 2;
             uint32_t sel = 0;
@@ -913,7 +909,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             moff[j] = F8 ? sste_meta_atom_byte8(m, k) : sste_meta_atom_byte16(m, k);
         }
         // loader cursor: (unit, stage) of the next loads
-        int e_unit = pair, e_kb = 0, e_kend = 0;
+        int e_j = 0, e_unit = seq.first(), e_kb = 0, e_kend = 0;
         const uint8_t *e_vals = nullptr, *e_meta = nullptr;
         bool e_cols = false;
         auto e_setup = [&]() {
@@ -945,7 +941,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                 }
             }
             if (++e_kb >= e_kend) {
-                e_unit += num_pairs;
+                ++e_j;
+                e_unit = seq.next(e_unit, e_j);
                 e_setup();
             }
             return true;
@@ -956,7 +953,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         uint32_t m0[UNITS], m1[UNITS], m2[UNITS];
         bool h0 = e_issue(v0, m0), h1 = e_issue(v1, m1), h2 = e_issue(v2, m2);
         uint32_t it = 0;
-        uint8_t *const ring = smem_raw + (smem_base - smem_u32(smem_raw));
+        uint8_t *const ring = ctrl_generic + CTRL_BYTES;
         while (h0) {
             const int s = it % NS;
             const uint32_t ph = (it / NS) & 1u;
@@ -997,15 +994,105 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             ++it;
         }
     }
+}
 
-    // ---------------------------------------------------------------- teardown
+// Shared-memory control block, tensor memory and the pair's barriers around one or two products.
+struct Frame {
+    uint8_t *ctrl;               // generic address of the control block
+    uint32_t ctrl_u32, data_u32; // shared addresses: control block, first stage
+    uint32_t tmem_base;
+    WaitCtx wc;
+};
+template <typename F>
+__device__ __forceinline__ Frame frame_begin(uint8_t *smem_raw, const GemmParams &p, F init)
+{
+    Frame f;
+    f.ctrl_u32 = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    f.data_u32 = f.ctrl_u32 + CTRL_BYTES;
+    f.ctrl = smem_raw + (f.ctrl_u32 - smem_u32(smem_raw));
+    volatile int *abort_flag = reinterpret_cast<volatile int *>(f.ctrl + CTRL_ABORT);
+    f.wc = WaitCtx{p.status, abort_flag, p.wait_limit_ns};
+    if (threadIdx.x == 0) {
+        init(f);
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if ((threadIdx.x >> 5) == 1) {
+        tmem_alloc(f.ctrl_u32 + CTRL_TMEM, TMEM_COLS);
+        tmem_relinquish();
+    }
     tc_fence_before();
     __syncthreads();
-    cluster_sync();          // neither CTA frees tensor memory while the pair still uses it
-    if (warp == 1) {
-        tc_fence_after();
-        tmem_dealloc(tmem_base, TMEM_COLS);
-    }
+    cluster_sync();          // the peer's barriers are initialised before anything signals them
+    tc_fence_after();
+    sste_pdl_wait();         // everything above overlapped the previous kernel; global memory from here on
+    f.tmem_base = *reinterpret_cast<volatile uint32_t *>(f.ctrl + CTRL_TMEM);
+    return f;
+}
+// every role of both CTAs is done: tensor memory and shared memory may be used for something else
+__device__ __forceinline__ void pair_sync()
+{
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync();
+    tc_fence_after();
+}
+
+template <bool SPARSE, BMajor BMAJ, int ELT, int BN, bool OUT_T, bool OUT_F32, bool BCOMP = false>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Cfg<SPARSE, ELT, BN, BCOMP>::THREADS, 1)
+gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
+            const __grid_constant__ CUtensorMap map_d, const __grid_constant__ CUtensorMap map_m,
+            const uint8_t *__restrict__ meta, const __grid_constant__ GemmParams p)
+{
+    extern __shared__ uint8_t smem_raw[];
+    sste_pdl_trigger();
+    const Frame f = frame_begin(smem_raw, p, [&](const Frame &fr) {
+        init_barriers<Cfg<SPARSE, ELT, BN, BCOMP>, BCOMP>(fr.ctrl_u32);
+        prefetch_tensormap(&map_a);
+        if (!BCOMP) prefetch_tensormap(&map_b);
+        if (SPARSE) prefetch_tensormap(&map_m);
+        if (!OUT_F32) prefetch_tensormap(&map_d);
+    });
+    const int pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
+    product<SPARSE, BMAJ, ELT, BN, OUT_T, OUT_F32, BCOMP, true>(map_a, map_b, map_d, map_m, meta, p,
+                                                               UnitSeq{0, 0, 0, 0, pairs, pair}, f.ctrl, f.ctrl_u32, f.data_u32,
+                                                               f.tmem_base, f.wc);
+    pair_sync();             // neither CTA frees tensor memory while the pair still uses it
+    if ((threadIdx.x >> 5) == 1) tmem_dealloc(f.tmem_base, TMEM_COLS);
+}
+
+// grad_W and grad_X of a layer in one launch.  They are independent, and each alone quantises badly into waves of CTA pairs
+// (3072 x 768, 8192 tokens: 36 and 96 tiles on 74 pairs).  Every pair computes its share of grad_W, then of grad_X: the
+// pairs that come out of grad_W a round earlier (`late_pairs` is the number of the others, the first ones) take `early`
+// rounds of grad_X tiles among themselves before all share the rest.
+struct GradsPlan { int late_pairs, early, early_first; };
+template <int ELT, int BNW, int BNX>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(320, 1)
+grads_kernel(const __grid_constant__ CUtensorMap wa, const __grid_constant__ CUtensorMap wb, const __grid_constant__ CUtensorMap wd,
+             const __grid_constant__ CUtensorMap wm, const __grid_constant__ CUtensorMap xa, const __grid_constant__ CUtensorMap xb,
+             const __grid_constant__ CUtensorMap xd, const __grid_constant__ GemmParams pw, const __grid_constant__ GemmParams px,
+             const GradsPlan g)
+{
+    extern __shared__ uint8_t smem_raw[];
+    sste_pdl_trigger();
+    const Frame f = frame_begin(smem_raw, pw, [&](const Frame &fr) {
+        init_barriers<Cfg<true, ELT, BNW>, false>(fr.ctrl_u32);
+        init_barriers<Cfg<false, ELT, BNX>, false>(fr.ctrl_u32 + CTRL_SECOND);
+        prefetch_tensormap(&wa); prefetch_tensormap(&wb); prefetch_tensormap(&wd); prefetch_tensormap(&wm);
+        prefetch_tensormap(&xa); prefetch_tensormap(&xb); prefetch_tensormap(&xd);
+    });
+    const int pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
+    product<true, BMajor::MN, ELT, BNW, false, false, false, false>(wa, wb, wd, wm, nullptr, pw, UnitSeq{0, 0, 0, 0, pairs, pair},
+                                                                    f.ctrl, f.ctrl_u32, f.data_u32, f.tmem_base, f.wc);
+    pair_sync();
+    const int n_early = pairs - g.late_pairs;
+    const bool late = pair < g.late_pairs;
+    const UnitSeq seq{late ? 0 : g.early, n_early, pair - g.late_pairs, g.early * n_early, pairs,
+                      g.early_first ? (late ? n_early + pair : pair - g.late_pairs) : pair};
+    product<false, BMajor::MN, ELT, BNX, false, false, false, true>(xa, xb, xd, xa, nullptr, px, seq, f.ctrl,
+                                                                    f.ctrl_u32 + CTRL_SECOND, f.data_u32, f.tmem_base, f.wc);
+    pair_sync();
+    if ((threadIdx.x >> 5) == 1) tmem_dealloc(f.tmem_base, TMEM_COLS);
 }
 
 // ------------------------------------------------------------------ host side
@@ -1079,7 +1166,22 @@ constexpr TileCost tile_cost(Product pr, int elt, int bn)
 }
 
 // Everything the host decides about one product launch.
-struct LaunchPlan { int bn, splits, split_from, group_m; };
+struct LaunchPlan { int bn, splits, split_from, group_m; double us; };
+
+// Microseconds that a split costs on top of its units' main loops: the exchange between `s` units, `bytes` of partials.
+double exchange_us(int s, int bn, double bytes)
+{
+    return (s == 2 ? 2.4 + 2.6 * bn / 256.0 : 2.5 + 0.65 * s + (2.6 + 0.4 * s) * bn / 256.0) + bytes / 15e6;
+}
+
+// L2-aware band height of a product with tiles `bn` wide.
+int plan_group_m(Product pr, int elt, bool bcomp, int bn, int pairs, int M, int N, int K)
+{
+    const bool sparse = (pr != GRAD_INPUT);
+    return pick_group_m((M + 2 * BM - 1) / (2 * BM), (N + bn - 1) / bn, pairs,
+                        static_cast<double>(K) * (sparse ? 0.5 * elt + 0.125 : 1.0 * elt) * 2 * BM,
+                        static_cast<double>(K) * ((bcomp ? 0.5 : 1.0) * elt) * bn);
+}
 
 // Tile width and split-K factor by the model's time.  Tiles that fill complete waves of CTA pairs are computed whole; the
 // tiles of the last, partial wave (all of them when there are fewer tiles than pairs, as for the weight gradient of a
@@ -1097,8 +1199,7 @@ LaunchPlan make_plan(Product pr, int elt, int only_bn, bool out_f32, bool bcomp,
     int forced = only_bn;
     for (int bn : widths.bn)
         if (!forced && bn && bn == g_force_bn) forced = bn;
-    LaunchPlan best{0, 1, 0, m_tiles};
-    double best_us = 0.0;
+    LaunchPlan best{0, 1, 0, m_tiles, 0.0};
     for (int bn : widths.bn) {
         if (!bn || (forced && bn != forced)) continue;
         const int tiles = m_tiles * ((N + bn - 1) / bn);
@@ -1114,23 +1215,151 @@ LaunchPlan make_plan(Product pr, int elt, int only_bn, bool out_f32, bool bcomp,
                 if (tail * 2 * 8 * MAX_PARTS > SSTE_SPLITK_TICKETS) continue;
                 const size_t bytes = static_cast<size_t>(tail) * s * 2 * BM * bn * sizeof(float);
                 if (bytes > partial_bytes) continue;
-                us += s == 2 ? 2.4 + 2.6 * bn / 256.0 : 2.5 + 0.65 * s + (2.6 + 0.4 * s) * bn / 256.0;
-                us += bytes / 15e6;
+                us += exchange_us(s, bn, static_cast<double>(bytes));
             }
             if (tail) us += ((tail * s + pairs - 1) / pairs) * ((k_blocks + s - 1) / s * c.stage_us + c.tile_us);
             const bool wanted = (g_force_splits == s && best.bn == bn);      // the hook applies where the shape allows it
-            if (!best.bn || us < best_us * (best.bn == bn ? 1.0 : 0.97) || wanted) {
+            if (!best.bn || us < best.us * (best.bn == bn ? 1.0 : 0.97) || wanted) {
                 if (g_force_splits && best.bn == bn && best.splits == g_force_splits) continue;
-                best = LaunchPlan{bn, s, s > 1 ? whole : tiles, m_tiles};
-                best_us = us;
+                best = LaunchPlan{bn, s, s > 1 ? whole : tiles, m_tiles, us};
             }
             if (g_force_splits == 1) break;
         }
     }
-    const int n_tiles = (N + best.bn - 1) / best.bn;
-    best.group_m = pick_group_m(m_tiles, n_tiles, pairs, static_cast<double>(K) * (sparse ? 0.5 * elt + 0.125 : 1.0 * elt) * 2 * BM,
-                                static_cast<double>(K) * ((bcomp ? 0.5 : 1.0) * elt) * best.bn);
+    best.group_m = plan_group_m(pr, elt, bcomp, best.bn, pairs, M, N, K);
     return best;
+}
+
+// One launch for both gradient products (grads_kernel): the plans of the two and how the pairs share grad_X.
+struct JointPlan { LaunchPlan w, x; int pairs; GradsPlan g; double us; };
+
+// grad_W units go round the pairs; the last, partial round leaves `late` pairs busy for one unit more.  For every width,
+// split and number of early rounds the model gives the time at which the last pair ends; a pair that changes over from one
+// product to the other drains and refills its pipeline (SWITCH_US, about what a kernel boundary costs).
+constexpr double SWITCH_US = 2.5;
+JointPlan make_joint_plan(int elt, int sm_count, size_t partial_bytes, int O, int I, int T)
+{
+    const int max_pairs = sm_count / 2;
+    const int wk = (T + 256 / elt - 1) / (256 / elt), xk = (O + 128 / elt - 1) / (128 / elt);      // stages
+    const Widths ww = widths_of(GRAD_WEIGHT, elt), xw = widths_of(GRAD_INPUT, elt);
+    JointPlan best{};
+    for (int bnw : ww.bn) {
+        if (!bnw) continue;
+        const TileCost cw = tile_cost(GRAD_WEIGHT, elt, bnw);
+        const int w_tiles = ((O + 2 * BM - 1) / (2 * BM)) * ((I + bnw - 1) / bnw);
+        for (int bnx : xw.bn) {
+            if (!bnx || (bnw == 256 && elt == 2 && bnx == 128)) continue;  // (no kernel for it)
+            const TileCost cx = tile_cost(GRAD_INPUT, elt, bnx);
+            const int x_tiles = ((T + 2 * BM - 1) / (2 * BM)) * ((I + bnx - 1) / bnx);
+            const double x_us = xk * cx.stage_us + cx.tile_us;
+            for (int s = 1; s <= MAX_SPLITS; ++s) {
+                const int all = w_tiles * s + x_tiles, P = all < max_pairs ? all : max_pairs;
+                const int whole = w_tiles / P * P, tail = w_tiles - whole;
+                double extra = 0.0;
+                if (s > 1) {
+                    if (tail == 0 || wk / s < 8 || (whole > 0 && wk % s != 0) || tail * s > P) continue;
+                    if (tail * 2 * 8 * MAX_PARTS > SSTE_SPLITK_TICKETS) continue;
+                    const size_t bytes = static_cast<size_t>(tail) * s * 2 * BM * bnw * sizeof(float);
+                    if (bytes > partial_bytes) continue;
+                    extra = exchange_us(s, bnw, static_cast<double>(bytes));
+                }
+                const int late = tail * s;                                  // pairs with one unit more
+                const double w_us = wk * cw.stage_us + cw.tile_us;
+                const double t_early = (whole / P) * w_us + (whole ? SWITCH_US : 0.0);
+                const double t_late = late ? (whole / P) * w_us + (wk + s - 1) / s * cw.stage_us + cw.tile_us + extra + SWITCH_US : 0.0;
+                const int n_early = P - late;
+                for (int early = 0; early == 0 || (late && n_early && t_early + (early - 1) * x_us < t_late); ++early) {
+                    const int rest = x_tiles - early * n_early;
+                    const int rounds = rest > 0 ? (rest + P - 1) / P : 0, last = rest > 0 ? rest - (rounds - 1) * P : 0;
+                    for (int ef = 0; ef < 2; ++ef) {
+                        // rounds of the early / late pairs: the group that comes second lacks the last one if `last` is short
+                        const int r_early = rounds - ((rounds && !ef && last <= late) ? 1 : 0);
+                        const int r_late = rounds - ((rounds && ef && last <= n_early) ? 1 : 0);
+                        double us = n_early ? t_early + (early + r_early) * x_us : 0.0;
+                        if (late && t_late + r_late * x_us > us) us = t_late + r_late * x_us;
+                        us += 0.05 * x_us;                                  // among equals the shorter tile
+                        if (best.pairs && us >= best.us - 1e-9) continue;
+                        best.w = LaunchPlan{bnw, s, s > 1 ? whole : w_tiles, 0, 0.0};
+                        best.x = LaunchPlan{bnx, 1, x_tiles, 0, 0.0};
+                        best.pairs = P;
+                        best.g = GradsPlan{late, early, ef};
+                        best.us = us;
+                    }
+                    if (rest <= 0) break;
+                }
+            }
+        }
+    }
+    best.w.group_m = plan_group_m(GRAD_WEIGHT, elt, false, best.w.bn, best.pairs, O, I, T);
+    best.x.group_m = plan_group_m(GRAD_INPUT, elt, false, best.x.bn, best.pairs, T, I, O);
+    return best;
+}
+
+// Tensor maps of a launch: A, B, output, metadata (those that it does not use repeat A's).
+struct Maps { CUtensorMap a, b, d, m; };
+template <bool SPARSE, BMajor BMAJ, int ELT, int BN, bool OUT_T, bool OUT_F32, bool BCOMP>
+bool make_maps(const sste_ctx *ctx, const void *A, const void *B, const void *meta, const GemmParams &p, Maps &maps)
+{
+    using C = Cfg<SPARSE, ELT, BN, BCOMP>;
+    constexpr int BK = (SPARSE ? 256 : 128) / ELT;
+    // A: compressed values [M, K/2] or [M, K], 128 bytes per row per stage
+    bool ok = make_map(ctx, &maps.a, A, ELT, p.M, SPARSE ? p.K / 2 : p.K, SPARSE ? BK / 2 : BK, BM, CU_TENSOR_MAP_SWIZZLE_128B);
+    maps.b = maps.d = maps.m = maps.a;
+    if (BCOMP) {             // B is expanded from its compressed form by the kernel
+    } else if (BMAJ == BMajor::K) {   // B stored [N, K]: sub-tiles of BN/2 rows by 128 bytes of K
+        ok = ok && make_map(ctx, &maps.b, B, ELT, p.N, p.K, 128 / ELT, BN / 2, CU_TENSOR_MAP_SWIZZLE_128B);
+    } else {                 // B stored [K, N]: chunks of 128 bytes of N by BK rows of K
+        ok = ok && make_map(ctx, &maps.b, B, ELT, p.K, p.N, 128 / ELT, BK, CU_TENSOR_MAP_SWIZZLE_128B);
+    }
+    if (OUT_F32) {           // the fp32 epilogue stores directly
+    } else if (OUT_T) {      // out[N, M] bf16: boxes of 64 m x 32 n
+        ok = ok && make_map(ctx, &maps.d, p.D, 2, p.N, p.M, 64, 32, CU_TENSOR_MAP_SWIZZLE_128B);
+    } else if (C::PANELS == 2) {   // out[M, N] bf16: boxes of 64 n x 32 m
+        ok = ok && make_map(ctx, &maps.d, p.D, 2, p.M, p.N, 64, 32, CU_TENSOR_MAP_SWIZZLE_128B);
+    } else {                 // out[M, N] bf16: boxes of 32 n x 32 m
+        ok = ok && make_map(ctx, &maps.d, p.D, 2, p.M, p.N, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B);
+    }
+    if (SPARSE)              // metadata image as rows of 512 bytes, four per atom
+        ok = ok && make_map(ctx, &maps.m, meta, 4, static_cast<uint64_t>(p.M / 128) * (p.K / 128) * 4, 128, 128, 4 * C::ATOMS,
+                            CU_TENSOR_MAP_SWIZZLE_NONE);
+    return ok;
+}
+
+// the fields of a launch that its plan decides
+void apply_plan(const sste_ctx *ctx, const LaunchPlan &plan, GemmParams &p)
+{
+    p.wait_limit_ns = WAIT_LIMIT_NS;
+    p.skip_last_stage = 0;
+    p.group_m = plan.group_m;
+    p.splits = plan.splits;
+    p.split_from = plan.split_from;
+    p.partials = ctx->splitk_partials;
+    p.tickets = ctx->splitk_tickets;
+}
+
+template <int ELT, int BNW, int BNX>
+sste_status launch_grads(const sste_ctx *ctx, const void *gvals, const void *gmeta, const void *X, const void *dY, const void *w,
+                         GemmParams pw, GemmParams px, const JointPlan &plan, cudaStream_t stream)
+{
+    Maps mw, mx;
+    if (!make_maps<true, BMajor::MN, ELT, BNW, false, false, false>(ctx, gvals, X, gmeta, pw, mw) ||
+        !make_maps<false, BMajor::MN, ELT, BNX, false, false, false>(ctx, dY, w, nullptr, px, mx))
+        return SSTE_ERR_CUDA;
+    auto kern = grads_kernel<ELT, BNW, BNX>;
+    constexpr int SMEM = Cfg<true, ELT, BNW>::SMEM_BYTES > Cfg<false, ELT, BNX>::SMEM_BYTES ? Cfg<true, ELT, BNW>::SMEM_BYTES
+                                                                                           : Cfg<false, ELT, BNX>::SMEM_BYTES;
+    static DeviceOnce attr_done;
+    if (!attr_done.run(ctx->device, [&] {
+            return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM) == cudaSuccess;
+        }))
+        return SSTE_ERR_CUDA;
+    apply_plan(ctx, plan.w, pw);
+    apply_plan(ctx, plan.x, px);
+    if (sste_launch(kern, dim3(2 * plan.pairs), dim3(320), SMEM, stream, mw.a, mw.b, mw.d, mw.m, mx.a, mx.b, mx.d, pw, px,
+                    plan.g) != cudaSuccess)
+        return SSTE_ERR_CUDA;
+    sste_count_launches(1);
+    return SSTE_OK;
 }
 
 template <bool SPARSE, BMajor BMAJ, int ELT, int BN, bool OUT_T, bool OUT_F32, bool BCOMP = false>
@@ -1138,34 +1367,8 @@ sste_status launch(const sste_ctx *ctx, const void *A, const void *B, const void
                    const LaunchPlan &plan, cudaStream_t stream)
 {
     using C = Cfg<SPARSE, ELT, BN, BCOMP>;
-    constexpr int BK = (SPARSE ? 256 : 128) / ELT;
-    CUtensorMap map_a, map_b, map_d, map_m;
-    bool ok;
-    if (SPARSE)   // compressed values [M, K/2]: 128 bytes per row per stage
-        ok = make_map(ctx, &map_a, A, ELT, p.M, p.K / 2, BK / 2, BM, CU_TENSOR_MAP_SWIZZLE_128B);
-    else
-        ok = make_map(ctx, &map_a, A, ELT, p.M, p.K, BK, BM, CU_TENSOR_MAP_SWIZZLE_128B);
-    if (BCOMP)               // B is expanded from its compressed form by the kernel: no map
-        map_b = map_a;
-    else if (BMAJ == BMajor::K)   // B stored [N, K]: sub-tiles of BN/2 rows by 128 bytes of K
-        ok = ok && make_map(ctx, &map_b, B, ELT, p.N, p.K, 128 / ELT, BN / 2, CU_TENSOR_MAP_SWIZZLE_128B);
-    else                     // B stored [K, N]: chunks of 128 bytes of N by BK rows of K
-        ok = ok && make_map(ctx, &map_b, B, ELT, p.K, p.N, 128 / ELT, BK, CU_TENSOR_MAP_SWIZZLE_128B);
-    if (OUT_F32) {
-        map_d = map_a;       // unused: the fp32 epilogue stores directly
-    } else if (OUT_T) {      // out[N, M] bf16: boxes of 64 m x 32 n
-        ok = ok && make_map(ctx, &map_d, p.D, 2, p.N, p.M, 64, 32, CU_TENSOR_MAP_SWIZZLE_128B);
-    } else if (C::PANELS == 2) {   // out[M, N] bf16: boxes of 64 n x 32 m
-        ok = ok && make_map(ctx, &map_d, p.D, 2, p.M, p.N, 64, 32, CU_TENSOR_MAP_SWIZZLE_128B);
-    } else {                 // out[M, N] bf16: boxes of 32 n x 32 m
-        ok = ok && make_map(ctx, &map_d, p.D, 2, p.M, p.N, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B);
-    }
-    if (SPARSE)              // metadata image as rows of 512 bytes, four per atom
-        ok = ok && make_map(ctx, &map_m, meta, 4, static_cast<uint64_t>(p.M / 128) * (p.K / 128) * 4, 128, 128, 4 * C::ATOMS,
-                            CU_TENSOR_MAP_SWIZZLE_NONE);
-    else
-        map_m = map_a;       // unused
-    if (!ok) return SSTE_ERR_CUDA;
+    Maps maps;
+    if (!make_maps<SPARSE, BMAJ, ELT, BN, OUT_T, OUT_F32, BCOMP>(ctx, A, B, meta, p, maps)) return SSTE_ERR_CUDA;
     auto kern = gemm_kernel<SPARSE, BMAJ, ELT, BN, OUT_T, OUT_F32, BCOMP>;
     // The opt-in to more than 48 KB of dynamic shared memory is a per-DEVICE attribute of the kernel:
     // set once per (instantiation, device), under a lock (contexts may be used from several host threads).
@@ -1176,8 +1379,7 @@ sste_status launch(const sste_ctx *ctx, const void *A, const void *B, const void
         return SSTE_ERR_CUDA;
     const int m_tiles = (p.M + 2 * BM - 1) / (2 * BM), n_tiles = (p.N + BN - 1) / BN;
     GemmParams pp = p;
-    pp.wait_limit_ns = WAIT_LIMIT_NS;
-    pp.skip_last_stage = 0;
+    apply_plan(ctx, plan, pp);
     if (g_inject_stall) {
         // Test hook (sste_debug_inject_stall): only a dense product of ONE output tile takes the fault, so that
         // exactly one CTA pair runs into the expired wait; every other launch refuses while the hook is armed.
@@ -1188,15 +1390,10 @@ sste_status launch(const sste_ctx *ctx, const void *A, const void *B, const void
     if (BCOMP) pp.b_vals = static_cast<const uint8_t *>(B);
     if (pp.out_amax && cudaMemsetAsync(pp.out_amax, 0, sizeof(unsigned int), stream) != cudaSuccess) return SSTE_ERR_CUDA;
     const int tiles = m_tiles * n_tiles;
-    pp.group_m = plan.group_m;
-    pp.splits = plan.splits;
-    pp.split_from = plan.split_from;
-    pp.partials = ctx->splitk_partials;
-    pp.tickets = ctx->splitk_tickets;
     const int n_split_tiles = tiles - pp.split_from;
     int pairs = pp.split_from + n_split_tiles * pp.splits;
     if (pairs > ctx->sm_count / 2) pairs = ctx->sm_count / 2;
-    if (sste_launch(kern, dim3(2 * pairs), dim3(C::THREADS), C::SMEM_BYTES, stream, map_a, map_b, map_d, map_m,
+    if (sste_launch(kern, dim3(2 * pairs), dim3(C::THREADS), C::SMEM_BYTES, stream, maps.a, maps.b, maps.d, maps.m,
                     static_cast<const uint8_t *>(meta), pp) != cudaSuccess)
         return SSTE_ERR_CUDA;
     if (cudaGetLastError() != cudaSuccess) return SSTE_ERR_CUDA;
@@ -1235,6 +1432,17 @@ sste_status launch_out(const sste_ctx *ctx, const void *A, const void *B, const 
     return launch<SPARSE, BMAJ, ELT, 256, OUT_T, false>(ctx, A, B, meta, p, plan, s);
 }
 
+// Room for a dense copy of a compressed weight in the last bytes of the workspace, null if the partials in front of it
+// would get too little; *partial_bytes: what is left to them.
+void *dense_copy_in_workspace(const sste_ctx *ctx, int O, int I, int elt, size_t *partial_bytes)
+{
+    const size_t dense_bytes = (static_cast<size_t>(O) * I * elt + 255) / 256 * 256;
+    if (!ctx->splitk_partials || dense_bytes + SSTE_DENSE_COPY_RESERVE > ctx->splitk_partial_bytes) return nullptr;
+    const size_t at = (ctx->splitk_partial_bytes - dense_bytes) / 256 * 256;
+    *partial_bytes = at;
+    return reinterpret_cast<char *>(ctx->splitk_partials) + at;
+}
+
 // FP8 operands come with the amax of the tensors they were quantised from (both or neither); bf16 with none.
 bool amax_args_ok(int elt, const float *a_amax, const float *b_amax)
 {
@@ -1266,6 +1474,20 @@ extern "C" sste_status sste_debug_plan(int product, sste_dtype opdt, int O, int 
     if (splits) *splits = plan.splits;
     if (split_from) *split_from = plan.split_from;
     if (group_m) *group_m = plan.group_m;
+    return SSTE_OK;
+}
+extern "C" sste_status sste_debug_joint_plan(sste_dtype opdt, int O, int I, int T, int sm_count, size_t workspace_bytes, int *out)
+{
+    int elt;
+    uint32_t code;
+    if (!fmt_code(opdt, &elt, &code) || sm_count < 2 || !out) return SSTE_ERR_INVALID_ARG;
+    if (!sste_mult128(T) || !sste_mult128(O) || !sste_mult128(I)) return SSTE_ERR_SHAPE;
+    const size_t partial_bytes =
+        workspace_bytes > SSTE_WS_SPLITK_PARTIALS_OFF + (size_t(1) << 20) ? workspace_bytes - SSTE_WS_SPLITK_PARTIALS_OFF : 0;
+    const JointPlan plan = make_joint_plan(elt, sm_count, partial_bytes, O, I, T);
+    const int v[10] = {plan.w.bn, plan.w.splits, plan.w.split_from, plan.w.group_m, plan.x.bn,
+                       plan.x.group_m, plan.pairs, plan.g.late_pairs, plan.g.early, plan.g.early_first};
+    for (int i = 0; i < 10; ++i) out[i] = v[i];
     return SSTE_OK;
 }
 // Host-only self-check of the once-per-device guard the launches use for per-device kernel attributes: `fn` must
@@ -1388,13 +1610,12 @@ extern "C" sste_status sste_linear_bwd_input(sste_ctx *ctx, const void *dY, int 
         // S(W) from the forward's compressed operand.  Where the workspace has room for the dense copy (in its last bytes;
         // split-K partials stay in front of it), it is expanded there first and the dense product runs on it: the same
         // bits, and one pass over the weight costs little (1280 x 5120, 16384 tokens, bf16: 511 -> 152 us for both).
-        const size_t dense_bytes = (static_cast<size_t>(O) * I * ea + 255) / 256 * 256;
-        if (ctx->splitk_partials && dense_bytes + SSTE_DENSE_COPY_RESERVE <= ctx->splitk_partial_bytes) {
-            char *copy = reinterpret_cast<char *>(ctx->splitk_partials) + (ctx->splitk_partial_bytes - dense_bytes) / 256 * 256;
+        size_t partial_bytes = 0;
+        if (void *copy = dense_copy_in_workspace(ctx, O, I, ea, &partial_bytes)) {
             const sste_status st = sste_decompress(ctx, vals, meta, O, I, wdt, copy, stream);
             if (st != SSTE_OK) return st;
             sste_ctx rest = *ctx;
-            rest.splitk_partial_bytes -= dense_bytes + 256;
+            rest.splitk_partial_bytes = partial_bytes;
             if (ea == 2) return launch_out<GRAD_INPUT, 2>(&rest, dY, copy, nullptr, p, xdt, s);
             return launch_out<GRAD_INPUT, 1>(&rest, dY, copy, nullptr, p, xdt, s);
         }
@@ -1410,4 +1631,65 @@ extern "C" sste_status sste_linear_bwd_input(sste_ctx *ctx, const void *dY, int 
     }
     if (ea == 2) return launch_out<GRAD_INPUT, 2>(ctx, dY, Wt_dense, nullptr, p, xdt, s);
     return launch_out<GRAD_INPUT, 1>(ctx, dY, Wt_dense, nullptr, p, xdt, s);
+}
+
+sste_status sste_bwd_products(sste_ctx *ctx, const void *gvals, const void *gmeta, const void *X, const void *dY, int O, int I,
+                              int T, sste_dtype gdt, sste_dtype wdt, const void *w_dense, const void *vals, const void *meta,
+                              const float *g_amax, const float *x_amax, const float *w_amax, void *dW, void *dX,
+                              sste_dtype odt, void *stream)
+{
+    const int elt = wdt == SSTE_BF16 ? 2 : 1;
+    const bool dims_ok = sste_mult128(T) && sste_mult128(O) && sste_mult128(I);
+    const bool aligned = sste_aligned(X, 128) && sste_aligned(gvals, 128) && sste_aligned(gmeta, 128) && sste_aligned(dW, 128) &&
+                         sste_aligned(dY, 128) && sste_aligned(w_dense, 128) && sste_aligned(vals, 128) &&
+                         sste_aligned(meta, 128) && sste_aligned(dX, 128);
+    const bool given = ctx && gvals && gmeta && X && dY && dW && dX && (w_dense || (vals && meta)) &&
+                       amax_args_ok(elt, g_amax, x_amax) && amax_args_ok(elt, g_amax, w_amax);
+    // One launch for bf16 outputs; the test hooks, fp32 outputs and everything that the single calls refuse go there.
+    if (given && dims_ok && aligned && odt == SSTE_BF16 && !g_inject_stall && !g_force_bn && !g_force_splits && !g_force_group_m) {
+        sste_device_guard guard(ctx->device);
+        if (!guard.ok) return SSTE_ERR_CUDA;
+        size_t partial_bytes = ctx->splitk_partials ? ctx->splitk_partial_bytes : 0;
+        const void *w = w_dense;
+        if (!w) {
+            if (void *copy = dense_copy_in_workspace(ctx, O, I, elt, &partial_bytes)) {
+                const sste_status st = sste_decompress(ctx, vals, meta, O, I, wdt, copy, stream);
+                if (st != SSTE_OK) return st;
+                w = copy;
+            }
+        }
+        if (w) {
+            const JointPlan plan = make_joint_plan(elt, ctx->sm_count, partial_bytes, O, I, T);
+            // (grad_X is not split here: with few tiles of a long reduction, a vocabulary projection, two launches win)
+            const double apart = make_plan(GRAD_WEIGHT, elt, 0, false, false, ctx->sm_count, partial_bytes, O, I, T).us +
+                                 make_plan(GRAD_INPUT, elt, 0, false, false, ctx->sm_count, partial_bytes, T, I, O).us + SWITCH_US;
+            uint32_t cg, cw;
+            int unused;
+            fmt_code(gdt, &unused, &cg);
+            fmt_code(wdt, &unused, &cw);
+            const GemmParams pw{O, I, T, dW, g_amax, x_amax, sste_fp8_max(gdt), sste_fp8_max(wdt), nullptr, ctx->status_dev, cg, cw, nullptr};
+            const GemmParams px{T, I, O, dX, g_amax, w_amax, sste_fp8_max(gdt), sste_fp8_max(wdt), nullptr, ctx->status_dev, cg, cw, nullptr};
+            cudaStream_t s = static_cast<cudaStream_t>(stream);
+            if (plan.us <= apart) {
+                if (elt == 1) return launch_grads<1, 256, 256>(ctx, gvals, gmeta, X, dY, w, pw, px, plan, s);
+                if (plan.w.bn == 256) return launch_grads<2, 256, 256>(ctx, gvals, gmeta, X, dY, w, pw, px, plan, s);
+                if (plan.x.bn == 256) return launch_grads<2, 128, 256>(ctx, gvals, gmeta, X, dY, w, pw, px, plan, s);
+                return launch_grads<2, 128, 128>(ctx, gvals, gmeta, X, dY, w, pw, px, plan, s);
+            }
+            if (!w_dense) {      // grad_W's partials stay clear of the copy
+                sste_ctx rest = *ctx;
+                rest.splitk_partial_bytes = partial_bytes;
+                sste_status st = elt == 2 ? launch_out<GRAD_WEIGHT, 2>(&rest, gvals, X, gmeta, pw, odt, s)
+                                          : launch_out<GRAD_WEIGHT, 1>(&rest, gvals, X, gmeta, pw, odt, s);
+                if (st == SSTE_OK)
+                    st = elt == 2 ? launch_out<GRAD_INPUT, 2>(&rest, dY, w, nullptr, px, odt, s)
+                                  : launch_out<GRAD_INPUT, 1>(&rest, dY, w, nullptr, px, odt, s);
+                return st;
+            }
+        }
+    }
+    const sste_status st = sste_linear_bwd_weight(ctx, gvals, gmeta, O, T, gdt, X, I, wdt, g_amax, x_amax, dW, odt, stream);
+    if (st != SSTE_OK) return st;
+    return sste_linear_bwd_input(ctx, dY, T, O, gdt, w_dense, w_dense ? nullptr : vals, w_dense ? nullptr : meta, I, wdt, g_amax,
+                                 w_amax, dX, odt, nullptr, stream);
 }

@@ -50,19 +50,24 @@ extern "C" sste_status sste_layer_backward(sste_ctx *ctx, const sste_layer *l, c
 {
     if (!ctx || !layer_ok(l) || !dY) return SSTE_ERR_INVALID_ARG;
     const bool fp8 = fp8_of(l);
-    const sste_dtype gdt = fp8 ? SSTE_E5M2 : SSTE_BF16, wdt = static_cast<sste_dtype>(l->op_dtype);
-    const sste_dtype odt = static_cast<sste_dtype>(l->out_dtype);
-    float *x_amax = fp8 ? l->amax : nullptr, *w_amax = fp8 ? l->amax + 1 : nullptr, *g_amax = fp8 ? l->amax + 2 : nullptr;
+    const sste_dtype gdt = fp8 ? SSTE_E5M2 : SSTE_BF16;
+    float *g_amax = fp8 ? l->amax + 2 : nullptr;
     if (fp8) {
         const sste_status st = sste_amax_scratch(ctx, dY, static_cast<size_t>(l->T) * l->O, g_amax, l->scratch, stream);
         if (st != SSTE_OK) return st;
     }
-    sste_status st = sste_mvue_sparsify(ctx, dY, l->T, l->O, SSTE_BF16, l->seed, l->tensor_id, step, token_offset,
+    const sste_status st = sste_mvue_sparsify(ctx, dY, l->T, l->O, SSTE_BF16, l->seed, l->tensor_id, step, token_offset,
                                         l->counter_cols, g_amax, gdt, l->gvals, l->gmeta, fp8 ? l->dYq : nullptr, stream);
     if (st != SSTE_OK) return st;
-    st = sste_linear_bwd_weight(ctx, l->gvals, l->gmeta, l->O, l->T, gdt, fp8 ? l->Xq : X, l->I, wdt, g_amax, x_amax, l->dW,
-                                odt, stream);
-    if (st != SSTE_OK) return st;
-    return sste_linear_bwd_input(ctx, fp8 ? l->dYq : dY, l->T, l->O, gdt, l->w_dense, l->w_dense ? nullptr : l->vals,
-                                 l->w_dense ? nullptr : l->meta, l->I, wdt, g_amax, w_amax, l->dX, odt, nullptr, stream);
+    return sste_layer_grads(ctx, l, X, dY, stream);
+}
+
+extern "C" sste_status sste_layer_grads(sste_ctx *ctx, const sste_layer *l, const void *X, const void *dY, void *stream)
+{
+    if (!ctx || !layer_ok(l) || !dY) return SSTE_ERR_INVALID_ARG;
+    const bool fp8 = fp8_of(l);
+    return sste_bwd_products(ctx, l->gvals, l->gmeta, fp8 ? l->Xq : X, fp8 ? l->dYq : dY, l->O, l->I, l->T,
+                             fp8 ? SSTE_E5M2 : SSTE_BF16, static_cast<sste_dtype>(l->op_dtype), l->w_dense, l->vals, l->meta,
+                             fp8 ? l->amax + 2 : nullptr, fp8 ? l->amax : nullptr, fp8 ? l->amax + 1 : nullptr, l->dW, l->dX,
+                             static_cast<sste_dtype>(l->out_dtype), stream);
 }

@@ -51,7 +51,7 @@ class SsteLinear:
         self.Y = torch.empty((T, O), dtype=out_dtype, device=dev)
         self.dX = torch.empty((T, I), dtype=out_dtype, device=dev)
         self.dW = torch.empty((O, I), dtype=out_dtype, device=dev)
-        self.launches = 0
+        self.launches = 0      # library calls, also those that a phase call stands for
         self.mark = None       # optional callback(label), called before every C-ABI call (a benchmark records events)
         self.track_flips = track_flips
         if track_flips:
@@ -91,7 +91,8 @@ class SsteLinear:
                                       and self.dYq.dtype is gdt and self.dYq.shape == g_shape)))
         lib = self.ctx.lib
         self.__dict__["_desc"] = desc = (fits, ctypes.addressof(d), self.W.data_ptr(), lib.sste_layer_prune,
-                                         lib.sste_layer_forward, lib.sste_layer_backward, x_shape, g_shape, d)
+                                         lib.sste_layer_forward, lib.sste_layer_backward, x_shape, g_shape, d,
+                                         lib.sste_layer_grads)
         return desc
 
     def _amax(self, k):
@@ -210,9 +211,20 @@ class SsteLinear:
         return self.dX
 
     def grad_weight_and_input(self, dY, side_ctx: B.Context, side_stream: torch.cuda.Stream):
-        """grad_W on `side_stream` (through `side_ctx`: its own split-K workspace) while grad_X runs on the
-        current stream: the two products are independent once MVUE has run, and the tail, second split-K pass
-        and ramp-up of one overlap the other.  Both are complete in current-stream order on return."""
+        """grad_W and grad_X at the same time: they are independent once MVUE has run.  With bf16 results one launch on
+        the current stream does both and shares the SMs between them; otherwise grad_W runs on `side_stream` (through
+        `side_ctx`: its own split-K workspace) beside grad_X.  Both are complete in current-stream order on return."""
+        if self.mark is None:
+            desc = self._desc or self._describe()
+            X = None if self.fp8 else self.X
+            if (desc[0] and self.Y.dtype is _bf16 and dY.dtype is _bf16 and dY.shape == desc[7] and dY.is_cuda
+                    and dY.is_contiguous() and (X is None or X.shape == desc[6])):
+                st = desc[9](self.ctx.handle, desc[1], None if X is None else X.data_ptr(), dY.data_ptr(),
+                             _raw_stream(_device()))
+                if st:
+                    self.ctx._check(st)
+                self.__dict__["launches"] += 2
+                return self.dX, self.dW
         main = torch.cuda.current_stream()
         side_stream.wait_stream(main)
         with torch.cuda.stream(side_stream):

@@ -71,3 +71,25 @@ def test_described_buffers_follow_the_attributes(ctx):
     lin.Y.fill_(7.0)
     lin.forward(X[:128])                                     # a shorter batch fills the first rows only
     assert torch.equal(lin.Y[:128], Y2[:128]) and bool((lin.Y[128:] == 7.0).all())
+
+
+@pytest.mark.parametrize("fp8", [False, True])
+@pytest.mark.parametrize("O,I,T", [(128, 128, 128), (128, 256, 4096), (768, 768, 2048), (3072, 768, 1024), (1280, 1280, 2176),
+                                   (2432, 2560, 512), (384, 5120, 640)])
+def test_one_launch_gradients_equal_two_launches(ctx, O, I, T, fp8):
+    """sste_layer_grads against the two single calls: the same sums, of which only the split may differ.
+
+    Another split of an fp32 sum changes it by about 1e-6 of the sum of magnitudes, which moves the bf16 result by at most
+    one unit in the last place (2^-7 of the value at the start of a binade) wherever it is not much smaller than those."""
+    from paper_2409_09099_b200.layer import SsteLinear
+    W = dbf16(synth.gaussian_bf16(O + 61, (O, I), 0.02))
+    X = dbf16(synth.gaussian_bf16(O + 62, (T, I), 1.0))
+    dY = dbf16(synth.gaussian_bf16(O + 63, (T, O), 1e-2))
+    lin = SsteLinear(ctx, W, T, tensor_id=4, seed=17, fp8=fp8)
+    lin.init_beta(); lin.prune(); lin.forward(X)
+    for rep in range(2):                                     # the tickets of split tiles must be left at zero
+        lin.dX.fill_(7.0); lin.dW.fill_(7.0)
+        dX, dW = (t.clone() for t in lin.backward(dY, step=3))
+        ref_w, ref_x = lin.grad_weight().float(), lin.grad_input(dY).float()
+        for got, ref in ((dW.float(), ref_w), (dX.float(), ref_x)):
+            assert bool(((got - ref).abs() <= 2.0 ** -7 * ref.abs() + 1e-5 * ref.abs().max()).all())
