@@ -281,6 +281,25 @@ sste_status sste_layer_backward(sste_ctx *ctx, const sste_layer *layer, const vo
  * on grad_X's.  (The split of grad_W's reduction may then differ from the single call's: same sums, other rounding.) */
 sste_status sste_layer_grads(sste_ctx *ctx, const sste_layer *layer, const void *X, const void *dY, void *stream);
 
+/*
+ * A layer of ANY shape (see sste_pad_2d): `inner` is the layer of the padded sizes, O, I, T the real ones.  Xp [inner.T,
+ * inner.I] and dYp [inner.T, inner.O] receive the padded X and dY.  Y [T, O], dX [T, I], dW [O, I], bf16: cropped copies of
+ * inner's results; NULL for one that the caller reads in place (its columns need no crop).  inner.out_dtype is SSTE_BF16.
+ */
+typedef struct sste_padded_layer {
+    sste_layer inner;
+    int O, I, T;
+    unsigned int reserved;      /* 0 */
+    void *Xp, *dYp;
+    void *Y, *dX, *dW;
+} sste_padded_layer;
+
+/* sste_pad_2d of X [T, I], sste_layer_forward, sste_crop_2d of Y. */
+sste_status sste_padded_forward(sste_ctx *ctx, const sste_padded_layer *layer, const void *X, void *stream);
+/* sste_pad_2d of dY [T, O], sste_layer_backward, sste_crop_2d of dX and dW. */
+sste_status sste_padded_backward(sste_ctx *ctx, const sste_padded_layer *layer, const void *dY, uint32_t step,
+                                 uint64_t token_offset, void *stream);
+
 /* ---- ablation variants of the pruning step (the axes of the paper's ablations; not on the default path) ---- */
 
 typedef enum { SSTE_PRUNE_SOFT = 0, SSTE_PRUNE_HARD = 1 } sste_pruning;

@@ -34,6 +34,7 @@ EXPORTS = [
     "sste_debug_force_tile_order", "sste_debug_plan", "sste_debug_tile_coords",
     "sste_debug_mvue_groups", "sste_debug_selftest_device_once", "sste_layer_prune", "sste_layer_forward",
     "sste_layer_backward", "sste_layer_grads", "sste_debug_joint_plan",
+    "sste_padded_forward", "sste_padded_backward",
 ]
 
 _P, _I, _Z, _U32, _U64, _F = (ctypes.c_void_p, ctypes.c_int, ctypes.c_size_t, ctypes.c_uint32, ctypes.c_uint64,
@@ -56,6 +57,8 @@ _ARGTYPES = {
     "sste_layer_forward": [_P, _P, _P, _P, _P],
     "sste_layer_backward": [_P, _P, _P, _P, _U32, _U64, _P],
     "sste_layer_grads": [_P, _P, _P, _P, _P],
+    "sste_padded_forward": [_P, _P, _P, _P],
+    "sste_padded_backward": [_P, _P, _P, _U32, _U64, _P],
 }
 
 
@@ -71,6 +74,12 @@ class SsteError(RuntimeError):
     def __init__(self, code: int, what: str):
         super().__init__(f"libsste: {what} (status {code})")
         self.code = code
+
+
+class PaddedLayerBuffers(ctypes.Structure):
+    """sste_padded_layer."""
+    _fields_ = [("inner", LayerBuffers), ("O", _I), ("I", _I), ("T", _I), ("reserved", _U32), ("Xp", _P), ("dYp", _P),
+                ("Y", _P), ("dX", _P), ("dW", _P)]
 
 
 _lib = None

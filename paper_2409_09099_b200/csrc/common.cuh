@@ -164,3 +164,7 @@ sste_status sste_bwd_products(sste_ctx *ctx, const void *gvals, const void *gmet
                               int T, sste_dtype gdt, sste_dtype wdt, const void *w_dense, const void *vals, const void *meta,
                               const float *g_amax, const float *x_amax, const float *w_amax, void *dW, void *dX,
                               sste_dtype odt, void *stream);
+
+// two sste_crop_2d in one launch (arguments as checked by that call)
+sste_status sste_crop_two(sste_ctx *ctx, const void *src0, int rows_p0, int cols_p0, void *dst0, int rows0, int cols0,
+                          const void *src1, int rows_p1, int cols_p1, void *dst1, int rows1, int cols1, void *stream);

@@ -868,25 +868,38 @@ pad_2d_kernel(const uint16_t *__restrict__ src, uint32_t rows, uint32_t cols, ui
 }
 
 // dst [rows, cols] <- top-left corner of src [rows_p, cols_p] (16-byte aligned rows or not); one thread per aligned vector
-// of dst, n = rows * cols elements.
+// of dst, n = rows * cols elements.  Up to two tensors per launch: the blocks from `blocks` on work on the second.
+struct CropJob {
+    const uint16_t *src;
+    size_t src_elements;
+    uint16_t *dst;
+    uint32_t cols_p, cols;
+    size_t n, n_vec;
+    uint32_t blocks;
+};
 template <typename INDEX>
 __global__ void __launch_bounds__(EW_THREADS)
-crop_2d_kernel(const uint16_t *__restrict__ src, uint32_t cols_p, size_t src_elements, uint16_t *__restrict__ dst, uint32_t cols,
-               INDEX n, INDEX n_vec)
+crop_2d_kernel(const CropJob job0, const CropJob job1)
 {
     sste_pdl_trigger();
     sste_pdl_wait();
+    const bool second = blockIdx.x >= job0.blocks;
+    const CropJob &job = second ? job1 : job0;
+    const uint16_t *__restrict__ src = job.src;
+    uint16_t *__restrict__ dst = job.dst;
+    const uint32_t cols = job.cols, cols_p = job.cols_p, block = blockIdx.x - (second ? job0.blocks : 0u);
+    const INDEX n = static_cast<INDEX>(job.n), n_vec = static_cast<INDEX>(job.n_vec);
     const size_t lead = (reinterpret_cast<uintptr_t>(src) & 15u) / 2;
     const uint4 *base = reinterpret_cast<const uint4 *>(src - lead);
     const INDEX dlead = static_cast<INDEX>((reinterpret_cast<uintptr_t>(dst) & 15u) / 2);
-    for (INDEX v = static_cast<INDEX>(blockIdx.x) * EW_THREADS + threadIdx.x; v < n_vec;
-         v += static_cast<INDEX>(gridDim.x) * EW_THREADS) {
+    for (INDEX v = static_cast<INDEX>(block) * EW_THREADS + threadIdx.x; v < n_vec;
+         v += static_cast<INDEX>(job.blocks) * EW_THREADS) {
         // elements [e0, e1) of dst
         const INDEX e0 = v == 0 ? 0 : v * 8 - dlead, e1 = (v + 1) * 8 - dlead < n ? (v + 1) * 8 - dlead : n;
         INDEX r = e0 / cols;
         uint32_t c = static_cast<uint32_t>(e0 - r * cols);
         const size_t first = lead + static_cast<size_t>(r) * cols_p + c;
-        if (e1 - e0 == 8 && c + 8 <= cols && load8_fits(first, lead, lead + src_elements)) {
+        if (e1 - e0 == 8 && c + 8 <= cols && load8_fits(first, lead, lead + job.src_elements)) {
             *reinterpret_cast<uint4 *>(dst + e0) = load8(base, first);
         } else {
             for (INDEX e = e0; e < e1; ++e) {
@@ -1303,6 +1316,35 @@ extern "C" sste_status sste_pad_2d(sste_ctx *ctx, const void *src, int rows, int
     return launch_result();
 }
 
+namespace {
+
+CropJob crop_job(const sste_ctx *ctx, const void *src, int rows_p, int cols_p, void *dst, int rows, int cols)
+{
+    CropJob j{};
+    j.src = static_cast<const uint16_t *>(src);
+    j.src_elements = static_cast<size_t>(rows_p) * cols_p;
+    j.dst = static_cast<uint16_t *>(dst);
+    j.cols_p = static_cast<uint32_t>(cols_p);
+    j.cols = static_cast<uint32_t>(cols);
+    j.n = static_cast<size_t>(rows) * cols;
+    j.n_vec = (j.n + (reinterpret_cast<uintptr_t>(dst) & 15u) / 2 + 7) / 8;
+    j.blocks = static_cast<uint32_t>(grid_for(j.n_vec, ctx->sm_count));
+    return j;
+}
+
+sste_status crop_launch(const sste_ctx *, const CropJob &a, const CropJob &b, void *stream)
+{
+    const dim3 grid(a.blocks + b.blocks);
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    if (a.n < (size_t(1) << 31) && b.n < (size_t(1) << 31))
+        sste_launch(crop_2d_kernel<uint32_t>, grid, dim3(EW_THREADS), 0, s, a, b);
+    else
+        sste_launch(crop_2d_kernel<uint64_t>, grid, dim3(EW_THREADS), 0, s, a, b);
+    return launch_result();
+}
+
+}  // namespace
+
 extern "C" sste_status sste_crop_2d(sste_ctx *ctx, const void *src, int rows_p, int cols_p, void *dst, int rows, int cols,
                                     void *stream)
 {
@@ -1311,18 +1353,16 @@ extern "C" sste_status sste_crop_2d(sste_ctx *ctx, const void *src, int rows_p, 
     if (!sste_aligned(src, 2) || !sste_aligned(dst, 2)) return SSTE_ERR_ALIGN;
     sste_device_guard guard(ctx->device);
     if (!guard.ok) return SSTE_ERR_CUDA;
-    const size_t n = static_cast<size_t>(rows) * cols;
-    const size_t n_vec = (n + (reinterpret_cast<uintptr_t>(dst) & 15u) / 2 + 7) / 8;
-    const size_t src_elements = static_cast<size_t>(rows_p) * cols_p;
-    const dim3 grid(grid_for(n_vec, ctx->sm_count));
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (n < (size_t(1) << 31))
-        sste_launch(crop_2d_kernel<uint32_t>, grid, dim3(EW_THREADS), 0, s, static_cast<const uint16_t *>(src), cols_p,
-                    src_elements, static_cast<uint16_t *>(dst), cols, n, n_vec);
-    else
-        sste_launch(crop_2d_kernel<uint64_t>, grid, dim3(EW_THREADS), 0, s, static_cast<const uint16_t *>(src), cols_p,
-                    src_elements, static_cast<uint16_t *>(dst), cols, n, n_vec);
-    return launch_result();
+    return crop_launch(ctx, crop_job(ctx, src, rows_p, cols_p, dst, rows, cols), CropJob{}, stream);
+}
+
+sste_status sste_crop_two(sste_ctx *ctx, const void *src0, int rows_p0, int cols_p0, void *dst0, int rows0, int cols0,
+                          const void *src1, int rows_p1, int cols_p1, void *dst1, int rows1, int cols1, void *stream)
+{
+    sste_device_guard guard(ctx->device);
+    if (!guard.ok) return SSTE_ERR_CUDA;
+    return crop_launch(ctx, crop_job(ctx, src0, rows_p0, cols_p0, dst0, rows0, cols0),
+                       crop_job(ctx, src1, rows_p1, cols_p1, dst1, rows1, cols1), stream);
 }
 
 extern "C" sste_status sste_debug_mvue_groups(sste_ctx *ctx, const void *a, const void *k24, size_t n, void *pos_out,

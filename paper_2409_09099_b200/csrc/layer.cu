@@ -71,3 +71,38 @@ extern "C" sste_status sste_layer_grads(sste_ctx *ctx, const sste_layer *l, cons
                              fp8 ? l->amax + 2 : nullptr, fp8 ? l->amax : nullptr, fp8 ? l->amax + 1 : nullptr, l->dW, l->dX,
                              static_cast<sste_dtype>(l->out_dtype), stream);
 }
+
+namespace {
+
+bool padded_ok(const sste_padded_layer *l)
+{
+    return l && layer_ok(&l->inner) && l->inner.out_dtype == SSTE_BF16 && l->Xp && l->dYp && l->O > 0 && l->I > 0 && l->T > 0 &&
+           l->O <= l->inner.O && l->I <= l->inner.I && l->T <= l->inner.T;
+}
+
+}  // namespace
+
+extern "C" sste_status sste_padded_forward(sste_ctx *ctx, const sste_padded_layer *l, const void *X, void *stream)
+{
+    if (!ctx || !padded_ok(l) || !X) return SSTE_ERR_INVALID_ARG;
+    const sste_layer &in = l->inner;
+    sste_status st = sste_pad_2d(ctx, X, l->T, l->I, l->Xp, in.T, in.I, stream);
+    if (st == SSTE_OK) st = sste_layer_forward(ctx, &in, l->Xp, nullptr, stream);
+    if (st == SSTE_OK && l->Y) st = sste_crop_2d(ctx, in.Y, in.T, in.O, l->Y, l->T, l->O, stream);
+    return st;
+}
+
+extern "C" sste_status sste_padded_backward(sste_ctx *ctx, const sste_padded_layer *l, const void *dY, uint32_t step,
+                                            uint64_t token_offset, void *stream)
+{
+    if (!ctx || !padded_ok(l) || !dY) return SSTE_ERR_INVALID_ARG;
+    const sste_layer &in = l->inner;
+    sste_status st = sste_pad_2d(ctx, dY, l->T, l->O, l->dYp, in.T, in.O, stream);
+    if (st == SSTE_OK) st = sste_layer_backward(ctx, &in, l->Xp, l->dYp, step, token_offset, stream);
+    if (st != SSTE_OK) return st;
+    if (l->dX && l->dW)
+        return sste_crop_two(ctx, in.dX, in.T, in.I, l->dX, l->T, l->I, in.dW, in.O, in.I, l->dW, l->O, l->I, stream);
+    if (l->dX) return sste_crop_2d(ctx, in.dX, in.T, in.I, l->dX, l->T, l->I, stream);
+    if (l->dW) return sste_crop_2d(ctx, in.dW, in.O, in.I, l->dW, l->O, l->I, stream);
+    return SSTE_OK;
+}

@@ -274,7 +274,8 @@ class SsteLinearPadded:
     The library's kernels want multiples of 128.  Zero groups are fixed points of the projection (Eq. 4) and of
     the MVUE rule and add nothing to beta, to an amax or to a product, so padding W, X and dY with zeros and
     cropping Y, dX and dW gives the unpadded results; the MVUE counter runs over the unpadded column count.
-    The pad and crop passes are library kernels too (sste_pad_2d / sste_crop_2d).
+    The pad and crop passes are library kernels too (sste_pad_2d / sste_crop_2d); a result whose columns need no
+    cropping is the first rows of the inner layer's buffer.
     """
 
     def __init__(self, ctx: B.Context, O: int, I: int, T: int, **kw):
@@ -286,9 +287,9 @@ class SsteLinearPadded:
         self.Xp = torch.empty((self.Tp, self.Ip), **bf)
         self.dYp = torch.empty((self.Tp, self.Op), **bf)
         self.inner = SsteLinear(ctx, self.Wp, self.Tp, counter_cols=O, **kw)
-        self.Y = torch.empty((T, O), **bf)
-        self.dX = torch.empty((T, I), **bf)
-        self.dW = torch.empty((O, I), **bf)
+        rows = lambda t, r, c: t[:r] if t.dtype is _bf16 and t.shape[1] == c else torch.empty((r, c), **bf)
+        self.Y, self.dX, self.dW = rows(self.inner.Y, T, O), rows(self.inner.dX, T, I), rows(self.inner.dW, O, I)
+        self._desc = None
 
     @property
     def beta(self):
@@ -303,15 +304,56 @@ class SsteLinearPadded:
     def prune(self):
         self.inner.prune()
 
+    # Descriptor of the one-call path, made anew when the inner layer's changes or a buffer of this layer is replaced.
+    def _described(self, X, shape):
+        inner = self.inner
+        if inner.mark is not None or X.dtype is not _bf16 or X.shape != shape or not X.is_cuda or not X.is_contiguous():
+            return None
+        of = inner._desc or inner._describe()
+        bufs = (self.Xp, self.dYp, self.Y, self.dX, self.dW)
+        d = self._desc
+        if d is None or d[0] is not of or any(a is not b for a, b in zip(d[1], bufs)):
+            crop = lambda t, whole: None if t.data_ptr() == whole.data_ptr() else B._ptr(t)
+            p = B.PaddedLayerBuffers(of[8], self.O, self.I, self.T, 0, B._ptr(self.Xp), B._ptr(self.dYp),
+                                     crop(self.Y, inner.Y), crop(self.dX, inner.dX), crop(self.dW, inner.dW))
+            fits = (of[0] and inner.Y.dtype is _bf16 and tuple(self.Xp.shape) == (self.Tp, self.Ip)
+                    and tuple(self.dYp.shape) == (self.Tp, self.Op) and tuple(self.Y.shape) == (self.T, self.O)
+                    and tuple(self.dX.shape) == (self.T, self.I) and tuple(self.dW.shape) == (self.O, self.I)
+                    and all(t.dtype is _bf16 for t in bufs))
+            lib = self.ctx.lib
+            self._desc = d = (of, bufs, fits, ctypes.addressof(p), lib.sste_padded_forward, lib.sste_padded_backward, p)
+        return d if d[2] else None
+
+    def _crop(self, src, dst):
+        if src.data_ptr() != dst.data_ptr():
+            self.ctx.crop_2d(src, dst)
+
     def forward(self, X):
+        d = self._described(X, (self.T, self.I))
+        if d is not None:
+            st = d[4](self.ctx.handle, d[3], X.data_ptr(), _raw_stream(_device()))
+            if st:
+                self.ctx._check(st)
+            inner = self.inner.__dict__
+            if not self.inner.fp8:
+                inner["X"] = self.Xp
+            inner["launches"] += 3 if self.inner.fp8 else 1
+            return self.Y
         self.ctx.pad_2d(X, self.Xp)
         self.inner.forward(self.Xp)
-        self.ctx.crop_2d(self.inner.Y, self.Y)
+        self._crop(self.inner.Y, self.Y)
         return self.Y
 
     def backward(self, dY, step: int = 0):
+        d = self._described(dY, (self.T, self.O))
+        if d is not None:
+            st = d[5](self.ctx.handle, d[3], dY.data_ptr(), step, 0, _raw_stream(_device()))
+            if st:
+                self.ctx._check(st)
+            self.inner.__dict__["launches"] += 4 if self.inner.fp8 else 3
+            return self.dX, self.dW
         self.ctx.pad_2d(dY, self.dYp)
         self.inner.backward(self.dYp, step=step)
-        self.ctx.crop_2d(self.inner.dX, self.dX)
-        self.ctx.crop_2d(self.inner.dW, self.dW)
+        self._crop(self.inner.dX, self.dX)
+        self._crop(self.inner.dW, self.dW)
         return self.dX, self.dW

@@ -93,3 +93,27 @@ def test_one_launch_gradients_equal_two_launches(ctx, O, I, T, fp8):
         ref_w, ref_x = lin.grad_weight().float(), lin.grad_input(dY).float()
         for got, ref in ((dW.float(), ref_w), (dX.float(), ref_x)):
             assert bool(((got - ref).abs() <= 2.0 ** -7 * ref.abs() + 1e-5 * ref.abs().max()).all())
+
+
+@pytest.mark.parametrize("fp8", [False, True])
+@pytest.mark.parametrize("O,I,T", [(203, 80, 72), (128, 80, 128), (200, 128, 1000), (1, 3, 5)])
+def test_padded_calls_equal_single_calls(ctx, O, I, T, fp8):
+    """sste_padded_forward / _backward against the single calls; columns that need a crop, rows only, neither."""
+    from paper_2409_09099_b200.layer import SsteLinearPadded
+    W = dbf16(synth.gaussian_bf16(O + 81, (O, I), 0.02))
+    layers = [SsteLinearPadded(ctx, O, I, T, tensor_id=4, seed=17, fp8=fp8) for _ in range(2)]
+    layers[1].inner.mark = lambda label: None               # the single calls
+    for step in range(2):
+        X = dbf16(synth.gaussian_bf16(O + 82 + step, (T, I), 1.0))
+        dY = dbf16(synth.gaussian_bf16(O + 92 + step, (T, O), 1e-2))
+        for lin in layers:
+            lin.set_weight(W)
+            if step == 0:
+                lin.init_beta()
+            lin.prune()
+            assert lin.forward(X) is lin.Y
+            lin.backward(dY, step=step)
+        a, b = layers
+        for name in ("Y", "dX", "dW"):
+            assert torch.equal(_bits(getattr(a, name)), _bits(getattr(b, name))), (step, name)
+        assert tuple(a.Y.shape) == (T, O) and tuple(a.dX.shape) == (T, I) and tuple(a.dW.shape) == (O, I)
