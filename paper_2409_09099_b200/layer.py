@@ -36,64 +36,69 @@ class SsteLinear:
                  fp8: bool = False, out_dtype: torch.dtype = torch.bfloat16, track_flips: bool = False,
                  dense_copy: bool = True, counter_cols: int = 0):
         assert W.dtype == torch.bfloat16 and W.is_cuda
-        self.ctx, self.W, self.T, self.tensor_id, self.seed, self.fp8 = ctx, W, T, tensor_id, seed, fp8
-        self.O, self.I = W.shape
-        self.counter_cols = counter_cols
-        O, I, dev = self.O, self.I, W.device
-        f32 = dict(dtype=torch.float32, device=dev)
-        self.beta = torch.zeros(1, **f32)
-        self.beta_ready = False
-        wdt = B.E4M3 if fp8 else B.BF16
-        gdt = B.E5M2 if fp8 else B.BF16
-        self.vals, self.meta = ctx.alloc_compressed(O, I, wdt)
-        self.w_dense = torch.empty((O, I), dtype=B._TORCH_DT[wdt], device=dev) if dense_copy else None
-        self.gvals, self.gmeta = ctx.alloc_compressed(O, T, gdt)
-        self.Y = torch.empty((T, O), dtype=out_dtype, device=dev)
-        self.dX = torch.empty((T, I), dtype=out_dtype, device=dev)
-        self.dW = torch.empty((O, I), dtype=out_dtype, device=dev)
-        self.launches = 0      # library calls, also those that a phase call stands for
-        self.mark = None       # optional callback(label), called before every C-ABI call (a benchmark records events)
-        self.track_flips = track_flips
+        O, I = W.shape
+        dev, empty = W.device, torch.empty
+        wdt, gdt = (B._TORCH_DT[B.E4M3], B._TORCH_DT[B.E5M2]) if fp8 else (_bf16, _bf16)
+        # scalars in one zeroed tensor: beta; FP8: max|X|, max|w~| (bf16 projection), max|dY| and the amax passes' scratch
+        scalars = torch.zeros(6 if fp8 else 1, dtype=torch.float32, device=dev)
+        buffers = dict(
+            ctx=ctx, W=W, T=T, tensor_id=tensor_id, seed=seed, fp8=fp8, O=O, I=I, counter_cols=counter_cols,
+            beta=scalars[0:1] if fp8 else scalars, beta_ready=False,
+            vals=empty((O, I // 2), dtype=wdt, device=dev), meta=empty(O * I // 8, dtype=torch.uint8, device=dev),
+            w_dense=empty((O, I), dtype=wdt, device=dev) if dense_copy else None,
+            gvals=empty((O, T // 2), dtype=gdt, device=dev), gmeta=empty(O * T // 8, dtype=torch.uint8, device=dev),
+            Y=empty((T, O), dtype=out_dtype, device=dev), dX=empty((T, I), dtype=out_dtype, device=dev),
+            dW=empty((O, I), dtype=out_dtype, device=dev),
+            launches=0,        # library calls, also those that a phase call stands for
+            mark=None,         # optional callback(label), called before every C-ABI call (a benchmark records events)
+            track_flips=track_flips,
+            amax=scalars[1:4] if fp8 else None,
+            Xq=empty((T, I), dtype=wdt, device=dev) if fp8 else None,
+            dYq=empty((T, O), dtype=gdt, device=dev) if fp8 else None,
+            _scratch=scalars[4:6] if fp8 else None,
+            _desc=None, _as_made=W.is_contiguous())
+        self.__dict__.update(buffers)
         if track_flips:
             self.meta_prev = torch.empty_like(self.meta)
             self.flips = torch.zeros(1, dtype=torch.int64, device=dev)   # mask entries changed by the last prune
             self._have_prev = False
-        self.amax = torch.zeros(3, **f32) if fp8 else None     # max|X|, max|w~| (bf16 projection), max|dY|
-        self.Xq = self.dYq = self._scratch = None
-        if fp8:
-            self._scratch = torch.zeros(2, dtype=torch.int32, device=dev)
-            self.Xq = torch.empty((T, I), dtype=torch.float8_e4m3fn, device=dev)
-            self.dYq = torch.empty((T, O), dtype=torch.float8_e5m2, device=dev)
 
     def __setattr__(self, name, value):
+        d = self.__dict__
         if name in _DESCRIBED:
-            self.__dict__["_desc"] = None
-        self.__dict__[name] = value
+            d["_desc"] = None
+            d["_as_made"] = False
+        d[name] = value
 
     # One C call per phase (prune, forward, backward) on buffers described once: what a small layer costs is host time.
     # The per-call path below it runs when something wants to see the single calls or the tensors are of other sizes.
     def _describe(self):
-        d = B.LayerBuffers(self.O, self.I, self.T, B.E4M3 if self.fp8 else B.BF16, B._CODE_OF[self.Y.dtype],
-                           self.counter_cols, self.tensor_id & 0xffffffff, 0, self.seed & 0xffffffffffffffff,
-                           *[B._ptr(t) for t in (self.W, self.beta, self.amax, self.vals, self.meta, self.w_dense,
-                                                 self.gvals, self.gmeta, self.Xq, self.dYq, self.Y, self.dX, self.dW,
-                                                 self._scratch)])
+        tensors = (self.W, self.beta, self.amax, self.vals, self.meta, self.w_dense, self.gvals, self.gmeta, self.Xq,
+                   self.dYq, self.Y, self.dX, self.dW, self._scratch)
         x_shape, g_shape = torch.Size((self.T, self.I)), torch.Size((self.T, self.O))
         # a layer whose buffers were replaced by ones of other sizes or types is not described: the single calls check it
-        wdt, gdt = (B._TORCH_DT[B.E4M3], B._TORCH_DT[B.E5M2]) if self.fp8 else (_bf16, _bf16)
-        fits = (self.W.dtype is _bf16 and tuple(self.W.shape) == (self.O, self.I) and self.beta.dtype is torch.float32
-                and self.vals.dtype is wdt and tuple(self.vals.shape) == (self.O, self.I // 2)
-                and self.gvals.dtype is gdt and tuple(self.gvals.shape) == (self.O, self.T // 2)
-                and (self.w_dense is None or (self.w_dense.dtype is wdt and tuple(self.w_dense.shape) == (self.O, self.I)))
-                and self.Y.shape == g_shape and self.dX.shape == x_shape and tuple(self.dW.shape) == (self.O, self.I)
-                and self.dX.dtype is self.Y.dtype and self.dW.dtype is self.Y.dtype
-                and (not self.fp8 or (self.Xq.dtype is wdt and self.Xq.shape == x_shape
-                                      and self.dYq.dtype is gdt and self.dYq.shape == g_shape)))
+        fits = self._as_made or self._replaced_fit(x_shape, g_shape, tensors)
+        d = B.LayerBuffers(self.O, self.I, self.T, B.E4M3 if self.fp8 else B.BF16, B._CODE_OF[self.Y.dtype],
+                           self.counter_cols, self.tensor_id & 0xffffffff, 0, self.seed & 0xffffffffffffffff,
+                           *[None if t is None else t.data_ptr() for t in tensors])
         lib = self.ctx.lib
         self.__dict__["_desc"] = desc = (fits, ctypes.addressof(d), self.W.data_ptr(), lib.sste_layer_prune,
                                          lib.sste_layer_forward, lib.sste_layer_backward, x_shape, g_shape, d,
                                          lib.sste_layer_grads)
         return desc
+
+    def _replaced_fit(self, x_shape, g_shape, tensors):
+        wdt, gdt = (B._TORCH_DT[B.E4M3], B._TORCH_DT[B.E5M2]) if self.fp8 else (_bf16, _bf16)
+        w_shape = (self.O, self.I)
+        return (all(t is None or (t.is_cuda and t.is_contiguous()) for t in tensors)
+                and self.W.dtype is _bf16 and tuple(self.W.shape) == w_shape and self.beta.dtype is torch.float32
+                and self.vals.dtype is wdt and tuple(self.vals.shape) == (self.O, self.I // 2)
+                and self.gvals.dtype is gdt and tuple(self.gvals.shape) == (self.O, self.T // 2)
+                and (self.w_dense is None or (self.w_dense.dtype is wdt and tuple(self.w_dense.shape) == w_shape))
+                and self.Y.shape == g_shape and self.dX.shape == x_shape and tuple(self.dW.shape) == w_shape
+                and self.dX.dtype is self.Y.dtype and self.dW.dtype is self.Y.dtype
+                and (not self.fp8 or (self.Xq.dtype is wdt and self.Xq.shape == x_shape
+                                      and self.dYq.dtype is gdt and self.dYq.shape == g_shape)))
 
     def _amax(self, k):
         return self.amax[k:k + 1] if self.fp8 else None
