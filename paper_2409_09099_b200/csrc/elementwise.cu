@@ -11,6 +11,59 @@ constexpr int EW_THREADS = 256;
 constexpr int PC_ROWS = 32;                                  // rows of W per project+compress CTA
 constexpr int PC_CHUNKS = PC_ROWS * 16 / EW_THREADS;         // 16-byte chunks per thread
 
+// ---------------------------------------------------------------- two fp32 values per instruction
+
+// Two fp32 values in one register pair: one instruction per operation for both (sm_100 f32x2), each lane a single
+// rounded operation, subnormals included.
+using f32x2 = unsigned long long;
+// byte permute with the selector as the instruction takes it (four nibbles in the low half)
+__device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel)
+{
+    uint32_t r;
+    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(sel));
+    return r;
+}
+__device__ __forceinline__ f32x2 pack2(float lo, float hi)
+{
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float &lo, float &hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
+{
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f32x2 both(float v) { return pack2(v, v); }
+// a <= b, a >= b as 1.0f / 0.0f (0 if either is a NaN), one instruction
+__device__ __forceinline__ float one_if_le(float a, float b)
+{
+    float r;
+    asm("set.le.f32.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 one_if_le2(f32x2 a, f32x2 b)
+{
+    float a0, a1, b0, b1;
+    unpack2(a, a0, a1);
+    unpack2(b, b0, b1);
+    return pack2(one_if_le(a0, b0), one_if_le(a1, b1));
+}
+
 // ---------------------------------------------------------------- group of four: S_soft + kept pair
 
 struct SoftGroup {
@@ -73,6 +126,67 @@ __device__ __forceinline__ SoftGroup soft_group(uint32_t w01, uint32_t w23, floa
     return r;
 }
 
+// What the six comparisons of a group's magnitudes (i < j: m_i >= m_j, so that ties go to the lower index) come to, by table:
+//   x: byte-permute selector of the two kept halfwords | kept nibble p0 | p1 << 2 in bits 16-19 | selector of the threshold's
+//      halfword (the third in rank, the second-smallest magnitude) into the upper half of a word, in bits 24-31
+//   y: 0x80 in byte i where position i is kept
+// Entry number: bit k of the comparison (0,1) (0,2) (0,3) (1,2) (1,3) (2,3).  Codes that no order gives are filled alike.
+constexpr int PROJECT_ENTRIES = 64;
+struct ProjectTable { uint2 e[PROJECT_ENTRIES]; };
+constexpr ProjectTable project_table()
+{
+    ProjectTable t{};
+    for (int n = 0; n < PROJECT_ENTRIES; ++n) {
+        int wins[4] = {0, 0, 0, 0}, k = 0;
+        for (int i = 0; i < 4; ++i)
+            for (int j = i + 1; j < 4; ++j, ++k) ++wins[(n >> k) & 1 ? i : j];
+        int order[4] = {0, 1, 2, 3};       // by wins, descending (they are 3, 2, 1, 0 for every order of magnitudes)
+        for (int a = 0; a < 4; ++a)
+            for (int b = a + 1; b < 4; ++b)
+                if (wins[order[b]] > wins[order[a]]) { const int o = order[a]; order[a] = order[b]; order[b] = o; }
+        const int p0 = order[0] < order[1] ? order[0] : order[1], p1 = order[0] < order[1] ? order[1] : order[0], th = order[2];
+        t.e[n].x = (0x1010u + 0x22u * p0 + 0x2200u * p1) | (static_cast<uint32_t>(p0 | (p1 << 2)) << 16) |
+                   (static_cast<uint32_t>((2 * th) | ((2 * th + 1) << 4)) << 24);
+        t.e[n].y = (0x80u << (8 * p0)) | (0x80u << (8 * p1));
+    }
+    return t;
+}
+__device__ const ProjectTable project_table_dev = project_table();
+
+// The method's projection of one group by that table: w01 = a0 | a1 << 16, w23 = a2 | a3 << 16; v: the values before the
+// cast, right in the kept positions only (a kept |a| = t gives +0: the fma adds +0 to an exact zero of either sign).
+// The kernel is bound by instruction issue: sums and products run for two values at once, comparisons give 1.0 / 0.0 and are
+// added up as subnormal floats whose bit pattern is the byte offset of the table entry (about 40 instructions per group,
+// 84 with the rank by integer keys).
+struct Projected { uint2 e; f32x2 v01, v23; };
+template <bool FP8>
+__device__ __forceinline__ Projected project_group(uint32_t w01, uint32_t w23, f32x2 beta2, f32x2 wscale2, const uint8_t *lut)
+{
+    const uint32_t a0 = w01 << 16, a1 = w01 & 0xffff0000u, a2 = w23 << 16, a3 = w23 & 0xffff0000u;
+    const float m0 = fabsf(__uint_as_float(a0)), m1 = fabsf(__uint_as_float(a1));
+    const float m2 = fabsf(__uint_as_float(a2)), m3 = fabsf(__uint_as_float(a3));
+    constexpr int UNIT = 8;
+    auto unit2 = [](int lo, int hi) { return pack2(__int_as_float(UNIT << lo), __int_as_float(UNIT << hi)); };
+    f32x2 off2 = mul2(pack2(one_if_le(m1, m0), one_if_le(m2, m0)), unit2(0, 1));
+    off2 = fma2(pack2(one_if_le(m3, m0), one_if_le(m2, m1)), unit2(2, 3), off2);
+    off2 = fma2(pack2(one_if_le(m3, m1), one_if_le(m3, m2)), unit2(4, 5), off2);
+    float o0, o1;
+    unpack2(off2, o0, o1);
+    Projected r;
+    r.e = *reinterpret_cast<const uint2 *>(lut + __float_as_uint(o0) + __float_as_uint(o1));
+    const uint32_t t = prmt(w01, w23, r.e.x >> 16) & 0x7fff0000u;         // fp32 bits of the threshold
+    // sign(a) (|a| - t) as the single subtraction a - copysign(t, a)
+    auto st = [&](uint32_t a) { return __uint_as_float((~a & 0x80000000u) | t); };       // -copysign(t, a)
+    const f32x2 zero2 = both(0.0f);
+    r.v01 = fma2(add2(pack2(__uint_as_float(a0), __uint_as_float(a1)), pack2(st(a0), st(a1))), beta2, zero2);
+    r.v23 = fma2(add2(pack2(__uint_as_float(a2), __uint_as_float(a3)), pack2(st(a2), st(a3))), beta2, zero2);
+    if (FP8) {
+        r.v01 = mul2(r.v01, wscale2);
+        r.v23 = mul2(r.v23, wscale2);
+    }
+    return r;
+}
+
 // ---------------------------------------------------------------- project + compress
 
 // One CTA: 32 rows x 128 input features of W (a quarter of a metadata atom, 512 contiguous bytes of its
@@ -85,8 +199,10 @@ project_compress_kernel(const uint4 *__restrict__ W, int I, const float *__restr
                         uint8_t *__restrict__ meta, void *__restrict__ dense)
 {
     __shared__ __align__(16) uint8_t meta_s[512];
+    __shared__ uint2 lut[PROJECT_ENTRIES];
     const int tid = threadIdx.x;
     const int kb = blockIdx.x, rb = blockIdx.y;
+    if (MODE == 0 && tid < PROJECT_ENTRIES) lut[tid] = project_table_dev.e[tid];
     sste_pdl_trigger();
     sste_pdl_wait();
     const float beta = *beta_dev;
@@ -100,6 +216,8 @@ project_compress_kernel(const uint4 *__restrict__ W, int I, const float *__restr
         const int row = c >> 4, kc = c & 15;
         in[i] = __ldg(W + (static_cast<size_t>(rb) * PC_ROWS + row) * row_chunks + kb * 16 + kc);
     }
+    if (MODE == 0) __syncthreads();              // the table is in place
+    const f32x2 beta2 = both(beta), wscale2 = both(wscale);
 #pragma unroll
     for (int i = 0; i < PC_CHUNKS; ++i) {
         const int c = i * EW_THREADS + tid;
@@ -110,6 +228,29 @@ project_compress_kernel(const uint4 *__restrict__ W, int I, const float *__restr
         uint32_t mbyte = 0;
 #pragma unroll
         for (int g = 0; g < 2; ++g) {
+            if (MODE == 0) {
+                const Projected s = project_group<FP8>(raw[2 * g], raw[2 * g + 1], beta2, wscale2, reinterpret_cast<const uint8_t *>(lut));
+                const uint32_t nib = (s.e.x >> 16) & 0xfu;
+                float v[4];
+                unpack2(s.v01, v[0], v[1]);
+                unpack2(s.v23, v[2], v[3]);
+                // masks of the kept positions: the selector's high bit replicates a byte's sign bit
+                if (FP8) {
+                    const uint32_t e01 = __nv_cvt_float2_to_fp8x2(make_float2(v[0], v[1]), __NV_SATFINITE, __NV_E4M3);
+                    const uint32_t e23 = __nv_cvt_float2_to_fp8x2(make_float2(v[2], v[3]), __NV_SATFINITE, __NV_E4M3);
+                    const uint32_t all = prmt(e01, e23, 0x5410);
+                    dn[g][0] = all & prmt(s.e.y, 0, 0xba98);
+                    kept[g] = prmt(all, 0, 0x4400u | (nib & 3u) | ((nib & 12u) << 2));
+                } else {
+                    const __nv_bfloat162 d01 = __floats2bfloat162_rn(v[0], v[1]), d23 = __floats2bfloat162_rn(v[2], v[3]);
+                    const uint32_t w01 = *reinterpret_cast<const uint32_t *>(&d01), w23 = *reinterpret_cast<const uint32_t *>(&d23);
+                    dn[g][0] = w01 & prmt(s.e.y, 0, 0x9988);
+                    dn[g][1] = w23 & prmt(s.e.y, 0, 0xbbaa);
+                    kept[g] = prmt(w01, w23, s.e.x);
+                }
+                mbyte |= nib << (4 * g);
+                continue;
+            }
             const SoftGroup s = soft_group<FP8, MODE>(raw[2 * g], raw[2 * g + 1], beta, wscale, gamma);
             if (FP8) {
                 const uint32_t e01 = __nv_cvt_float2_to_fp8x2(make_float2(s.w[0], s.w[1]), __NV_SATFINITE, __NV_E4M3);
@@ -256,57 +397,6 @@ __device__ __forceinline__ void philox4x32_10(uint32_t c0, uint32_t c1, uint32_t
 }
 
 // ---------------------------------------------------------------- MVUE of two groups
-
-// Two fp32 values in one register pair: one instruction per operation for both (sm_100 f32x2), each lane a single
-// rounded operation, subnormals included.
-using f32x2 = unsigned long long;
-// byte permute with the selector as the instruction takes it (four nibbles in the low half)
-__device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel)
-{
-    uint32_t r;
-    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(sel));
-    return r;
-}
-__device__ __forceinline__ f32x2 pack2(float lo, float hi)
-{
-    f32x2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void unpack2(f32x2 v, float &lo, float &hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b)
-{
-    f32x2 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b)
-{
-    f32x2 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
-{
-    f32x2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-__device__ __forceinline__ f32x2 both(float v) { return pack2(v, v); }
-// a <= b, a >= b as 1.0f / 0.0f (0 if either is a NaN), one instruction
-__device__ __forceinline__ float one_if_le(float a, float b)
-{
-    float r;
-    asm("set.le.f32.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ f32x2 one_if_le2(f32x2 a, f32x2 b)
-{
-    float a0, a1, b0, b1;
-    unpack2(a, a0, a1);
-    unpack2(b, b0, b1);
-    return pack2(one_if_le(a0, b0), one_if_le(a1, b1));
-}
 
 // What a group's draw comes to, by table: the kept positions q0 < q1 and how to pick their bits.
 //   x: byte-permute selector over (a0 a1 | a2 a3) for the two kept elements | (q0 | q1 << 2) << 16
