@@ -168,3 +168,8 @@ sste_status sste_bwd_products(sste_ctx *ctx, const void *gvals, const void *gmet
 // two sste_crop_2d in one launch (arguments as checked by that call)
 sste_status sste_crop_two(sste_ctx *ctx, const void *src0, int rows_p0, int cols_p0, void *dst0, int rows0, int cols0,
                           const void *src1, int rows_p1, int cols_p1, void *dst1, int rows1, int cols1, void *stream);
+
+// sste_pad_2d of dY [rows, cols] into dYp [T, O] and sste_mvue_sparsify (bf16) of the result, in one pass.
+sste_status sste_mvue_padded(sste_ctx *ctx, const void *dY, int rows, int cols, void *dYp, int T, int O, uint64_t seed,
+                             uint32_t tensor_id, uint32_t step, uint64_t token_offset, int counter_cols, void *gvals,
+                             void *gmeta, void *stream);

@@ -557,6 +557,50 @@ mvue_groups_kernel(const uint2 *__restrict__ a, const uint32_t *__restrict__ k24
     }
 }
 
+// ---------------------------------------------------------------- rows of any length, eight elements at a time
+
+// Eight elements from element offset `first` (may be anything) of the array [begin, end) of elements counted from the
+// 16-byte aligned address `base`; the caller has checked begin <= first, first + 8 <= end.
+__device__ __forceinline__ bool load8_fits(size_t first, size_t begin, size_t end)
+{
+    // the aligned vectors touched lie inside the array
+    return (first & ~static_cast<size_t>(7)) >= begin && ((first + 7) | 7) < end;
+}
+__device__ __forceinline__ uint4 load8(const uint4 *__restrict__ base, size_t first)
+{
+    const uint4 a = __ldg(base + (first >> 3));
+    const uint32_t sh = static_cast<uint32_t>(first) & 7u;
+    if (sh == 0) return a;
+    const uint4 b = __ldg(base + (first >> 3) + 1);
+    const uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+    uint32_t u[6], t[5], o[4];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) u[k] = (sh & 4u) ? w[k + 2] : w[k];
+#pragma unroll
+    for (int k = 0; k < 5; ++k) t[k] = (sh & 2u) ? u[k + 1] : u[k];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) o[k] = __funnelshift_r(t[k], t[k + 1], 16u * (sh & 1u));
+    return make_uint4(o[0], o[1], o[2], o[3]);
+}
+
+// A [rows, cols] array of 2-byte elements whose rows may start anywhere, seen as the top-left corner of a larger one of zeros.
+struct RaggedRows {
+    const uint16_t *src;
+    uint32_t rows, cols;
+    // elements [c0, c0 + 8) of row r; c0 a multiple of 8
+    __device__ __forceinline__ uint4 load(uint32_t r, uint32_t c0) const
+    {
+        if (r >= rows || c0 >= cols) return make_uint4(0u, 0u, 0u, 0u);
+        const size_t lead = (reinterpret_cast<uintptr_t>(src) & 15u) / 2;       // src starts `lead` elements into its vector
+        const size_t first = lead + static_cast<size_t>(r) * cols + c0, end = lead + static_cast<size_t>(rows) * cols;
+        if (c0 + 8 <= cols && load8_fits(first, lead, end)) return load8(reinterpret_cast<const uint4 *>(src - lead), first);
+        uint32_t e[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) e[i] = (c0 + i < cols) ? __ldg(src + static_cast<size_t>(r) * cols + c0 + i) : 0u;
+        return make_uint4(e[0] | (e[1] << 16), e[2] | (e[3] << 16), e[4] | (e[5] << 16), e[6] | (e[7] << 16));
+    }
+};
+
 // ---------------------------------------------------------------- MVUE + compress (transposing)
 
 // One CTA: 128 tokens x 64 output columns of dY (half a metadata atom).  A thread handles 4 tokens x 8 columns
@@ -566,12 +610,14 @@ mvue_groups_kernel(const uint2 *__restrict__ a, const uint32_t *__restrict__ k24
 // the loads); two tasks of 128 columns, tasks of 4 columns, and persistent CTAs with cp.async prefetch were slower.
 // ANY_COUNTER: counter_cols is not a multiple of 4 (a padded, odd column count), so a thread's eight
 // consecutive group indices do not start on a Philox block and span three blocks instead of two.
-template <bool FP8, bool ANY_COUNTER>
+// PADDED: dY is given as ragged rows; the kernel also writes the zero-padded copy that grad_X reads (a padding pass of its
+// own took 35 us of reading and writing for 1000 rows of 50257).
+template <bool FP8, bool ANY_COUNTER, bool PADDED = false>
 __global__ void __launch_bounds__(EW_THREADS, 4)
 mvue_kernel(const uint4 *__restrict__ dY, int O, int T, uint32_t key0, uint32_t key1, uint32_t tensor_id,
             uint32_t step, uint64_t tg_offset, uint32_t counter_cols, const float *__restrict__ g_amax_dev,
             void *__restrict__ gvals,
-            uint8_t *__restrict__ gmeta, void *__restrict__ dense_q)
+            uint8_t *__restrict__ gmeta, void *__restrict__ dense_q, const RaggedRows rag, uint4 *__restrict__ padded)
 {
     // bf16: 64 rows x 32 words; fp8: 64 rows x 16 words
     __shared__ __align__(16) uint32_t vals_s[64 * (FP8 ? 16 : 32)];
@@ -592,7 +638,14 @@ mvue_kernel(const uint4 *__restrict__ dY, int O, int T, uint32_t key0, uint32_t 
         const size_t tok0 = static_cast<size_t>(tb) * 128 + 4 * tgl;
         uint4 in[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) in[i] = __ldg(dY + (tok0 + i) * row_chunks + jb * 8 + jc);
+        for (int i = 0; i < 4; ++i) {
+            if (PADDED) {
+                in[i] = rag.load(static_cast<uint32_t>(tok0) + i, jb * 64u + jc * 8u);
+                padded[(tok0 + i) * row_chunks + jb * 8 + jc] = in[i];
+            } else {
+                in[i] = __ldg(dY + (tok0 + i) * row_chunks + jb * 8 + jc);
+            }
+        }
 
         const uint64_t g0 = (tg_offset + static_cast<uint64_t>(tb) * 32 + tgl) * static_cast<uint64_t>(counter_cols) +
                             static_cast<uint64_t>(jb) * 64 + jc * 8;
@@ -901,59 +954,18 @@ decompress_kernel(const uint4 *__restrict__ vals, const uint8_t *__restrict__ me
 // accesses only where a vector is cut by a row end or an array end.  Element by element, with a 64-bit division for each,
 // 1000 rows of 50257 took 50 us to pad and 119 us to crop; now 35 us each (about 6 TB/s).
 
-// Eight elements from element offset `first` (may be anything) of the array [begin, end) of elements counted from the
-// 16-byte aligned address `base`; the caller has checked begin <= first, first + 8 <= end.
-__device__ __forceinline__ bool load8_fits(size_t first, size_t begin, size_t end)
-{
-    // the aligned vectors touched lie inside the array
-    return (first & ~static_cast<size_t>(7)) >= begin && ((first + 7) | 7) < end;
-}
-__device__ __forceinline__ uint4 load8(const uint4 *__restrict__ base, size_t first)
-{
-    const uint4 a = __ldg(base + (first >> 3));
-    const uint32_t sh = static_cast<uint32_t>(first) & 7u;
-    if (sh == 0) return a;
-    const uint4 b = __ldg(base + (first >> 3) + 1);
-    const uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-    uint32_t u[6], t[5], o[4];
-#pragma unroll
-    for (int k = 0; k < 6; ++k) u[k] = (sh & 4u) ? w[k + 2] : w[k];
-#pragma unroll
-    for (int k = 0; k < 5; ++k) t[k] = (sh & 2u) ? u[k + 1] : u[k];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) o[k] = __funnelshift_r(t[k], t[k + 1], 16u * (sh & 1u));
-    return make_uint4(o[0], o[1], o[2], o[3]);
-}
-
 // dst [rows_p, cols_p] <- src [rows, cols] in the top-left corner, zeros elsewhere; one thread per 8 destination elements.
 // INDEX: unsigned type that holds the number of destination vectors (a 64-bit division costs more than the copy).
 template <typename INDEX>
 __global__ void __launch_bounds__(EW_THREADS)
-pad_2d_kernel(const uint16_t *__restrict__ src, uint32_t rows, uint32_t cols, uint4 *__restrict__ dst, uint32_t vec_per_row,
-              INDEX n_vec)
+pad_2d_kernel(const RaggedRows src, uint4 *__restrict__ dst, uint32_t vec_per_row, INDEX n_vec)
 {
     sste_pdl_trigger();
     sste_pdl_wait();
-    const size_t lead = (reinterpret_cast<uintptr_t>(src) & 15u) / 2;       // src starts `lead` elements into its vector
-    const uint4 *base = reinterpret_cast<const uint4 *>(src - lead);
-    const size_t end = lead + static_cast<size_t>(rows) * cols;
     for (INDEX v = static_cast<INDEX>(blockIdx.x) * EW_THREADS + threadIdx.x; v < n_vec;
          v += static_cast<INDEX>(gridDim.x) * EW_THREADS) {
-        const uint32_t r = static_cast<uint32_t>(v / vec_per_row), c0 = static_cast<uint32_t>(v - static_cast<INDEX>(r) * vec_per_row) * 8u;
-        uint4 out = make_uint4(0u, 0u, 0u, 0u);
-        if (r < rows && c0 < cols) {
-            const size_t first = lead + static_cast<size_t>(r) * cols + c0;
-            if (c0 + 8 <= cols && load8_fits(first, lead, end)) {
-                out = load8(base, first);
-            } else {
-                uint32_t e[8];
-#pragma unroll
-                for (int i = 0; i < 8; ++i)
-                    e[i] = (c0 + i < cols) ? __ldg(src + static_cast<size_t>(r) * cols + c0 + i) : 0u;
-                out = make_uint4(e[0] | (e[1] << 16), e[2] | (e[3] << 16), e[4] | (e[5] << 16), e[6] | (e[7] << 16));
-            }
-        }
-        dst[v] = out;
+        const uint32_t r = static_cast<uint32_t>(v / vec_per_row);
+        dst[v] = src.load(r, static_cast<uint32_t>(v - static_cast<INDEX>(r) * vec_per_row) * 8u);
     }
 }
 
@@ -1224,10 +1236,31 @@ extern "C" sste_status sste_mvue_sparsify(sste_ctx *ctx, const void *dY, int T, 
     const bool f8 = (odt == SSTE_E5M2), any = (ccols % 4) != 0;
 #define SSTE_MVUE_LAUNCH(F8, ANY)                                                                                   \
     sste_launch(mvue_kernel<F8, ANY>, dim3(grid), dim3(EW_THREADS), 0, s, g, O, T, key0, key1, tensor_id, step, tg0, \
-                ccols, F8 ? g_amax_dev : nullptr, gvals, gm, F8 ? dense_q_out : nullptr)
+                ccols, F8 ? g_amax_dev : nullptr, gvals, gm, F8 ? dense_q_out : nullptr, RaggedRows{}, nullptr)
     if (f8) { if (any) SSTE_MVUE_LAUNCH(true, true); else SSTE_MVUE_LAUNCH(true, false); }
     else { if (any) SSTE_MVUE_LAUNCH(false, true); else SSTE_MVUE_LAUNCH(false, false); }
 #undef SSTE_MVUE_LAUNCH
+    return launch_result();
+}
+
+sste_status sste_mvue_padded(sste_ctx *ctx, const void *dY, int rows, int cols, void *dYp, int T, int O, uint64_t seed,
+                             uint32_t tensor_id, uint32_t step, uint64_t token_offset, int counter_cols, void *gvals,
+                             void *gmeta, void *stream)
+{
+    if (!ctx || !dY || !dYp || !gvals || !gmeta || counter_cols < 0 || counter_cols > O) return SSTE_ERR_INVALID_ARG;
+    if (!sste_mult128(O) || !sste_mult128(T) || rows <= 0 || cols <= 0 || rows > T || cols > O || token_offset % 4 != 0)
+        return SSTE_ERR_SHAPE;
+    if (!sste_aligned(dY, 2) || !sste_aligned(dYp, 128) || !sste_aligned(gvals, 128) || !sste_aligned(gmeta, 128))
+        return SSTE_ERR_ALIGN;
+    sste_device_guard guard(ctx->device);
+    if (!guard.ok) return SSTE_ERR_CUDA;
+    const uint32_t ccols = static_cast<uint32_t>(counter_cols == 0 ? O : counter_cols);
+    const RaggedRows rag{static_cast<const uint16_t *>(dY), static_cast<uint32_t>(rows), static_cast<uint32_t>(cols)};
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    auto kern = ccols % 4 ? mvue_kernel<false, true, true> : mvue_kernel<false, false, true>;
+    sste_launch(kern, dim3(O / 64, T / 128), dim3(EW_THREADS), 0, s, nullptr, O, T, static_cast<uint32_t>(seed),
+                static_cast<uint32_t>(seed >> 32), tensor_id, step, token_offset / 4, ccols, nullptr, gvals,
+                static_cast<uint8_t *>(gmeta), nullptr, rag, static_cast<uint4 *>(dYp));
     return launch_result();
 }
 
@@ -1396,13 +1429,12 @@ extern "C" sste_status sste_pad_2d(sste_ctx *ctx, const void *src, int rows, int
     const size_t n_vec = static_cast<size_t>(rows_p) * cols_p / 8;
     const dim3 grid(grid_for(n_vec, ctx->sm_count));
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    const RaggedRows rag{static_cast<const uint16_t *>(src), static_cast<uint32_t>(rows), static_cast<uint32_t>(cols)};
     // 32-bit indices with room for one grid stride beyond the end
     if (n_vec < (size_t(1) << 31))
-        sste_launch(pad_2d_kernel<uint32_t>, grid, dim3(EW_THREADS), 0, s, static_cast<const uint16_t *>(src), rows, cols,
-                    static_cast<uint4 *>(dst), cols_p / 8, n_vec);
+        sste_launch(pad_2d_kernel<uint32_t>, grid, dim3(EW_THREADS), 0, s, rag, static_cast<uint4 *>(dst), cols_p / 8, n_vec);
     else
-        sste_launch(pad_2d_kernel<uint64_t>, grid, dim3(EW_THREADS), 0, s, static_cast<const uint16_t *>(src), rows, cols,
-                    static_cast<uint4 *>(dst), cols_p / 8, n_vec);
+        sste_launch(pad_2d_kernel<uint64_t>, grid, dim3(EW_THREADS), 0, s, rag, static_cast<uint4 *>(dst), cols_p / 8, n_vec);
     return launch_result();
 }
 

@@ -97,8 +97,15 @@ extern "C" sste_status sste_padded_backward(sste_ctx *ctx, const sste_padded_lay
 {
     if (!ctx || !padded_ok(l) || !dY) return SSTE_ERR_INVALID_ARG;
     const sste_layer &in = l->inner;
-    sste_status st = sste_pad_2d(ctx, dY, l->T, l->O, l->dYp, in.T, in.O, stream);
-    if (st == SSTE_OK) st = sste_layer_backward(ctx, &in, l->Xp, l->dYp, step, token_offset, stream);
+    sste_status st;
+    if (fp8_of(&in)) {       // the quantisation needs max|dY| before the sparsification reads it
+        st = sste_pad_2d(ctx, dY, l->T, l->O, l->dYp, in.T, in.O, stream);
+        if (st == SSTE_OK) st = sste_layer_backward(ctx, &in, l->Xp, l->dYp, step, token_offset, stream);
+    } else {
+        st = sste_mvue_padded(ctx, dY, l->T, l->O, l->dYp, in.T, in.O, in.seed, in.tensor_id, step, token_offset, in.counter_cols,
+                              in.gvals, in.gmeta, stream);
+        if (st == SSTE_OK) st = sste_layer_grads(ctx, &in, l->Xp, l->dYp, stream);
+    }
     if (st != SSTE_OK) return st;
     if (l->dX && l->dW)
         return sste_crop_two(ctx, in.dX, in.T, in.I, l->dX, l->T, l->I, in.dW, in.O, in.I, l->dW, l->O, l->I, stream);
