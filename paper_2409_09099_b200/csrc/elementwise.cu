@@ -566,12 +566,9 @@ __device__ __forceinline__ bool load8_fits(size_t first, size_t begin, size_t en
     // the aligned vectors touched lie inside the array
     return (first & ~static_cast<size_t>(7)) >= begin && ((first + 7) | 7) < end;
 }
-__device__ __forceinline__ uint4 load8(const uint4 *__restrict__ base, size_t first)
+// the eight elements from element `sh` of the two consecutive vectors a, b on
+__device__ __forceinline__ uint4 shift8(const uint4 &a, const uint4 &b, uint32_t sh)
 {
-    const uint4 a = __ldg(base + (first >> 3));
-    const uint32_t sh = static_cast<uint32_t>(first) & 7u;
-    if (sh == 0) return a;
-    const uint4 b = __ldg(base + (first >> 3) + 1);
     const uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
     uint32_t u[6], t[5], o[4];
 #pragma unroll
@@ -581,6 +578,12 @@ __device__ __forceinline__ uint4 load8(const uint4 *__restrict__ base, size_t fi
 #pragma unroll
     for (int k = 0; k < 4; ++k) o[k] = __funnelshift_r(t[k], t[k + 1], 16u * (sh & 1u));
     return make_uint4(o[0], o[1], o[2], o[3]);
+}
+__device__ __forceinline__ uint4 load8(const uint4 *__restrict__ base, size_t first)
+{
+    const uint4 a = __ldg(base + (first >> 3));
+    const uint32_t sh = static_cast<uint32_t>(first) & 7u;
+    return sh == 0 ? a : shift8(a, __ldg(base + (first >> 3) + 1), sh);
 }
 
 // A [rows, cols] array of 2-byte elements whose rows may start anywhere, seen as the top-left corner of a larger one of zeros.
@@ -598,6 +601,28 @@ struct RaggedRows {
 #pragma unroll
         for (int i = 0; i < 8; ++i) e[i] = (c0 + i < cols) ? __ldg(src + static_cast<size_t>(r) * cols + c0 + i) : 0u;
         return make_uint4(e[0] | (e[1] << 16), e[2] | (e[3] << 16), e[4] | (e[5] << 16), e[6] | (e[7] << 16));
+    }
+    // the same of four consecutive rows; all their loads are under way before the first is used
+    __device__ __forceinline__ void load4(uint32_t r, uint32_t c0, uint4 (&out)[4]) const
+    {
+        const size_t lead = (reinterpret_cast<uintptr_t>(src) & 15u) / 2;
+        const size_t first = lead + static_cast<size_t>(r) * cols + c0;
+        if (r + 3 < rows && c0 + 8 <= cols && (first & ~static_cast<size_t>(7)) >= lead &&
+            first + 3u * static_cast<size_t>(cols) + 16 <= lead + static_cast<size_t>(rows) * cols) {
+            const uint4 *base = reinterpret_cast<const uint4 *>(src - lead);
+            uint4 a[4], b[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const uint4 *v = base + ((first + static_cast<size_t>(i) * cols) >> 3);
+                a[i] = __ldg(v);
+                b[i] = __ldg(v + 1);
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) out[i] = shift8(a[i], b[i], static_cast<uint32_t>(first + static_cast<size_t>(i) * cols) & 7u);
+        } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) out[i] = load(r + i, c0);
+        }
     }
 };
 
@@ -638,13 +663,12 @@ mvue_kernel(const uint4 *__restrict__ dY, int O, int T, uint32_t key0, uint32_t 
         const size_t tok0 = static_cast<size_t>(tb) * 128 + 4 * tgl;
         uint4 in[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            if (PADDED) {
-                in[i] = rag.load(static_cast<uint32_t>(tok0) + i, jb * 64u + jc * 8u);
-                padded[(tok0 + i) * row_chunks + jb * 8 + jc] = in[i];
-            } else {
-                in[i] = __ldg(dY + (tok0 + i) * row_chunks + jb * 8 + jc);
-            }
+        for (int i = 0; i < 4; ++i)
+            if (!PADDED) in[i] = __ldg(dY + (tok0 + i) * row_chunks + jb * 8 + jc);
+        if (PADDED) {
+            rag.load4(static_cast<uint32_t>(tok0), jb * 64u + jc * 8u, in);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) padded[(tok0 + i) * row_chunks + jb * 8 + jc] = in[i];
         }
 
         const uint64_t g0 = (tg_offset + static_cast<uint64_t>(tb) * 32 + tgl) * static_cast<uint64_t>(counter_cols) +
