@@ -61,6 +61,7 @@ extern "C" sste_status sste_create(sste_ctx **out, int device, void *workspace, 
     ctx->splitk_partials = nullptr;
     ctx->splitk_tickets = nullptr;
     ctx->splitk_partial_bytes = 0;
+    ctx->zero_after = nullptr;
     if (workspace_bytes > SSTE_WS_SPLITK_PARTIALS_OFF + (size_t(1) << 20)) {
         ctx->splitk_partials = reinterpret_cast<float *>(ws + SSTE_WS_SPLITK_PARTIALS_OFF);
         ctx->splitk_partial_bytes = workspace_bytes - SSTE_WS_SPLITK_PARTIALS_OFF;

@@ -22,6 +22,7 @@ struct sste_ctx {
     float *splitk_partials;         // fp32 partial tiles of split-K products; null if the workspace is minimal
     unsigned int *splitk_tickets;   // arrival counters of the split tiles, zero between launches
     size_t splitk_partial_bytes;
+    unsigned int *zero_after;       // a word that every product empties when it starts; null but in a layer call's own copy
 };
 
 constexpr int SSTE_MAX_REDUCE_BLOCKS = 1024;
@@ -152,9 +153,15 @@ inline cudaError_t sste_launch(void (*kern)(KArgs...), dim3 grid, dim3 block, si
 // Process-wide count of kernels this library has launched (read by sste_debug_launch_count).
 void sste_count_launches(int n);
 
-// sste_amax / sste_project_amax without a memset in front: the running maximum and the arrival counter live in 8 bytes of
-// the caller's (zero before and after every call) and the block that arrives last stores the result.
+// An amax pass and the kernel that quantises with its result, without a memset in front: the pass leaves the maximum in
+// *scratch (zero before), the second kernel stores it in *amax_dev, and the next product of a context whose zero_after is
+// scratch empties it.
 sste_status sste_amax_scratch(sste_ctx *ctx, const void *x, size_t n, float *amax_dev, void *scratch, void *stream);
+sste_status sste_quantize_scratch(sste_ctx *ctx, const void *x, size_t n, float *amax_dev, void *scratch, void *q, void *stream);
+sste_status sste_mvue_scratch(sste_ctx *ctx, const void *dY, int T, int O, uint64_t seed, uint32_t tensor_id, uint32_t step,
+                              uint64_t token_offset, int counter_cols, float *g_amax_dev, void *scratch, void *gvals,
+                              void *gmeta, void *dense_q_out, void *stream);
+// sste_project_amax without a memset: 8 bytes of scratch, zero before and after.
 sste_status sste_project_amax_scratch(sste_ctx *ctx, const void *W, int O, int I, const float *beta_dev, float *amax_dev,
                                       void *scratch, void *stream);
 

@@ -11,6 +11,22 @@ constexpr int EW_THREADS = 256;
 constexpr int PC_ROWS = 32;                                  // rows of W per project+compress CTA
 constexpr int PC_CHUNKS = PC_ROWS * 16 / EW_THREADS;         // 16-byte chunks per thread
 
+// ---------------------------------------------------------------- an amax that the kernel in front has found
+
+// The amax a kernel quantises with.  scratch NULL: it is in *amax.  Otherwise the kernel in front of this one has left it in
+// *scratch only (as the bits of a non-negative fp32); this kernel publishes it in *amax, and the product behind it empties
+// the scratch.  That keeps the amax kernel free of a last block's chain of atomics and fences, which was 2 of the 3-4 us
+// that a small tensor's took.  (Counting this kernel's blocks to empty it here made them queue up at that address:
+// project + compress of 45 M weights 35 -> 85 us.)
+struct AmaxIn { float *amax; const unsigned int *scratch; };
+__device__ __forceinline__ float amax_take(const AmaxIn &a, bool publish)
+{
+    if (!a.scratch) return *a.amax;
+    const float v = __uint_as_float(*a.scratch);
+    if (publish) *a.amax = v;
+    return v;
+}
+
 // ---------------------------------------------------------------- two fp32 values per instruction
 
 // Two fp32 values in one register pair: one instruction per operation for both (sm_100 f32x2), each lane a single
@@ -640,7 +656,7 @@ struct RaggedRows {
 template <bool FP8, bool ANY_COUNTER, bool PADDED = false>
 __global__ void __launch_bounds__(EW_THREADS, 4)
 mvue_kernel(const uint4 *__restrict__ dY, int O, int T, uint32_t key0, uint32_t key1, uint32_t tensor_id,
-            uint32_t step, uint64_t tg_offset, uint32_t counter_cols, const float *__restrict__ g_amax_dev,
+            uint32_t step, uint64_t tg_offset, uint32_t counter_cols, const AmaxIn g_amax,
             void *__restrict__ gvals,
             uint8_t *__restrict__ gmeta, void *__restrict__ dense_q, const RaggedRows rag, uint4 *__restrict__ padded)
 {
@@ -651,10 +667,10 @@ mvue_kernel(const uint4 *__restrict__ dY, int O, int T, uint32_t key0, uint32_t 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int jb = blockIdx.x, tb = blockIdx.y;   // column block (64), token block
     if (tid < MVUE_ENTRIES) lut[tid] = FP8 ? mvue_table_fp8.e[tid] : mvue_table_bf16.e[tid];
-    __syncthreads();
     sste_pdl_trigger();
     sste_pdl_wait();
-    const float gscale = FP8 ? sste_scale_from_amax(*g_amax_dev, 57344.0f) : 1.0f;
+    const float gscale = FP8 ? sste_scale_from_amax(amax_take(g_amax, jb == 0 && tb == 0 && tid == 0), 57344.0f) : 1.0f;
+    __syncthreads();                              // the table is in place
     const size_t row_chunks = static_cast<size_t>(O) / 8;
 
     {
@@ -785,33 +801,24 @@ mvue_kernel(const uint4 *__restrict__ dY, int O, int T, uint32_t key0, uint32_t 
 
 // ---------------------------------------------------------------- FP8 helpers
 
-// *amax_dev = max over the grid of every thread's `bits`, the bit patterns of non-negative fp32 values, which order like
-// unsigned integers.  One atomic per block: with one per warp the 9472 of a full grid queued up at the one address for
-// 9 us, whatever the tensor's size (amax of 12.6 MB: 10.3 -> 6.1 us).  scratch NULL: *amax_dev was zeroed by a memset in
-// front of the kernel.  Otherwise scratch[0] takes the running maximum and scratch[1] counts the blocks; the last one
-// stores the result and leaves both zero: no memset, which would also keep this kernel from starting early (-2 us).
-__device__ __forceinline__ void grid_max_to(uint32_t bits, float *amax_dev, unsigned int *scratch)
+// *acc = max(*acc, every thread's `bits`), the bit patterns of non-negative fp32 values, which order like unsigned
+// integers.  One atomic per block: with one per warp the 9472 of a full grid queued up at the one address for 9 us,
+// whatever the tensor's size (amax of 12.6 MB: 10.3 -> 6.1 us).  True in the thread that did it, false in all others.
+__device__ __forceinline__ bool grid_max_to(uint32_t bits, unsigned int *acc)
 {
     __shared__ unsigned int best_s[EW_THREADS / 32];
     bits = __reduce_max_sync(0xffffffffu, bits);
     if ((threadIdx.x & 31) == 0) best_s[threadIdx.x >> 5] = bits;
     __syncthreads();
-    if (threadIdx.x != 0) return;
+    if (threadIdx.x != 0) return false;
 #pragma unroll
     for (int w = 1; w < EW_THREADS / 32; ++w) bits = max(bits, best_s[w]);
-    unsigned int *acc = scratch ? scratch : reinterpret_cast<unsigned int *>(amax_dev);
     if (bits != 0) atomicMax(acc, bits);
-    if (!scratch) return;
-    __threadfence();
-    if (atomicAdd(scratch + 1, 1u) == gridDim.x - 1) {
-        __threadfence();
-        *reinterpret_cast<unsigned int *>(amax_dev) = atomicExch(scratch, 0u);
-        scratch[1] = 0u;
-    }
+    return true;
 }
 
 __global__ void __launch_bounds__(EW_THREADS)
-amax_kernel(const uint4 *__restrict__ x, size_t n_chunks, float *__restrict__ amax_dev, unsigned int *__restrict__ scratch)
+amax_kernel(const uint4 *__restrict__ x, size_t n_chunks, unsigned int *__restrict__ acc)
 {
     uint32_t best2 = 0;   // magnitude bits of bf16 compare like unsigned integers: running maximum in both halves
     sste_pdl_trigger();
@@ -830,7 +837,7 @@ amax_kernel(const uint4 *__restrict__ x, size_t n_chunks, float *__restrict__ am
             best2 = __vmaxu2(best2, v[j].w & 0x7fff7fffu);
         }
     }
-    grid_max_to(max(best2 & 0xffffu, best2 >> 16) << 16, amax_dev, scratch);
+    grid_max_to(max(best2 & 0xffffu, best2 >> 16) << 16, acc);
 }
 
 // amax of the bf16 projection w~ = bf16(beta * S_soft(W)) without writing it: rounding to bf16 is monotone,
@@ -863,7 +870,17 @@ project_amax_kernel(const uint4 *__restrict__ W, size_t n_chunks, const float *_
             }
         }
     }
-    grid_max_to(sste_f32_to_bf16_bits(best) << 16, amax_dev, scratch);
+    // scratch NULL: *amax_dev was zeroed by a memset.  Otherwise scratch[0] takes the maximum, scratch[1] counts the blocks,
+    // and the last one stores the result and leaves both zero.
+    unsigned int *acc = scratch ? scratch : reinterpret_cast<unsigned int *>(amax_dev);
+    if (grid_max_to(sste_f32_to_bf16_bits(best) << 16, acc) && scratch) {
+        __threadfence();
+        if (atomicAdd(scratch + 1, 1u) == gridDim.x - 1) {
+            __threadfence();
+            *reinterpret_cast<unsigned int *>(amax_dev) = atomicExch(scratch, 0u);
+            scratch[1] = 0u;
+        }
+    }
 }
 
 __global__ void fp8_scale_kernel(const float *amax_dev, float fp8_max, float *scale_dev, float *inv_scale_dev)
@@ -878,12 +895,12 @@ __global__ void fp8_scale_kernel(const float *amax_dev, float fp8_max, float *sc
 
 template <bool E5M2>
 __global__ void __launch_bounds__(EW_THREADS)
-quantize_kernel(const uint4 *__restrict__ x, size_t n_chunks, const float *__restrict__ amax_dev,
+quantize_kernel(const uint4 *__restrict__ x, size_t n_chunks, const AmaxIn amax,
                 uint2 *__restrict__ q)
 {
     sste_pdl_trigger();
     sste_pdl_wait();
-    const float scale = sste_scale_from_amax(*amax_dev, E5M2 ? 57344.0f : 448.0f);
+    const float scale = sste_scale_from_amax(amax_take(amax, blockIdx.x == 0 && threadIdx.x == 0), E5M2 ? 57344.0f : 448.0f);
     const size_t stride = static_cast<size_t>(gridDim.x) * EW_THREADS;
     for (size_t c = static_cast<size_t>(blockIdx.x) * EW_THREADS + threadIdx.x; c < n_chunks; c += 4 * stride) {
         uint4 v[4];
@@ -1234,10 +1251,11 @@ extern "C" sste_status sste_srste_decay(sste_ctx *ctx, const void *W, const void
     return launch_result();
 }
 
-extern "C" sste_status sste_mvue_sparsify(sste_ctx *ctx, const void *dY, int T, int O, sste_dtype gdt, uint64_t seed,
-                                          uint32_t tensor_id, uint32_t step, uint64_t token_offset, int counter_cols,
-                                          const float *g_amax_dev, sste_dtype odt, void *gvals, void *gmeta,
-                                          void *dense_q_out, void *stream)
+namespace {
+
+sste_status mvue_launch(sste_ctx *ctx, const void *dY, int T, int O, sste_dtype gdt, uint64_t seed, uint32_t tensor_id,
+                        uint32_t step, uint64_t token_offset, int counter_cols, const float *g_amax_dev, void *scratch,
+                        sste_dtype odt, void *gvals, void *gmeta, void *dense_q_out, void *stream)
 {
     if (!ctx || !dY || !gvals || !gmeta) return SSTE_ERR_INVALID_ARG;
     if (gdt != SSTE_BF16 || (odt != SSTE_BF16 && odt != SSTE_E5M2)) return SSTE_ERR_DTYPE;
@@ -1258,13 +1276,33 @@ extern "C" sste_status sste_mvue_sparsify(sste_ctx *ctx, const void *dY, int T, 
     uint8_t *gm = static_cast<uint8_t *>(gmeta);
     const uint64_t tg0 = token_offset / 4;
     const bool f8 = (odt == SSTE_E5M2), any = (ccols % 4) != 0;
+    const AmaxIn g_amax{const_cast<float *>(g_amax_dev), static_cast<unsigned int *>(scratch)};
 #define SSTE_MVUE_LAUNCH(F8, ANY)                                                                                   \
     sste_launch(mvue_kernel<F8, ANY>, dim3(grid), dim3(EW_THREADS), 0, s, g, O, T, key0, key1, tensor_id, step, tg0, \
-                ccols, F8 ? g_amax_dev : nullptr, gvals, gm, F8 ? dense_q_out : nullptr, RaggedRows{}, nullptr)
+                ccols, F8 ? g_amax : AmaxIn{}, gvals, gm, F8 ? dense_q_out : nullptr, RaggedRows{}, nullptr)
     if (f8) { if (any) SSTE_MVUE_LAUNCH(true, true); else SSTE_MVUE_LAUNCH(true, false); }
     else { if (any) SSTE_MVUE_LAUNCH(false, true); else SSTE_MVUE_LAUNCH(false, false); }
 #undef SSTE_MVUE_LAUNCH
     return launch_result();
+}
+
+}  // namespace
+
+extern "C" sste_status sste_mvue_sparsify(sste_ctx *ctx, const void *dY, int T, int O, sste_dtype gdt, uint64_t seed,
+                                          uint32_t tensor_id, uint32_t step, uint64_t token_offset, int counter_cols,
+                                          const float *g_amax_dev, sste_dtype odt, void *gvals, void *gmeta,
+                                          void *dense_q_out, void *stream)
+{
+    return mvue_launch(ctx, dY, T, O, gdt, seed, tensor_id, step, token_offset, counter_cols, g_amax_dev, nullptr, odt, gvals,
+                       gmeta, dense_q_out, stream);
+}
+
+sste_status sste_mvue_scratch(sste_ctx *ctx, const void *dY, int T, int O, uint64_t seed, uint32_t tensor_id, uint32_t step,
+                              uint64_t token_offset, int counter_cols, float *g_amax_dev, void *scratch, void *gvals,
+                              void *gmeta, void *dense_q_out, void *stream)
+{
+    return mvue_launch(ctx, dY, T, O, SSTE_BF16, seed, tensor_id, step, token_offset, counter_cols, g_amax_dev, scratch, SSTE_E5M2,
+                       gvals, gmeta, dense_q_out, stream);
 }
 
 sste_status sste_mvue_padded(sste_ctx *ctx, const void *dY, int rows, int cols, void *dYp, int T, int O, uint64_t seed,
@@ -1283,7 +1321,7 @@ sste_status sste_mvue_padded(sste_ctx *ctx, const void *dY, int rows, int cols, 
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     auto kern = ccols % 4 ? mvue_kernel<false, true, true> : mvue_kernel<false, false, true>;
     sste_launch(kern, dim3(O / 64, T / 128), dim3(EW_THREADS), 0, s, nullptr, O, T, static_cast<uint32_t>(seed),
-                static_cast<uint32_t>(seed >> 32), tensor_id, step, token_offset / 4, ccols, nullptr, gvals,
+                static_cast<uint32_t>(seed >> 32), tensor_id, step, token_offset / 4, ccols, AmaxIn{}, gvals,
                 static_cast<uint8_t *>(gmeta), nullptr, rag, static_cast<uint4 *>(dYp));
     return launch_result();
 }
@@ -1301,7 +1339,7 @@ sste_status amax_launch(sste_ctx *ctx, const void *x, size_t n, float *amax_dev,
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (!scratch) SSTE_CUDA_TRY(cudaMemsetAsync(amax_dev, 0, sizeof(float), s));
     sste_launch(amax_kernel, dim3(grid_for(n_chunks, ctx->sm_count)), dim3(EW_THREADS), 0, s, static_cast<const uint4 *>(x),
-                n_chunks, amax_dev, static_cast<unsigned int *>(scratch));
+                n_chunks, static_cast<unsigned int *>(scratch ? scratch : amax_dev));
     return launch_result();
 }
 
@@ -1361,8 +1399,10 @@ extern "C" sste_status sste_fp8_scale(sste_ctx *ctx, const float *amax_dev, sste
     return launch_result();
 }
 
-extern "C" sste_status sste_quantize_fp8(sste_ctx *ctx, const void *x, size_t n, const float *amax_dev,
-                                         sste_dtype odt, void *q, void *stream)
+namespace {
+
+sste_status quantize_launch(sste_ctx *ctx, const void *x, size_t n, const float *amax_dev, void *scratch, sste_dtype odt, void *q,
+                            void *stream)
 {
     if (!ctx || !x || !amax_dev || !q) return SSTE_ERR_INVALID_ARG;
     if (odt != SSTE_E4M3 && odt != SSTE_E5M2) return SSTE_ERR_DTYPE;
@@ -1371,15 +1411,29 @@ extern "C" sste_status sste_quantize_fp8(sste_ctx *ctx, const void *x, size_t n,
     sste_device_guard guard(ctx->device);
     if (!guard.ok) return SSTE_ERR_CUDA;
     const size_t n_chunks = n / 8;
+    const AmaxIn amax{const_cast<float *>(amax_dev), static_cast<unsigned int *>(scratch)};
     const int grid = grid_for(n_chunks, ctx->sm_count);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (odt == SSTE_E5M2)
         sste_launch(quantize_kernel<true>, dim3(grid), dim3(EW_THREADS), 0, s, static_cast<const uint4 *>(x),
-                    n_chunks, amax_dev, static_cast<uint2 *>(q));
+                    n_chunks, amax, static_cast<uint2 *>(q));
     else
         sste_launch(quantize_kernel<false>, dim3(grid), dim3(EW_THREADS), 0, s, static_cast<const uint4 *>(x),
-                    n_chunks, amax_dev, static_cast<uint2 *>(q));
+                    n_chunks, amax, static_cast<uint2 *>(q));
     return launch_result();
+}
+
+}  // namespace
+
+extern "C" sste_status sste_quantize_fp8(sste_ctx *ctx, const void *x, size_t n, const float *amax_dev,
+                                         sste_dtype odt, void *q, void *stream)
+{
+    return quantize_launch(ctx, x, n, amax_dev, nullptr, odt, q, stream);
+}
+
+sste_status sste_quantize_scratch(sste_ctx *ctx, const void *x, size_t n, float *amax_dev, void *scratch, void *q, void *stream)
+{
+    return quantize_launch(ctx, x, n, amax_dev, scratch, SSTE_E4M3, q, stream);
 }
 
 extern "C" sste_status sste_meta_to_canonical(sste_ctx *ctx, const void *meta, int rows, int k, sste_dtype dt,

@@ -344,6 +344,7 @@ struct GemmParams {
     float *partials;        // split-K: fp32 partial tiles [split tile][cta][split][row quarter][BN / 4][32 lanes][4]
     unsigned int *tickets;  // split-K: claims (low half) and finished partials (high half) per [split tile][cta][epilogue
                             // warp][part]; zero between launches
+    unsigned int *zero_after; // nullable: a word to be zeroed once the kernels in front are done
 };
 
 
@@ -1026,6 +1027,7 @@ __device__ __forceinline__ Frame frame_begin(uint8_t *smem_raw, const GemmParams
     cluster_sync();          // the peer's barriers are initialised before anything signals them
     tc_fence_after();
     sste_pdl_wait();         // everything above overlapped the previous kernel; global memory from here on
+    if (blockIdx.x == 0 && threadIdx.x == 32 && p.zero_after) *p.zero_after = 0u;
     f.tmem_base = *reinterpret_cast<volatile uint32_t *>(f.ctrl + CTRL_TMEM);
     return f;
 }
@@ -1335,6 +1337,7 @@ void apply_plan(const sste_ctx *ctx, const LaunchPlan &plan, GemmParams &p)
     p.split_from = plan.split_from;
     p.partials = ctx->splitk_partials;
     p.tickets = ctx->splitk_tickets;
+    p.zero_after = ctx->zero_after;
 }
 
 template <int ELT, int BNW, int BNX>

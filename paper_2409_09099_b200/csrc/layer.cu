@@ -14,18 +14,25 @@ bool layer_ok(const sste_layer *l)
     return !fp8_of(l) || (l->amax && l->Xq && l->dYq && l->scratch);
 }
 
+// The status of the product that should have emptied the layer's scratch; if a call was refused, a memset does.
+sste_status emptied(const sste_layer *l, sste_status st, void *stream)
+{
+    if (st != SSTE_OK) cudaMemsetAsync(l->scratch, 0, 8, static_cast<cudaStream_t>(stream));
+    return st;
+}
+
 }  // namespace
 
 extern "C" sste_status sste_layer_prune(sste_ctx *ctx, const sste_layer *l, void *stream)
 {
     if (!ctx || !layer_ok(l)) return SSTE_ERR_INVALID_ARG;
-    float *w_amax = fp8_of(l) ? l->amax + 1 : nullptr;
-    if (fp8_of(l)) {
-        const sste_status st = sste_project_amax_scratch(ctx, l->W, l->O, l->I, l->beta, w_amax, l->scratch, stream);
-        if (st != SSTE_OK) return st;
-    }
-    return sste_project_compress(ctx, l->W, l->O, l->I, SSTE_BF16, l->beta, w_amax, static_cast<sste_dtype>(l->op_dtype),
-                                 l->vals, l->meta, l->w_dense, stream);
+    if (!fp8_of(l))
+        return sste_project_compress(ctx, l->W, l->O, l->I, SSTE_BF16, l->beta, nullptr, SSTE_BF16, l->vals, l->meta, l->w_dense,
+                                     stream);
+    sste_status st = sste_project_amax_scratch(ctx, l->W, l->O, l->I, l->beta, l->amax + 1, l->scratch, stream);
+    if (st != SSTE_OK) return st;
+    return sste_project_compress(ctx, l->W, l->O, l->I, SSTE_BF16, l->beta, l->amax + 1, SSTE_E4M3, l->vals, l->meta, l->w_dense,
+                                 stream);
 }
 
 extern "C" sste_status sste_layer_forward(sste_ctx *ctx, const sste_layer *l, const void *X, float *y_amax_out_dev, void *stream)
@@ -37,27 +44,41 @@ extern "C" sste_status sste_layer_forward(sste_ctx *ctx, const sste_layer *l, co
         w_amax = l->amax + 1;
         const size_t n = static_cast<size_t>(l->T) * l->I;
         sste_status st = sste_amax_scratch(ctx, X, n, x_amax, l->scratch, stream);
-        if (st == SSTE_OK) st = sste_quantize_fp8(ctx, X, n, x_amax, SSTE_E4M3, l->Xq, stream);
         if (st != SSTE_OK) return st;
-        X = l->Xq;
+        st = sste_quantize_scratch(ctx, X, n, x_amax, l->scratch, l->Xq, stream);
+        if (st == SSTE_OK) {
+            sste_ctx emptying = *ctx;
+            emptying.zero_after = static_cast<unsigned int *>(l->scratch);
+            st = sste_linear_fwd(&emptying, l->Xq, l->T, l->vals, l->meta, l->O, l->I, SSTE_E4M3, x_amax, w_amax, l->Y,
+                                 static_cast<sste_dtype>(l->out_dtype), y_amax_out_dev, stream);
+        }
+        return emptied(l, st, stream);
     }
-    return sste_linear_fwd(ctx, X, l->T, l->vals, l->meta, l->O, l->I, static_cast<sste_dtype>(l->op_dtype), x_amax, w_amax,
-                           l->Y, static_cast<sste_dtype>(l->out_dtype), y_amax_out_dev, stream);
+    return sste_linear_fwd(ctx, X, l->T, l->vals, l->meta, l->O, l->I, SSTE_BF16, nullptr, nullptr, l->Y,
+                           static_cast<sste_dtype>(l->out_dtype), y_amax_out_dev, stream);
 }
 
 extern "C" sste_status sste_layer_backward(sste_ctx *ctx, const sste_layer *l, const void *X, const void *dY, uint32_t step,
                                            uint64_t token_offset, void *stream)
 {
     if (!ctx || !layer_ok(l) || !dY) return SSTE_ERR_INVALID_ARG;
-    const bool fp8 = fp8_of(l);
-    const sste_dtype gdt = fp8 ? SSTE_E5M2 : SSTE_BF16;
-    float *g_amax = fp8 ? l->amax + 2 : nullptr;
-    if (fp8) {
-        const sste_status st = sste_amax_scratch(ctx, dY, static_cast<size_t>(l->T) * l->O, g_amax, l->scratch, stream);
+    sste_status st;
+    if (fp8_of(l)) {
+        float *g_amax = l->amax + 2;
+        st = sste_amax_scratch(ctx, dY, static_cast<size_t>(l->T) * l->O, g_amax, l->scratch, stream);
         if (st != SSTE_OK) return st;
+        st = sste_mvue_scratch(ctx, dY, l->T, l->O, l->seed, l->tensor_id, step, token_offset, l->counter_cols, g_amax,
+                               l->scratch, l->gvals, l->gmeta, l->dYq, stream);
+        if (st == SSTE_OK) {
+            sste_ctx emptying = *ctx;
+            emptying.zero_after = static_cast<unsigned int *>(l->scratch);
+            st = sste_layer_grads(&emptying, l, X, dY, stream);
+        }
+        return emptied(l, st, stream);
+    } else {
+        st = sste_mvue_sparsify(ctx, dY, l->T, l->O, SSTE_BF16, l->seed, l->tensor_id, step, token_offset, l->counter_cols, nullptr,
+                                SSTE_BF16, l->gvals, l->gmeta, nullptr, stream);
     }
-    const sste_status st = sste_mvue_sparsify(ctx, dY, l->T, l->O, SSTE_BF16, l->seed, l->tensor_id, step, token_offset,
-                                        l->counter_cols, g_amax, gdt, l->gvals, l->gmeta, fp8 ? l->dYq : nullptr, stream);
     if (st != SSTE_OK) return st;
     return sste_layer_grads(ctx, l, X, dY, stream);
 }
