@@ -1328,6 +1328,15 @@ sste_status sste_mvue_padded(sste_ctx *ctx, const void *dY, int rows, int cols, 
 
 namespace {
 
+// Blocks of an amax pass: as few as four loads per thread allow, because each ends with atomics at one address (the E4M3
+// prune of 1.6 M weights: 8.9 us with 800 blocks, 7.2 with 200), and eight per SM where the tensor is large (with four, 12 MB
+// take 1 us longer).
+int amax_grid(size_t n_chunks, int sm_count)
+{
+    const size_t blocks = (n_chunks + 4 * EW_THREADS - 1) / (4 * EW_THREADS), cap = static_cast<size_t>(sm_count) * 8;
+    return static_cast<int>(blocks < cap ? blocks : cap);
+}
+
 sste_status amax_launch(sste_ctx *ctx, const void *x, size_t n, float *amax_dev, void *scratch, void *stream)
 {
     if (!ctx || !x || !amax_dev) return SSTE_ERR_INVALID_ARG;
@@ -1338,7 +1347,7 @@ sste_status amax_launch(sste_ctx *ctx, const void *x, size_t n, float *amax_dev,
     const size_t n_chunks = n / 8;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (!scratch) SSTE_CUDA_TRY(cudaMemsetAsync(amax_dev, 0, sizeof(float), s));
-    sste_launch(amax_kernel, dim3(grid_for(n_chunks, ctx->sm_count)), dim3(EW_THREADS), 0, s, static_cast<const uint4 *>(x),
+    sste_launch(amax_kernel, dim3(amax_grid(n_chunks, ctx->sm_count)), dim3(EW_THREADS), 0, s, static_cast<const uint4 *>(x),
                 n_chunks, static_cast<unsigned int *>(scratch ? scratch : amax_dev));
     return launch_result();
 }
@@ -1354,7 +1363,7 @@ sste_status project_amax_launch(sste_ctx *ctx, const void *W, int O, int I, cons
     const size_t n_chunks = static_cast<size_t>(O) * I / 8;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (!scratch) SSTE_CUDA_TRY(cudaMemsetAsync(amax_dev, 0, sizeof(float), s));
-    sste_launch(project_amax_kernel, dim3(grid_for(n_chunks, ctx->sm_count)), dim3(EW_THREADS), 0, s,
+    sste_launch(project_amax_kernel, dim3(amax_grid(n_chunks, ctx->sm_count)), dim3(EW_THREADS), 0, s,
                 static_cast<const uint4 *>(W), n_chunks, beta_dev, amax_dev, static_cast<unsigned int *>(scratch));
     return launch_result();
 }
