@@ -412,8 +412,8 @@ sste_status sste_debug_plan(int product, sste_dtype opdt, int O, int I, int T, i
 /* The plan of a one-launch grad_W + grad_X (sste_layer_grads), host only; out: grad_W's tile width, split factor, first
  * split tile, band height; grad_X's tile width, band height; CTA pairs; how many of them have a grad_W unit more than the
  * others; the rounds of grad_X tiles that the others take among themselves first; whether they also come first in the
- * rounds after. */
-sste_status sste_debug_joint_plan(sste_dtype opdt, int O, int I, int T, int sm_count, size_t workspace_bytes, int out[10]);
+ * rounds after; grad_X's split factor (all tiles, summed afterwards); whether grad_W's partials are summed afterwards. */
+sste_status sste_debug_joint_plan(sste_dtype opdt, int O, int I, int T, int sm_count, size_t workspace_bytes, int out[12]);
 sste_status sste_debug_tile_coords(int tile, int m_tiles, int n_tiles, int group_m, int *mt, int *nt);
 
 /* Host-only self-check of the once-per-device bookkeeping behind per-device kernel attributes (a context may live on

@@ -141,10 +141,10 @@ def plan(product: int, opdt: int, O: int, I: int, T: int, sm_count: int = 148, w
 
 
 def joint_plan(opdt: int, O: int, I: int, T: int, sm_count: int = 148, workspace_bytes: int | None = None):
-    """sste_debug_joint_plan: the ten numbers of a one-launch grad_W + grad_X, in the order of the header; host only."""
+    """sste_debug_joint_plan: the twelve numbers of a one-launch grad_W + grad_X, in the order of the header; host only."""
     lib = load()
     ws = lib.sste_workspace_bytes_recommended() if workspace_bytes is None else workspace_bytes
-    out = (ctypes.c_int * 10)()
+    out = (ctypes.c_int * 12)()
     st = lib.sste_debug_joint_plan(opdt, O, I, T, sm_count, ctypes.c_size_t(ws), out)
     if st != OK:
         raise SsteError(st, lib.sste_status_string(st).decode())

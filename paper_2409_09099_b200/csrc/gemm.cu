@@ -19,6 +19,7 @@
 // Every wait is bounded: on expiry the CTA records SSTE_ERR_TIMEOUT and leaves.
 #include <cuda.h>
 
+#include <array>
 #include <type_traits>
 
 #include "common.cuh"
@@ -30,7 +31,7 @@ constexpr int TMEM_COLS = 512;
 // Shared memory starts with a control block: barriers of the kernel's first product at 0 and of its second at 512, the
 // expander's selector table at 256, the tensor-memory address at 1008 and the abort flag at 1016.
 constexpr int CTRL_BYTES = 1024, CTRL_SECOND = 512, CTRL_LUT = 256, CTRL_TMEM = 1008, CTRL_ABORT = 1016;
-constexpr int MAX_SPLITS = 16;     // split-K factor limit
+constexpr int MAX_SPLITS = 16;     // split-K factor limit where the units exchange their partials
 constexpr int MAX_PARTS = 2;       // parts that a warp's share of a split tile is exchanged in
 constexpr int PANEL_BYTES = 2048;  // epilogue panel: 32 rows x 32 columns of bf16
 constexpr unsigned long long WAIT_LIMIT_NS = 2000000000ull;   // two seconds of wall time (%globaltimer)
@@ -342,7 +343,7 @@ struct GemmParams {
     int splits;             // split-K factor of the tiles from `split_from` on (1 = none)
     int split_from;         // first split tile: tiles below it are computed whole
     float *partials;        // split-K: fp32 partial tiles [split tile][cta][split][row quarter][BN / 4][32 lanes][4]
-    unsigned int *tickets;  // split-K: claims (low half) and finished partials (high half) per [split tile][cta][epilogue
+    unsigned int *tickets;  // split-K, null where splitk_sum_kernel follows: claims (low half) and finished partials (high half) per [split tile][cta][epilogue
                             // warp][part]; zero between launches
     unsigned int *zero_after; // nullable: a word to be zeroed once the kernels in front are done
 };
@@ -711,6 +712,23 @@ product(const CUtensorMap &map_a, const CUtensorMap &map_b, const CUtensorMap &m
                 const int parts = min(n_box, MAX_PARTS);
                 constexpr int AHEAD = 2;               // (three spill registers of the ordinary epilogue)
                 bool ok = true;
+                if (!p.tickets) {
+                    // summed by splitk_sum_kernel: lane = row, whatever the output's orientation
+                    float4 *mine = part0 + static_cast<size_t>(u.split) * 4 * PART;
+#pragma unroll 1
+                    for (int pnl = pnl0; pnl < pnl0 + n_pnl; ++pnl) {
+                        uint32_t r[32];
+                        tmem_ld_32x32(acc_base + 32 * pnl, r);
+                        tmem_ld_wait();
+#pragma unroll
+                        for (int i = 0; i < 8; ++i)
+                            __stcg(mine + (8 * pnl + i) * 32,
+                                   make_float4(__uint_as_float(r[4 * i]), __uint_as_float(r[4 * i + 1]),
+                                               __uint_as_float(r[4 * i + 2]), __uint_as_float(r[4 * i + 3])));
+                    }
+                    release_acc();
+                    continue;
+                }
                 uint32_t drawn = 0;
                 if (elect) drawn = atomicAdd(tickets + u.split % parts, 1u);
 #pragma unroll 1
@@ -1063,6 +1081,74 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     if ((threadIdx.x >> 5) == 1) tmem_dealloc(f.tmem_base, TMEM_COLS);
 }
 
+// Sum of the partial tiles of a product whose few tiles were cut into many K ranges (p.tickets null).  In the product itself
+// one warp would read the partials of all other units, a few at a time: at 16 ranges that chain of L2 round trips took 10 us
+// and more.  Here every thread of a small grid adds up one float4 of the ranges, eight loads in flight, in split order.
+// (Blocks from `blocks` on do the same for a second product.)
+template <bool OUT_T>
+__global__ void __launch_bounds__(128) splitk_sum_kernel(const __grid_constant__ GemmParams p1, int bn1, int blocks,
+                                                         const __grid_constant__ GemmParams p2, int bn2)
+{
+    sste_pdl_trigger();
+    const bool second = static_cast<int>(blockIdx.x) >= blocks;
+    const GemmParams &p = second ? p2 : p1;
+    const int bn = second ? bn2 : bn1;
+    const int lane = threadIdx.x & 31, warp = (blockIdx.x - (second ? blocks : 0)) * 4 + (threadIdx.x >> 5);
+    const int groups = bn / 4;                               // warps per 32 rows of a tile
+    const int q = warp / groups, g = warp - q * groups;
+    const int slot = q >> 2, quarter = q & 3;                // slot: [split tile][cta]
+    // row-major output: eight rows x 16 columns per warp (whole sectors); transposed: 32 rows x 4 columns
+    const int c4 = OUT_T ? g : (g >> 2) * 4 + (lane & 3), row = OUT_T ? lane : (g & 3) * 8 + (lane >> 2);
+    int mt, nt;
+    tile_coords(p.split_from + (slot >> 1), (p.M + 2 * BM - 1) / (2 * BM), (p.N + bn - 1) / bn, p.group_m, mt, nt);
+    const int m = mt * 2 * BM + (slot & 1) * BM + quarter * 32 + row, n = nt * bn + 4 * c4;
+    const bool inside = m < p.M && n < p.N;
+    sste_pdl_wait();
+    const float scale = sste_out_scale(p.a_amax, p.a_fp8_max, p.b_amax, p.b_fp8_max);
+    uint32_t best = 0;
+    if (inside) {
+        const size_t step = static_cast<size_t>(4) * groups * 32;       // float4 between two splits
+        const float4 *src = reinterpret_cast<const float4 *>(p.partials) +
+                            (static_cast<size_t>(slot) * p.splits * 4 + quarter) * (groups * 32) + c4 * 32 + row;
+        float4 v = __ldcg(src);
+        auto add = [&](const float4 &x) {
+            v.x = __fadd_rn(v.x, x.x); v.y = __fadd_rn(v.y, x.y); v.z = __fadd_rn(v.z, x.z); v.w = __fadd_rn(v.w, x.w);
+        };
+        int sp = 1;
+        for (; sp + 8 <= p.splits; sp += 8) {
+            float4 x[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) x[i] = __ldcg(src + (sp + i) * step);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) add(x[i]);
+        }
+        float4 x[7];
+#pragma unroll
+        for (int i = 0; i < 7; ++i) if (sp + i < p.splits) x[i] = __ldcg(src + (sp + i) * step);
+#pragma unroll
+        for (int i = 0; i < 7; ++i) if (sp + i < p.splits) add(x[i]);
+        const __nv_bfloat162 lo = __floats2bfloat162_rn(__fmul_rn(v.x, scale), __fmul_rn(v.y, scale));
+        const __nv_bfloat162 hi = __floats2bfloat162_rn(__fmul_rn(v.z, scale), __fmul_rn(v.w, scale));
+        const uint32_t w0 = *reinterpret_cast<const uint32_t *>(&lo), w1 = *reinterpret_cast<const uint32_t *>(&hi);
+        __nv_bfloat16 *out = static_cast<__nv_bfloat16 *>(p.D);
+        if (OUT_T) {
+            out[static_cast<size_t>(n) * p.M + m] = lo.x;
+            out[static_cast<size_t>(n + 1) * p.M + m] = lo.y;
+            out[static_cast<size_t>(n + 2) * p.M + m] = hi.x;
+            out[static_cast<size_t>(n + 3) * p.M + m] = hi.y;
+        } else {
+            *reinterpret_cast<uint2 *>(out + static_cast<size_t>(m) * p.N + n) = make_uint2(w0, w1);
+        }
+        const uint32_t a = __vmaxu2(w0 & 0x7fff7fffu, w1 & 0x7fff7fffu);
+        best = max(a & 0xffffu, a >> 16) << 16;
+    }
+    if (p.out_amax) {
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) best = max(best, __shfl_xor_sync(0xffffffffu, best, off));
+        if (lane == 0 && best != 0) atomicMax(p.out_amax, best);
+    }
+}
+
 // grad_W and grad_X of a layer in one launch.  They are independent, and each alone quantises badly into waves of CTA pairs
 // (3072 x 768, 8192 tokens: 36 and 96 tiles on 74 pairs).  Every pair computes its share of grad_W, then of grad_X: the
 // pairs that come out of grad_W a round earlier (`late_pairs` is the number of the others, the first ones) take `early`
@@ -1168,13 +1254,19 @@ constexpr TileCost tile_cost(Product pr, int elt, int bn)
 }
 
 // Everything the host decides about one product launch.
-struct LaunchPlan { int bn, splits, split_from, group_m; double us; };
+struct LaunchPlan { int bn, splits, split_from, group_m; double us; bool sum_after; };
 
 // Microseconds that a split costs on top of its units' main loops: the exchange between `s` units, `bytes` of partials.
 double exchange_us(int s, int bn, double bytes)
 {
     return (s == 2 ? 2.4 + 2.6 * bn / 256.0 : 2.5 + 0.65 * s + (2.6 + 0.4 * s) * bn / 256.0) + bytes / 15e6;
 }
+
+// The same where splitk_sum_kernel follows the product: its launch, the fp32 stores that the units end with, their bytes.
+// (Measured against whole tiles and exchanges at 1 ... 32 tiles, 2 ... 44 ranges.)
+double sum_us(int s, int bn, double bytes) { return 0.4 + 2.4 * bn / 256.0 + 0.04 * s + bytes / 2.9e6; }
+// split factors tried there (0: none)
+constexpr int SUM_SPLITS[] = {2, 3, 4, 6, 8, 11, 16, 22, 32, 44, 64};
 
 // L2-aware band height of a product with tiles `bn` wide.
 int plan_group_m(Product pr, int elt, bool bcomp, int bn, int pairs, int M, int N, int K)
@@ -1185,13 +1277,30 @@ int plan_group_m(Product pr, int elt, bool bcomp, int bn, int pairs, int M, int 
                         static_cast<double>(K) * ((bcomp ? 0.5 : 1.0) * elt) * bn);
 }
 
+// The plans of the last shapes of a thread: trying every width and split takes up to some 20 us of host time.
+template <typename Plan>
+struct PlanMemo {
+    typedef std::array<long long, 6> Key;
+    static constexpr int ENTRIES = 64;
+    struct Entry { Key key{}; Plan plan{}; bool set = false; } entry[ENTRIES];
+    template <typename F>
+    const Plan &get(const Key &key, F make)
+    {
+        unsigned long long h = 0;
+        for (long long k : key) h = (h ^ static_cast<unsigned long long>(k)) * 0x9e3779b97f4a7c15ull;
+        Entry &e = entry[h >> 58];
+        if (!e.set || e.key != key) e = Entry{key, make(), true};
+        return e.plan;
+    }
+};
+
 // Tile width and split-K factor by the model's time.  Tiles that fill complete waves of CTA pairs are computed whole; the
 // tiles of the last, partial wave (all of them when there are fewer tiles than pairs, as for the weight gradient of a
 // GPT-2-sized layer: 36 tiles, 74 pairs) may be cut into `splits` K ranges of at least eight stages, so that the wave
 // takes 1/splits of a tile time and the exchange of the partials on top: 2.4 + 2.6 bn/256 us between two units,
-// 4.4 + 3.8 bn/256 between three and so on (measured at 9 ... 36 tiles), and their bytes.  Among widths within 3 % the
-// first wins.
-LaunchPlan make_plan(Product pr, int elt, int only_bn, bool out_f32, bool bcomp, int sm_count, size_t partial_bytes, int M,
+// 4.4 + 3.8 bn/256 between three and so on (measured at 9 ... 36 tiles), and their bytes.  Few tiles (all ranges run at once)
+// of a long reduction take many short ranges and a sum afterwards instead.  Among widths within 3 % the first wins.
+LaunchPlan find_plan(Product pr, int elt, int only_bn, bool out_f32, bool bcomp, int sm_count, size_t partial_bytes, int M,
                      int N, int K)
 {
     const bool sparse = (pr != GRAD_INPUT);
@@ -1201,7 +1310,7 @@ LaunchPlan make_plan(Product pr, int elt, int only_bn, bool out_f32, bool bcomp,
     int forced = only_bn;
     for (int bn : widths.bn)
         if (!forced && bn && bn == g_force_bn) forced = bn;
-    LaunchPlan best{0, 1, 0, m_tiles, 0.0};
+    LaunchPlan best{0, 1, 0, m_tiles, 0.0, false};
     for (int bn : widths.bn) {
         if (!bn || (forced && bn != forced)) continue;
         const int tiles = m_tiles * ((N + bn - 1) / bn);
@@ -1223,13 +1332,30 @@ LaunchPlan make_plan(Product pr, int elt, int only_bn, bool out_f32, bool bcomp,
             const bool wanted = (g_force_splits == s && best.bn == bn);      // the hook applies where the shape allows it
             if (!best.bn || us < best.us * (best.bn == bn ? 1.0 : 0.97) || wanted) {
                 if (g_force_splits && best.bn == bn && best.splits == g_force_splits) continue;
-                best = LaunchPlan{bn, s, s > 1 ? whole : tiles, m_tiles, us};
+                best = LaunchPlan{bn, s, s > 1 ? whole : tiles, m_tiles, us, false};
             }
             if (g_force_splits == 1) break;
+        }
+        for (int s : SUM_SPLITS) {
+            const size_t bytes = static_cast<size_t>(tail) * s * 2 * BM * bn * sizeof(float);
+            if (g_force_splits || g_inject_stall || out_f32 || whole > 0 || tail * s > pairs || k_blocks / s < 2 || bytes > partial_bytes) break;
+            const double us = (k_blocks + s - 1) / s * c.stage_us + c.tile_us + sum_us(s, bn, static_cast<double>(bytes));
+            if (us < best.us * (best.bn == bn ? 1.0 : 0.97)) best = LaunchPlan{bn, s, 0, m_tiles, us, true};
         }
     }
     best.group_m = plan_group_m(pr, elt, bcomp, best.bn, pairs, M, N, K);
     return best;
+}
+
+LaunchPlan make_plan(Product pr, int elt, int only_bn, bool out_f32, bool bcomp, int sm_count, size_t partial_bytes, int M,
+                     int N, int K)
+{
+    if (g_force_splits || g_force_bn || g_force_group_m || g_inject_stall)
+        return find_plan(pr, elt, only_bn, out_f32, bcomp, sm_count, partial_bytes, M, N, K);
+    static thread_local PlanMemo<LaunchPlan> memo;
+    const long long kind = (((pr * 4 + elt) * 2 + out_f32) * 2 + bcomp) * 1024 + only_bn;
+    return memo.get({kind, sm_count, static_cast<long long>(partial_bytes), M, N, K},
+                    [&] { return find_plan(pr, elt, only_bn, out_f32, bcomp, sm_count, partial_bytes, M, N, K); });
 }
 
 // One launch for both gradient products (grads_kernel): the plans of the two and how the pairs share grad_X.
@@ -1238,8 +1364,8 @@ struct JointPlan { LaunchPlan w, x; int pairs; GradsPlan g; double us; };
 // grad_W units go round the pairs; the last, partial round leaves `late` pairs busy for one unit more.  For every width,
 // split and number of early rounds the model gives the time at which the last pair ends; a pair that changes over from one
 // product to the other drains and refills its pipeline (SWITCH_US, about what a kernel boundary costs).
-constexpr double SWITCH_US = 2.5;
-JointPlan make_joint_plan(int elt, int sm_count, size_t partial_bytes, int O, int I, int T)
+constexpr double SWITCH_US = 2.5, LAUNCH_US = 3.0;      // (a second launch: what a product of one stage takes besides it)
+JointPlan find_joint_plan(int elt, int sm_count, size_t partial_bytes, int O, int I, int T)
 {
     const int max_pairs = sm_count / 2;
     const int wk = (T + 256 / elt - 1) / (256 / elt), xk = (O + 128 / elt - 1) / (128 / elt);      // stages
@@ -1253,25 +1379,39 @@ JointPlan make_joint_plan(int elt, int sm_count, size_t partial_bytes, int O, in
             if (!bnx || (bnw == 256 && elt == 2 && bnx == 128)) continue;  // (no kernel for it)
             const TileCost cx = tile_cost(GRAD_INPUT, elt, bnx);
             const int x_tiles = ((T + 2 * BM - 1) / (2 * BM)) * ((I + bnx - 1) / bnx);
-            const double x_us = xk * cx.stage_us + cx.tile_us;
-            for (int s = 1; s <= MAX_SPLITS; ++s) {
-                const int all = w_tiles * s + x_tiles, P = all < max_pairs ? all : max_pairs;
+            // grad_W whole, split with an exchange (s = 2 .. MAX_SPLITS) or with a sum afterwards (the rest); grad_X whole or with
+            // a sum.  Sums are for few tiles: everything has to fit into one round of the pairs.
+            constexpr int SUMS = sizeof(SUM_SPLITS) / sizeof(SUM_SPLITS[0]);
+            for (int o = 1; o <= MAX_SPLITS + SUMS; ++o)
+            for (int ox = -1; ox < SUMS; ++ox) {
+                const bool w_sum = o > MAX_SPLITS;
+                const int s = w_sum ? SUM_SPLITS[o - MAX_SPLITS - 1] : o, sx = ox < 0 ? 1 : SUM_SPLITS[ox];
+                if (ox >= 0 && (w_tiles * s + x_tiles * sx > max_pairs || xk / sx < 2)) break;
+                const double x_us = (xk + sx - 1) / sx * cx.stage_us + cx.tile_us;
+                const int x_units = x_tiles * sx;
+                const int all = w_tiles * s + x_units, P = all < max_pairs ? all : max_pairs;
                 const int whole = w_tiles / P * P, tail = w_tiles - whole;
-                double extra = 0.0;
-                if (s > 1) {
+                const size_t w_bytes = s > 1 ? static_cast<size_t>(tail) * s * 2 * BM * bnw * sizeof(float) : 0;
+                const size_t x_bytes = sx > 1 ? static_cast<size_t>(x_tiles) * sx * 2 * BM * bnx * sizeof(float) : 0;
+                if (w_bytes + x_bytes > partial_bytes) continue;
+                double extra = 0.0, after = 0.0;
+                if (w_sum) {
+                    if (whole > 0 || w_tiles * s > max_pairs || wk / s < 2) continue;
+                } else if (s > 1) {
                     if (tail == 0 || wk / s < 8 || (whole > 0 && wk % s != 0) || tail * s > P) continue;
                     if (tail * 2 * 8 * MAX_PARTS > SSTE_SPLITK_TICKETS) continue;
-                    const size_t bytes = static_cast<size_t>(tail) * s * 2 * BM * bnw * sizeof(float);
-                    if (bytes > partial_bytes) continue;
-                    extra = exchange_us(s, bnw, static_cast<double>(bytes));
+                    extra = exchange_us(s, bnw, static_cast<double>(w_bytes));
                 }
+                if (w_sum || sx > 1)
+                    after = sum_us(w_sum && s > sx ? s : sx, sx > 1 && (!w_sum || bnx > bnw) ? bnx : bnw,
+                                   static_cast<double>((w_sum ? w_bytes : 0) + x_bytes));
                 const int late = tail * s;                                  // pairs with one unit more
                 const double w_us = wk * cw.stage_us + cw.tile_us;
                 const double t_early = (whole / P) * w_us + (whole ? SWITCH_US : 0.0);
                 const double t_late = late ? (whole / P) * w_us + (wk + s - 1) / s * cw.stage_us + cw.tile_us + extra + SWITCH_US : 0.0;
                 const int n_early = P - late;
                 for (int early = 0; early == 0 || (late && n_early && t_early + (early - 1) * x_us < t_late); ++early) {
-                    const int rest = x_tiles - early * n_early;
+                    const int rest = x_units - early * n_early;
                     const int rounds = rest > 0 ? (rest + P - 1) / P : 0, last = rest > 0 ? rest - (rounds - 1) * P : 0;
                     for (int ef = 0; ef < 2; ++ef) {
                         // rounds of the early / late pairs: the group that comes second lacks the last one if `last` is short
@@ -1279,10 +1419,10 @@ JointPlan make_joint_plan(int elt, int sm_count, size_t partial_bytes, int O, in
                         const int r_late = rounds - ((rounds && ef && last <= n_early) ? 1 : 0);
                         double us = n_early ? t_early + (early + r_early) * x_us : 0.0;
                         if (late && t_late + r_late * x_us > us) us = t_late + r_late * x_us;
-                        us += 0.05 * x_us;                                  // among equals the shorter tile
+                        us += 0.05 * x_us + after;                          // among equals the shorter tile
                         if (best.pairs && us >= best.us - 1e-9) continue;
-                        best.w = LaunchPlan{bnw, s, s > 1 ? whole : w_tiles, 0, 0.0};
-                        best.x = LaunchPlan{bnx, 1, x_tiles, 0, 0.0};
+                        best.w = LaunchPlan{bnw, s, s > 1 ? whole : w_tiles, 0, 0.0, w_sum};
+                        best.x = LaunchPlan{bnx, sx, sx > 1 ? 0 : x_tiles, 0, 0.0, sx > 1};
                         best.pairs = P;
                         best.g = GradsPlan{late, early, ef};
                         best.us = us;
@@ -1295,6 +1435,14 @@ JointPlan make_joint_plan(int elt, int sm_count, size_t partial_bytes, int O, in
     best.w.group_m = plan_group_m(GRAD_WEIGHT, elt, false, best.w.bn, best.pairs, O, I, T);
     best.x.group_m = plan_group_m(GRAD_INPUT, elt, false, best.x.bn, best.pairs, T, I, O);
     return best;
+}
+
+JointPlan make_joint_plan(int elt, int sm_count, size_t partial_bytes, int O, int I, int T)
+{
+    if (g_force_splits || g_force_bn || g_force_group_m) return find_joint_plan(elt, sm_count, partial_bytes, O, I, T);
+    static thread_local PlanMemo<JointPlan> memo;
+    return memo.get({elt, sm_count, static_cast<long long>(partial_bytes), O, I, T},
+                    [&] { return find_joint_plan(elt, sm_count, partial_bytes, O, I, T); });
 }
 
 // Tensor maps of a launch: A, B, output, metadata (those that it does not use repeat A's).
@@ -1336,8 +1484,26 @@ void apply_plan(const sste_ctx *ctx, const LaunchPlan &plan, GemmParams &p)
     p.splits = plan.splits;
     p.split_from = plan.split_from;
     p.partials = ctx->splitk_partials;
-    p.tickets = ctx->splitk_tickets;
+    p.tickets = plan.sum_after ? nullptr : ctx->splitk_tickets;
     p.zero_after = ctx->zero_after;
+}
+
+template <int BN>
+int split_tiles(const GemmParams &p)
+{
+    return (p.M + 2 * BM - 1) / (2 * BM) * ((p.N + BN - 1) / BN) - p.split_from;
+}
+
+// The sum of a product's partials (the first `tiles` split tiles) and of a second one's.
+template <bool OUT_T>
+sste_status launch_sum(const GemmParams &p, int bn, int tiles, const GemmParams &p2, int bn2, int tiles2, cudaStream_t stream)
+{
+    // a thread per four elements: 2 CTAs x 4 row quarters x bn / 4 warps per tile, four warps a block
+    const int blocks = tiles * bn / 2, blocks2 = tiles2 * bn2 / 2;
+    if (sste_launch(splitk_sum_kernel<OUT_T>, dim3(blocks + blocks2), dim3(128), 0, stream, p, bn, blocks, p2, bn2) != cudaSuccess)
+        return SSTE_ERR_CUDA;
+    sste_count_launches(1);
+    return SSTE_OK;
 }
 
 template <int ELT, int BNW, int BNX>
@@ -1358,10 +1524,14 @@ sste_status launch_grads(const sste_ctx *ctx, const void *gvals, const void *gme
         return SSTE_ERR_CUDA;
     apply_plan(ctx, plan.w, pw);
     apply_plan(ctx, plan.x, px);
+    if (plan.x.sum_after && plan.w.splits > 1)      // behind grad_W's partials
+        px.partials += split_tiles<BNW>(pw) * static_cast<size_t>(plan.w.splits) * 2 * BM * BNW;
     if (sste_launch(kern, dim3(2 * plan.pairs), dim3(320), SMEM, stream, mw.a, mw.b, mw.d, mw.m, mx.a, mx.b, mx.d, pw, px,
                     plan.g) != cudaSuccess)
         return SSTE_ERR_CUDA;
     sste_count_launches(1);
+    if (plan.w.sum_after) return launch_sum<false>(pw, BNW, split_tiles<BNW>(pw), px, BNX, plan.x.sum_after ? split_tiles<BNX>(px) : 0, stream);
+    if (plan.x.sum_after) return launch_sum<false>(px, BNX, split_tiles<BNX>(px), px, BNX, 0, stream);
     return SSTE_OK;
 }
 
@@ -1401,6 +1571,7 @@ sste_status launch(const sste_ctx *ctx, const void *A, const void *B, const void
         return SSTE_ERR_CUDA;
     if (cudaGetLastError() != cudaSuccess) return SSTE_ERR_CUDA;
     sste_count_launches(1);
+    if (plan.sum_after) return launch_sum<OUT_T>(pp, BN, n_split_tiles, pp, BN, 0, stream);
     return SSTE_OK;
 }
 
@@ -1488,9 +1659,10 @@ extern "C" sste_status sste_debug_joint_plan(sste_dtype opdt, int O, int I, int 
     const size_t partial_bytes =
         workspace_bytes > SSTE_WS_SPLITK_PARTIALS_OFF + (size_t(1) << 20) ? workspace_bytes - SSTE_WS_SPLITK_PARTIALS_OFF : 0;
     const JointPlan plan = make_joint_plan(elt, sm_count, partial_bytes, O, I, T);
-    const int v[10] = {plan.w.bn, plan.w.splits, plan.w.split_from, plan.w.group_m, plan.x.bn,
-                       plan.x.group_m, plan.pairs, plan.g.late_pairs, plan.g.early, plan.g.early_first};
-    for (int i = 0; i < 10; ++i) out[i] = v[i];
+    const int v[12] = {plan.w.bn, plan.w.splits, plan.w.split_from, plan.w.group_m, plan.x.bn,
+                       plan.x.group_m, plan.pairs, plan.g.late_pairs, plan.g.early, plan.g.early_first,
+                       plan.x.splits, plan.w.sum_after};
+    for (int i = 0; i < 12; ++i) out[i] = v[i];
     return SSTE_OK;
 }
 // Host-only self-check of the once-per-device guard the launches use for per-device kernel attributes: `fn` must
@@ -1667,7 +1839,7 @@ sste_status sste_bwd_products(sste_ctx *ctx, const void *gvals, const void *gmet
             // whose last wave costs little and whose tiles run 10 % slower beside the other product's (1280 x 5120, 16384
             // tokens, bf16: 248 us apart, 260 us together; 3840 x 1280: 194 and 180).
             const double apart = make_plan(GRAD_WEIGHT, elt, 0, false, false, ctx->sm_count, partial_bytes, O, I, T).us +
-                                 make_plan(GRAD_INPUT, elt, 0, false, false, ctx->sm_count, partial_bytes, T, I, O).us + SWITCH_US;
+                                 make_plan(GRAD_INPUT, elt, 0, false, false, ctx->sm_count, partial_bytes, T, I, O).us + LAUNCH_US;
             uint32_t cg, cw;
             int unused;
             fmt_code(gdt, &unused, &cg);

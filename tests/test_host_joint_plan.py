@@ -37,16 +37,20 @@ def _units_of(pair, pairs, late, early, early_first, n):
 def test_every_unit_once(dt, sms):
     for O, I, T in _shapes():
         for ws in (None, B.load().sste_workspace_bytes()):
-            bw, splits, split_from, gw, bx, gx, pairs, late, early, ef = B.joint_plan(dt, O, I, T, sms, ws)
+            bw, splits, split_from, gw, bx, gx, pairs, late, early, ef, sx, w_sum = B.joint_plan(dt, O, I, T, sms, ws)
             elt = 2 if dt == B.BF16 else 1
             wt, xt = -(-O // 256) * -(-I // bw), -(-T // 256) * -(-I // bx)
             assert bw in (128, 256) and bx in (128, 256) and 1 <= pairs <= sms // 2 and 0 <= late <= pairs
             assert 1 <= gw <= -(-O // 256) and 1 <= gx <= -(-T // 256)
             w_units = split_from + (wt - split_from) * splits
             if splits > 1:
-                assert ws is None and -(-T // (256 // elt)) // splits >= 8 and split_from % pairs == 0
+                assert ws is None and -(-T // (256 // elt)) // splits >= (2 if w_sum else 8) and split_from % pairs == 0
             else:
                 assert split_from == wt
             assert late == w_units % pairs or (late == pairs and w_units % pairs == 0)   # pairs with a unit more come first
-            seen = sorted(u for p in range(pairs) for u in _units_of(p, pairs, late, early, ef, xt))
-            assert seen == list(range(xt)), (O, I, T)
+            if w_sum:                                # sums only where all ranges run at once
+                assert ws is None and split_from == 0 and splits > 1 and wt * splits <= sms // 2
+            if sx > 1:
+                assert ws is None and wt * splits + xt * sx <= sms // 2 and -(-O // (128 // elt)) // sx >= 2
+            seen = sorted(u for p in range(pairs) for u in _units_of(p, pairs, late, early, ef, xt * sx))
+            assert seen == list(range(xt * sx)), (O, I, T)
