@@ -1084,6 +1084,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
 // Sum of the partial tiles of a product whose few tiles were cut into many K ranges (p.tickets null).  In the product itself
 // one warp would read the partials of all other units, a few at a time: at 16 ranges that chain of L2 round trips took 10 us
 // and more.  Here every thread of a small grid adds up one float4 of the ranges, eight loads in flight, in split order.
+// 128 x 8192, 128 tokens, bf16 forward: 13.3 us with 5 ranges that exchange -> 7.4 with 16; 8192 x 128, 128 tokens, both
+// gradients: 21.7 -> 10.0; 128 x 128, 8192 tokens: 17.7 -> 8.6.  With many tiles the exchange moves half of the bytes and
+// needs no second launch: it stays.
 // (Blocks from `blocks` on do the same for a second product.)
 template <bool OUT_T>
 __global__ void __launch_bounds__(128) splitk_sum_kernel(const __grid_constant__ GemmParams p1, int bn1, int blocks,
@@ -1265,7 +1268,7 @@ double exchange_us(int s, int bn, double bytes)
 // The same where splitk_sum_kernel follows the product: its launch, the fp32 stores that the units end with, their bytes.
 // (Measured against whole tiles and exchanges at 1 ... 32 tiles, 2 ... 44 ranges.)
 double sum_us(int s, int bn, double bytes) { return 0.4 + 2.4 * bn / 256.0 + 0.04 * s + bytes / 2.9e6; }
-// split factors tried there (0: none)
+// split factors tried there
 constexpr int SUM_SPLITS[] = {2, 3, 4, 6, 8, 11, 16, 22, 32, 44, 64};
 
 // L2-aware band height of a product with tiles `bn` wide.
@@ -1364,13 +1367,14 @@ struct JointPlan { LaunchPlan w, x; int pairs; GradsPlan g; double us; };
 // grad_W units go round the pairs; the last, partial round leaves `late` pairs busy for one unit more.  For every width,
 // split and number of early rounds the model gives the time at which the last pair ends; a pair that changes over from one
 // product to the other drains and refills its pipeline (SWITCH_US, about what a kernel boundary costs).
-constexpr double SWITCH_US = 2.5, LAUNCH_US = 3.0;      // (a second launch: what a product of one stage takes besides it)
+constexpr double SWITCH_US = 2.5, SUM_WAIT_US = 1.5, LAUNCH_US = 3.0;      // (a second launch: what a product of one stage takes besides it)
 JointPlan find_joint_plan(int elt, int sm_count, size_t partial_bytes, int O, int I, int T)
 {
     const int max_pairs = sm_count / 2;
     const int wk = (T + 256 / elt - 1) / (256 / elt), xk = (O + 128 / elt - 1) / (128 / elt);      // stages
     const Widths ww = widths_of(GRAD_WEIGHT, elt), xw = widths_of(GRAD_INPUT, elt);
     JointPlan best{};
+    double best_rank = 0.0;
     for (int bnw : ww.bn) {
         if (!bnw) continue;
         const TileCost cw = tile_cost(GRAD_WEIGHT, elt, bnw);
@@ -1380,7 +1384,9 @@ JointPlan find_joint_plan(int elt, int sm_count, size_t partial_bytes, int O, in
             const TileCost cx = tile_cost(GRAD_INPUT, elt, bnx);
             const int x_tiles = ((T + 2 * BM - 1) / (2 * BM)) * ((I + bnx - 1) / bnx);
             // grad_W whole, split with an exchange (s = 2 .. MAX_SPLITS) or with a sum afterwards (the rest); grad_X whole or with
-            // a sum.  Sums are for few tiles: everything has to fit into one round of the pairs.
+            // a sum.  Sums are for few tiles whose ranges all run at once; they wait for the last tile of the other product
+            // too, which an exchange does not (128 x 2048, 8192 tokens, FP8: 19.1 us with an exchange, 21.4 with a sum): against
+            // other plans of one launch they count SUM_WAIT_US more.
             constexpr int SUMS = sizeof(SUM_SPLITS) / sizeof(SUM_SPLITS[0]);
             for (int o = 1; o <= MAX_SPLITS + SUMS; ++o)
             for (int ox = -1; ox < SUMS; ++ox) {
@@ -1417,10 +1423,14 @@ JointPlan find_joint_plan(int elt, int sm_count, size_t partial_bytes, int O, in
                         // rounds of the early / late pairs: the group that comes second lacks the last one if `last` is short
                         const int r_early = rounds - ((rounds && !ef && last <= late) ? 1 : 0);
                         const int r_late = rounds - ((rounds && ef && last <= n_early) ? 1 : 0);
-                        double us = n_early ? t_early + (early + r_early) * x_us : 0.0;
-                        if (late && t_late + r_late * x_us > us) us = t_late + r_late * x_us;
+                        // (a pair that gets no grad_X tile does not change over)
+                        double us = n_early ? t_early + (early + r_early ? (early + r_early) * x_us : whole ? -SWITCH_US : 0.0) : 0.0;
+                        const double late_us = t_late + (r_late ? r_late * x_us : -SWITCH_US);
+                        if (late && late_us > us) us = late_us;
                         us += 0.05 * x_us + after;                          // among equals the shorter tile
-                        if (best.pairs && us >= best.us - 1e-9) continue;
+                        const double rank = us + (after > 0.0 ? SUM_WAIT_US : 0.0);
+                        if (best.pairs && rank >= best_rank - 1e-9) continue;
+                        best_rank = rank;
                         best.w = LaunchPlan{bnw, s, s > 1 ? whole : w_tiles, 0, 0.0, w_sum};
                         best.x = LaunchPlan{bnx, sx, sx > 1 ? 0 : x_tiles, 0, 0.0, sx > 1};
                         best.pairs = P;
