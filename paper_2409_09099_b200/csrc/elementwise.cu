@@ -93,8 +93,8 @@ struct SoftGroup {
 // subtraction a - copysign(t, a), and the kept pair is the top two of four integer keys
 // (magnitude << 2 | 3 - index: magnitude descending, index ascending; pairwise distinct) found with a
 // seven-operation min/max network.
-// MODE 0: the method's projection (threshold |t2|); MODE 1: interpolated threshold
-// t = (1 - gamma) |t2| + gamma |t3| (Sec. 4.1); MODE 2: hard thresholding (Eq. 2), the kept pair unchanged.
+// MODE 1: interpolated threshold t = (1 - gamma) |t2| + gamma |t3| (Sec. 4.1); MODE 2: hard thresholding (Eq. 2), the kept
+// pair unchanged.  (MODE 0, the method's own projection, is project_group.)
 template <bool FP8, int MODE>
 __device__ __forceinline__ SoftGroup soft_group(uint32_t w01, uint32_t w23, float beta, float wscale, float gamma)
 {
