@@ -101,7 +101,8 @@ sste_status sste_create(sste_ctx **ctx, int device, void *workspace, size_t work
 sste_status sste_destroy(sste_ctx *ctx);
 const char *sste_status_string(sste_status s);
 
-/* Synchronise `stream`, read and clear the device status word.  SSTE_OK if nothing was recorded. */
+/* Synchronise `stream`, read and clear the device status word.  SSTE_OK if nothing was recorded.  SSTE_ERR_TIMEOUT: the
+ * products launched on this context since the expired wait are not to be trusted; those launched after this call are. */
 sste_status sste_poll_device_status(sste_ctx *ctx, void *stream);
 
 /* Sizes of a compressed operand of a logical [rows, k] matrix. */

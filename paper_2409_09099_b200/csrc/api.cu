@@ -94,9 +94,12 @@ extern "C" sste_status sste_poll_device_status(sste_ctx *ctx, void *stream)
     SSTE_CUDA_TRY(cudaMemcpyAsync(&word, ctx->status_dev, sizeof word, cudaMemcpyDeviceToHost, s));
     SSTE_CUDA_TRY(cudaMemsetAsync(ctx->status_dev, 0, sizeof word, s));
     SSTE_CUDA_TRY(cudaStreamSynchronize(s));
-    // a product that gave up on a wait may have left split tiles half counted
-    if (word == SSTE_ERR_TIMEOUT && ctx->splitk_tickets)
+    // A product that gave up on a wait may have left split tiles half counted, and the word keeps only one of several
+    // errors: whatever it says, the counters are zero again when this returns.
+    if (word != SSTE_OK && ctx->splitk_tickets) {
         SSTE_CUDA_TRY(cudaMemsetAsync(ctx->splitk_tickets, 0, SSTE_SPLITK_TICKETS * sizeof(unsigned int), s));
+        SSTE_CUDA_TRY(cudaStreamSynchronize(s));
+    }
     if (word > SSTE_ERR_TIMEOUT) return SSTE_ERR_CUDA;
     return static_cast<sste_status>(word);
 }

@@ -109,7 +109,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, const W
         if (mbar_try_wait(bar, parity)) return true;
         if (*wc.abort_flag) return false;
         if (global_ns() - start > wc.limit_ns) {
-            atomicCAS(wc.status, 0u, static_cast<unsigned int>(SSTE_ERR_TIMEOUT));
+            atomicMax(wc.status, static_cast<unsigned int>(SSTE_ERR_TIMEOUT));      // also over a recorded degenerate beta
             *wc.abort_flag = 1;
             return false;
         }
@@ -765,7 +765,7 @@ product(const CUtensorMap &map_a, const CUtensorMap &map_b, const CUtensorMap &m
                             while (ok && ld_acquire_gpu(ticket) != all) {
                                 if (*wc.abort_flag) ok = false;
                                 else if (global_ns() - start > wc.limit_ns) {
-                                    atomicCAS(wc.status, 0u, static_cast<unsigned int>(SSTE_ERR_TIMEOUT));
+                                    atomicMax(wc.status, static_cast<unsigned int>(SSTE_ERR_TIMEOUT));      // also over a recorded degenerate beta
                                     *wc.abort_flag = 1;
                                     ok = false;
                                 }
