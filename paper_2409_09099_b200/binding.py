@@ -180,6 +180,8 @@ class Context:
         self.device = device
         n = self.lib.sste_workspace_bytes() if minimal_workspace else self.lib.sste_workspace_bytes_recommended()
         self.workspace = torch.zeros(n, dtype=torch.uint8, device=f"cuda:{device}")
+        # the first call may be on any stream: the fill (and whoever had this memory before) is done by then
+        torch.cuda.current_stream(device).synchronize()
         handle = ctypes.c_void_p()
         st = self.lib.sste_create(ctypes.byref(handle), device, _vp(self.workspace), ctypes.c_size_t(n))
         self._check(st)

@@ -69,7 +69,8 @@ extern "C" sste_status sste_create(sste_ctx **out, int device, void *workspace, 
     if (ctx->splitk_partials) ctx->splitk_tickets = reinterpret_cast<unsigned int *>(ws + SSTE_WS_SPLITK_TICKETS_OFF);
     if (cudaMemset(ws, 0, SSTE_WS_PARTIALS_OFF) != cudaSuccess ||
         (ctx->splitk_tickets &&
-         cudaMemset(ctx->splitk_tickets, 0, SSTE_SPLITK_TICKETS * sizeof(unsigned int)) != cudaSuccess)) {
+         cudaMemset(ctx->splitk_tickets, 0, SSTE_SPLITK_TICKETS * sizeof(unsigned int)) != cudaSuccess) ||
+        cudaStreamSynchronize(nullptr) != cudaSuccess) {     // (a memset may return first: the next call may be on any stream)
         delete ctx;
         return SSTE_ERR_CUDA;
     }
