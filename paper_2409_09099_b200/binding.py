@@ -190,8 +190,7 @@ class Context:
     def close(self):
         if getattr(self, "handle", None):
             self.lib.sste_destroy(self.handle)
-            self.handle = None
-            self.workspace = None      # 192 MB: not kept by whatever still refers to a closed context
+            self.handle = None         # (the workspace goes with this object: work on other streams may still use it)
 
     def __del__(self):
         try:

@@ -39,3 +39,17 @@ def test_first_product_on_another_stream(own_stream):
     torch.cuda.synchronize()
     assert torch.equal(got.view(torch.int16), want.view(torch.int16)) and ctx.poll_device_status() == B.OK
     ctx.close()
+
+
+def test_close_leaves_the_workspace_to_work_in_flight():
+    """Closing frees nothing: memory allocated right afterwards is not the workspace of a product that has yet to run."""
+    gvals, gmeta, X, want = _operands()
+    got, side = torch.empty_like(want), torch.cuda.Stream()
+    ctx = B.Context(0)
+    with torch.cuda.stream(side):
+        torch.cuda._sleep(BUSY)
+        ctx.linear_bwd_weight(gvals, gmeta, X, got)
+    ctx.close()
+    other = torch.full_like(ctx.workspace, 0x5a)             # on this stream, beside the side stream's work
+    torch.cuda.synchronize()
+    assert torch.equal(got.view(torch.int16), want.view(torch.int16)) and bool((other == 0x5a).all())
