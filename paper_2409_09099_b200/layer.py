@@ -19,6 +19,11 @@ _DESCRIBED = frozenset(("ctx", "W", "T", "tensor_id", "seed", "fp8", "counter_co
 _bf16, _raw_stream, _device = torch.bfloat16, torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
 
 
+def _takes(t, shape):
+    """Whether a one-call phase can read `t` as it is; anything else goes to the single calls, which check it."""
+    return t.dtype is _bf16 and t.shape == shape and t.is_cuda and t.is_contiguous()
+
+
 class SsteLinear:
     """W[O, I] dense master weight (bf16); forward Y = X S(W)^T, backward (dX, dW).
 
@@ -150,7 +155,7 @@ class SsteLinear:
     def forward(self, X, y_amax_out=None):
         if self.mark is None:
             desc = self._desc or self._describe()
-            if desc[0] and X.dtype is _bf16 and X.shape == desc[6] and X.is_cuda and X.is_contiguous():
+            if desc[0] and _takes(X, desc[6]):
                 st = desc[4](self.ctx.handle, desc[1], X.data_ptr(), B._ptr(y_amax_out), _raw_stream(_device()))
                 if st:
                     self.ctx._check(st)
@@ -183,8 +188,7 @@ class SsteLinear:
         if self.mark is None:
             desc = self._desc or self._describe()
             X = None if self.fp8 else self.X
-            if (desc[0] and dY.dtype is _bf16 and dY.shape == desc[7] and dY.is_cuda and dY.is_contiguous()
-                    and (X is None or X.shape == desc[6])):
+            if desc[0] and _takes(dY, desc[7]) and (X is None or _takes(X, desc[6])):
                 st = desc[5](self.ctx.handle, desc[1], None if X is None else X.data_ptr(), dY.data_ptr(), step, token_offset,
                              _raw_stream(_device()))
                 if st:
@@ -222,8 +226,7 @@ class SsteLinear:
         if self.mark is None:
             desc = self._desc or self._describe()
             X = None if self.fp8 else self.X
-            if (desc[0] and self.Y.dtype is _bf16 and dY.dtype is _bf16 and dY.shape == desc[7] and dY.is_cuda
-                    and dY.is_contiguous() and (X is None or X.shape == desc[6])):
+            if desc[0] and self.Y.dtype is _bf16 and _takes(dY, desc[7]) and (X is None or _takes(X, desc[6])):
                 st = desc[9](self.ctx.handle, desc[1], None if X is None else X.data_ptr(), dY.data_ptr(),
                              _raw_stream(_device()))
                 if st:
@@ -312,7 +315,7 @@ class SsteLinearPadded:
     # Descriptor of the one-call path, made anew when the inner layer's changes or a buffer of this layer is replaced.
     def _described(self, X, shape):
         inner = self.inner
-        if inner.mark is not None or X.dtype is not _bf16 or X.shape != shape or not X.is_cuda or not X.is_contiguous():
+        if inner.mark is not None or not _takes(X, shape):
             return None
         of = inner._desc or inner._describe()
         bufs = (self.Xp, self.dYp, self.Y, self.dX, self.dW)
