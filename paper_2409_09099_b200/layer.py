@@ -24,6 +24,11 @@ def _takes(t, shape):
     return t.dtype is _bf16 and t.shape == shape and t.is_cuda and t.is_contiguous()
 
 
+class _Described:
+    """sste_layer of a layer's buffers; per phase the C call, the tensors it works on and the addresses put down for them."""
+    __slots__ = ("fits", "buffers", "at", "x_shape", "g_shape", "w_shape", "prune", "forward", "backward", "grads")
+
+
 class SsteLinear:
     """W[O, I] dense master weight (bf16); forward Y = X S(W)^T, backward (dX, dW).
 
@@ -87,22 +92,45 @@ class SsteLinear:
                            self.counter_cols, self.tensor_id & 0xffffffff, 0, self.seed & 0xffffffffffffffff,
                            *[None if t is None else t.data_ptr() for t in tensors])
         lib = self.ctx.lib
-        self.__dict__["_desc"] = desc = (fits, ctypes.addressof(d), self.W.data_ptr(), lib.sste_layer_prune,
-                                         lib.sste_layer_forward, lib.sste_layer_backward, x_shape, g_shape, d,
-                                         lib.sste_layer_grads)
+        self.__dict__["_desc"] = desc = _Described()
+        desc.fits, desc.buffers, desc.at, desc.x_shape, desc.g_shape = fits, d, ctypes.addressof(d), x_shape, g_shape
+        desc.w_shape = torch.Size((self.O, self.I))
+        w = (self.vals, self.meta) if self.w_dense is None else (self.w_dense,)
+        for name, call, read in (
+                ("prune", lib.sste_layer_prune, (self.W, self.beta, self.vals, self.meta, self.w_dense, self.amax, self._scratch)),
+                ("forward", lib.sste_layer_forward, (self.vals, self.meta, self.Y, self.Xq, self.amax, self._scratch)),
+                ("backward", lib.sste_layer_backward, (self.gvals, self.gmeta, self.dW, self.dX, *w, self.Xq, self.dYq, self.amax,
+                                                       self._scratch)),
+                ("grads", lib.sste_layer_grads, (self.gvals, self.gmeta, self.dW, self.dX, *w, self.Xq, self.dYq, self.amax))):
+            read = tuple(t for t in read if t is not None)
+            setattr(desc, name, (call, read, [t.data_ptr() for t in read]))
         return desc
+
+    def _described(self, phase):
+        """The descriptor, with the addresses that the buffers of `phase` have now; None: the single calls take it.
+
+        A tensor may be given other storage without being replaced (`t.data = ...`, a storage resized to 0 and back)."""
+        desc = self._desc or self._describe()
+        _, read, at = getattr(desc, phase)
+        if [t.data_ptr() for t in read] != at:
+            self.__dict__["_as_made"] = False
+            desc = self._describe()
+        return desc if desc.fits else None
 
     def _replaced_fit(self, x_shape, g_shape, tensors):
         wdt, gdt = (B._TORCH_DT[B.E4M3], B._TORCH_DT[B.E5M2]) if self.fp8 else (_bf16, _bf16)
         w_shape = (self.O, self.I)
         return (all(t is None or (t.is_cuda and t.is_contiguous()) for t in tensors)
                 and self.W.dtype is _bf16 and tuple(self.W.shape) == w_shape and self.beta.dtype is torch.float32
+                and self.beta.numel() >= 1 and self.meta.nbytes == self.O * self.I // 8
+                and self.gmeta.nbytes == self.O * self.T // 8
                 and self.vals.dtype is wdt and tuple(self.vals.shape) == (self.O, self.I // 2)
                 and self.gvals.dtype is gdt and tuple(self.gvals.shape) == (self.O, self.T // 2)
                 and (self.w_dense is None or (self.w_dense.dtype is wdt and tuple(self.w_dense.shape) == w_shape))
                 and self.Y.shape == g_shape and self.dX.shape == x_shape and tuple(self.dW.shape) == w_shape
                 and self.dX.dtype is self.Y.dtype and self.dW.dtype is self.Y.dtype
-                and (not self.fp8 or (self.Xq.dtype is wdt and self.Xq.shape == x_shape
+                and (not self.fp8 or (self.amax.dtype is torch.float32 and self.amax.numel() == 3
+                                      and self._scratch.nbytes == 8 and self.Xq.dtype is wdt and self.Xq.shape == x_shape
                                       and self.dYq.dtype is gdt and self.dYq.shape == g_shape)))
 
     def _amax(self, k):
@@ -122,9 +150,9 @@ class SsteLinear:
     def prune(self):
         assert self.beta_ready, "call init_beta() in the first iteration"
         if self.mark is None and not self.track_flips:
-            desc = self._desc or self._describe()
-            if desc[0] and self.W.data_ptr() == desc[2]:          # W is the caller's: its storage may have been exchanged
-                st = desc[3](self.ctx.handle, desc[1], _raw_stream(_device()))
+            desc = self._described("prune")
+            if desc and _takes(self.W, desc.w_shape):             # W is the caller's: it may be another view by now
+                st = desc.prune[0](self.ctx.handle, desc.at, _raw_stream(_device()))
                 if st:
                     self.ctx._check(st)
                 self.__dict__["launches"] += 2 if self.fp8 else 1
@@ -154,9 +182,9 @@ class SsteLinear:
     # (2a) forward with the sparse weight
     def forward(self, X, y_amax_out=None):
         if self.mark is None:
-            desc = self._desc or self._describe()
-            if desc[0] and _takes(X, desc[6]):
-                st = desc[4](self.ctx.handle, desc[1], X.data_ptr(), B._ptr(y_amax_out), _raw_stream(_device()))
+            desc = self._described("forward")
+            if desc and _takes(X, desc.x_shape):
+                st = desc.forward[0](self.ctx.handle, desc.at, X.data_ptr(), B._ptr(y_amax_out), _raw_stream(_device()))
                 if st:
                     self.ctx._check(st)
                 d = self.__dict__
@@ -186,11 +214,11 @@ class SsteLinear:
     # (2b) backward: MVUE on the output gradient for grad_W, dense product for grad_X
     def backward(self, dY, step: int = 0, token_offset: int = 0):
         if self.mark is None:
-            desc = self._desc or self._describe()
+            desc = self._described("backward")
             X = None if self.fp8 else self.X
-            if desc[0] and _takes(dY, desc[7]) and (X is None or _takes(X, desc[6])):
-                st = desc[5](self.ctx.handle, desc[1], None if X is None else X.data_ptr(), dY.data_ptr(), step, token_offset,
-                             _raw_stream(_device()))
+            if desc and _takes(dY, desc.g_shape) and (X is None or _takes(X, desc.x_shape)):
+                st = desc.backward[0](self.ctx.handle, desc.at, None if X is None else X.data_ptr(), dY.data_ptr(), step,
+                                      token_offset, _raw_stream(_device()))
                 if st:
                     self.ctx._check(st)
                 self.__dict__["launches"] += 4 if self.fp8 else 3
@@ -224,11 +252,11 @@ class SsteLinear:
         the current stream does both and shares the SMs between them; otherwise grad_W runs on `side_stream` (through
         `side_ctx`: its own split-K workspace) beside grad_X.  Both are complete in current-stream order on return."""
         if self.mark is None:
-            desc = self._desc or self._describe()
+            desc = self._described("grads")
             X = None if self.fp8 else self.X
-            if desc[0] and self.Y.dtype is _bf16 and _takes(dY, desc[7]) and (X is None or _takes(X, desc[6])):
-                st = desc[9](self.ctx.handle, desc[1], None if X is None else X.data_ptr(), dY.data_ptr(),
-                             _raw_stream(_device()))
+            if desc and self.Y.dtype is _bf16 and _takes(dY, desc.g_shape) and (X is None or _takes(X, desc.x_shape)):
+                st = desc.grads[0](self.ctx.handle, desc.at, None if X is None else X.data_ptr(), dY.data_ptr(),
+                                   _raw_stream(_device()))
                 if st:
                     self.ctx._check(st)
                 self.__dict__["launches"] += 2
@@ -312,34 +340,37 @@ class SsteLinearPadded:
     def prune(self):
         self.inner.prune()
 
-    # Descriptor of the one-call path, made anew when the inner layer's changes or a buffer of this layer is replaced.
-    def _described(self, X, shape):
+    # Descriptor of the one-call path, made anew when the inner layer's changes or a buffer of this layer is replaced or
+    # given other storage.
+    def _described(self, phase, X, shape):
         inner = self.inner
         if inner.mark is not None or not _takes(X, shape):
             return None
-        of = inner._desc or inner._describe()
+        of = inner._described(phase)
+        if of is None:
+            return None
         bufs = (self.Xp, self.dYp, self.Y, self.dX, self.dW)
+        at = [t.data_ptr() for t in bufs]
         d = self._desc
-        if d is None or d[0] is not of or any(a is not b for a, b in zip(d[1], bufs)):
+        if d is None or d[0] is not of or d[2] != at or any(a is not b for a, b in zip(d[1], bufs)):
             crop = lambda t, whole: None if t.data_ptr() == whole.data_ptr() else B._ptr(t)
-            p = B.PaddedLayerBuffers(of[8], self.O, self.I, self.T, 0, B._ptr(self.Xp), B._ptr(self.dYp),
+            p = B.PaddedLayerBuffers(of.buffers, self.O, self.I, self.T, 0, B._ptr(self.Xp), B._ptr(self.dYp),
                                      crop(self.Y, inner.Y), crop(self.dX, inner.dX), crop(self.dW, inner.dW))
-            fits = (of[0] and inner.Y.dtype is _bf16 and tuple(self.Xp.shape) == (self.Tp, self.Ip)
+            fits = (inner.Y.dtype is _bf16 and tuple(self.Xp.shape) == (self.Tp, self.Ip)
                     and tuple(self.dYp.shape) == (self.Tp, self.Op) and tuple(self.Y.shape) == (self.T, self.O)
                     and tuple(self.dX.shape) == (self.T, self.I) and tuple(self.dW.shape) == (self.O, self.I)
-                    and all(t.dtype is _bf16 for t in bufs))
-            lib = self.ctx.lib
-            self._desc = d = (of, bufs, fits, ctypes.addressof(p), lib.sste_padded_forward, lib.sste_padded_backward, p)
-        return d if d[2] else None
+                    and all(t.dtype is _bf16 and t.is_cuda and t.is_contiguous() for t in bufs))
+            self._desc = d = (of, bufs, at, fits, ctypes.addressof(p), p)
+        return d if d[3] else None
 
     def _crop(self, src, dst):
         if src.data_ptr() != dst.data_ptr():
             self.ctx.crop_2d(src, dst)
 
     def forward(self, X):
-        d = self._described(X, (self.T, self.I))
+        d = self._described("forward", X, (self.T, self.I))
         if d is not None:
-            st = d[4](self.ctx.handle, d[3], X.data_ptr(), _raw_stream(_device()))
+            st = self.ctx.lib.sste_padded_forward(self.ctx.handle, d[4], X.data_ptr(), _raw_stream(_device()))
             if st:
                 self.ctx._check(st)
             inner = self.inner.__dict__
@@ -353,9 +384,9 @@ class SsteLinearPadded:
         return self.Y
 
     def backward(self, dY, step: int = 0):
-        d = self._described(dY, (self.T, self.O))
+        d = self._described("backward", dY, (self.T, self.O))
         if d is not None:
-            st = d[5](self.ctx.handle, d[3], dY.data_ptr(), step, 0, _raw_stream(_device()))
+            st = self.ctx.lib.sste_padded_backward(self.ctx.handle, d[4], dY.data_ptr(), step, 0, _raw_stream(_device()))
             if st:
                 self.ctx._check(st)
             self.inner.__dict__["launches"] += 4 if self.inner.fp8 else 3

@@ -52,3 +52,48 @@ def test_a_saved_input_that_the_products_cannot_read_is_refused(ctx, call, what)
     ref.forward(X.t().contiguous())
     ref.backward(dY)
     assert _same(lin.dW, ref.dW)
+
+
+@pytest.mark.parametrize("fp8", [False, True])
+def test_buffers_given_other_storage(ctx, fp8):
+    """`t.data = ...` on any buffer between two phases: the next phase works on the new storage and leaves the old alone."""
+    lin, ref, X, dY = _layer(ctx, fp8=fp8), _layer(ctx, fp8=fp8), X1(), DY()
+    names = ["W", "beta", "vals", "meta", "w_dense", "gvals", "gmeta", "Y", "dX", "dW"] + (["amax", "Xq", "dYq"] if fp8 else [])
+    for l in (ref, lin):
+        l.prune(); l.forward(X); l.backward(dY, step=1)
+    old = {}
+    for phase in ("prune", "forward", "backward"):
+        for n in names:
+            t = getattr(lin, n)
+            old[n] = t.data
+            t.data = t.data.clone()
+            old[n].view(torch.uint8).fill_(0x55)
+        for l in (ref, lin):
+            {"prune": l.prune, "forward": lambda: l.forward(X), "backward": lambda: l.backward(dY, step=2)}[phase]()
+        for n in names:
+            assert bool((old[n].view(torch.uint8) == 0x55).all()), (phase, n)
+            assert _same(getattr(lin, n), getattr(ref, n)), (phase, n)
+    assert lin._desc.fits and lin._desc.buffers.W == lin.W.data_ptr()      # described again, not left to the single calls
+
+
+def test_padded_buffers_given_other_storage(ctx):
+    lin = SsteLinearPadded(ctx, 200, 100, 72, seed=5)
+    W, X, dY = (dbf16(synth.gaussian_bf16(s, sh, sg)) for s, sh, sg in ((51, (200, 100), 0.02), (52, (72, 100), 1.0), (53, (72, 200), 1e-2)))
+    lin.set_weight(W); lin.init_beta(); lin.prune()
+    want = [lin.forward(X).clone()] + [t.clone() for t in lin.backward(dY, step=1)]
+    old = []
+    for t in (lin.Xp, lin.dYp, lin.Y, lin.dX, lin.dW):
+        old.append(t.data)
+        t.data = torch.zeros_like(t.data)
+        old[-1].view(torch.int16).fill_(0x5555)
+    got = [lin.forward(X), *lin.backward(dY, step=1)]
+    assert all(_same(a, b) for a, b in zip(got, want)) and all(bool((t.view(torch.int16) == 0x5555).all()) for t in old)
+
+
+def test_a_weight_turned_into_a_view_that_is_not_contiguous_is_refused(ctx):
+    W = dbf16(synth.gaussian_bf16(61, (256, 256), 0.02))
+    lin = SsteLinear(ctx, W, T)
+    lin.init_beta(); lin.prune()
+    lin.W.data = lin.W.data.t()                          # same address, same sizes
+    with pytest.raises(AssertionError):
+        lin.prune()
