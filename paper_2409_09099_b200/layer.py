@@ -15,8 +15,18 @@ from . import binding as B
 
 # attributes the sste_layer descriptor is made of: setting one makes the next call build it anew
 _DESCRIBED = frozenset(("ctx", "W", "T", "tensor_id", "seed", "fp8", "counter_cols", "beta", "vals", "meta", "w_dense",
-                        "gvals", "gmeta", "Y", "dX", "dW", "amax", "Xq", "dYq", "_scratch"))
+                        "gvals", "gmeta", "Y", "dX", "dW", "amax", "Xq", "dYq", "_scratch", "sparsify_grad", "grad_weight",
+                        "grad_input"))
+# what a one-call phase stands for; a layer or context that brings its own version of one of these gets the single calls
+_LAYER_CALLS = ("sparsify_grad", "grad_weight", "grad_input")
+_CONTEXT_CALLS = ("project_amax", "project_compress", "amax", "quantize_fp8", "linear_fwd", "mvue_sparsify", "linear_bwd_weight",
+                  "linear_bwd_input", "pad_2d", "crop_2d")
 _bf16, _raw_stream, _device = torch.bfloat16, torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+
+
+def _as_defined(obj, cls, names):
+    """Whether `obj` is a `cls` whose methods `names` are those of `cls` (no subclass, no attribute, overrides them)."""
+    return isinstance(obj, cls) and not any(getattr(type(obj), n) is not getattr(cls, n) or n in vars(obj) for n in names)
 
 
 def _takes(t, shape):
@@ -86,14 +96,18 @@ class SsteLinear:
         tensors = (self.W, self.beta, self.amax, self.vals, self.meta, self.w_dense, self.gvals, self.gmeta, self.Xq,
                    self.dYq, self.Y, self.dX, self.dW, self._scratch)
         x_shape, g_shape = torch.Size((self.T, self.I)), torch.Size((self.T, self.O))
+        self.__dict__["_desc"] = desc = _Described()
         # a layer whose buffers were replaced by ones of other sizes or types is not described: the single calls check it
-        fits = self._as_made or self._replaced_fit(x_shape, g_shape, tensors)
+        desc.fits = (_as_defined(self, SsteLinear, _LAYER_CALLS) and _as_defined(self.ctx, B.Context, _CONTEXT_CALLS)
+                     and (self._as_made or self._replaced_fit(x_shape, g_shape, tensors)))
+        if not desc.fits:
+            desc.prune = desc.forward = desc.backward = desc.grads = (None, (), [])
+            return desc
         d = B.LayerBuffers(self.O, self.I, self.T, B.E4M3 if self.fp8 else B.BF16, B._CODE_OF[self.Y.dtype],
                            self.counter_cols, self.tensor_id & 0xffffffff, 0, self.seed & 0xffffffffffffffff,
                            *[None if t is None else t.data_ptr() for t in tensors])
         lib = self.ctx.lib
-        self.__dict__["_desc"] = desc = _Described()
-        desc.fits, desc.buffers, desc.at, desc.x_shape, desc.g_shape = fits, d, ctypes.addressof(d), x_shape, g_shape
+        desc.buffers, desc.at, desc.x_shape, desc.g_shape = d, ctypes.addressof(d), x_shape, g_shape
         desc.w_shape = torch.Size((self.O, self.I))
         w = (self.vals, self.meta) if self.w_dense is None else (self.w_dense,)
         for name, call, read in (
@@ -264,7 +278,11 @@ class SsteLinear:
         main = torch.cuda.current_stream()
         side_stream.wait_stream(main)
         with torch.cuda.stream(side_stream):
-            self.grad_weight(side_ctx)
+            saved, self.__dict__["ctx"] = self.ctx, side_ctx       # (not a new context of the layer: nothing to describe)
+            try:
+                self.grad_weight()
+            finally:
+                self.__dict__["ctx"] = saved
         self.grad_input(dY)
         main.wait_stream(side_stream)
         return self.dX, self.dW
@@ -286,7 +304,7 @@ class SsteLinear:
     def grad_weight(self, ctx: B.Context | None = None):
         self._m("linear_bwd_weight")
         (ctx or self.ctx).linear_bwd_weight(self.gvals, self.gmeta, self.Xq if self.fp8 else self.X, self.dW,
-                                   g_amax_dev=self._amax(2), x_amax_dev=self._amax(0))
+                                            g_amax_dev=self._amax(2), x_amax_dev=self._amax(0))
         self.launches += 1
         return self.dW
 

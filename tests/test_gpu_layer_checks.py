@@ -97,3 +97,38 @@ def test_a_weight_turned_into_a_view_that_is_not_contiguous_is_refused(ctx):
     lin.W.data = lin.W.data.t()                          # same address, same sizes
     with pytest.raises(AssertionError):
         lin.prune()
+
+
+@pytest.mark.parametrize("how", ["subclass", "attribute", "context"])
+@pytest.mark.parametrize("call", ["backward", "overlap"])
+def test_single_calls_that_someone_overrides_are_still_made(ctx, how, call):
+    """A layer whose grad_weight does something more (an all-reduce, a count), or a context that watches its calls."""
+    seen = []
+
+    class Watching(SsteLinear):
+        def grad_weight(self):
+            seen.append("W")
+            return super().grad_weight()
+
+    class WatchingContext(B.Context):
+        def linear_bwd_weight(self, *a, **kw):
+            seen.append("W")
+            return super().linear_bwd_weight(*a, **kw)
+
+    ctx_ = WatchingContext(0) if how == "context" else ctx
+    side_ctx, side = (WatchingContext if how == "context" else B.Context)(0), torch.cuda.Stream()
+    lin, X, dY = _layer(ctx_, cls=Watching if how == "subclass" else SsteLinear), X1(), DY()
+    lin.forward(X)
+    if how == "attribute":
+        plain = lin.grad_weight
+        lin.grad_weight = lambda: (seen.append("W"), plain())[1]
+    if call == "backward":
+        lin.backward(dY)
+    else:
+        lin.sparsify_grad(dY)
+        lin.grad_weight_and_input(dY, side_ctx, side)
+    assert seen == ["W"]
+    ref = _layer(ctx)
+    ref.forward(X); ref.backward(dY)
+    torch.testing.assert_close(lin.dW.float(), ref.dW.float(), rtol=2.0 ** -7, atol=1e-5 * float(ref.dW.float().abs().max()))
+    assert lin.ctx is ctx_
