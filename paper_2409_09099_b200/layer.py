@@ -402,7 +402,9 @@ class SsteLinearPadded:
         return self.Y
 
     def backward(self, dY, step: int = 0):
-        d = self._described("backward", dY, (self.T, self.O))
+        # (the inner layer's input is Xp after a forward; without one, or after somebody gave it another, the single calls tell)
+        read_xp = self.inner.fp8 or self.inner.__dict__.get("X") is self.Xp
+        d = self._described("backward", dY, (self.T, self.O)) if read_xp else None
         if d is not None:
             st = self.ctx.lib.sste_padded_backward(self.ctx.handle, d[4], dY.data_ptr(), step, 0, _raw_stream(_device()))
             if st:

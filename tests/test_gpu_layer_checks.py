@@ -132,3 +132,18 @@ def test_single_calls_that_someone_overrides_are_still_made(ctx, how, call):
     ref.forward(X); ref.backward(dY)
     torch.testing.assert_close(lin.dW.float(), ref.dW.float(), rtol=2.0 ** -7, atol=1e-5 * float(ref.dW.float().abs().max()))
     assert lin.ctx is ctx_
+
+
+def test_padded_backward_uses_the_inner_layers_input(ctx):
+    """No forward, no input: refused.  An input that somebody gave the inner layer (recomputed activations) is the one used."""
+    W, X, dY = (dbf16(synth.gaussian_bf16(s, sh, sg)) for s, sh, sg in ((71, (200, 100), 0.02), (72, (72, 100), 1.0), (73, (72, 200), 1e-2)))
+    lin, ref = (SsteLinearPadded(ctx, 200, 100, 72, seed=5) for _ in range(2))
+    for l in (lin, ref):
+        l.set_weight(W); l.init_beta(); l.prune()
+    with pytest.raises(AttributeError):
+        lin.backward(dY)
+    lin.forward(torch.zeros_like(X))
+    ref.forward(X)
+    lin.inner.X = ref.Xp
+    for a, b in zip(lin.backward(dY), ref.backward(dY)):
+        assert _same(a, b)
