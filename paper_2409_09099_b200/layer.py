@@ -8,6 +8,7 @@ sparse weight and is meant to be applied to the dense weight unchanged.
 from __future__ import annotations
 
 import ctypes
+from operator import index
 
 import torch
 
@@ -104,7 +105,7 @@ class SsteLinear:
             desc.prune = desc.forward = desc.backward = desc.grads = (None, (), [])
             return desc
         d = B.LayerBuffers(self.O, self.I, self.T, B.E4M3 if self.fp8 else B.BF16, B._CODE_OF[self.Y.dtype],
-                           self.counter_cols, self.tensor_id & 0xffffffff, 0, self.seed & 0xffffffffffffffff,
+                           self.counter_cols, index(self.tensor_id) & 0xffffffff, 0, index(self.seed) & 0xffffffffffffffff,
                            *[None if t is None else t.data_ptr() for t in tensors])
         lib = self.ctx.lib
         desc.buffers, desc.at, desc.x_shape, desc.g_shape = d, ctypes.addressof(d), x_shape, g_shape

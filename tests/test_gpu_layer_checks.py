@@ -147,3 +147,15 @@ def test_padded_backward_uses_the_inner_layers_input(ctx):
     lin.inner.X = ref.Xp
     for a, b in zip(lin.backward(dY), ref.backward(dY)):
         assert _same(a, b)
+
+
+@pytest.mark.parametrize("kind", ["int64", "uint64", "int32"])
+def test_seeds_and_ids_from_numpy(ctx, kind):
+    import numpy as np
+    n = getattr(np, kind)
+    lin, ref, X, dY = _layer(ctx), _layer(ctx), X1(), DY()
+    lin.seed, lin.tensor_id, lin.T, lin.counter_cols = n(77), n(3), n(T), n(0)
+    ref.seed, ref.tensor_id = 77, 3
+    for l in (lin, ref):
+        l.prune(); l.forward(X); l.backward(dY, step=n(4), token_offset=n(8))
+    assert _same(lin.dW, ref.dW) and _same(lin.gmeta, ref.gmeta)
