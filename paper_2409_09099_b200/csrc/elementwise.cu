@@ -466,6 +466,7 @@ struct MvuePair {
     uint2 e0, e1;     // table entries of the two groups
     f32x2 h;          // magnitude of a kept value other than a clipped maximum
     f32x2 mx;         // largest magnitude
+    f32x2 sum;        // of the four magnitudes; where it is not finite, the rest does not hold (mvue_group does)
 };
 
 // Inclusion probabilities p_i = min(1, c |a_i|) with sum 2, kept values a_i / p_i, systematic sampling
@@ -480,7 +481,8 @@ struct MvuePair {
 // f32x2 arithmetic on the FMA pipe (a selection is a multiply by an exact 0 or 1), comparisons give 1.0 / 0.0, their
 // counts are added up as subnormal floats whose bit pattern IS the byte offset of the table entry that holds the kept
 // pair.  118 -> about 70 issued instructions per group, of them about 31 (from 78) on the half-rate pipe.  No branches;
-// every fp32 step is a single rounded operation in the oracle's order.
+// every fp32 step is a single rounded operation in the oracle's order.  (A product with an exact 0 is 0 for finite values
+// only: a sum that overflows, an infinity or a NaN make a group one for mvue_group.)
 __device__ __forceinline__ MvuePair mvue_pair(const uint32_t (&w)[4], uint32_t k_lo, uint32_t k_hi, const uint8_t *lut)
 {
     float lo[4], hi[4];
@@ -540,7 +542,110 @@ __device__ __forceinline__ MvuePair mvue_pair(const uint32_t (&w)[4], uint32_t k
     g.e1 = *reinterpret_cast<const uint2 *>(lut + __float_as_uint(o1));
     g.h = h;
     g.mx = mx;
+    g.sum = s3;
     return g;
+}
+
+// a <= b as an integer mask (all ones / zero)
+__device__ __forceinline__ int fset_le(float a, float b)
+{
+    int r;
+    asm("set.le.s32.f32 %0, %1, %2;" : "=r"(r) : "f"(a), "f"(b));
+    return r;
+}
+
+// The same rule for one group of any values, by selections: p01 = a0 | a1 << 16, p23 = a2 | a3 << 16 (bf16), u the uniform.
+// Sums may overflow; comparisons with a NaN are false, and a NaN is never the maximum.
+struct MvueGroup {
+    uint32_t q0, q1;  // kept positions q0 < q1
+    float v0, v1;     // their values before the cast
+};
+__device__ __forceinline__ MvueGroup mvue_group(uint32_t p01, uint32_t p23, float u)
+{
+    const float m0 = fabsf(__uint_as_float(p01 << 16)), m1 = fabsf(__uint_as_float(p01 & 0xffff0000u));
+    const float m2 = fabsf(__uint_as_float(p23 << 16)), m3 = fabsf(__uint_as_float(p23 & 0xffff0000u));
+    const float mx = fmaxf(fmaxf(m0, m1), fmaxf(m2, m3));
+    const bool e0 = (m0 == mx), e1 = !e0 && (m1 == mx), e2 = !e0 && !e1 && (m2 == mx), e3 = !e0 && !e1 && !e2;
+    const uint32_t xi = e0 ? 0u : e1 ? 1u : e2 ? 2u : 3u;
+    // cumulative sums without the maximum and with it
+    const float z0 = e0 ? 0.0f : m0, z1 = __fadd_rn(z0, e1 ? 0.0f : m1), z2 = __fadd_rn(z1, e2 ? 0.0f : m2);
+    const float rest = __fadd_rn(z2, e3 ? 0.0f : m3);
+    const float s1 = __fadd_rn(m0, m1), s2 = __fadd_rn(s1, m2), s3 = __fadd_rn(s2, m3);
+    const bool clipped = (mx >= rest);
+    const float h = clipped ? rest : __fmul_rn(0.5f, s3);
+    const float c0 = clipped ? z0 : m0, c1 = clipped ? z1 : s1, c2 = clipped ? z2 : s2;
+    const float r1 = __fmul_rn(u, h), r2 = __fadd_rn(r1, h);
+    // (a point AT rest counts as just below it; rest == 0 makes the bound a NaN, which fminf passes over)
+    const float r1c = clipped ? fminf(r1, __uint_as_float(__float_as_uint(rest) - 1u)) : r1;
+    const int j1 = -(fset_le(c0, r1c) + fset_le(c1, r1c) + fset_le(c2, r1c));
+    const int n2 = -(fset_le(c0, r2) + fset_le(c1, r2) + fset_le(c2, r2));
+    const uint32_t ia = static_cast<uint32_t>(!clipped ? min(j1, 2) : rest == 0.0f ? (e0 ? 1 : 0) : j1);
+    const uint32_t ib = clipped ? xi : static_cast<uint32_t>(min(max(j1 + 1, n2), 3));
+    // bf16 bits of a_ia and a_ib in the upper half (lower half: don't care)
+    const uint32_t sa = __byte_perm(p01, p23, ia * 0x2200u + 0x1000u), sb = __byte_perm(p01, p23, ib * 0x2200u + 0x1000u);
+    const uint32_t hb = __float_as_uint(h), sgn = (hb == 0u) ? 0u : 0x80000000u;
+    const float va = __uint_as_float((sa & sgn) | hb);
+    const float vb = __uint_as_float(clipped ? (sb & 0xffff0000u) : ((sb & sgn) | hb));
+    const bool swap = ia > ib;
+    return MvueGroup{min(ia, ib), max(ia, ib), swap ? vb : va, swap ? va : vb};
+}
+
+// Metadata bytes of a thread's eight columns (nibs: a nibble per column): two token groups share a byte, lane ^ 8 holds the
+// neighbouring one.
+template <bool FP8>
+__device__ __forceinline__ void mvue_put_meta(uint32_t nibs, int jc, int tgl, uint8_t *meta_s)
+{
+    const uint32_t other = __shfl_xor_sync(0xffffffffu, nibs, 8);
+    if ((tgl & 1) == 0) {
+        const uint32_t k = 4u * tgl;
+        // the eight bytes (own nibble | neighbour's nibble << 4) of columns e = 0..7, four at a time:
+        // even columns from the low nibbles of each byte of `nibs`, odd columns from the high ones
+        const uint32_t even = (nibs & 0x0f0f0f0fu) | ((other << 4) & 0xf0f0f0f0u);
+        const uint32_t odd = ((nibs >> 4) & 0x0f0f0f0fu) | (other & 0xf0f0f0f0u);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const uint32_t jl = jc * 8 + e;
+            const uint32_t byte = ((e & 1) ? odd : even) >> (8 * (e >> 1));
+            meta_s[FP8 ? sste_meta_atom_byte8(jl, k) : sste_meta_atom_byte16(jl, k)] = static_cast<uint8_t>(byte);
+        }
+    }
+}
+
+// A block's groups by that rule (mvue_kernel's rare path; all threads): rows of dY or of its padded copy from `src` on, group
+// g0 + e of the thread uses word (g0 + e) & 3 of Philox block (g0 + e) >> 2.
+template <bool FP8>
+__device__ __noinline__ void mvue_any_values(const uint4 *src, size_t row_chunks, uint64_t g0, uint32_t tensor_id, uint32_t step,
+                                             uint32_t key0, uint32_t key1, float gscale, uint32_t *vals_s, uint8_t *meta_s,
+                                             uint2 *dense_q)
+{
+    const int lane = threadIdx.x & 31, jc = lane & 7, tgl = (threadIdx.x >> 5) * 4 + (lane >> 3);
+    uint32_t nibs = 0, rnd[4];
+#pragma unroll 1
+    for (int e = 0; e < 8; ++e) {
+        const uint64_t g = g0 + e;
+        philox4x32_10(static_cast<uint32_t>(g >> 2), static_cast<uint32_t>(g >> 34), tensor_id, step, key0, key1, rnd);
+        const uint32_t r01 = (g & 1u) ? rnd[1] : rnd[0], r23 = (g & 1u) ? rnd[3] : rnd[2], k = (g & 2u) ? r23 : r01;
+        uint32_t a[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) a[i] = reinterpret_cast<const uint16_t *>(src + i * row_chunks)[e];
+        const MvueGroup r = mvue_group(a[0] | (a[1] << 16), a[2] | (a[3] << 16), __uint2float_rn(k >> 8) * 0x1p-24f);
+        nibs |= (r.q0 | (r.q1 << 2)) << (4 * e);
+        const int jl = jc * 8 + e;
+        if (FP8) {
+            reinterpret_cast<uint16_t *>(vals_s)[jl * 32 + (tgl ^ (8 * (jc & 3)))] = static_cast<uint16_t>(__nv_cvt_float2_to_fp8x2(
+                make_float2(__fmul_rn(r.v0, gscale), __fmul_rn(r.v1, gscale)), __NV_SATFINITE, __NV_E5M2));
+            if (dense_q) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    reinterpret_cast<uint8_t *>(dense_q + i * row_chunks)[e] =
+                        static_cast<uint8_t>(sste_f32_to_e5m2(__fmul_rn(sste_bf16_bits_to_f32(a[i]), gscale)));
+            }
+        } else {
+            const __nv_bfloat162 pair = __floats2bfloat162_rn(r.v0, r.v1);
+            vals_s[jl * 32 + (tgl ^ (4 * (jc & 7)))] = *reinterpret_cast<const uint32_t *>(&pair);
+        }
+    }
+    mvue_put_meta<FP8>(nibs, jc, tgl, meta_s);
 }
 
 // The group rule on explicit inputs (test / debug): group i = four bf16 values a[4 i .. 4 i + 3] and the uniform
@@ -562,7 +667,14 @@ mvue_groups_kernel(const uint2 *__restrict__ a, const uint32_t *__restrict__ k24
         const uint32_t w[4] = {__byte_perm(g.x, g.y, 0x7610), __byte_perm(g.x, g.y, 0x5432), __byte_perm(g.y, g.x, 0x7610),
                                __byte_perm(g.y, g.x, 0x5432)};
         const MvuePair r = mvue_pair(w, k, ~k, reinterpret_cast<const uint8_t *>(lut));
-        float h, other;
+        float h, sum, other;
+        unpack2(r.sum, sum, other);
+        if (!(sum < INFINITY)) {
+            const MvueGroup any = mvue_group(g.x, g.y, __uint2float_rn(k >> 8) * 0x1p-24f);
+            pos[i] = any.q0 | (any.q1 << 2);
+            val[i] = make_float2(any.v0, any.v1);
+            continue;
+        }
         unpack2(r.h, h, other);
         const uint32_t kept = prmt(g.x, g.y, r.e0.x), mask = r.e0.y;
         pos[i] = (r.e0.x >> 16) & 0xfu;
@@ -672,6 +784,7 @@ mvue_kernel(const uint4 *__restrict__ dY, int O, int T, uint32_t key0, uint32_t 
     const float gscale = FP8 ? sste_scale_from_amax(amax_take(g_amax, jb == 0 && tb == 0 && tid == 0), 57344.0f) : 1.0f;
     __syncthreads();                              // the table is in place
     const size_t row_chunks = static_cast<size_t>(O) / 8;
+    bool plain = !FP8 || gscale < INFINITY;              // every sum of a group's magnitudes is finite
 
     {
         const int jc = lane & 7;                         // column chunk 0..7
@@ -708,6 +821,7 @@ mvue_kernel(const uint4 *__restrict__ dY, int O, int T, uint32_t key0, uint32_t 
                                     {in[2].x, in[2].y, in[2].z, in[2].w},
                                     {in[3].x, in[3].y, in[3].z, in[3].w}};
         uint32_t ex[8];                                 // first table word of every group: its nibble in byte 2
+        f32x2 sums;
 #pragma unroll
         for (int c = 0; c < 4; ++c) {                   // columns 2c, 2c + 1: one word of each token row
             if (!ANY_COUNTER && c % 2 == 0)             // drawn when needed: fewer registers live
@@ -717,6 +831,13 @@ mvue_kernel(const uint4 *__restrict__ dY, int O, int T, uint32_t key0, uint32_t 
             const MvuePair g = mvue_pair(w, rnd[2 * c], rnd[2 * c + 1], reinterpret_cast<const uint8_t *>(lut));
             ex[2 * c] = g.e0.x;
             ex[2 * c + 1] = g.e1.x;
+            if (FP8) {                                  // (no registers to spare for a running sum)
+                float sum0, sum1;
+                unpack2(g.sum, sum0, sum1);
+                plain = plain && sum0 + sum1 < INFINITY;
+            } else {
+                sums = c == 0 ? g.sum : add2(sums, g.sum);
+            }
             float h[2], mx[2];
             unpack2(FP8 ? mul2(g.h, both(gscale)) : g.h, h[0], h[1]);
             if (FP8) unpack2(mul2(g.mx, both(gscale)), mx[0], mx[1]);
@@ -764,24 +885,23 @@ mvue_kernel(const uint4 *__restrict__ dY, int O, int T, uint32_t key0, uint32_t 
         // nibbles of the even columns in the low halves of the bytes, of the odd ones in the high halves
         const uint32_t ev = __byte_perm(__byte_perm(ex[0], ex[2], 0x0062), __byte_perm(ex[4], ex[6], 0x0062), 0x5410);
         const uint32_t od = __byte_perm(__byte_perm(ex[1], ex[3], 0x0062), __byte_perm(ex[5], ex[7], 0x0062), 0x5410);
-        const uint32_t nibs = ev | (od << 4);
-        // two token groups share a metadata byte: lane ^ 8 holds the neighbouring token group
-        const uint32_t other = __shfl_xor_sync(0xffffffffu, nibs, 8);
-        if ((tgl & 1) == 0) {
-            const uint32_t k = 4u * tgl;
-            // the eight bytes (own nibble | neighbour's nibble << 4) of columns e = 0..7, four at a time:
-            // even columns from the low nibbles of each byte of `nibs`, odd columns from the high ones
-            const uint32_t even = (nibs & 0x0f0f0f0fu) | ((other << 4) & 0xf0f0f0f0u);
-            const uint32_t odd = ((nibs >> 4) & 0x0f0f0f0fu) | (other & 0xf0f0f0f0u);
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const uint32_t jl = jc * 8 + e;
-                const uint32_t byte = ((e & 1) ? odd : even) >> (8 * (e >> 1));
-                meta_s[FP8 ? sste_meta_atom_byte8(jl, k) : sste_meta_atom_byte16(jl, k)] = static_cast<uint8_t>(byte);
-            }
+        mvue_put_meta<FP8>(ev | (od << 4), jc, tgl, meta_s);
+        if (!FP8) {
+            float sum0, sum1;
+            unpack2(sums, sum0, sum1);
+            plain = sum0 + sum1 < INFINITY;
         }
     }
-    __syncthreads();
+    // A group of this block whose sum is not finite (or, FP8, a scale that is not): all of them again, by the rule for any values.
+    if (!__syncthreads_and(plain)) {
+        const size_t at = (static_cast<size_t>(tb) * 128 + warp * 16 + (lane >> 3) * 4) * row_chunks + jb * 8 + (lane & 7);
+        mvue_any_values<FP8>((PADDED ? padded : dY) + at, row_chunks,
+                             (tg_offset + static_cast<uint64_t>(tb) * 32 + warp * 4 + (lane >> 3)) * static_cast<uint64_t>(counter_cols) +
+                                 static_cast<uint64_t>(jb) * 64 + (lane & 7) * 8,
+                             tensor_id, step, key0, key1, gscale, vals_s, meta_s,
+                             FP8 && dense_q ? reinterpret_cast<uint2 *>(dense_q) + at : nullptr);
+        __syncthreads();
+    }
     // rows of the transposed tile: bf16 128 B (8 vectors of 16 B), fp8 64 B (4 vectors)
     constexpr int VECS = FP8 ? 4 : 8;
     const size_t out_row_vecs = static_cast<size_t>(T) / (FP8 ? 32 : 16);   // 16-byte vectors per output row
