@@ -93,8 +93,9 @@ struct SoftGroup {
 // subtraction a - copysign(t, a), and the kept pair is the top two of four integer keys
 // (magnitude << 2 | 3 - index: magnitude descending, index ascending; pairwise distinct) found with a
 // seven-operation min/max network.
-// MODE 1: interpolated threshold t = (1 - gamma) |t2| + gamma |t3| (Sec. 4.1); MODE 2: hard thresholding (Eq. 2), the kept
-// pair unchanged.  (MODE 0, the method's own projection, is project_group.)
+// MODE 0: the method's projection of a group with values that are not finite (project_group takes the others); MODE 1:
+// interpolated threshold t = (1 - gamma) |t2| + gamma |t3| (Sec. 4.1); MODE 2: hard thresholding (Eq. 2), the kept pair
+// unchanged.
 template <bool FP8, int MODE>
 __device__ __forceinline__ SoftGroup soft_group(uint32_t w01, uint32_t w23, float beta, float wscale, float gamma)
 {
@@ -205,6 +206,68 @@ __device__ __forceinline__ Projected project_group(uint32_t w01, uint32_t w23, f
 
 // ---------------------------------------------------------------- project + compress
 
+// The two groups of eight consecutive features after the projection: kept values packed (bf16: 32 bits, FP8: 16 bits per group),
+// all values packed (bf16: two words, FP8: word 0 per group), the metadata byte.
+struct ProjectedChunk { uint32_t kept[2], dn[2][2], mbyte; };
+
+// By rank on integer keys (soft_group), whatever the values.
+template <bool FP8, int MODE>
+__device__ __forceinline__ ProjectedChunk project_by_keys(const uint4 &in, float beta, float wscale, float gamma)
+{
+    const uint32_t raw[4] = {in.x, in.y, in.z, in.w};
+    ProjectedChunk o;
+    o.mbyte = 0;
+#pragma unroll
+    for (int g = 0; g < 2; ++g) {
+        const SoftGroup s = soft_group<FP8, MODE>(raw[2 * g], raw[2 * g + 1], beta, wscale, gamma);
+        if (FP8) {
+            const uint32_t e01 = __nv_cvt_float2_to_fp8x2(make_float2(s.w[0], s.w[1]), __NV_SATFINITE, __NV_E4M3);
+            const uint32_t e23 = __nv_cvt_float2_to_fp8x2(make_float2(s.w[2], s.w[3]), __NV_SATFINITE, __NV_E4M3);
+            o.dn[g][0] = e01 | (e23 << 16);
+            o.kept[g] = __byte_perm(o.dn[g][0], 0, s.p0 | (s.p1 << 4) | 0x4400u);
+        } else {
+            const __nv_bfloat162 d01 = __floats2bfloat162_rn(s.w[0], s.w[1]);
+            const __nv_bfloat162 d23 = __floats2bfloat162_rn(s.w[2], s.w[3]);
+            o.dn[g][0] = *reinterpret_cast<const uint32_t *>(&d01);
+            o.dn[g][1] = *reinterpret_cast<const uint32_t *>(&d23);
+            // halfword p0 -> low half, halfword p1 -> high half
+            o.kept[g] = __byte_perm(o.dn[g][0], o.dn[g][1], 0x1010u + 0x22u * s.p0 + 0x2200u * s.p1);
+        }
+        o.mbyte |= (s.p0 | (s.p1 << 2)) << (4 * g);
+    }
+    return o;
+}
+
+// Chunk c (of PC_ROWS x 16) of CTA (kb, rb) to where it belongs.
+template <bool FP8>
+__device__ __forceinline__ void put_chunk(const ProjectedChunk &o, int c, int kb, int rb, size_t row_chunks, void *vals,
+                                          uint8_t *meta_s, void *dense)
+{
+    const int row = c >> 4, kc = c & 15;
+    const uint32_t k = 8u * kc;
+    const uint32_t arow = (rb & 3) * PC_ROWS + row;   // row inside the 128-row atom
+    meta_s[(FP8 ? sste_meta_atom_byte8(arow, k) : sste_meta_atom_byte16(arow, k)) - 512u * (rb & 3)] = static_cast<uint8_t>(o.mbyte);
+    const size_t chunk = (static_cast<size_t>(rb) * PC_ROWS + row) * row_chunks + kb * 16 + kc;   // in units of 8 input features
+    if (FP8) {
+        reinterpret_cast<uint32_t *>(vals)[chunk] = o.kept[0] | (o.kept[1] << 16);
+        if (dense) reinterpret_cast<uint2 *>(dense)[chunk] = make_uint2(o.dn[0][0], o.dn[1][0]);
+    } else {
+        reinterpret_cast<uint2 *>(vals)[chunk] = make_uint2(o.kept[0], o.kept[1]);
+        if (dense) reinterpret_cast<uint4 *>(dense)[chunk] = make_uint4(o.dn[0][0], o.dn[0][1], o.dn[1][0], o.dn[1][1]);
+    }
+}
+
+// A CTA's groups once more, by keys (the method's projection of values that are not all finite; all threads).
+template <bool FP8>
+__device__ __noinline__ void project_any_values(const uint4 *W, size_t row_chunks, float beta, float wscale, void *vals,
+                                                uint8_t *meta_s, void *dense)
+{
+    for (int c = threadIdx.x; c < PC_ROWS * 16; c += EW_THREADS) {
+        const uint4 in = W[(static_cast<size_t>(blockIdx.y) * PC_ROWS + (c >> 4)) * row_chunks + blockIdx.x * 16 + (c & 15)];
+        put_chunk<FP8>(project_by_keys<FP8, 0>(in, beta, wscale, 0.0f), c, blockIdx.x, blockIdx.y, row_chunks, vals, meta_s, dense);
+    }
+}
+
 // One CTA: 32 rows x 128 input features of W (a quarter of a metadata atom, 512 contiguous bytes of its
 // image); a thread handles two chunks of 8 consecutive features.  Small tiles keep even the 2.4 M-element
 // GPT-2 weights spread over several CTAs per SM.
@@ -234,19 +297,22 @@ project_compress_kernel(const uint4 *__restrict__ W, int I, const float *__restr
     }
     if (MODE == 0) __syncthreads();              // the table is in place
     const f32x2 beta2 = both(beta), wscale2 = both(wscale);
+    // An infinity or a NaN in a group or in a scale makes the sum of its values one (so may huge values, which only costs
+    // time): the table's order of magnitudes is for numbers, and inf - inf is not the 0 of |a| = t.  Nor is a product with
+    // beta = 0 (-0 for a negative value, which the fma's + 0 loses).
+    bool plain = beta != 0.0f;
 #pragma unroll
     for (int i = 0; i < PC_CHUNKS; ++i) {
-        const int c = i * EW_THREADS + tid;
-        const int row = c >> 4, kc = c & 15;
-        const uint32_t raw[4] = {in[i].x, in[i].y, in[i].z, in[i].w};
-        uint32_t kept[2];      // per group: the two kept values, packed (bf16: 32 bits, fp8: 16 bits)
-        uint32_t dn[2][2];     // per group: the four projected values, packed (bf16: two words, fp8: word 0)
-        uint32_t mbyte = 0;
+        ProjectedChunk o;
+        if (MODE == 0) {
+            const uint32_t raw[4] = {in[i].x, in[i].y, in[i].z, in[i].w};
+            f32x2 sum;
+            o.mbyte = 0;
 #pragma unroll
-        for (int g = 0; g < 2; ++g) {
-            if (MODE == 0) {
+            for (int g = 0; g < 2; ++g) {
                 const Projected s = project_group<FP8>(raw[2 * g], raw[2 * g + 1], beta2, wscale2, reinterpret_cast<const uint8_t *>(lut));
                 const uint32_t nib = (s.e.x >> 16) & 0xfu;
+                sum = g == 0 ? add2(s.v01, s.v23) : add2(sum, add2(s.v01, s.v23));
                 float v[4];
                 unpack2(s.v01, v[0], v[1]);
                 unpack2(s.v23, v[2], v[3]);
@@ -255,49 +321,31 @@ project_compress_kernel(const uint4 *__restrict__ W, int I, const float *__restr
                     const uint32_t e01 = __nv_cvt_float2_to_fp8x2(make_float2(v[0], v[1]), __NV_SATFINITE, __NV_E4M3);
                     const uint32_t e23 = __nv_cvt_float2_to_fp8x2(make_float2(v[2], v[3]), __NV_SATFINITE, __NV_E4M3);
                     const uint32_t all = prmt(e01, e23, 0x5410);
-                    dn[g][0] = all & prmt(s.e.y, 0, 0xba98);
-                    kept[g] = prmt(all, 0, 0x4400u | (nib & 3u) | ((nib & 12u) << 2));
+                    o.dn[g][0] = all & prmt(s.e.y, 0, 0xba98);
+                    o.kept[g] = prmt(all, 0, 0x4400u | (nib & 3u) | ((nib & 12u) << 2));
                 } else {
                     const __nv_bfloat162 d01 = __floats2bfloat162_rn(v[0], v[1]), d23 = __floats2bfloat162_rn(v[2], v[3]);
                     const uint32_t w01 = *reinterpret_cast<const uint32_t *>(&d01), w23 = *reinterpret_cast<const uint32_t *>(&d23);
-                    dn[g][0] = w01 & prmt(s.e.y, 0, 0x9988);
-                    dn[g][1] = w23 & prmt(s.e.y, 0, 0xbbaa);
-                    kept[g] = prmt(w01, w23, s.e.x);
+                    o.dn[g][0] = w01 & prmt(s.e.y, 0, 0x9988);
+                    o.dn[g][1] = w23 & prmt(s.e.y, 0, 0xbbaa);
+                    o.kept[g] = prmt(w01, w23, s.e.x);
                 }
-                mbyte |= nib << (4 * g);
-                continue;
+                o.mbyte |= nib << (4 * g);
             }
-            const SoftGroup s = soft_group<FP8, MODE>(raw[2 * g], raw[2 * g + 1], beta, wscale, gamma);
-            if (FP8) {
-                const uint32_t e01 = __nv_cvt_float2_to_fp8x2(make_float2(s.w[0], s.w[1]), __NV_SATFINITE, __NV_E4M3);
-                const uint32_t e23 = __nv_cvt_float2_to_fp8x2(make_float2(s.w[2], s.w[3]), __NV_SATFINITE, __NV_E4M3);
-                dn[g][0] = e01 | (e23 << 16);
-                kept[g] = __byte_perm(dn[g][0], 0, s.p0 | (s.p1 << 4) | 0x4400u);
-            } else {
-                const __nv_bfloat162 d01 = __floats2bfloat162_rn(s.w[0], s.w[1]);
-                const __nv_bfloat162 d23 = __floats2bfloat162_rn(s.w[2], s.w[3]);
-                dn[g][0] = *reinterpret_cast<const uint32_t *>(&d01);
-                dn[g][1] = *reinterpret_cast<const uint32_t *>(&d23);
-                // halfword p0 -> low half, halfword p1 -> high half
-                kept[g] = __byte_perm(dn[g][0], dn[g][1], 0x1010u + 0x22u * s.p0 + 0x2200u * s.p1);
-            }
-            mbyte |= (s.p0 | (s.p1 << 2)) << (4 * g);
-        }
-        const uint32_t k = 8u * kc;
-        const uint32_t arow = (rb & 3) * PC_ROWS + row;   // row inside the 128-row atom
-        meta_s[(FP8 ? sste_meta_atom_byte8(arow, k) : sste_meta_atom_byte16(arow, k)) - 512u * (rb & 3)] =
-            static_cast<uint8_t>(mbyte);
-        const size_t grow = static_cast<size_t>(rb) * PC_ROWS + row;
-        const size_t chunk = grow * row_chunks + kb * 16 + kc;   // index in units of 8 input features
-        if (FP8) {
-            reinterpret_cast<uint32_t *>(vals)[chunk] = kept[0] | (kept[1] << 16);
-            if (dense) reinterpret_cast<uint2 *>(dense)[chunk] = make_uint2(dn[0][0], dn[1][0]);
+            float lo, hi;
+            unpack2(sum, lo, hi);
+            plain = plain && fabsf(lo + hi) < INFINITY;
         } else {
-            reinterpret_cast<uint2 *>(vals)[chunk] = make_uint2(kept[0], kept[1]);
-            if (dense) reinterpret_cast<uint4 *>(dense)[chunk] = make_uint4(dn[0][0], dn[0][1], dn[1][0], dn[1][1]);
+            o = project_by_keys<FP8, MODE>(in[i], beta, wscale, gamma);
         }
+        put_chunk<FP8>(o, i * EW_THREADS + tid, kb, rb, row_chunks, vals, meta_s, dense);
     }
-    __syncthreads();
+    if (MODE != 0) {
+        __syncthreads();
+    } else if (!__syncthreads_and(plain)) {
+        project_any_values<FP8>(W, row_chunks, beta, wscale, vals, meta_s, dense);
+        __syncthreads();
+    }
     if (tid < 32) {
         const size_t atom = static_cast<size_t>(rb >> 2) * (I / 128) + kb;
         reinterpret_cast<uint4 *>(meta + atom * 2048 + 512 * (rb & 3))[tid] = reinterpret_cast<const uint4 *>(meta_s)[tid];

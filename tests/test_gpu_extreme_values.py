@@ -152,3 +152,38 @@ def _uniforms(seed, tid, step, g):
     for i in range(first, last + 1):
         words[i - first] = orc.philox4x32_10((i & 0xffffffff, i >> 32, tid, step), (seed & 0xffffffff, seed >> 32))
     return (words[(block - np.uint64(first)).astype(np.int64), (g & np.uint64(3)).astype(np.int64)] >> 8).astype(np.float32)
+
+
+def projection_rule(a, beta, s):
+    """Kept positions and the four values of groups a [n, 4] (bf16 values): rank by magnitude bits, t the second-smallest."""
+    key = (a.view(np.uint32) & np.uint32(0x7fffffff)).astype(np.int64) * 4 + (3 - np.arange(4))
+    order = np.argsort(-key, axis=1)
+    p = np.sort(order[:, :2], axis=1)
+    with np.errstate(all="ignore"):
+        t = np.abs(a[np.arange(len(a)), order[:, 2]])[:, None]
+        v = (a - np.copysign(t, a)) * np.float32(beta) * np.float32(s)
+        v = np.where(np.abs(a) > t, v, np.float32(0))
+    return p, v.astype(np.float32)
+
+
+@pytest.mark.parametrize("beta", [1.5, 0.0, np.inf, np.nan])
+@pytest.mark.parametrize("fp8", [False, True])
+def test_projection(ctx, fp8, beta):
+    a = np.zeros((128 * 768 // 4, 4), np.float32)
+    a[: len(_groups())] = _groups()
+    W = synth.to_bf16_bits(a.reshape(128, 768))
+    a = synth.bf16_bits_to_f32(W).reshape(-1, 4)
+    dt = B.E4M3 if fp8 else B.BF16
+    for amax in ((1.0, 2.0 ** 127, 2.0 ** -140, np.inf, np.nan) if fp8 else (None,)):
+        vals, meta = ctx.alloc_compressed(128, 768, dt)
+        dense = torch.empty((128, 768), dtype=B._TORCH_DT[dt], device=DEV)
+        f32 = lambda x: torch.tensor([x], dtype=torch.float32, device=DEV)
+        ctx.project_compress(dbf16(W), f32(beta), vals, meta, dense, w_amax_dev=f32(amax) if fp8 else None)
+        with np.errstate(all="ignore"):
+            p, v = projection_rule(a, beta, np.float32(448) / np.float32(amax) if fp8 else 1.0)
+        code, nan, bits = ((lambda x: orc.f32_to_fp8(x, orc.E4M3), _nan_e4m3, bits8) if fp8 else (orc.f32_to_bf16, _nan16, bits16))
+        assert _equal(bits(dense), code(v).reshape(128, 768), nan)
+        assert _equal(bits(vals), code(np.take_along_axis(v, p, 1)).reshape(128, 384), nan)
+        nib = (p[:, 0] | (p[:, 1] << 2)).reshape(128, 48, 4).astype(np.uint16)
+        want = nib[..., 0] | (nib[..., 1] << 4) | (nib[..., 2] << 8) | (nib[..., 3] << 12)
+        assert np.array_equal(canonical_meta(ctx, meta, 128, 768, dt), want)
