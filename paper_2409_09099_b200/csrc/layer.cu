@@ -1,6 +1,8 @@
 // One call per phase of a layer's iteration (prune, forward, backward): the calls of the path in order, on the buffers of an
 // sste_layer.  A caller in an interpreted language pays for one call instead of two to four, each with a dozen arguments
 // to convert: on a 256 x 256 layer that conversion, not the GPU, set the pace.
+#include <initializer_list>
+
 #include "common.cuh"
 
 namespace {
@@ -14,6 +16,41 @@ bool layer_ok(const sste_layer *l)
     return !fp8_of(l) || (l->amax && l->Xq && l->dYq && l->scratch);
 }
 
+// What the kernels of a phase ask of the layer, looked at before the first of them is launched: sizes, and the buffers that
+// they need.  (A prune does not look at T.)
+sste_status phase_ok(const sste_layer *l, int T, std::initializer_list<const void *> needed)
+{
+    for (const void *b : needed)
+        if (!b) return SSTE_ERR_INVALID_ARG;
+    if (!sste_mult128(l->O) || !sste_mult128(l->I) || !sste_mult128(T)) return SSTE_ERR_SHAPE;
+    for (const void *b : needed)
+        if (!sste_aligned(b, 128)) return SSTE_ERR_ALIGN;
+    return fp8_of(l) && (!sste_aligned(l->amax, 4) || !sste_aligned(l->scratch, 8)) ? SSTE_ERR_ALIGN : SSTE_OK;
+}
+bool out_dtype_ok(const sste_layer *l) { return l->out_dtype == SSTE_BF16 || l->out_dtype == SSTE_F32; }
+
+sste_status forward_ok(const sste_layer *l, const void *X)
+{
+    if (!out_dtype_ok(l)) return SSTE_ERR_DTYPE;
+    if (fp8_of(l) && !sste_aligned(X, 16)) return SSTE_ERR_ALIGN;      // read by the amax and quantising passes only
+    return phase_ok(l, l->T, {l->vals, l->meta, l->Y, fp8_of(l) ? l->Xq : X});
+}
+sste_status grads_ok(const sste_layer *l, const void *X, const void *dY)
+{
+    if (!out_dtype_ok(l)) return SSTE_ERR_DTYPE;
+    const bool fp8 = fp8_of(l);
+    const void *v = l->w_dense ? l->w_dense : l->vals, *m = l->w_dense ? l->w_dense : l->meta;
+    return phase_ok(l, l->T, {l->gvals, l->gmeta, fp8 ? l->Xq : X, fp8 ? l->dYq : dY, v, m, l->dW, l->dX});
+}
+sste_status backward_ok(const sste_layer *l, const void *X, const void *dY, uint64_t token_offset)
+{
+    const sste_status st = grads_ok(l, X, dY);
+    if (st != SSTE_OK) return st;
+    if (l->counter_cols < 0 || l->counter_cols > l->O) return SSTE_ERR_INVALID_ARG;
+    if (token_offset % 4 != 0) return SSTE_ERR_SHAPE;
+    return sste_aligned(dY, 128) ? SSTE_OK : SSTE_ERR_ALIGN;
+}
+
 // The status of the product that should have emptied the layer's scratch; if a call was refused, a memset does.
 sste_status emptied(const sste_layer *l, sste_status st, void *stream)
 {
@@ -25,7 +62,9 @@ sste_status emptied(const sste_layer *l, sste_status st, void *stream)
 
 extern "C" sste_status sste_layer_prune(sste_ctx *ctx, const sste_layer *l, void *stream)
 {
-    if (!ctx || !layer_ok(l)) return SSTE_ERR_INVALID_ARG;
+    if (!ctx || !layer_ok(l) || !l->beta) return SSTE_ERR_INVALID_ARG;
+    const sste_status ok = phase_ok(l, 128, {l->W, l->vals, l->meta, l->w_dense ? l->w_dense : l->vals});
+    if (ok != SSTE_OK) return ok;
     if (!fp8_of(l))
         return sste_project_compress(ctx, l->W, l->O, l->I, SSTE_BF16, l->beta, nullptr, SSTE_BF16, l->vals, l->meta, l->w_dense,
                                      stream);
@@ -38,6 +77,8 @@ extern "C" sste_status sste_layer_prune(sste_ctx *ctx, const sste_layer *l, void
 extern "C" sste_status sste_layer_forward(sste_ctx *ctx, const sste_layer *l, const void *X, float *y_amax_out_dev, void *stream)
 {
     if (!ctx || !layer_ok(l) || !X) return SSTE_ERR_INVALID_ARG;
+    const sste_status ok = forward_ok(l, X);
+    if (ok != SSTE_OK) return ok;
     float *x_amax = nullptr, *w_amax = nullptr;
     if (fp8_of(l)) {
         x_amax = l->amax;
@@ -62,7 +103,8 @@ extern "C" sste_status sste_layer_backward(sste_ctx *ctx, const sste_layer *l, c
                                            uint64_t token_offset, void *stream)
 {
     if (!ctx || !layer_ok(l) || !dY) return SSTE_ERR_INVALID_ARG;
-    sste_status st;
+    sste_status st = backward_ok(l, X, dY, token_offset);
+    if (st != SSTE_OK) return st;
     if (fp8_of(l)) {
         float *g_amax = l->amax + 2;
         st = sste_amax_scratch(ctx, dY, static_cast<size_t>(l->T) * l->O, g_amax, l->scratch, stream);
@@ -86,6 +128,8 @@ extern "C" sste_status sste_layer_backward(sste_ctx *ctx, const sste_layer *l, c
 extern "C" sste_status sste_layer_grads(sste_ctx *ctx, const sste_layer *l, const void *X, const void *dY, void *stream)
 {
     if (!ctx || !layer_ok(l) || !dY) return SSTE_ERR_INVALID_ARG;
+    const sste_status ok = grads_ok(l, X, dY);
+    if (ok != SSTE_OK) return ok;
     const bool fp8 = fp8_of(l);
     return sste_bwd_products(ctx, l->gvals, l->gmeta, fp8 ? l->Xq : X, fp8 ? l->dYq : dY, l->O, l->I, l->T,
                              fp8 ? SSTE_E5M2 : SSTE_BF16, static_cast<sste_dtype>(l->op_dtype), l->w_dense, l->vals, l->meta,
@@ -107,7 +151,9 @@ extern "C" sste_status sste_padded_forward(sste_ctx *ctx, const sste_padded_laye
 {
     if (!ctx || !padded_ok(l) || !X) return SSTE_ERR_INVALID_ARG;
     const sste_layer &in = l->inner;
-    sste_status st = sste_pad_2d(ctx, X, l->T, l->I, l->Xp, in.T, in.I, stream);
+    sste_status st = forward_ok(&in, l->Xp);
+    if (st == SSTE_OK && (!sste_aligned(X, 2) || !sste_aligned(l->Y, 2))) st = SSTE_ERR_ALIGN;
+    if (st == SSTE_OK) st = sste_pad_2d(ctx, X, l->T, l->I, l->Xp, in.T, in.I, stream);
     if (st == SSTE_OK) st = sste_layer_forward(ctx, &in, l->Xp, nullptr, stream);
     if (st == SSTE_OK && l->Y) st = sste_crop_2d(ctx, in.Y, in.T, in.O, l->Y, l->T, l->O, stream);
     return st;
@@ -118,7 +164,9 @@ extern "C" sste_status sste_padded_backward(sste_ctx *ctx, const sste_padded_lay
 {
     if (!ctx || !padded_ok(l) || !dY) return SSTE_ERR_INVALID_ARG;
     const sste_layer &in = l->inner;
-    sste_status st;
+    sste_status st = backward_ok(&in, l->Xp, l->dYp, token_offset);
+    if (st == SSTE_OK && (!sste_aligned(dY, 2) || !sste_aligned(l->dX, 2) || !sste_aligned(l->dW, 2))) st = SSTE_ERR_ALIGN;
+    if (st != SSTE_OK) return st;
     if (fp8_of(&in)) {       // the quantisation needs max|dY| before the sparsification reads it
         st = sste_pad_2d(ctx, dY, l->T, l->O, l->dYp, in.T, in.O, stream);
         if (st == SSTE_OK) st = sste_layer_backward(ctx, &in, l->Xp, l->dYp, step, token_offset, stream);
