@@ -1627,6 +1627,19 @@ void *dense_copy_in_workspace(const sste_ctx *ctx, int O, int I, int elt, size_t
     return reinterpret_cast<char *>(ctx->splitk_partials) + at;
 }
 
+bool test_hook_set() { return g_inject_stall || g_force_bn || g_force_splits || g_force_group_m; }
+
+// The plan of both gradient products in one launch; whether that beats two in a row.  Two win where grad_X has few tiles of a
+// long reduction, and for large products, whose last wave costs little and whose tiles run 10 % slower beside the other
+// product's (1280 x 5120, 16384 tokens, bf16: 248 us apart, 260 us together; 3840 x 1280: 194 and 180).
+bool joint_wins(const sste_ctx *ctx, int elt, size_t partial_bytes, int O, int I, int T, JointPlan *plan)
+{
+    *plan = make_joint_plan(elt, ctx->sm_count, partial_bytes, O, I, T);
+    const double apart = make_plan(GRAD_WEIGHT, elt, 0, false, false, ctx->sm_count, partial_bytes, O, I, T).us +
+                         make_plan(GRAD_INPUT, elt, 0, false, false, ctx->sm_count, partial_bytes, T, I, O).us + LAUNCH_US;
+    return 1.1 * plan->us <= apart;
+}
+
 // FP8 operands come with the amax of the tensors they were quantised from (both or neither); bf16 with none.
 bool amax_args_ok(int elt, const float *a_amax, const float *b_amax)
 {
@@ -1818,6 +1831,15 @@ extern "C" sste_status sste_linear_bwd_input(sste_ctx *ctx, const void *dY, int 
     return launch_out<GRAD_INPUT, 1>(ctx, dY, Wt_dense, nullptr, p, xdt, s);
 }
 
+bool sste_bwd_in_one_launch(const sste_ctx *ctx, int elt, int O, int I, int T, bool dense_copy, sste_dtype odt)
+{
+    size_t partial_bytes = ctx->splitk_partials ? ctx->splitk_partial_bytes : 0;
+    if (odt != SSTE_BF16 || test_hook_set()) return false;
+    if (!dense_copy && !dense_copy_in_workspace(ctx, O, I, elt, &partial_bytes)) return false;
+    JointPlan plan;
+    return joint_wins(ctx, elt, partial_bytes, O, I, T, &plan);
+}
+
 sste_status sste_bwd_products(sste_ctx *ctx, const void *gvals, const void *gmeta, const void *X, const void *dY, int O, int I,
                               int T, sste_dtype gdt, sste_dtype wdt, const void *w_dense, const void *vals, const void *meta,
                               const float *g_amax, const float *x_amax, const float *w_amax, void *dW, void *dX,
@@ -1831,7 +1853,7 @@ sste_status sste_bwd_products(sste_ctx *ctx, const void *gvals, const void *gmet
     const bool given = ctx && gvals && gmeta && X && dY && dW && dX && (w_dense || (vals && meta)) &&
                        amax_args_ok(elt, g_amax, x_amax) && amax_args_ok(elt, g_amax, w_amax);
     // One launch for bf16 outputs; the test hooks, fp32 outputs and everything that the single calls refuse go there.
-    if (given && dims_ok && aligned && odt == SSTE_BF16 && !g_inject_stall && !g_force_bn && !g_force_splits && !g_force_group_m) {
+    if (given && dims_ok && aligned && odt == SSTE_BF16 && !test_hook_set()) {
         sste_device_guard guard(ctx->device);
         if (!guard.ok) return SSTE_ERR_CUDA;
         size_t partial_bytes = ctx->splitk_partials ? ctx->splitk_partial_bytes : 0;
@@ -1844,12 +1866,6 @@ sste_status sste_bwd_products(sste_ctx *ctx, const void *gvals, const void *gmet
             }
         }
         if (w) {
-            const JointPlan plan = make_joint_plan(elt, ctx->sm_count, partial_bytes, O, I, T);
-            // Two launches where they win: few grad_X tiles of a long reduction (it is not split here), and large products,
-            // whose last wave costs little and whose tiles run 10 % slower beside the other product's (1280 x 5120, 16384
-            // tokens, bf16: 248 us apart, 260 us together; 3840 x 1280: 194 and 180).
-            const double apart = make_plan(GRAD_WEIGHT, elt, 0, false, false, ctx->sm_count, partial_bytes, O, I, T).us +
-                                 make_plan(GRAD_INPUT, elt, 0, false, false, ctx->sm_count, partial_bytes, T, I, O).us + LAUNCH_US;
             uint32_t cg, cw;
             int unused;
             fmt_code(gdt, &unused, &cg);
@@ -1857,7 +1873,8 @@ sste_status sste_bwd_products(sste_ctx *ctx, const void *gvals, const void *gmet
             const GemmParams pw{O, I, T, dW, g_amax, x_amax, sste_fp8_max(gdt), sste_fp8_max(wdt), nullptr, ctx->status_dev, cg, cw, nullptr};
             const GemmParams px{T, I, O, dX, g_amax, w_amax, sste_fp8_max(gdt), sste_fp8_max(wdt), nullptr, ctx->status_dev, cg, cw, nullptr};
             cudaStream_t s = static_cast<cudaStream_t>(stream);
-            if (1.1 * plan.us <= apart) {
+            JointPlan plan;
+            if (joint_wins(ctx, elt, partial_bytes, O, I, T, &plan)) {
                 if (elt == 1) return launch_grads<1, 256, 256>(ctx, gvals, gmeta, X, dY, w, pw, px, plan, s);
                 if (plan.w.bn == 256) return launch_grads<2, 256, 256>(ctx, gvals, gmeta, X, dY, w, pw, px, plan, s);
                 if (plan.x.bn == 256) return launch_grads<2, 128, 256>(ctx, gvals, gmeta, X, dY, w, pw, px, plan, s);

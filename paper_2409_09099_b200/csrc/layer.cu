@@ -137,6 +137,13 @@ extern "C" sste_status sste_layer_grads(sste_ctx *ctx, const sste_layer *l, cons
                              static_cast<sste_dtype>(l->out_dtype), stream);
 }
 
+extern "C" int sste_layer_grads_joint(const sste_ctx *ctx, const sste_layer *l)
+{
+    if (!ctx || !layer_ok(l) || !sste_mult128(l->O) || !sste_mult128(l->I) || !sste_mult128(l->T)) return 0;
+    return sste_bwd_in_one_launch(ctx, fp8_of(l) ? 1 : 2, l->O, l->I, l->T, l->w_dense != nullptr,
+                                  static_cast<sste_dtype>(l->out_dtype));
+}
+
 namespace {
 
 bool padded_ok(const sste_padded_layer *l)

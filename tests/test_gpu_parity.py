@@ -283,28 +283,34 @@ def test_argument_validation_launches_nothing(ctx):
     assert ctx.poll_device_status() == 0
 
 
+# 768 x 3072, 2048 tokens: one launch for both products, the side stream where a `mark` wants to see the calls; the others: two
+# products side by side
+@pytest.mark.parametrize("O,I,T,marked", [(768, 3072, 2048, True), (2048, 2048, 2048, False), (4864, 1152, 640, False)])
 @pytest.mark.parametrize("fp8", [False, True])
-def test_overlapped_backward_equals_serial(ctx, fp8):
+def test_overlapped_backward_equals_serial(ctx, fp8, O, I, T, marked):
     """grad_W on a side stream (own context, own split-K workspace) beside grad_X gives the same bits as the
     two calls back to back, also when both products split their reduction."""
     from paper_2409_09099_b200 import binding as B
     from paper_2409_09099_b200.layer import SsteLinear
-    O, I, T = 768, 3072, 2048
     W = dbf16(synth.gaussian_bf16(71, (O, I), 0.02))
     X = dbf16(synth.gaussian_bf16(72, (T, I), 1.0))
     dY = dbf16(synth.gaussian_bf16(73, (T, O), 1e-2))
     side_ctx, side = B.Context(0), torch.cuda.Stream()
+    calls = []
+    plain = side_ctx.linear_bwd_weight
+    side_ctx.linear_bwd_weight = lambda *a, **kw: (calls.append(torch.cuda.current_stream()), plain(*a, **kw))
     try:
         lin = SsteLinear(ctx, W, T, tensor_id=1, seed=9, fp8=fp8)
         lin.init_beta(); lin.prune(); lin.forward(X)
-        lin.backward(dY, step=2)
-        torch.cuda.synchronize()
-        dW0, dX0 = lin.dW.clone(), lin.dX.clone()
+        lin.sparsify_grad(dY, 2)
+        dW0, dX0 = lin.grad_weight().clone(), lin.grad_input(dY).clone()
         lin.dW.zero_(); lin.dX.zero_()
+        lin.mark = (lambda label: None) if marked else None
         for _ in range(3):
             lin.sparsify_grad(dY, 2)
             lin.grad_weight_and_input(dY, side_ctx, side)
         torch.cuda.synchronize()
+        assert calls == [side] * 3
         assert torch.equal(lin.dW.view(torch.int16), dW0.view(torch.int16))
         assert torch.equal(lin.dX.view(torch.int16), dX0.view(torch.int16))
         assert side_ctx.poll_device_status() == 0
