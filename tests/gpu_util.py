@@ -27,3 +27,16 @@ def canonical_meta(ctx, meta, rows, k, dt):
     out = torch.empty((rows, k // 16), dtype=torch.int16, device=DEV)
     ctx.meta_to_canonical(meta, rows, k, dt, out)
     return out.cpu().numpy().view(np.uint16)
+
+
+def context_with_workspace(nbytes):
+    """A Context whose workspace has `nbytes` bytes."""
+    import ctypes
+
+    from paper_2409_09099_b200 import binding as B
+    c = B.Context(0, minimal_workspace=True)
+    workspace, handle = torch.zeros(nbytes, dtype=torch.uint8, device=DEV), ctypes.c_void_p()
+    c._check(c.lib.sste_create(ctypes.byref(handle), 0, ctypes.c_void_p(workspace.data_ptr()), ctypes.c_size_t(nbytes)))
+    c.lib.sste_destroy(c.handle)
+    c.handle, c.workspace = handle, workspace
+    return c
