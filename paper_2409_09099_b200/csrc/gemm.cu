@@ -1303,8 +1303,9 @@ struct PlanMemo {
 // takes 1/splits of a tile time and the exchange of the partials on top: 2.4 + 2.6 bn/256 us between two units,
 // 4.4 + 3.8 bn/256 between three and so on (measured at 9 ... 36 tiles), and their bytes.  Few tiles (all ranges run at once)
 // of a long reduction take many short ranges and a sum afterwards instead.  Among widths within 3 % the first wins.
+// (estimate: for the time of grad_X in joint_wins, whose line was drawn with these constants as they are.)
 LaunchPlan find_plan(Product pr, int elt, int only_bn, bool out_f32, bool bcomp, int sm_count, size_t partial_bytes, int M,
-                     int N, int K)
+                     int N, int K, bool estimate)
 {
     const bool sparse = (pr != GRAD_INPUT);
     const int bk = (sparse ? 256 : 128) / elt, k_blocks = (K + bk - 1) / bk, pairs = sm_count / 2;
@@ -1318,7 +1319,13 @@ LaunchPlan find_plan(Product pr, int elt, int only_bn, bool out_f32, bool bcomp,
         if (!bn || (forced && bn != forced)) continue;
         const int tiles = m_tiles * ((N + bn - 1) / bn);
         const int whole = tiles / pairs * pairs, tail = tiles - whole;
-        const TileCost c = tile_cost(pr, elt, bn);
+        TileCost c = tile_cost(pr, elt, bn);
+        // grad_X by itself, measured at 110 shapes with every width and split: a 128-wide stage costs more than beside grad_W
+        // (few tiles, each paced by its own loads), and an exchange between more than two units 2 us more.  With both the
+        // plan is within 0.6 % of the best on the mean and 10 % at worst, without 1.0 and 19 % (4864 x 1152, 640 tokens, bf16:
+        // 21.3 -> 17.8 us; 4096 x 1664, 3200: 40.6 -> 38.1).
+        const bool dense = pr == GRAD_INPUT && !estimate;
+        if (dense && bn == 128) c.stage_us = 0.30;
         const double whole_us = (whole / pairs) * (k_blocks * c.stage_us + c.tile_us);
         for (int s = 1; s <= MAX_SPLITS; ++s) {
             double us = whole_us;
@@ -1329,7 +1336,7 @@ LaunchPlan find_plan(Product pr, int elt, int only_bn, bool out_f32, bool bcomp,
                 if (tail * 2 * 8 * MAX_PARTS > SSTE_SPLITK_TICKETS) continue;
                 const size_t bytes = static_cast<size_t>(tail) * s * 2 * BM * bn * sizeof(float);
                 if (bytes > partial_bytes) continue;
-                us += exchange_us(s, bn, static_cast<double>(bytes));
+                us += exchange_us(s, bn, static_cast<double>(bytes)) + (dense && s > 2 ? 2.0 : 0.0);
             }
             if (tail) us += ((tail * s + pairs - 1) / pairs) * ((k_blocks + s - 1) / s * c.stage_us + c.tile_us);
             const bool wanted = (g_force_splits == s && best.bn == bn);      // the hook applies where the shape allows it
@@ -1351,14 +1358,14 @@ LaunchPlan find_plan(Product pr, int elt, int only_bn, bool out_f32, bool bcomp,
 }
 
 LaunchPlan make_plan(Product pr, int elt, int only_bn, bool out_f32, bool bcomp, int sm_count, size_t partial_bytes, int M,
-                     int N, int K)
+                     int N, int K, bool estimate = false)
 {
     if (g_force_splits || g_force_bn || g_force_group_m || g_inject_stall)
-        return find_plan(pr, elt, only_bn, out_f32, bcomp, sm_count, partial_bytes, M, N, K);
+        return find_plan(pr, elt, only_bn, out_f32, bcomp, sm_count, partial_bytes, M, N, K, estimate);
     static thread_local PlanMemo<LaunchPlan> memo;
-    const long long kind = (((pr * 4 + elt) * 2 + out_f32) * 2 + bcomp) * 1024 + only_bn;
+    const long long kind = ((((pr * 4 + elt) * 2 + out_f32) * 2 + bcomp) * 2 + estimate) * 1024 + only_bn;
     return memo.get({kind, sm_count, static_cast<long long>(partial_bytes), M, N, K},
-                    [&] { return find_plan(pr, elt, only_bn, out_f32, bcomp, sm_count, partial_bytes, M, N, K); });
+                    [&] { return find_plan(pr, elt, only_bn, out_f32, bcomp, sm_count, partial_bytes, M, N, K, estimate); });
 }
 
 // One launch for both gradient products (grads_kernel): the plans of the two and how the pairs share grad_X.
@@ -1636,7 +1643,7 @@ bool joint_wins(const sste_ctx *ctx, int elt, size_t partial_bytes, int O, int I
 {
     *plan = make_joint_plan(elt, ctx->sm_count, partial_bytes, O, I, T);
     const double apart = make_plan(GRAD_WEIGHT, elt, 0, false, false, ctx->sm_count, partial_bytes, O, I, T).us +
-                         make_plan(GRAD_INPUT, elt, 0, false, false, ctx->sm_count, partial_bytes, T, I, O).us + LAUNCH_US;
+                         make_plan(GRAD_INPUT, elt, 0, false, false, ctx->sm_count, partial_bytes, T, I, O, true).us + LAUNCH_US;
     return 1.1 * plan->us <= apart;
 }
 
