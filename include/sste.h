@@ -419,6 +419,8 @@ sste_status sste_debug_plan(int product, sste_dtype opdt, int O, int I, int T, i
  * others; the rounds of grad_X tiles that the others take among themselves first; whether they also come first in the
  * rounds after; grad_X's split factor (all tiles, summed afterwards); whether grad_W's partials are summed afterwards. */
 sste_status sste_debug_joint_plan(sste_dtype opdt, int O, int I, int T, int sm_count, size_t workspace_bytes, int out[12]);
+/* Searches for a plan so far in this process: launches of shapes that the thread's memory of plans does not hold. */
+unsigned long long sste_debug_plan_searches(void);
 sste_status sste_debug_tile_coords(int tile, int m_tiles, int n_tiles, int group_m, int *mt, int *nt);
 
 /* Host-only self-check of the once-per-device bookkeeping behind per-device kernel attributes (a context may live on

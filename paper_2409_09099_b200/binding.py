@@ -34,6 +34,7 @@ EXPORTS = [
     "sste_debug_force_tile_order", "sste_debug_plan", "sste_debug_tile_coords",
     "sste_debug_mvue_groups", "sste_debug_selftest_device_once", "sste_layer_prune", "sste_layer_forward",
     "sste_layer_backward", "sste_layer_grads", "sste_layer_grads_joint", "sste_debug_joint_plan",
+    "sste_debug_plan_searches",
     "sste_padded_forward", "sste_padded_backward",
 ]
 

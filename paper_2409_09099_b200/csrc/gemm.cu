@@ -20,6 +20,7 @@
 #include <cuda.h>
 
 #include <array>
+#include <atomic>
 #include <type_traits>
 
 #include "common.cuh"
@@ -1280,19 +1281,28 @@ int plan_group_m(Product pr, int elt, bool bcomp, int bn, int pairs, int M, int 
                         static_cast<double>(K) * ((bcomp ? 0.5 : 1.0) * elt) * bn);
 }
 
-// The plans of the last shapes of a thread: trying every width and split takes up to some 20 us of host time.
+// The plans of the last shapes of a thread: a search takes 0.4 us of host time for most products and 1.2 for most pairs of
+// gradients, but some 30 us for 16384 tokens through 11008 x 4096 and more with more tokens (it tries every number of early
+// rounds).  Sets of four: with one place per shape two products of a GPT-2-large block pushed each other out every step.
+std::atomic<unsigned long long> g_plan_searches{0};
 template <typename Plan>
 struct PlanMemo {
     typedef std::array<long long, 6> Key;
-    static constexpr int ENTRIES = 64;
-    struct Entry { Key key{}; Plan plan{}; bool set = false; } entry[ENTRIES];
+    static constexpr int SETS = 32, WAYS = 4;
+    struct Entry { Key key{}; Plan plan{}; bool set = false; };
+    struct Set { Entry entry[WAYS]; int oldest = 0; } sets[SETS];
     template <typename F>
     const Plan &get(const Key &key, F make)
     {
         unsigned long long h = 0;
         for (long long k : key) h = (h ^ static_cast<unsigned long long>(k)) * 0x9e3779b97f4a7c15ull;
-        Entry &e = entry[h >> 58];
-        if (!e.set || e.key != key) e = Entry{key, make(), true};
+        Set &set = sets[h >> 59];
+        for (const Entry &e : set.entry)
+            if (e.set && e.key == key) return e.plan;
+        g_plan_searches.fetch_add(1, std::memory_order_relaxed);
+        Entry &e = set.entry[set.oldest];
+        set.oldest = (set.oldest + 1) % WAYS;
+        e = Entry{key, make(), true};
         return e.plan;
     }
 };
@@ -1695,6 +1705,7 @@ extern "C" sste_status sste_debug_joint_plan(sste_dtype opdt, int O, int I, int 
     for (int i = 0; i < 12; ++i) out[i] = v[i];
     return SSTE_OK;
 }
+extern "C" unsigned long long sste_debug_plan_searches(void) { return g_plan_searches.load(std::memory_order_relaxed); }
 // Host-only self-check of the once-per-device guard the launches use for per-device kernel attributes: `fn` must
 // run once per device ordinal, again after a failure, and never for a device that already succeeded.
 extern "C" sste_status sste_debug_selftest_device_once(void)

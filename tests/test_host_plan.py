@@ -92,3 +92,24 @@ def test_grad_x_alone_at_shapes_where_the_model_was_wrong():
     """Measured best (us): 256 wide in four ranges 17.8 (128 wide in two: 21.3); two ranges of the last 17 tiles 38.1 (four: 40.6)."""
     assert B.plan(2, B.BF16, 4864, 1152, 640)[:3] == (256, 4, 0)
     assert B.plan(2, B.BF16, 4096, 1664, 3200)[:3] == (256, 2, 74)
+
+
+def test_plans_of_a_model_are_kept():
+    """Every product of a model's layers, step after step: no plan is searched for twice."""
+    lib = B.load()
+    lib.sste_debug_plan_searches.restype = ctypes.c_ulonglong
+    models = [[(3840, 1280), (1280, 1280), (5120, 1280), (1280, 5120)], [(2304, 768), (768, 768), (3072, 768), (768, 3072)],
+              [(11008, 4096), (4096, 11008)]]
+    for tokens in (8192, 16384):
+        for layers in models:
+            def step():
+                for O, I in layers:
+                    for dt in (B.BF16, B.E4M3):
+                        for product in (0, 1, 2):
+                            B.plan(product, dt, O, I, tokens)
+                        B.joint_plan(dt, O, I, tokens)
+            step()
+            before = lib.sste_debug_plan_searches()
+            for _ in range(3):
+                step()
+            assert lib.sste_debug_plan_searches() == before, layers
