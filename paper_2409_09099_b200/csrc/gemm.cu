@@ -478,10 +478,12 @@ product(const CUtensorMap &map_a, const CUtensorMap &map_b, const CUtensorMap &m
                     const uint32_t b_dst = a_dst + C::A_STAGE;
                     // A: 128 bytes per row = BK/2 compressed (sparse) or BK dense elements
                     tma_load_2d(a_dst, &map_a, lead_full, kb * (SPARSE ? BK / 2 : BK), m0);
-                    // metadata: the atoms of this K, 2 KB each, as rows of 512 bytes.  (With an odd number of atoms the
-                    // last 8-bit stage also fetches the first atom of the next row block: it meets zero-filled K.)
+                    // metadata: the atoms of this K, 2 KB each, as rows of 512 bytes.  Rows beyond M (zero-filled values) take the
+                    // codes of the last row block: zero is not one of the six codes.  (With an odd number of atoms the last
+                    // 8-bit stage also fetches what follows; the MMAs stop in front of it.)
                     if (SPARSE)
-                        tma_load_2d(b_dst + C::B_STAGE, &map_m, lead_full, 0, ((m0 / BM) * k_atoms + kb * C::ATOMS) * 4);
+                        tma_load_2d(b_dst + C::B_STAGE, &map_m, lead_full, 0,
+                                    (min(m0 / BM, p.M / BM - 1) * k_atoms + kb * C::ATOMS) * 4);
                     if (BCOMP) {
                         // B is written into the stage by the expander warps
                     } else if (BMAJ == BMajor::K) {
@@ -526,8 +528,11 @@ product(const CUtensorMap &map_a, const CUtensorMap &map_b, const CUtensorMap &m
                         for (int i = 0; i < C::ATOMS; ++i)
                             tc_cp_meta_atom(meta_cols + 4 * i, smem_desc(b_src + C::B_STAGE + 2048 * i, 128, 128, 0));
                     }
+                    // the last stage of an 8-bit sparse product with an odd number of atoms is half a stage
+                    const bool half = SPARSE && F8 && (kb + 1) * BK > p.K;
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
+                        if (half && j >= 2) break;
                         const uint64_t adesc = smem_desc(a_src + 32 * j, 16, 1024, 2);
                         uint64_t bdesc;
                         if (BMAJ == BMajor::K) {
