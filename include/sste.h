@@ -175,9 +175,10 @@ sste_status sste_mvue_sparsify(sste_ctx *ctx, const void *dY, int T, int O, sste
  * Sec. 5.1: grad_X = grad_Z S(W), a dense product (the 2:4 structure of S(W) lies along I, which
  * is not the reduction dimension here).  dY [T, O] of dtype gdt (SSTE_BF16 / SSTE_E5M2).  S(W) [O, I] of
  * dtype wdt (SSTE_BF16 / SSTE_E4M3) is given EITHER as the dense copy Wt_dense written by
- * sste_project_compress, OR (Wt_dense = NULL) as the forward's compressed operand (vals, meta): the kernel then
- * expands each K slice into the dense shared-memory operand itself (+0 in the pruned positions), the same
- * product bit for bit, and the dense copy need not exist.  dX [T, I] of dtype xdt = acc [* 1/s_g * 1/s_w for FP8
+ * sste_project_compress, OR (Wt_dense = NULL) as the forward's compressed operand (vals, meta), and the caller keeps
+ * no dense copy: the call expands it (+0 in the pruned positions) into the context's workspace where that has room for
+ * it beside 80 MB of partial sums, and else slice by slice inside the product (slower); the same sums of the same
+ * values either way.  dX [T, I] of dtype xdt = acc [* 1/s_g * 1/s_w for FP8
  * operands, from g_amax_dev / w_amax_dev; NULL for bf16].  dx_amax_out_dev: nullable, max|dX| as for the forward.
  */
 sste_status sste_linear_bwd_input(sste_ctx *ctx, const void *dY, int T, int O, sste_dtype gdt,
@@ -368,7 +369,7 @@ sste_status sste_pad_2d(sste_ctx *ctx, const void *src, int rows, int cols, void
 sste_status sste_crop_2d(sste_ctx *ctx, const void *src, int rows_p, int cols_p, void *dst, int rows, int cols,
                          void *stream);
 
-/* ---- test / debug helpers ---- */
+/* ---- inspection and test helpers ---- */
 
 /* Compressed operand (vals [rows, k/2] + metadata image) -> dense [rows, k] of the same dtype dt (SSTE_BF16,
  * SSTE_E4M3 or SSTE_E5M2), +0 in the pruned positions: the matrix the sparse tensor-core instruction sees. */

@@ -1112,7 +1112,7 @@ meta_to_canonical_kernel(const uint8_t *__restrict__ meta, int rows, int k, uint
     }
 }
 
-// ---------------------------------------------------------------- compressed operand -> dense (test / debug)
+// ---------------------------------------------------------------- compressed operand -> dense (grad_X of a layer without a dense copy)
 
 // One thread per 16 bytes of values: bf16 4 groups (16 dense elements), fp8 8 groups (32 dense elements).
 template <bool EIGHT_BIT>

@@ -4,7 +4,7 @@
 //   grad input   grad_X = grad_Z S(W)        dense A, MN-major B
 //
 // One persistent, warp-specialised kernel template run by CTA PAIRS (cluster of two,
-// tcgen05 cta_group::2).  A pair owns a 256 x 256 output tile: each CTA holds its own
+// tcgen05 cta_group::2).  A pair owns an output tile of 256 rows and 128 to 256 columns: each CTA holds its own
 // 128 rows of A and HALF of the B tile, so the B operand is streamed from shared memory
 // at half the rate per SM -- with one CTA per tile the sparse instruction is bound by that
 // stream and runs no faster than the dense one -- and L2 -> SM traffic per flop drops.
@@ -1651,8 +1651,7 @@ void *dense_copy_in_workspace(const sste_ctx *ctx, int O, int I, int elt, size_t
 
 bool test_hook_set() { return g_inject_stall || g_force_bn || g_force_splits || g_force_group_m; }
 
-// The plan of both gradient products in one launch; whether that beats two in a row.  Two win where grad_X has few tiles of a
-// long reduction, and for large products, whose last wave costs little and whose tiles run 10 % slower beside the other
+// The plan of both gradient products in one launch; whether that beats two in a row.  Two win for large products, whose last wave costs little and whose tiles run 10 % slower beside the other
 // product's (1280 x 5120, 16384 tokens, bf16: 248 us apart, 260 us together; 3840 x 1280: 194 and 180).
 bool joint_wins(const sste_ctx *ctx, int elt, size_t partial_bytes, int O, int I, int T, JointPlan *plan)
 {
@@ -1875,7 +1874,7 @@ sste_status sste_bwd_products(sste_ctx *ctx, const void *gvals, const void *gmet
                          sste_aligned(meta, 128) && sste_aligned(dX, 128);
     const bool given = ctx && gvals && gmeta && X && dY && dW && dX && (w_dense || (vals && meta)) &&
                        amax_args_ok(elt, g_amax, x_amax) && amax_args_ok(elt, g_amax, w_amax);
-    // One launch for bf16 outputs; the test hooks, fp32 outputs and everything that the single calls refuse go there.
+    // One launch for bf16 outputs where joint_wins says so; test hooks, fp32 outputs and whatever the single calls refuse go there.
     if (given && dims_ok && aligned && odt == SSTE_BF16 && !test_hook_set()) {
         sste_device_guard guard(ctx->device);
         if (!guard.ok) return SSTE_ERR_CUDA;

@@ -47,8 +47,8 @@ class SsteLinear:
     operands, E5M2 output gradient, per-tensor scale = fp8_max / amax; the state of a
     quantised tensor is its amax (one device float), from which every consumer forms the
     scale itself.  ``dense_copy=True`` (the default, the faster route on B200) also keeps w~ as a
-    dense [O, I] tensor and feeds grad_X from it; with ``dense_copy=False`` no dense w~ exists and
-    grad_X expands the compressed operand inside the product (same bits, less memory, slower).
+    dense [O, I] tensor and feeds grad_X from it; with ``dense_copy=False`` the layer keeps none and
+    grad_X expands the compressed operand for the length of the call (less memory, slower).
     ``track_flips=True`` keeps the previous iteration's metadata and counts the mask entries
     that changed at every prune (flip rate, Sec. 3.1).
     """

@@ -1,7 +1,9 @@
 """Few output tiles of a long reduction: K ranges on every CTA pair, their fp32 partials added by a second kernel.
 
-Against the fp64 product of the same operands.  Bound: a bf16 result is off by half an ulp (at most 2^-8 relative); the fp32 sums
-over K terms add at most K 2^-24 of the sum of |terms|.
+Against the fp64 product of the same operands.  Bound: a bf16 result is off by half an ulp (at most 2^-8 relative).  Each of the
+fp32 additions is off by at most 2^-23 of a partial sum (the adder truncates), itself about sqrt(K) of a term where signs are
+random; the sum of |terms| is about K of a term, so the errors add up to about 2^-23 of it: four times that.  (A dropped stage of
+64 terms at K = 8192 is some sqrt(64) / 8192 = 2^-10 of it.)
 """
 import gc
 
@@ -20,9 +22,9 @@ def give_memory_back():
     gc.collect()
 
 
-def _close(got, a, b, K):
+def _close(got, a, b):
     ref, mag = a.double() @ b.double(), a.double().abs() @ b.double().abs()
-    bound = ref.abs() * 2.0 ** -8 + mag * K * 2.0 ** -23 + 1e-30
+    bound = ref.abs() * 2.0 ** -8 + mag * 2.0 ** -21 + 1e-30
     assert bool(((got.double() - ref).abs() <= bound).all())
 
 
@@ -65,11 +67,11 @@ def test_products_and_layer(shape, fp8):
     ctx.decompress(lin.gvals, lin.gmeta, G)
     Gd = G.double() * inv[2]
     for y in (Y, Y1):
-        _close(y, xd, wd.T, I)
+        _close(y, xd, wd.T)
     for w in (dW, dW1):
-        _close(w, Gd, xd, T)
+        _close(w, Gd, xd)
     for x in (dX, dX1):
-        _close(x, gd, wd, O)
+        _close(x, gd, wd)
 
 
 def test_shapes_take_the_path():
@@ -93,5 +95,5 @@ def test_same_bits_every_time_and_without_workspace():
     Z = torch.empty_like(Y)
     small.linear_fwd(X, lin.vals, lin.meta, Z)
     wd = lin.w_dense.double()
-    _close(Y, X.double(), wd.T, 8192)
-    _close(Z, X.double(), wd.T, 8192)
+    _close(Y, X.double(), wd.T)
+    _close(Z, X.double(), wd.T)
