@@ -35,9 +35,27 @@ def _takes(t, shape):
     return t.dtype is _bf16 and t.shape == shape and t.is_cuda and t.is_contiguous()
 
 
+def _same_places(tensors):
+    """A check that the storage of `tensors` is where it is now.
+
+    Unrolled for the bf16 phases of a layer with a dense copy, where the host sets the pace (0.3 us for five tensors, 0.5 in a
+    loop)."""
+    calls, at = [t.data_ptr for t in tensors], [t.data_ptr() for t in tensors]
+    if len(calls) == 3:
+        (a, b, c), (p, q, r) = calls, at
+        return lambda: a() == p and b() == q and c() == r
+    if len(calls) == 5:
+        (a, b, c, d, e), (p, q, r, s, t) = calls, at
+        return lambda: a() == p and b() == q and c() == r and d() == s and e() == t
+    return lambda: [call() for call in calls] == at
+
+
 class _Described:
-    """sste_layer of a layer's buffers; per phase the C call, the tensors it works on and the addresses put down for them."""
-    __slots__ = ("fits", "buffers", "at", "x_shape", "g_shape", "w_shape", "prune", "forward", "backward", "grads")
+    """sste_layer of a layer's buffers; per phase the C call and the check that the buffers it works on are where they were.
+
+    A tensor may be given other storage without being replaced (`t.data = ...`, a storage resized to 0 and back)."""
+    __slots__ = ("fits", "buffers", "at", "x_shape", "g_shape", "w_shape", "prune", "prune_there", "forward", "forward_there",
+                 "backward", "backward_there", "grads")
 
 
 class SsteLinear:
@@ -102,7 +120,7 @@ class SsteLinear:
         desc.fits = (_as_defined(self, SsteLinear, _LAYER_CALLS) and _as_defined(self.ctx, B.Context, _CONTEXT_CALLS)
                      and (self._as_made or self._replaced_fit(x_shape, g_shape, tensors)))
         if not desc.fits:
-            desc.prune = desc.forward = desc.backward = desc.grads = (None, (), [])
+            desc.prune_there = desc.forward_there = desc.backward_there = lambda: True
             return desc
         d = B.LayerBuffers(self.O, self.I, self.T, B.E4M3 if self.fp8 else B.BF16, B._CODE_OF[self.Y.dtype],
                            self.counter_cols, index(self.tensor_id) & 0xffffffff, 0, index(self.seed) & 0xffffffffffffffff,
@@ -111,26 +129,18 @@ class SsteLinear:
         desc.buffers, desc.at, desc.x_shape, desc.g_shape = d, ctypes.addressof(d), x_shape, g_shape
         desc.w_shape = torch.Size((self.O, self.I))
         w = (self.vals, self.meta) if self.w_dense is None else (self.w_dense,)
-        for name, call, read in (
-                ("prune", lib.sste_layer_prune, (self.W, self.beta, self.vals, self.meta, self.w_dense, self.amax, self._scratch)),
-                ("forward", lib.sste_layer_forward, (self.vals, self.meta, self.Y, self.Xq, self.amax, self._scratch)),
-                ("backward", lib.sste_layer_backward, (self.gvals, self.gmeta, self.dW, self.dX, *w, self.Xq, self.dYq, self.amax,
-                                                       self._scratch)),
-                ("grads", lib.sste_layer_grads, (self.gvals, self.gmeta, self.dW, self.dX, *w, self.Xq, self.dYq, self.amax))):
-            read = tuple(t for t in read if t is not None)
-            setattr(desc, name, (call, read, [t.data_ptr() for t in read]))
+        there = lambda *tensors: _same_places([t for t in tensors if t is not None])
+        desc.prune, desc.forward, desc.backward, desc.grads = (lib.sste_layer_prune, lib.sste_layer_forward,
+                                                               lib.sste_layer_backward, lib.sste_layer_grads)
+        fp8 = (self.amax, self._scratch)
+        desc.prune_there = there(self.W, self.beta, self.vals, self.meta, self.w_dense, *fp8)
+        desc.forward_there = there(self.vals, self.meta, self.Y, self.Xq, *fp8)
+        desc.backward_there = there(self.gvals, self.gmeta, self.dW, self.dX, *w, self.Xq, self.dYq, *fp8)
         return desc
 
-    def _described(self, phase):
-        """The descriptor, with the addresses that the buffers of `phase` have now; None: the single calls take it.
-
-        A tensor may be given other storage without being replaced (`t.data = ...`, a storage resized to 0 and back)."""
-        desc = self._desc or self._describe()
-        _, read, at = getattr(desc, phase)
-        if [t.data_ptr() for t in read] != at:
-            self.__dict__["_as_made"] = False
-            desc = self._describe()
-        return desc if desc.fits else None
+    def _moved(self):
+        self.__dict__["_as_made"] = False
+        return self._describe()
 
     def _replaced_fit(self, x_shape, g_shape, tensors):
         wdt, gdt = (B._TORCH_DT[B.E4M3], B._TORCH_DT[B.E5M2]) if self.fp8 else (_bf16, _bf16)
@@ -165,9 +175,12 @@ class SsteLinear:
     def prune(self):
         assert self.beta_ready, "call init_beta() in the first iteration"
         if self.mark is None and not self.track_flips:
-            desc = self._described("prune")
-            if desc and _takes(self.W, desc.w_shape):             # W is the caller's: it may be another view by now
-                st = desc.prune[0](self.ctx.handle, desc.at, _raw_stream(_device()))
+            desc = self._desc or self._describe()
+            if not desc.prune_there():
+                desc = self._moved()
+            W = self.W                                            # the caller's: it may be another view by now
+            if desc.fits and W.dtype is _bf16 and W.shape == desc.w_shape and W.is_contiguous():
+                st = desc.prune(self.ctx.handle, desc.at, _raw_stream(_device()))
                 if st:
                     self.ctx._check(st)
                 self.__dict__["launches"] += 2 if self.fp8 else 1
@@ -197,9 +210,12 @@ class SsteLinear:
     # (2a) forward with the sparse weight
     def forward(self, X, y_amax_out=None):
         if self.mark is None:
-            desc = self._described("forward")
-            if desc and _takes(X, desc.x_shape):
-                st = desc.forward[0](self.ctx.handle, desc.at, X.data_ptr(), B._ptr(y_amax_out), _raw_stream(_device()))
+            desc = self._desc or self._describe()
+            if not desc.forward_there():
+                desc = self._moved()
+            if desc.fits and _takes(X, desc.x_shape):
+                st = desc.forward(self.ctx.handle, desc.at, X.data_ptr(), None if y_amax_out is None else B._ptr(y_amax_out),
+                                  _raw_stream(_device()))
                 if st:
                     self.ctx._check(st)
                 d = self.__dict__
@@ -229,10 +245,12 @@ class SsteLinear:
     # (2b) backward: MVUE on the output gradient for grad_W, dense product for grad_X
     def backward(self, dY, step: int = 0, token_offset: int = 0):
         if self.mark is None:
-            desc = self._described("backward")
+            desc = self._desc or self._describe()
+            if not desc.backward_there():
+                desc = self._moved()
             X = None if self.fp8 else self.X
-            if desc and _takes(dY, desc.g_shape) and (X is None or _takes(X, desc.x_shape)):
-                st = desc.backward[0](self.ctx.handle, desc.at, None if X is None else X.data_ptr(), dY.data_ptr(), step,
+            if desc.fits and _takes(dY, desc.g_shape) and (X is None or _takes(X, desc.x_shape)):
+                st = desc.backward(self.ctx.handle, desc.at, None if X is None else X.data_ptr(), dY.data_ptr(), step,
                                       token_offset, _raw_stream(_device()))
                 if st:
                     self.ctx._check(st)
@@ -269,11 +287,13 @@ class SsteLinear:
         after the other (4096 x 11008, 2048 tokens, bf16: 213 against 228 us; 1280 x 5120, 16384 tokens: 229 against 240).
         Both are complete in current-stream order on return."""
         if self.mark is None:
-            desc = self._described("grads")
+            desc = self._desc or self._describe()
+            if not desc.backward_there():
+                desc = self._moved()
             X = None if self.fp8 else self.X
-            if (desc and _takes(dY, desc.g_shape) and (X is None or _takes(X, desc.x_shape))
+            if (desc.fits and _takes(dY, desc.g_shape) and (X is None or _takes(X, desc.x_shape))
                     and self.ctx.lib.sste_layer_grads_joint(self.ctx.handle, desc.at)):
-                st = desc.grads[0](self.ctx.handle, desc.at, None if X is None else X.data_ptr(), dY.data_ptr(),
+                st = desc.grads(self.ctx.handle, desc.at, None if X is None else X.data_ptr(), dY.data_ptr(),
                                    _raw_stream(_device()))
                 if st:
                     self.ctx._check(st)
@@ -362,40 +382,42 @@ class SsteLinearPadded:
     def prune(self):
         self.inner.prune()
 
-    # Descriptor of the one-call path, made anew when the inner layer's changes or a buffer of this layer is replaced or
-    # given other storage.
-    def _described(self, phase, X, shape):
-        inner = self.inner
-        if inner.mark is not None or not _takes(X, shape):
-            return None
-        of = inner._described(phase)
-        if of is None:
-            return None
-        bufs = (self.Xp, self.dYp, self.Y, self.dX, self.dW)
-        at = [t.data_ptr() for t in bufs]
+    # Descriptor of the one-call path for the inner layer's `of`, made anew when that is or when a buffer of this layer is
+    # replaced or given other storage; None: the single calls take it.
+    def _described(self, of):
         d = self._desc
-        if d is None or d[0] is not of or d[2] != at or any(a is not b for a, b in zip(d[1], bufs)):
-            crop = lambda t, whole: None if t.data_ptr() == whole.data_ptr() else B._ptr(t)
-            p = B.PaddedLayerBuffers(of.buffers, self.O, self.I, self.T, 0, B._ptr(self.Xp), B._ptr(self.dYp),
-                                     crop(self.Y, inner.Y), crop(self.dX, inner.dX), crop(self.dW, inner.dW))
-            fits = (inner.Y.dtype is _bf16 and tuple(self.Xp.shape) == (self.Tp, self.Ip)
-                    and tuple(self.dYp.shape) == (self.Tp, self.Op) and tuple(self.Y.shape) == (self.T, self.O)
-                    and tuple(self.dX.shape) == (self.T, self.I) and tuple(self.dW.shape) == (self.O, self.I)
-                    and all(t.dtype is _bf16 and t.is_cuda and t.is_contiguous() for t in bufs))
-            self._desc = d = (of, bufs, at, fits, ctypes.addressof(p), p)
-        return d if d[3] else None
+        if d is not None and d[0] is of and d[2]():
+            xp, dyp, y, dx, dw = d[1]
+            if self.Xp is xp and self.dYp is dyp and self.Y is y and self.dX is dx and self.dW is dw:
+                return d[4] if d[3] else None
+        bufs, inner = (self.Xp, self.dYp, self.Y, self.dX, self.dW), self.inner
+        crop = lambda t, whole: None if t.data_ptr() == whole.data_ptr() else B._ptr(t)
+        p = B.PaddedLayerBuffers(of.buffers, self.O, self.I, self.T, 0, B._ptr(self.Xp), B._ptr(self.dYp),
+                                 crop(self.Y, inner.Y), crop(self.dX, inner.dX), crop(self.dW, inner.dW))
+        fits = (inner.Y.dtype is _bf16 and tuple(self.Xp.shape) == (self.Tp, self.Ip)
+                and tuple(self.dYp.shape) == (self.Tp, self.Op) and tuple(self.Y.shape) == (self.T, self.O)
+                and tuple(self.dX.shape) == (self.T, self.I) and tuple(self.dW.shape) == (self.O, self.I)
+                and all(t.dtype is _bf16 and t.is_cuda and t.is_contiguous() for t in bufs))
+        self._desc = of, bufs, _same_places(bufs), fits, ctypes.addressof(p), p
+        return ctypes.addressof(p) if fits else None
 
     def _crop(self, src, dst):
         if src.data_ptr() != dst.data_ptr():
             self.ctx.crop_2d(src, dst)
 
     def forward(self, X):
-        d = self._described("forward", X, (self.T, self.I))
-        if d is not None:
-            st = self.ctx.lib.sste_padded_forward(self.ctx.handle, d[4], X.data_ptr(), _raw_stream(_device()))
+        inner = self.inner
+        at = None
+        if inner.mark is None and _takes(X, (self.T, self.I)):
+            of = inner._desc or inner._describe()
+            if not of.forward_there():
+                of = inner._moved()
+            at = self._described(of) if of.fits else None
+        if at is not None:
+            st = self.ctx.lib.sste_padded_forward(self.ctx.handle, at, X.data_ptr(), _raw_stream(_device()))
             if st:
                 self.ctx._check(st)
-            inner = self.inner.__dict__
+            inner = inner.__dict__
             if not self.inner.fp8:
                 inner["X"] = self.Xp
             inner["launches"] += 3 if self.inner.fp8 else 1
@@ -407,10 +429,15 @@ class SsteLinearPadded:
 
     def backward(self, dY, step: int = 0):
         # (the inner layer's input is Xp after a forward; without one, or after somebody gave it another, the single calls tell)
-        read_xp = self.inner.fp8 or self.inner.__dict__.get("X") is self.Xp
-        d = self._described("backward", dY, (self.T, self.O)) if read_xp else None
-        if d is not None:
-            st = self.ctx.lib.sste_padded_backward(self.ctx.handle, d[4], dY.data_ptr(), step, 0, _raw_stream(_device()))
+        inner = self.inner
+        at = None
+        if inner.mark is None and (inner.fp8 or inner.__dict__.get("X") is self.Xp) and _takes(dY, (self.T, self.O)):
+            of = inner._desc or inner._describe()
+            if not of.backward_there():
+                of = inner._moved()
+            at = self._described(of) if of.fits else None
+        if at is not None:
+            st = self.ctx.lib.sste_padded_backward(self.ctx.handle, at, dY.data_ptr(), step, 0, _raw_stream(_device()))
             if st:
                 self.ctx._check(st)
             self.inner.__dict__["launches"] += 4 if self.inner.fp8 else 3
