@@ -468,6 +468,8 @@ product(const CUtensorMap &map_a, const CUtensorMap &map_b, const CUtensorMap &m
                 tile_coords(u.tile, m_tiles, n_tiles, p.group_m, mt, nt);
                 const int m0 = mt * 2 * BM + static_cast<int>(rank) * BM;      // this CTA's rows of A
                 const int n0 = nt * BN + static_cast<int>(rank) * (BN / 2);    // this CTA's half of B
+                // rows beyond M (zero-filled values) take the codes of the last row block: zero is not one of the six codes
+                const int meta_row = min(m0 / BM, p.M / BM - 1) * k_atoms * 4;
                 for (int kb = u.kb0; kb < u.kb1; ++kb) {
                     // test hook: the stage is never loaded nor announced, so the MMA warp's wait for it runs out
                     if (p.skip_last_stage && seq.next(unit, j + 1) >= num_units && kb == u.kb1 - 1) break;
@@ -478,12 +480,9 @@ product(const CUtensorMap &map_a, const CUtensorMap &map_b, const CUtensorMap &m
                     const uint32_t b_dst = a_dst + C::A_STAGE;
                     // A: 128 bytes per row = BK/2 compressed (sparse) or BK dense elements
                     tma_load_2d(a_dst, &map_a, lead_full, kb * (SPARSE ? BK / 2 : BK), m0);
-                    // metadata: the atoms of this K, 2 KB each, as rows of 512 bytes.  Rows beyond M (zero-filled values) take the
-                    // codes of the last row block: zero is not one of the six codes.  (With an odd number of atoms the last
-                    // 8-bit stage also fetches what follows; the MMAs stop in front of it.)
-                    if (SPARSE)
-                        tma_load_2d(b_dst + C::B_STAGE, &map_m, lead_full, 0,
-                                    (min(m0 / BM, p.M / BM - 1) * k_atoms + kb * C::ATOMS) * 4);
+                    // metadata: the atoms of this K, 2 KB each, as rows of 512 bytes.  (With an odd number of atoms the last
+                    // 8-bit stage also fetches what follows; no MMA reads it.)
+                    if (SPARSE) tma_load_2d(b_dst + C::B_STAGE, &map_m, lead_full, 0, meta_row + kb * C::ATOMS * 4);
                     if (BCOMP) {
                         // B is written into the stage by the expander warps
                     } else if (BMAJ == BMajor::K) {
@@ -504,6 +503,7 @@ product(const CUtensorMap &map_a, const CUtensorMap &map_b, const CUtensorMap &m
         // ------------------------------------------------------------ MMA issuer (leader CTA only)
         if (leader && lane == 0) {
             const uint32_t idesc = instr_desc(SPARSE, p.afmt, p.bfmt, BMAJ == BMajor::MN, BN);
+            const int half_kb = p.K % BK != 0 ? k_blocks_total - 1 : -1;
             uint32_t s = 0, ph = 0, local_tile = 0;
             bool ok = true;
             for (int unit = seq.first(); unit < num_units && ok; ++local_tile, unit = seq.next(unit, local_tile)) {
@@ -528,11 +528,11 @@ product(const CUtensorMap &map_a, const CUtensorMap &map_b, const CUtensorMap &m
                         for (int i = 0; i < C::ATOMS; ++i)
                             tc_cp_meta_atom(meta_cols + 4 * i, smem_desc(b_src + C::B_STAGE + 2048 * i, 128, 128, 0));
                     }
-                    // the last stage of an 8-bit sparse product with an odd number of atoms is half a stage
-                    const bool half = SPARSE && F8 && (kb + 1) * BK > p.K;
+                    // the second half of the last stage of an 8-bit sparse product with an odd number of atoms (zero-filled
+                    // values) takes the first half's metadata columns
+                    const uint32_t back = (SPARSE && F8 && kb == half_kb) ? 4u : 0u;
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
-                        if (half && j >= 2) break;
                         const uint64_t adesc = smem_desc(a_src + 32 * j, 16, 1024, 2);
                         uint64_t bdesc;
                         if (BMAJ == BMajor::K) {
@@ -545,7 +545,7 @@ product(const CUtensorMap &map_a, const CUtensorMap &map_b, const CUtensorMap &m
                         if (SPARSE) {
                             // bf16: one 32-bit metadata column per instruction, the column pair is addressed and
                             // the descriptor's sparse selector picks the column; fp8: two columns per instruction
-                            const uint32_t e = meta_cols + (F8 ? 2 * j : (j & 2));
+                            const uint32_t e = meta_cols + (F8 ? 2 * j - (j >= 2 ? back : 0u) : (j & 2));
                             const uint32_t id2 = F8 ? 0u : static_cast<uint32_t>(j & 1);
                             tc_mma_sparse<F8>(d_tmem, adesc, bdesc, e, idesc | id2, acc);
                         } else {
