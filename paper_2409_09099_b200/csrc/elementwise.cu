@@ -807,7 +807,7 @@ struct RaggedRows {
 // One CTA: 128 tokens x 64 output columns of dY (half a metadata atom).  A thread handles 4 tokens x 8 columns
 // (8 groups, two Philox calls); results are transposed through shared memory so that every
 // output row (= column of dY) receives whole 128-byte lines.  dY[8192, 3072], bf16 / FP8: 35.6 / 38.1 us with the
-// scalar rule, 24.2 / 30.3 us with mvue_pair (15.6 us is what the loads and stores take alone, 20.0 us the rule without
+// scalar rule, 24.7 / 30.9 us with mvue_pair (15.6 us is what the loads and stores take alone, 20.0 us the rule without
 // the loads); two tasks of 128 columns, tasks of 4 columns, and persistent CTAs with cp.async prefetch were slower.
 // ANY_COUNTER: counter_cols is not a multiple of 4 (a padded, odd column count), so a thread's eight
 // consecutive group indices do not start on a Philox block and span three blocks instead of two.
