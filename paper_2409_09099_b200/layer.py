@@ -27,7 +27,9 @@ _bf16, _raw_stream, _device = torch.bfloat16, torch._C._cuda_getCurrentRawStream
 
 def _as_defined(obj, cls, names):
     """Whether `obj` is a `cls` whose methods `names` are those of `cls` (no subclass, no attribute, overrides them)."""
-    return isinstance(obj, cls) and not any(getattr(type(obj), n) is not getattr(cls, n) or n in vars(obj) for n in names)
+    t = type(obj)
+    return (isinstance(obj, cls) and vars(obj).keys().isdisjoint(names)
+            and (t is cls or all(getattr(t, n) is getattr(cls, n) for n in names)))
 
 
 def _takes(t, shape):
