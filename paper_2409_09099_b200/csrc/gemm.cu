@@ -69,24 +69,41 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t byt
 {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
-// arrive on a barrier that may live in the peer CTA (shared::cluster address)
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr)
+// Arrive on a barrier that may live in the peer CTA (shared::cluster address).  CLUSTER: what this thread wrote to shared memory is
+// for the peer too.  Without it the arrival only says that something has been read (tensor memory, behind its own fence), and
+// need not wait until the thread's writes are visible in the cluster.  (With cluster scope on every arrival and wait, a forward of 3072 x
+// 768 with 8192 tokens took 26.8 us in bf16 and 23.5 in FP8, now 24.1 and 20.0; with 128 tokens 7.4 and 6.8; a shape whose
+// epilogue sets the pace gains most: 1024 x 50304 60 -> 55.)
+template <bool CLUSTER>
+__device__ __forceinline__ void mbar_arrive_at(uint32_t cluster_addr)
 {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+    if (CLUSTER) asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+    else asm volatile("mbarrier.arrive.release.cta.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
 // One try: the thread is suspended by the hardware until the phase completes or a time limit of
 // about a millisecond passes, so a waiting thread does not poll shared memory (the sparse MMA streams
 // its operands at 3/4 of the shared-memory bandwidth and is slowed down by pollers).
+// CLUSTER: the thread goes on to what the peer CTA's threads wrote (the others go on to what copies and MMAs, or nobody, wrote).
+template <bool CLUSTER>
 __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
 {
     uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\n\t"
-        "selp.b32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity), "r"(1000000u)
-        : "memory");
+    if (CLUSTER)
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\n\t"
+            "selp.b32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(bar), "r"(parity), "r"(1000000u)
+            : "memory");
+    else
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cta.shared::cta.b64 p, [%1], %2, %3;\n\t"
+            "selp.b32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(bar), "r"(parity), "r"(1000000u)
+            : "memory");
     return ok != 0;
 }
 __device__ __forceinline__ unsigned long long global_ns()
@@ -102,12 +119,13 @@ struct WaitCtx {
     volatile int *abort_flag;          // this CTA's "a wait has expired" flag (shared memory)
     unsigned long long limit_ns;       // WAIT_LIMIT_NS, or the short limit of the stall-injection test hook
 };
+template <bool CLUSTER>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, const WaitCtx &wc)
 {
-    if (mbar_try_wait(bar, parity)) return true;
+    if (mbar_try_wait<CLUSTER>(bar, parity)) return true;
     const unsigned long long start = global_ns();
     while (true) {
-        if (mbar_try_wait(bar, parity)) return true;
+        if (mbar_try_wait<CLUSTER>(bar, parity)) return true;
         if (*wc.abort_flag) return false;
         if (global_ns() - start > wc.limit_ns) {
             atomicMax(wc.status, static_cast<unsigned int>(SSTE_ERR_TIMEOUT));      // also over a recorded degenerate beta
@@ -117,10 +135,11 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, const W
     }
 }
 // Bounded wait of a whole warp: lane 0 waits, the others park at the warp barrier.
+template <bool CLUSTER>
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, const WaitCtx &wc)
 {
     uint32_t ok = 1;
-    if ((threadIdx.x & 31) == 0) ok = mbar_wait(bar, parity, wc) ? 1u : 0u;
+    if ((threadIdx.x & 31) == 0) ok = mbar_wait<CLUSTER>(bar, parity, wc) ? 1u : 0u;
     ok = __shfl_sync(0xffffffffu, ok, 0);
     return ok != 0;
 }
@@ -473,7 +492,7 @@ product(const CUtensorMap &map_a, const CUtensorMap &map_b, const CUtensorMap &m
                 for (int kb = u.kb0; kb < u.kb1; ++kb) {
                     // test hook: the stage is never loaded nor announced, so the MMA warp's wait for it runs out
                     if (p.skip_last_stage && seq.next(unit, j + 1) >= num_units && kb == u.kb1 - 1) break;
-                    if (!mbar_wait(empty_bar(s), ph ^ 1u, wc)) { ok = false; break; }
+                    if (!mbar_wait<BCOMP>(empty_bar(s), ph ^ 1u, wc)) { ok = false; break; }
                     const uint32_t lead_full = map_to_cta(full_bar(s), 0);
                     if (leader) mbar_arrive_expect_tx(full_bar(s), STAGE_TX);
                     const uint32_t a_dst = smem_base + s * C::STAGE;
@@ -509,12 +528,12 @@ product(const CUtensorMap &map_a, const CUtensorMap &map_b, const CUtensorMap &m
             for (int unit = seq.first(); unit < num_units && ok; ++local_tile, unit = seq.next(unit, local_tile)) {
                 const Unit u = decode(unit);
                 const uint32_t buf = local_tile % NB, use = local_tile / NB;
-                if (!mbar_wait(acc_empty_bar(buf), (use & 1u) ^ 1u, wc)) { ok = false; break; }
+                if (!mbar_wait<BCOMP>(acc_empty_bar(buf), (use & 1u) ^ 1u, wc)) { ok = false; break; }
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + buf * BN;
                 uint32_t acc = 0;
                 for (int kb = u.kb0; kb < u.kb1; ++kb) {
-                    if (!mbar_wait(full_bar(s), ph, wc)) { ok = false; break; }
+                    if (!mbar_wait<BCOMP>(full_bar(s), ph, wc)) { ok = false; break; }
                     tc_fence_after();
                     const uint32_t a_src = smem_base + s * C::STAGE;
                     const uint32_t b_src = a_src + C::A_STAGE;
@@ -632,10 +651,10 @@ product(const CUtensorMap &map_a, const CUtensorMap &map_b, const CUtensorMap &m
             auto release_acc = [&] {       // this warp has read its rows: count towards the buffer's release
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive_cluster(map_to_cta(acc_empty_bar(buf), 0));
+                if (lane == 0) mbar_arrive_at<BCOMP>(map_to_cta(acc_empty_bar(buf), 0));
             };
             // (a pair of warps leaves together when a wait expired: its barriers need both)
-            if (!group_all(mbar_wait_warp(acc_full_bar(buf), use & 1u, wc))) break;
+            if (!group_all(mbar_wait_warp<BCOMP>(acc_full_bar(buf), use & 1u, wc))) break;
             tc_fence_after();
             if (OUT_F32) {
                 const int m = m0 + quarter * 32 + lane;
@@ -982,7 +1001,7 @@ product(const CUtensorMap &map_a, const CUtensorMap &map_b, const CUtensorMap &m
         while (h0) {
             const int s = it % NS;
             const uint32_t ph = (it / NS) & 1u;
-            if (!mbar_wait_warp(empty_bar(s), ph ^ 1u, wc)) break;
+            if (!mbar_wait_warp<BCOMP>(empty_bar(s), ph ^ 1u, wc)) break;
             uint8_t *b_dst = ring + s * C::STAGE + C::A_STAGE + (seg >> 2) * (BK * 128);
             const int j0 = (seg & 3) * 2;
 #pragma unroll
@@ -1010,7 +1029,7 @@ product(const CUtensorMap &map_a, const CUtensorMap &map_b, const CUtensorMap &m
             }
             fence_proxy_async();        // the tensor core reads the stage through the async proxy
             __syncwarp();
-            if (lane == 0) mbar_arrive_cluster(map_to_cta(full_bar(s), 0));
+            if (lane == 0) mbar_arrive_at<BCOMP>(map_to_cta(full_bar(s), 0));
 #pragma unroll
             for (int j = 0; j < UNITS; ++j) { v0[j] = v1[j]; m0[j] = m1[j]; v1[j] = v2[j]; m1[j] = m2[j]; }
             h0 = h1;
