@@ -705,13 +705,8 @@ product(const CUtensorMap &map_a, const CUtensorMap &map_b, const CUtensorMap &m
                 release_acc();
                 continue;
             }
-            // BOXP packed panels of this warp -> staging (swizzled as the TMA store expects, conflict-free) -> output
-            auto store_box = [&](int pnl, const uint32_t *w) {
-                const uint32_t sb = my_staging + (BOXES == 2 ? (box_it & 1u) * (2 * PANEL_BYTES) : 0u);
-                ++box_it;
-                // the buffer is writable once the store issued from it last has read it
-                if (elect) asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(BOXES - 1) : "memory");
-                group_sync();
+            // packed panels of this warp -> staging (swizzled as the TMA store expects, conflict-free): one box of BOXP panels
+            auto stage_box = [&](uint32_t sb, const uint32_t *w) {
                 if (OUT_T) {
                     // staging row = column n of the accumulator, 64 m of the pair; matrix k = rows m 8k .. 8k + 7 of the warp
 #pragma unroll
@@ -731,11 +726,38 @@ product(const CUtensorMap &map_a, const CUtensorMap &map_b, const CUtensorMap &m
                         st_shared_v4(sb + lane * 64 + ((c ^ ((lane >> 1) & 3)) << 4), w[4 * c], w[4 * c + 1], w[4 * c + 2],
                                      w[4 * c + 3]);
                 }
+            };
+            // -> output, by one thread of the group
+            auto put_box = [&](uint32_t sb, int pnl) {
+                if (OUT_T) tma_store_2d(&map_d, sb, m0 + 64 * (quarter >> 1), n0 + 32 * pnl);
+                else tma_store_2d(&map_d, sb, n0 + 32 * pnl, m0 + 32 * quarter);
+            };
+            auto store_box = [&](int pnl, const uint32_t *w) {
+                const uint32_t sb = my_staging + (BOXES == 2 ? (box_it & 1u) * (2 * PANEL_BYTES) : 0u);
+                ++box_it;
+                // the buffer is writable once the store issued from it last has read it
+                if (elect) asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(BOXES - 1) : "memory");
+                group_sync();
+                stage_box(sb, w);
                 fence_proxy_async();
                 group_sync();
                 if (elect) {
-                    if (OUT_T) tma_store_2d(&map_d, sb, m0 + 64 * (quarter >> 1), n0 + 32 * pnl);
-                    else tma_store_2d(&map_d, sb, n0 + 32 * pnl, m0 + 32 * quarter);
+                    put_box(sb, pnl);
+                    tma_store_commit();
+                }
+            };
+            // both buffers at once: one wait, one fence and two barriers for two boxes (the second is there if `two`; FP8 forward of
+            // 3072 x 768, 8192 tokens: 18.8 -> 17.9 us, bf16 24.0 -> 23.8)
+            auto store_two = [&](int pnl, const uint32_t *w, bool two) {
+                if (elect) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+                group_sync();
+                stage_box(my_staging, w);
+                if (two) stage_box(my_staging + 2 * PANEL_BYTES, w + 16);
+                fence_proxy_async();
+                group_sync();
+                if (elect) {
+                    put_box(my_staging, pnl);
+                    if (two) put_box(my_staging + 2 * PANEL_BYTES, pnl + 1);
                     tma_store_commit();
                 }
             };
@@ -916,9 +938,13 @@ product(const CUtensorMap &map_a, const CUtensorMap &map_b, const CUtensorMap &m
                         if (second) pack_chunk(r + 32, pk + 16 * i + 16);
                     }
                     if (h0 + HOLD == PANELS_MAX) release_acc();
+                    if constexpr (BOXES == 2 && HOLD == 2) {
+                        if (h0 < n_pnl) store_two(pnl0 + h0, pk, h0 + 1 < n_pnl);
+                    } else {
 #pragma unroll
-                    for (int i = 0; i < HOLD; i += BOXP)
-                        if (h0 + i < n_pnl) store_box(pnl0 + h0 + i, pk + 16 * i);
+                        for (int i = 0; i < HOLD; i += BOXP)
+                            if (h0 + i < n_pnl) store_box(pnl0 + h0 + i, pk + 16 * i);
+                    }
                 }
             }
         }
