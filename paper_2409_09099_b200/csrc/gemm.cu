@@ -508,6 +508,7 @@ product(const CUtensorMap &map_a, const CUtensorMap &map_b, const CUtensorMap &m
                 const int n0 = nt * BN + static_cast<int>(rank) * (BN / 2);    // this CTA's half of B
                 // rows beyond M (zero-filled values) take the codes of the last row block: zero is not one of the six codes
                 const int meta_row = min(m0 / BM, p.M / BM - 1) * k_atoms * 4;
+                if (j == 0) sste_pdl_wait();
                 for (int kb = u.kb0; kb < u.kb1; ++kb) {
                     // test hook: the stage is never loaded nor announced, so the MMA warp's wait for it runs out
                     if (p.skip_last_stage && seq.next(unit, j + 1) >= num_units && kb == u.kb1 - 1) break;
@@ -544,6 +545,7 @@ product(const CUtensorMap &map_a, const CUtensorMap &map_b, const CUtensorMap &m
             const int half_kb = p.K % BK != 0 ? k_blocks_total - 1 : -1;
             uint32_t s = 0, ph = 0, local_tile = 0;
             bool ok = true;
+            sste_pdl_wait();                 // (the bounded waits below do not count the previous kernel's time)
             for (int unit = seq.first(); unit < num_units && ok; ++local_tile, unit = seq.next(unit, local_tile)) {
                 const Unit u = decode(unit);
                 const uint32_t buf = local_tile % NB, use = local_tile / NB;
@@ -615,6 +617,7 @@ product(const CUtensorMap &map_a, const CUtensorMap &map_b, const CUtensorMap &m
         const bool elect = lane == 0 && (!OUT_T || (warp & 1) == 0); // issues the group's stores
         auto group_sync = [&] { if (OUT_T) pair_barrier(group_bar); else __syncwarp(); };
         auto group_all = [&](bool ok) -> bool { return OUT_T ? pair_barrier_and(group_bar, ok) : __all_sync(0xffffffffu, ok); };
+        sste_pdl_wait();
         const float scale = sste_out_scale(p.a_amax, p.a_fp8_max, p.b_amax, p.b_fp8_max);
         const bool want_amax = (p.out_amax != nullptr);
         const int kind = want_amax ? 2 : scale != 1.0f ? 1 : 0;      // what a stored value needs besides the rounding
@@ -1037,6 +1040,7 @@ product(const CUtensorMap &map_a, const CUtensorMap &map_b, const CUtensorMap &m
             return true;
         };
         e_setup();
+        sste_pdl_wait();
         // three stages of loads in flight in registers: a round trip to L2 is longer than two stages of MMAs
         uint4 v0[UNITS], v1[UNITS], v2[UNITS];
         uint32_t m0[UNITS], m1[UNITS], m2[UNITS];
@@ -1114,8 +1118,13 @@ __device__ __forceinline__ Frame frame_begin(uint8_t *smem_raw, const GemmParams
     __syncthreads();
     cluster_sync();          // the peer's barriers are initialised before anything signals them
     tc_fence_after();
-    sste_pdl_wait();         // everything above overlapped the previous kernel; global memory from here on
-    if (blockIdx.x == 0 && threadIdx.x == 32 && p.zero_after) *p.zero_after = 0u;
+    // (everything up to here overlaps the previous kernel.  Each role waits for it in front of its own first access to global
+    // memory or bounded wait, the producer with the first tile's coordinates worked out: 0.2 to 0.4 us of every product, a forward of
+    // 3072 x 768 with 128 tokens 6.55 -> 6.35.)
+    if (blockIdx.x == 0 && threadIdx.x == 32 && p.zero_after) {
+        sste_pdl_wait();
+        *p.zero_after = 0u;
+    }
     f.tmem_base = *reinterpret_cast<volatile uint32_t *>(f.ctrl + CTRL_TMEM);
     return f;
 }
