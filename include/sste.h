@@ -24,8 +24,9 @@
  *     completed, so stream order holds for every caller-visible effect, also
  *     between these calls and the caller's own kernels, copies and captures.
  *   - Two calls that may overlap on the device (different streams) need
- *     different contexts if either is a product: the split-K workspace belongs
- *     to the context.
+ *     different contexts if either is a product, a beta or a phase of an FP8
+ *     layer: the split-K workspace, the reduction scratch and the slots of a
+ *     maximum that a kernel's blocks share belong to the context.
  *   - O = out features, I = in features, T = tokens.  O, I and T must be
  *     multiples of 128 and tensor pointers 128-byte aligned, otherwise
  *     SSTE_ERR_SHAPE / SSTE_ERR_ALIGN is returned BEFORE anything is launched.
@@ -271,9 +272,10 @@ typedef struct sste_layer {
     void *scratch;
 } sste_layer;
 
-/* sste_project_compress of the layer's weight (FP8: after sste_project_amax). */
+/* sste_project_compress of the layer's weight (FP8: after sste_project_amax, in one launch where the weight is small enough). */
 sste_status sste_layer_prune(sste_ctx *ctx, const sste_layer *layer, void *stream);
-/* sste_linear_fwd of X (FP8: after sste_amax and sste_quantize_fp8 of it).  X bf16 [T, I]. */
+/* sste_linear_fwd of X (FP8: after sste_amax and sste_quantize_fp8 of it, in one launch for a million elements up to as many as all
+ * SMs hold in registers).  X bf16 [T, I]. */
 sste_status sste_layer_forward(sste_ctx *ctx, const sste_layer *layer, const void *X, float *y_amax_out_dev, void *stream);
 /* sste_mvue_sparsify of dY (FP8: after sste_amax of it), then sste_layer_grads.  dY bf16 [T, O]. */
 sste_status sste_layer_backward(sste_ctx *ctx, const sste_layer *layer, const void *X, const void *dY, uint32_t step,

@@ -68,6 +68,8 @@ extern "C" sste_status sste_layer_prune(sste_ctx *ctx, const sste_layer *l, void
     if (!fp8_of(l))
         return sste_project_compress(ctx, l->W, l->O, l->I, SSTE_BF16, l->beta, nullptr, SSTE_BF16, l->vals, l->meta, l->w_dense,
                                      stream);
+    if (sste_project_fp8_fits(ctx, l->O, l->I))
+        return sste_project_fp8(ctx, l->W, l->O, l->I, l->beta, l->amax + 1, l->vals, l->meta, l->w_dense, stream);
     sste_status st = sste_project_amax_scratch(ctx, l->W, l->O, l->I, l->beta, l->amax + 1, l->scratch, stream);
     if (st != SSTE_OK) return st;
     return sste_project_compress(ctx, l->W, l->O, l->I, SSTE_BF16, l->beta, l->amax + 1, SSTE_E4M3, l->vals, l->meta, l->w_dense,
@@ -84,6 +86,12 @@ extern "C" sste_status sste_layer_forward(sste_ctx *ctx, const sste_layer *l, co
         x_amax = l->amax;
         w_amax = l->amax + 1;
         const size_t n = static_cast<size_t>(l->T) * l->I;
+        if (sste_amax_quantize_fits(ctx, n)) {
+            const sste_status st = sste_amax_quantize(ctx, X, n, x_amax, l->Xq, stream);
+            if (st != SSTE_OK) return st;
+            return sste_linear_fwd(ctx, l->Xq, l->T, l->vals, l->meta, l->O, l->I, SSTE_E4M3, x_amax, w_amax, l->Y,
+                                   static_cast<sste_dtype>(l->out_dtype), y_amax_out_dev, stream);
+        }
         sste_status st = sste_amax_scratch(ctx, X, n, x_amax, l->scratch, stream);
         if (st != SSTE_OK) return st;
         st = sste_quantize_scratch(ctx, X, n, x_amax, l->scratch, l->Xq, stream);

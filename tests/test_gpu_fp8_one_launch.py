@@ -1,0 +1,112 @@
+"""FP8 layers: maximum and quantisation of X, maximum and projection of W in one launch each, against the two single calls.
+
+Bit for bit, at the sizes where the work per block changes, at the largest that one launch takes and beyond it; also with most SMs
+busy, so that blocks which run work out the chunks of those that do not.
+"""
+import pytest
+import torch
+
+from paper_2409_09099_b200 import binding as B
+from paper_2409_09099_b200.layer import SsteLinear
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    c = B.Context(0)
+    yield c
+    assert c.poll_device_status() == 0
+    c.close()
+
+
+def _randn(rows, cols, seed):
+    return torch.empty((rows, cols), dtype=torch.bfloat16, device="cuda").normal_(
+        generator=torch.Generator(device="cuda").manual_seed(seed))
+
+
+def _bits(t):
+    return t.contiguous().view(torch.uint8)
+
+
+def _slots_empty(ctx):
+    """the context's counters and slots, in front of the partial tiles, are zero again"""
+    torch.cuda.synchronize()
+    return not ctx.workspace[17408:17408 + 4 * 8192].any()
+
+
+def _check_x(ctx, X, Xq, amax):
+    ref_amax, ref_q = torch.empty_like(amax), torch.empty_like(Xq)
+    ctx.amax(X, ref_amax)
+    ctx.quantize_fp8(X, ref_amax, ref_q)
+    assert torch.equal(amax, ref_amax) and torch.equal(_bits(Xq), _bits(ref_q))
+
+
+# T x I: the largest of two launches, the smallest of one; 296 blocks of one vector per thread, then two; four; the largest of one
+# launch, the next of two
+@pytest.mark.parametrize("T,I", [(1024, 896), (1024, 1024), (128, 9472), (128, 9600), (512, 9472), (1024, 9344), (1024, 9472), (1024, 9600)])
+def test_quantised_input(ctx, T, I):
+    W = _randn(128, I, 1) * 0.02
+    lin = SsteLinear(ctx, W, T, fp8=True)
+    lin.init_beta()
+    lin.prune()
+    X = _randn(T, I, T + I)
+    X[-1, -1] = 77.0                                  # the maximum in the last chunk, then everywhere zero, then small again
+    for scale in (1.0, 0.0, 0.25):
+        lin.forward(X * scale)
+        _check_x(ctx, X * scale, lin.Xq, lin.amax[0:1])
+        assert _slots_empty(ctx)
+
+
+# O x I: one tile of 32 x 128 per block up to 592 of them, two up to 1184, four up to 1776, then two launches
+@pytest.mark.parametrize("O,I", [(128, 128), (4736, 512), (2432, 1024), (4736, 1024), (4864, 1024), (7040, 1024), (7168, 1024)])
+@pytest.mark.parametrize("dense_copy", [True, False])
+def test_projected_weight(ctx, O, I, dense_copy):
+    W = _randn(O, I, O + I) * 0.02
+    W[-1, -4:] = torch.tensor([3.0, -2.0, 0.5, 0.25], dtype=torch.bfloat16)
+    layers = [SsteLinear(ctx, W, 128, fp8=True, dense_copy=dense_copy) for _ in range(2)]
+    layers[1].mark = lambda label: None               # the single calls
+    for factor in (1.0, 0.5):
+        for lin in layers:
+            lin.init_beta()
+            lin.prune()
+        a, b = layers
+        assert torch.equal(a.amax[1:2], b.amax[1:2])
+        for name in ("vals", "meta") + (("w_dense",) if dense_copy else ()):
+            assert torch.equal(_bits(getattr(a, name)), _bits(getattr(b, name))), name
+        assert _slots_empty(ctx)
+        W.mul_(factor * 0.5)
+
+
+def test_blocks_that_cannot_run_are_not_waited_for(ctx):
+    """A product on 80 SMs of another stream (its context cannot split it) leaves room for half of the blocks."""
+    other, side = B.Context(0, minimal_workspace=True), torch.cuda.Stream()
+    M, K = 10240, 16384
+    busy = SsteLinear(other, _randn(M, 256, 3) * 0.02, K)          # grad_W: 40 tiles of the whole reduction
+    busy.init_beta()
+    busy.prune()
+    busy.forward(_randn(K, 256, 4))
+    busy.sparsify_grad(_randn(K, M, 5))
+    T, I = 1024, 9472
+    lin = SsteLinear(ctx, _randn(3712, I // 74, 6) * 0.02, 128, fp8=True)
+    wide = SsteLinear(ctx, _randn(128, I, 7) * 0.02, T, fp8=True)
+    for l in (lin, wide):
+        l.init_beta()
+        l.prune()
+    X = _randn(T, I, 8)
+    wide.forward(X)
+    torch.cuda.synchronize()
+    vals, codes = lin.vals.clone(), wide.Xq.clone()
+    for _ in range(3):
+        lin.vals.zero_()
+        wide.Xq.zero_()
+        torch.cuda.synchronize()
+        with torch.cuda.stream(side):
+            for _ in range(3):
+                busy.grad_weight()
+        wide.forward(X)
+        lin.prune()
+        torch.cuda.synchronize()
+        assert torch.equal(_bits(wide.Xq), _bits(codes)) and torch.equal(_bits(lin.vals), _bits(vals))
+        assert _slots_empty(ctx)
+    assert other.poll_device_status() == 0
