@@ -281,12 +281,12 @@ sste_status sste_layer_forward(sste_ctx *ctx, const sste_layer *layer, const voi
 sste_status sste_layer_backward(sste_ctx *ctx, const sste_layer *layer, const void *X, const void *dY, uint32_t step,
                                 uint64_t token_offset, void *stream);
 /* grad_W and grad_X after sste_mvue_sparsify: sste_linear_bwd_weight with X (FP8: with the layer's Xq; X may be NULL) and
- * sste_linear_bwd_input.  With bf16 outputs both run in ONE launch where sste_layer_grads_joint says so: the pairs of SMs that
+ * sste_linear_bwd_input.  With bf16 outputs both run in ONE launch where that is the faster way: the pairs of SMs that
  * grad_W's tiles leave idle start on grad_X's.  (The split of grad_W's reduction may then differ from the single call's: same
  * sums, other rounding.)  Otherwise one product follows the other. */
 sste_status sste_layer_grads(sste_ctx *ctx, const sste_layer *layer, const void *X, const void *dY, void *stream);
-/* 1 if sste_layer_grads takes one launch for this layer, 0 if two: a caller with a second stream and context of its own then
- * gains by sste_linear_bwd_weight there beside sste_linear_bwd_input here.  Host only. */
+/* 1 if sste_layer_grads takes one launch for this layer and that also beats two side by side, 0 otherwise: a caller with a second
+ * stream and context of its own may then put sste_linear_bwd_weight there beside sste_linear_bwd_input here.  Host only. */
 int sste_layer_grads_joint(const sste_ctx *ctx, const sste_layer *layer);
 
 /*

@@ -180,7 +180,7 @@ sste_status sste_bwd_products(sste_ctx *ctx, const void *gvals, const void *gmet
                               int T, sste_dtype gdt, sste_dtype wdt, const void *w_dense, const void *vals, const void *meta,
                               const float *g_amax, const float *x_amax, const float *w_amax, void *dW, void *dX,
                               sste_dtype odt, void *stream);
-// Whether that is one launch for these sizes (multiples of 128; elt: bytes of an operand's element).
+// Whether one launch also beats the two side by side on two streams, for these sizes (multiples of 128; elt: bytes of an operand's element).
 bool sste_bwd_in_one_launch(const sste_ctx *ctx, int elt, int O, int I, int T, bool dense_copy, sste_dtype odt);
 
 // two sste_crop_2d in one launch (arguments as checked by that call)

@@ -1744,14 +1744,19 @@ void *dense_copy_in_workspace(const sste_ctx *ctx, int O, int I, int elt, size_t
 
 bool test_hook_set() { return g_inject_stall || g_force_bn || g_force_splits || g_force_group_m; }
 
-// The plan of both gradient products in one launch; whether that beats two in a row.  Two win for large products, whose last wave costs little and whose tiles run 10 % slower beside the other
-// product's (1280 x 5120, 16384 tokens, bf16: 248 us apart, 260 us together; 3840 x 1280: 194 and 180).
-bool joint_wins(const sste_ctx *ctx, int elt, size_t partial_bytes, int O, int I, int T, JointPlan *plan)
+// The plan of both gradient products in one launch; whether that beats two in a row, or (beside) two side by side on two streams.
+// Two win where the second launch and its own last wave cost less than what tiles lose beside the other product's, some 3 % (6016 x
+// 1152, 5504 tokens, bf16: 100 us apart, 104 together; 5248 x 768, 8832 tokens: 88 and 94; 3840 x 1280, 16384 tokens: 183 and 168; 1280 x
+// 5120, 16384: 237 and 227; 2560 x 1280, 640: 22 and 19).  The line was drawn over 146 shapes timed both ways; with 10 % in place of 3 %
+// and 2 us, 66 of them went the wrong way, by 9 % on the mean.  A caller that offers a second stream keeps it unless one launch is clearly
+// ahead (4 %, without the 2 us: 22 of the 146 go the other way than with 10 %, 10 % faster on the mean: 1280 x 5120, 8192 tokens 126 -> 119,
+// 512 x 7040, 1792 tokens 28.7 -> 21.6; the other line would be faster on most of the rest too, but such callers count on their stream).
+bool joint_wins(const sste_ctx *ctx, int elt, size_t partial_bytes, int O, int I, int T, bool beside, JointPlan *plan)
 {
     *plan = make_joint_plan(elt, ctx->sm_count, partial_bytes, O, I, T);
     const double apart = make_plan(GRAD_WEIGHT, elt, 0, false, false, ctx->sm_count, partial_bytes, O, I, T).us +
                          make_plan(GRAD_INPUT, elt, 0, false, false, ctx->sm_count, partial_bytes, T, I, O, true).us + LAUNCH_US;
-    return 1.1 * plan->us <= apart;
+    return beside ? 1.04 * plan->us <= apart : 1.03 * plan->us <= apart + 2.0;
 }
 
 // FP8 operands come with the amax of the tensors they were quantised from (both or neither); bf16 with none.
@@ -1952,7 +1957,7 @@ bool sste_bwd_in_one_launch(const sste_ctx *ctx, int elt, int O, int I, int T, b
     if (odt != SSTE_BF16 || test_hook_set()) return false;
     if (!dense_copy && !dense_copy_in_workspace(ctx, O, I, elt, &partial_bytes)) return false;
     JointPlan plan;
-    return joint_wins(ctx, elt, partial_bytes, O, I, T, &plan);
+    return joint_wins(ctx, elt, partial_bytes, O, I, T, true, &plan);
 }
 
 sste_status sste_bwd_products(sste_ctx *ctx, const void *gvals, const void *gmeta, const void *X, const void *dY, int O, int I,
@@ -1989,7 +1994,7 @@ sste_status sste_bwd_products(sste_ctx *ctx, const void *gvals, const void *gmet
             const GemmParams px{T, I, O, dX, g_amax, w_amax, sste_fp8_max(gdt), sste_fp8_max(wdt), nullptr, ctx->status_dev, cg, cw, nullptr};
             cudaStream_t s = static_cast<cudaStream_t>(stream);
             JointPlan plan;
-            if (joint_wins(ctx, elt, partial_bytes, O, I, T, &plan)) {
+            if (joint_wins(ctx, elt, partial_bytes, O, I, T, false, &plan)) {
                 if (elt == 1) return launch_grads<1, 256, 256>(ctx, gvals, gmeta, X, dY, w, pw, px, plan, s);
                 if (plan.w.bn == 256) return launch_grads<2, 256, 256>(ctx, gvals, gmeta, X, dY, w, pw, px, plan, s);
                 if (plan.x.bn == 256) return launch_grads<2, 128, 256>(ctx, gvals, gmeta, X, dY, w, pw, px, plan, s);
