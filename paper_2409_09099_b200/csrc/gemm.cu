@@ -751,6 +751,8 @@ product(const CUtensorMap &map_a, const CUtensorMap &map_b, const CUtensorMap &m
                 if (OUT_T) tma_store_2d(&map_d, sb, m0 + 64 * (quarter >> 1), n0 + 32 * pnl);
                 else tma_store_2d(&map_d, sb, n0 + 32 * pnl, m0 + 32 * quarter);
             };
+            // A box is a bulk group of its own, and box_it the number of the buffer that the next one takes: all but the newest
+            // group have then been read before a buffer is written again.
             auto store_box = [&](int pnl, const uint32_t *w) {
                 const uint32_t sb = my_staging + (BOXES == 2 ? (box_it & 1u) * (2 * PANEL_BYTES) : 0u);
                 ++box_it;
@@ -776,9 +778,13 @@ product(const CUtensorMap &map_a, const CUtensorMap &map_b, const CUtensorMap &m
                 group_sync();
                 if (elect) {
                     put_box(my_staging, pnl);
-                    if (two) put_box(my_staging + 2 * PANEL_BYTES, pnl + 1);
                     tma_store_commit();
+                    if (two) {
+                        put_box(my_staging + 2 * PANEL_BYTES, pnl + 1);
+                        tma_store_commit();
+                    }
                 }
+                box_it = two ? 0u : 1u;
             };
             if (unit >= p.split_from && p.splits > 1) {
                 // Split-K.  The group's panels are exchanged in up to MAX_PARTS parts, which the units of a tile take in

@@ -113,3 +113,11 @@ def test_plans_of_a_model_are_kept():
             for _ in range(3):
                 step()
             assert lib.sste_debug_plan_searches() == before, layers
+
+
+@pytest.mark.parametrize("O,I,T,dt", [(640, 5120, 8192, B.BF16), (5248, 5120, 1024, B.BF16), (8064, 8448, 640, B.BF16),
+                                      (1664, 8192, 8192, B.E4M3), (768, 10240, 8192, B.E4M3)])
+def test_plans_with_whole_tiles_and_then_split_ones(O, I, T, dt):
+    """(the sizes of test_gpu_split_tail.py: a pair stores its whole tiles two boxes at a time, then its part of a split one)"""
+    bn, splits, split_from, _ = B.plan(FWD, dt, O, I, T)
+    assert bn == 224 and splits > 1 and split_from >= 74
