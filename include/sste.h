@@ -438,6 +438,12 @@ sste_status sste_debug_selftest_device_once(void);
  * the hook is armed.  Process-wide; disarm with 0. */
 sste_status sste_debug_inject_stall(int on);
 
+/* Test hook for the one-launch maxima of an FP8 layer (sste_layer_prune, sste_layer_forward).  While armed (a device address of
+ * one uint32, not NULL), every other block keeps the maximum of its part to itself, so that the others work it out in its place
+ * as they do when a block does not run, and the parts that blocks worked out besides their own are added to *taken_dev.
+ * Results are the same.  Process-wide; disarm with NULL. */
+sste_status sste_debug_withhold_maxima(void *taken_dev);
+
 #ifdef __cplusplus
 }
 #endif

@@ -34,7 +34,7 @@ EXPORTS = [
     "sste_debug_force_tile_order", "sste_debug_plan", "sste_debug_tile_coords",
     "sste_debug_mvue_groups", "sste_debug_selftest_device_once", "sste_layer_prune", "sste_layer_forward",
     "sste_layer_backward", "sste_layer_grads", "sste_layer_grads_joint", "sste_debug_joint_plan",
-    "sste_debug_plan_searches",
+    "sste_debug_plan_searches", "sste_debug_withhold_maxima",
     "sste_padded_forward", "sste_padded_backward",
 ]
 
@@ -329,6 +329,10 @@ class Context:
 
     def debug_inject_stall(self, on: bool):
         self._check(self.lib.sste_debug_inject_stall(1 if on else 0))
+
+    def debug_withhold_maxima(self, taken_dev):
+        """sste_debug_withhold_maxima: armed with a counter (an int32 tensor of one element), disarmed with None."""
+        self._check(self.lib.sste_debug_withhold_maxima(_vp(taken_dev)))
 
     def debug_force_tile_width(self, bn: int):
         self._check(self.lib.sste_debug_force_tile_width(bn))

@@ -110,3 +110,33 @@ def test_blocks_that_cannot_run_are_not_waited_for(ctx):
         assert torch.equal(_bits(wide.Xq), _bits(codes)) and torch.equal(_bits(lin.vals), _bits(vals))
         assert _slots_empty(ctx)
     assert other.poll_device_status() == 0
+
+
+# one tile of W per block, two, four; one vector of X per thread, two, four, eight
+@pytest.mark.parametrize("O,I,T", [(4736, 512, 2176), (4736, 1024, 2304), (6912, 1024, 4608), (128, 1024, 9216)])
+def test_chunks_that_others_work_out(ctx, O, I, T):
+    """Every other block keeps its maximum to itself: the others take its chunk over, and the words are empty afterwards all the same."""
+    lin = SsteLinear(ctx, _randn(O, I, 1) * 0.02, T, fp8=True)
+    lin.init_beta()
+    lin.prune()
+    X = _randn(T, I, 2)
+    lin.forward(X)
+    want = [t.clone() for t in (lin.amax, lin.vals, lin.meta, lin.w_dense, lin.Xq, lin.Y)]
+    taken = torch.zeros(1, dtype=torch.int32, device="cuda")
+    tiles = O // 32 * (I // 128)
+    chunks = -(-tiles // (1 if tiles <= 592 else 2 if tiles <= 1184 else 4))
+    vectors = T * I // 8
+    chunks_x = -(-vectors // (512 * next(v for v in (1, 2, 4, 8) if vectors <= 296 * 512 * v)))
+    ctx.debug_withhold_maxima(taken)
+    try:
+        for _ in range(20):
+            lin.amax.zero_(), lin.vals.zero_(), lin.meta.zero_(), lin.w_dense.zero_(), lin.Xq.zero_(), taken.zero_()
+            lin.prune()
+            pruned = taken.clone()
+            lin.forward(X)
+            assert int(pruned) >= chunks // 2 and int(taken) - int(pruned) >= chunks_x // 2
+            assert _slots_empty(ctx)
+            for a, b in zip((lin.amax, lin.vals, lin.meta, lin.w_dense, lin.Xq, lin.Y), want):
+                assert torch.equal(_bits(a), _bits(b))
+    finally:
+        ctx.debug_withhold_maxima(None)
