@@ -24,9 +24,8 @@
  *     completed, so stream order holds for every caller-visible effect, also
  *     between these calls and the caller's own kernels, copies and captures.
  *   - Two calls that may overlap on the device (different streams) need
- *     different contexts if either is a product, a beta or a phase of an FP8
- *     layer: the split-K workspace, the reduction scratch and the slots of a
- *     maximum that a kernel's blocks share belong to the context.
+ *     different contexts if either is a product, or if both are a beta: the
+ *     split-K workspace and the reduction scratch belong to the context.
  *   - O = out features, I = in features, T = tokens.  O, I and T must be
  *     multiples of 128 and tensor pointers 128-byte aligned, otherwise
  *     SSTE_ERR_SHAPE / SSTE_ERR_ALIGN is returned BEFORE anything is launched.
@@ -251,16 +250,21 @@ sste_status sste_quantize_fp8(sste_ctx *ctx, const void *x, size_t n, const floa
  * The buffers of one S-STE linear, as the calls above take them; the caller fills it in once and keeps it.  All pointers
  * are device memory.  op_dtype SSTE_BF16: amax, Xq, dYq and scratch are NULL.  SSTE_E4M3 (the FP8 variant, gradients
  * E5M2): amax is three floats, max|X|, max|w~|, max|dY|; Xq [T, I] E4M3 and dYq [T, O] E5M2 receive the quantised tensors;
- * scratch is 8 bytes of the caller's, zero before the first call and left zero by every call (calls on one layer are
+ * scratch is SSTE_LAYER_SCRATCH_BYTES of the caller's, and scratch_bytes says so, or 8 bytes with scratch_bytes 0 (the maximum
+ * of X or W is then always a launch of its own); zero before the first call and left zero by every call (calls on one layer are
  * stream-ordered).  w_dense NULL: grad_X works from the compressed operand.
  */
+#define SSTE_LAYER_SCRATCH_BYTES 4104
 typedef struct sste_layer {
     int O, I, T;
     int op_dtype;               /* SSTE_BF16 or SSTE_E4M3 */
     int out_dtype;              /* of Y, dX and dW: SSTE_BF16 or SSTE_F32 */
     int counter_cols;           /* see sste_mvue_sparsify */
     unsigned int tensor_id;
-    unsigned int reserved;      /* 0 */
+    union {
+        unsigned int scratch_bytes; /* SSTE_LAYER_SCRATCH_BYTES or 0 */
+        unsigned int reserved;      /* the former name: 0 */
+    };
     unsigned long long seed;
     const void *W;              /* bf16 [O, I] */
     const float *beta;

@@ -64,10 +64,13 @@ _ARGTYPES = {
 }
 
 
+LAYER_SCRATCH_BYTES = 4104      # SSTE_LAYER_SCRATCH_BYTES
+
+
 class LayerBuffers(ctypes.Structure):
     """sste_layer: the buffers of one layer, filled in once (layer.py)."""
     _fields_ = [("O", _I), ("I", _I), ("T", _I), ("op_dtype", _I), ("out_dtype", _I), ("counter_cols", _I),
-                ("tensor_id", _U32), ("reserved", _U32), ("seed", _U64), ("W", _P), ("beta", _P), ("amax", _P),
+                ("tensor_id", _U32), ("scratch_bytes", _U32), ("seed", _U64), ("W", _P), ("beta", _P), ("amax", _P),
                 ("vals", _P), ("meta", _P), ("w_dense", _P), ("gvals", _P), ("gmeta", _P), ("Xq", _P), ("dYq", _P),
                 ("Y", _P), ("dX", _P), ("dW", _P), ("scratch", _P)]
 

@@ -60,20 +60,16 @@ extern "C" sste_status sste_create(sste_ctx **out, int device, void *workspace, 
     ctx->cu_tensor_map_encode = encode;
     ctx->splitk_partials = nullptr;
     ctx->splitk_tickets = nullptr;
-    ctx->slots = nullptr;
     ctx->splitk_partial_bytes = 0;
     ctx->zero_after = nullptr;
     if (workspace_bytes > SSTE_WS_SPLITK_PARTIALS_OFF + (size_t(1) << 20)) {
         ctx->splitk_partials = reinterpret_cast<float *>(ws + SSTE_WS_SPLITK_PARTIALS_OFF);
         ctx->splitk_partial_bytes = workspace_bytes - SSTE_WS_SPLITK_PARTIALS_OFF;
     }
-    if (ctx->splitk_partials) {
-        ctx->splitk_tickets = reinterpret_cast<unsigned int *>(ws + SSTE_WS_SPLITK_TICKETS_OFF);
-        ctx->slots = ctx->splitk_tickets + SSTE_SPLITK_TICKETS;
-    }
+    if (ctx->splitk_partials) ctx->splitk_tickets = reinterpret_cast<unsigned int *>(ws + SSTE_WS_SPLITK_TICKETS_OFF);
     if (cudaMemset(ws, 0, SSTE_WS_PARTIALS_OFF) != cudaSuccess ||
         (ctx->splitk_tickets &&
-         cudaMemset(ctx->splitk_tickets, 0, SSTE_COUNTERS * sizeof(unsigned int)) != cudaSuccess) ||
+         cudaMemset(ctx->splitk_tickets, 0, SSTE_SPLITK_TICKETS * sizeof(unsigned int)) != cudaSuccess) ||
         cudaStreamSynchronize(nullptr) != cudaSuccess) {     // (a memset may return first: the next call may be on any stream)
         delete ctx;
         return SSTE_ERR_CUDA;
@@ -102,7 +98,7 @@ extern "C" sste_status sste_poll_device_status(sste_ctx *ctx, void *stream)
     // A product that gave up on a wait may have left split tiles half counted, and the word keeps only one of several
     // errors: whatever it says, the counters are zero again when this returns.
     if (word != SSTE_OK && ctx->splitk_tickets) {
-        SSTE_CUDA_TRY(cudaMemsetAsync(ctx->splitk_tickets, 0, SSTE_COUNTERS * sizeof(unsigned int), s));
+        SSTE_CUDA_TRY(cudaMemsetAsync(ctx->splitk_tickets, 0, SSTE_SPLITK_TICKETS * sizeof(unsigned int), s));
         SSTE_CUDA_TRY(cudaStreamSynchronize(s));
     }
     if (word > SSTE_ERR_TIMEOUT) return SSTE_ERR_CUDA;

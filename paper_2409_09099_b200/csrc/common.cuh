@@ -22,7 +22,6 @@ struct sste_ctx {
     float *splitk_partials;         // fp32 partial tiles of split-K products; null if the workspace is minimal
     unsigned int *splitk_tickets;   // arrival counters of the split tiles, zero between launches
     size_t splitk_partial_bytes;
-    unsigned int *slots;            // SSTE_MAX_SLOTS words of a maximum that a kernel's blocks share, zero between launches; null as splitk_tickets is
     unsigned int *zero_after;       // a word that every product empties when it starts; null but in a layer call's own copy
 };
 
@@ -31,10 +30,10 @@ constexpr size_t SSTE_WS_STATUS_OFF = 0;
 constexpr size_t SSTE_WS_COUNTER_OFF = 64;
 constexpr size_t SSTE_WS_PARTIALS_OFF = 256;
 constexpr size_t SSTE_WS_BYTES = SSTE_WS_PARTIALS_OFF + 2 * sizeof(double) * SSTE_MAX_REDUCE_BLOCKS;
-// optional tail of the workspace: counters (of split-K products, then the slots), then partial tiles
-constexpr int SSTE_COUNTERS = 8192, SSTE_MAX_SLOTS = 1024, SSTE_SPLITK_TICKETS = SSTE_COUNTERS - SSTE_MAX_SLOTS;
+// optional tail of the workspace, used by split-K products: arrival counters, then partial tiles
+constexpr int SSTE_SPLITK_TICKETS = 8192;
 constexpr size_t SSTE_WS_SPLITK_TICKETS_OFF = (SSTE_WS_BYTES + 1023) / 1024 * 1024;
-constexpr size_t SSTE_WS_SPLITK_PARTIALS_OFF = SSTE_WS_SPLITK_TICKETS_OFF + SSTE_COUNTERS * sizeof(unsigned int);
+constexpr size_t SSTE_WS_SPLITK_PARTIALS_OFF = SSTE_WS_SPLITK_TICKETS_OFF + SSTE_SPLITK_TICKETS * sizeof(unsigned int);
 // room that a dense copy of the weight in the workspace leaves to the partials: the most a plan asks for on 148 SMs
 // (73 split tiles x 4 ranges x 256 KB)
 constexpr size_t SSTE_DENSE_COPY_RESERVE = size_t(80) << 20;
@@ -166,13 +165,15 @@ sste_status sste_mvue_scratch(sste_ctx *ctx, const void *dY, int T, int O, uint6
 sste_status sste_project_amax_scratch(sste_ctx *ctx, const void *W, int O, int I, const float *beta_dev, float *amax_dev,
                                       void *scratch, void *stream);
 
+// words of a maximum that a kernel's blocks share: the tail of a layer's scratch, zero between launches
+constexpr int SSTE_MAX_SLOTS = (SSTE_LAYER_SCRATCH_BYTES - 8) / 4;
 // sste_amax and sste_quantize_fp8 (E4M3) in one launch, where the tensor is small enough.
 bool sste_amax_quantize_fits(const sste_ctx *ctx, size_t n);
-sste_status sste_amax_quantize(sste_ctx *ctx, const void *x, size_t n, float *amax_dev, void *q, void *stream);
+sste_status sste_amax_quantize(sste_ctx *ctx, const void *x, size_t n, float *amax_dev, unsigned int *slots, void *q, void *stream);
 // The same for sste_project_amax and sste_project_compress (E4M3).
 bool sste_project_fp8_fits(const sste_ctx *ctx, int O, int I);
-sste_status sste_project_fp8(sste_ctx *ctx, const void *W, int O, int I, const float *beta_dev, float *amax_dev, void *vals,
-                             void *meta, void *dense_out, void *stream);
+sste_status sste_project_fp8(sste_ctx *ctx, const void *W, int O, int I, const float *beta_dev, float *amax_dev, unsigned int *slots,
+                             void *vals, void *meta, void *dense_out, void *stream);
 
 // grad_W and grad_X of a layer (the two products behind sste_linear_bwd_weight and sste_linear_bwd_input, same arguments), in
 // one launch where that is possible.

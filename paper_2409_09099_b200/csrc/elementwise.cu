@@ -1141,7 +1141,7 @@ quantize_kernel(const uint4 *__restrict__ x, size_t n_chunks, const AmaxIn amax,
 // ---------------------------------------------------------------- maximum of a tensor, then what is quantised with it, in one launch
 
 // Block b keeps chunk b of the tensor in registers and leaves the chunk's maximum (its bits with the lowest set: bf16
-// magnitudes end in zeros) in slot b of the context.  Block 0 reads the slots until none is empty and leaves the tensor's maximum in
+// magnitudes end in zeros) in slot b of the layer's scratch.  Block 0 reads the slots until none is empty and leaves the tensor's maximum in
 // one more word, which the others wait for; then each goes on with its chunk.  A word is both value and flag, so reading it needs
 // no order: a store, and a load that finds it.  (All blocks reading all slots held the stores up: 13 us for the weight of 3072 x
 // 768, 8 us in two launches.  A maximum and a count by atomics, with a fence between: 7.5 us, and 9.5 us instead of 8.6 for a
@@ -1951,14 +1951,14 @@ extern "C" sste_status sste_debug_withhold_maxima(void *taken_dev)
 bool sste_amax_quantize_fits(const sste_ctx *ctx, size_t n)
 {
     const size_t blocks = static_cast<size_t>(ctx->sm_count) * 2;
-    return ctx->slots && blocks <= GM_SLOTS && n >= (size_t(1) << 20) && n / 8 <= blocks * AQ_THREADS * 8;
+    return blocks <= GM_SLOTS && n >= (size_t(1) << 20) && n / 8 <= blocks * AQ_THREADS * 8;
 }
 
-sste_status sste_amax_quantize(sste_ctx *ctx, const void *x, size_t n, float *amax_dev, void *q, void *stream)
+sste_status sste_amax_quantize(sste_ctx *ctx, const void *x, size_t n, float *amax_dev, unsigned int *slots, void *q, void *stream)
 {
-    if (!ctx || !x || !amax_dev || !q) return SSTE_ERR_INVALID_ARG;
+    if (!ctx || !x || !amax_dev || !slots || !q) return SSTE_ERR_INVALID_ARG;
     if (n == 0 || n % 16 != 0 || !sste_amax_quantize_fits(ctx, n)) return SSTE_ERR_SHAPE;
-    if (!sste_aligned(x, 16) || !sste_aligned(amax_dev, 4) || !sste_aligned(q, 16)) return SSTE_ERR_ALIGN;
+    if (!sste_aligned(x, 16) || !sste_aligned(amax_dev, 4) || !sste_aligned(slots, 4) || !sste_aligned(q, 16)) return SSTE_ERR_ALIGN;
     sste_device_guard guard(ctx->device);
     if (!guard.ok) return SSTE_ERR_CUDA;
     const size_t n_vec = n / 8;
@@ -1968,7 +1968,7 @@ sste_status sste_amax_quantize(sste_ctx *ctx, const void *x, size_t n, float *am
     while (chunks() > static_cast<size_t>(ctx->sm_count) * 2) v *= 2;
     auto kern = v == 1 ? amax_quantize_kernel<1> : v == 2 ? amax_quantize_kernel<2> : v == 4 ? amax_quantize_kernel<4> : amax_quantize_kernel<8>;
     sste_launch(kern, dim3(static_cast<unsigned int>(chunks())), dim3(AQ_THREADS), 0, static_cast<cudaStream_t>(stream),
-                static_cast<const uint4 *>(x), n_vec, amax_dev, ctx->slots, static_cast<uint2 *>(q), ctx->status_dev, g_taken_test);
+                static_cast<const uint4 *>(x), n_vec, amax_dev, slots, static_cast<uint2 *>(q), ctx->status_dev, g_taken_test);
     return launch_result();
 }
 
@@ -1978,7 +1978,7 @@ namespace {
 int project_fp8_tiles(const sste_ctx *ctx, int O, int I)
 {
     const long long tiles = static_cast<long long>(I / 128) * (O / PC_ROWS), sms = ctx->sm_count;
-    if (!ctx->slots || sms * 4 > GM_SLOTS) return 0;
+    if (sms * 4 > GM_SLOTS) return 0;
     return tiles <= sms * 4 ? 1 : tiles <= sms * 8 ? 2 : tiles <= sms * 12 ? 4 : 0;
 }
 
@@ -1986,13 +1986,13 @@ int project_fp8_tiles(const sste_ctx *ctx, int O, int I)
 
 bool sste_project_fp8_fits(const sste_ctx *ctx, int O, int I) { return project_fp8_tiles(ctx, O, I) != 0; }
 
-sste_status sste_project_fp8(sste_ctx *ctx, const void *W, int O, int I, const float *beta_dev, float *amax_dev, void *vals,
-                             void *meta, void *dense_out, void *stream)
+sste_status sste_project_fp8(sste_ctx *ctx, const void *W, int O, int I, const float *beta_dev, float *amax_dev, unsigned int *slots,
+                             void *vals, void *meta, void *dense_out, void *stream)
 {
-    if (!ctx || !W || !beta_dev || !amax_dev || !vals || !meta) return SSTE_ERR_INVALID_ARG;
+    if (!ctx || !W || !beta_dev || !amax_dev || !slots || !vals || !meta) return SSTE_ERR_INVALID_ARG;
     if (!sste_mult128(O) || !sste_mult128(I) || !sste_project_fp8_fits(ctx, O, I)) return SSTE_ERR_SHAPE;
     if (!sste_aligned(W, 128) || !sste_aligned(vals, 128) || !sste_aligned(meta, 128) || !sste_aligned(dense_out, 128) ||
-        !sste_aligned(amax_dev, 4))
+        !sste_aligned(amax_dev, 4) || !sste_aligned(slots, 4))
         return SSTE_ERR_ALIGN;
     sste_device_guard guard(ctx->device);
     if (!guard.ok) return SSTE_ERR_CUDA;
@@ -2000,7 +2000,7 @@ sste_status sste_project_fp8(sste_ctx *ctx, const void *W, int O, int I, const f
     const uint32_t tiles = static_cast<uint32_t>(I / 128) * static_cast<uint32_t>(O / PC_ROWS), chunks = (tiles + r - 1) / r;
     auto kern = r == 1 ? project_fp8_kernel<1> : r == 2 ? project_fp8_kernel<2> : project_fp8_kernel<4>;
     sste_launch(kern, dim3(chunks), dim3(EW_THREADS), 0, static_cast<cudaStream_t>(stream), static_cast<const uint4 *>(W), I, tiles, beta_dev,
-                amax_dev, ctx->slots, vals, static_cast<uint8_t *>(meta), dense_out, ctx->status_dev, g_taken_test);
+                amax_dev, slots, vals, static_cast<uint8_t *>(meta), dense_out, ctx->status_dev, g_taken_test);
     return launch_result();
 }
 

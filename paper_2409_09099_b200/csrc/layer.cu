@@ -27,6 +27,12 @@ sste_status phase_ok(const sste_layer *l, int T, std::initializer_list<const voi
         if (!sste_aligned(b, 128)) return SSTE_ERR_ALIGN;
     return fp8_of(l) && (!sste_aligned(l->amax, 4) || !sste_aligned(l->scratch, 8)) ? SSTE_ERR_ALIGN : SSTE_OK;
 }
+// Where the blocks of a one-launch maximum leave theirs, behind the scratch's first 8 bytes; null if there is no room.
+unsigned int *slots_of(const sste_layer *l)
+{
+    return l->scratch_bytes == SSTE_LAYER_SCRATCH_BYTES ? static_cast<unsigned int *>(l->scratch) + 2 : nullptr;
+}
+
 bool out_dtype_ok(const sste_layer *l) { return l->out_dtype == SSTE_BF16 || l->out_dtype == SSTE_F32; }
 
 sste_status forward_ok(const sste_layer *l, const void *X)
@@ -68,8 +74,8 @@ extern "C" sste_status sste_layer_prune(sste_ctx *ctx, const sste_layer *l, void
     if (!fp8_of(l))
         return sste_project_compress(ctx, l->W, l->O, l->I, SSTE_BF16, l->beta, nullptr, SSTE_BF16, l->vals, l->meta, l->w_dense,
                                      stream);
-    if (sste_project_fp8_fits(ctx, l->O, l->I))
-        return sste_project_fp8(ctx, l->W, l->O, l->I, l->beta, l->amax + 1, l->vals, l->meta, l->w_dense, stream);
+    if (slots_of(l) && sste_project_fp8_fits(ctx, l->O, l->I))
+        return sste_project_fp8(ctx, l->W, l->O, l->I, l->beta, l->amax + 1, slots_of(l), l->vals, l->meta, l->w_dense, stream);
     sste_status st = sste_project_amax_scratch(ctx, l->W, l->O, l->I, l->beta, l->amax + 1, l->scratch, stream);
     if (st != SSTE_OK) return st;
     return sste_project_compress(ctx, l->W, l->O, l->I, SSTE_BF16, l->beta, l->amax + 1, SSTE_E4M3, l->vals, l->meta, l->w_dense,
@@ -86,8 +92,8 @@ extern "C" sste_status sste_layer_forward(sste_ctx *ctx, const sste_layer *l, co
         x_amax = l->amax;
         w_amax = l->amax + 1;
         const size_t n = static_cast<size_t>(l->T) * l->I;
-        if (sste_amax_quantize_fits(ctx, n)) {
-            const sste_status st = sste_amax_quantize(ctx, X, n, x_amax, l->Xq, stream);
+        if (slots_of(l) && sste_amax_quantize_fits(ctx, n)) {
+            const sste_status st = sste_amax_quantize(ctx, X, n, x_amax, slots_of(l), l->Xq, stream);
             if (st != SSTE_OK) return st;
             return sste_linear_fwd(ctx, l->Xq, l->T, l->vals, l->meta, l->O, l->I, SSTE_E4M3, x_amax, w_amax, l->Y,
                                    static_cast<sste_dtype>(l->out_dtype), y_amax_out_dev, stream);

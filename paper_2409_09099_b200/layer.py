@@ -81,7 +81,7 @@ class SsteLinear:
         dev, empty = W.device, torch.empty
         wdt, gdt = (B._TORCH_DT[B.E4M3], B._TORCH_DT[B.E5M2]) if fp8 else (_bf16, _bf16)
         # scalars in one zeroed tensor: beta; FP8: max|X|, max|w~| (bf16 projection), max|dY| and the amax passes' scratch
-        scalars = torch.zeros(6 if fp8 else 1, dtype=torch.float32, device=dev)
+        scalars = torch.zeros(4 + B.LAYER_SCRATCH_BYTES // 4 if fp8 else 1, dtype=torch.float32, device=dev)
         buffers = dict(
             ctx=ctx, W=W, T=T, tensor_id=tensor_id, seed=seed, fp8=fp8, O=O, I=I, counter_cols=counter_cols,
             beta=scalars[0:1] if fp8 else scalars, beta_ready=False,
@@ -96,7 +96,7 @@ class SsteLinear:
             amax=scalars[1:4] if fp8 else None,
             Xq=empty((T, I), dtype=wdt, device=dev) if fp8 else None,
             dYq=empty((T, O), dtype=gdt, device=dev) if fp8 else None,
-            _scratch=scalars[4:6] if fp8 else None,
+            _scratch=scalars[4:] if fp8 else None,
             _desc=None, _as_made=W.is_contiguous())
         self.__dict__.update(buffers)
         if track_flips:
@@ -124,8 +124,9 @@ class SsteLinear:
         if not desc.fits:
             desc.prune_there = desc.forward_there = desc.backward_there = lambda: True
             return desc
+        scratch_bytes = B.LAYER_SCRATCH_BYTES if self.fp8 and self._scratch.nbytes >= B.LAYER_SCRATCH_BYTES else 0
         d = B.LayerBuffers(self.O, self.I, self.T, B.E4M3 if self.fp8 else B.BF16, B._CODE_OF[self.Y.dtype],
-                           self.counter_cols, index(self.tensor_id) & 0xffffffff, 0, index(self.seed) & 0xffffffffffffffff,
+                           self.counter_cols, index(self.tensor_id) & 0xffffffff, scratch_bytes, index(self.seed) & 0xffffffffffffffff,
                            *[None if t is None else t.data_ptr() for t in tensors])
         lib = self.ctx.lib
         desc.buffers, desc.at, desc.x_shape, desc.g_shape = d, ctypes.addressof(d), x_shape, g_shape
@@ -157,7 +158,7 @@ class SsteLinear:
                 and self.Y.shape == g_shape and self.dX.shape == x_shape and tuple(self.dW.shape) == w_shape
                 and self.dX.dtype is self.Y.dtype and self.dW.dtype is self.Y.dtype
                 and (not self.fp8 or (self.amax.dtype is torch.float32 and self.amax.numel() == 3
-                                      and self._scratch.nbytes == 8 and self.Xq.dtype is wdt and self.Xq.shape == x_shape
+                                      and self._scratch.nbytes >= 8 and self.Xq.dtype is wdt and self.Xq.shape == x_shape
                                       and self.dYq.dtype is gdt and self.dYq.shape == g_shape)))
 
     def _amax(self, k):

@@ -64,3 +64,10 @@ def test_product_path_never_imports_the_oracle():
             if f.endswith((".py", ".cu", ".cuh", ".h")):
                 src = open(os.path.join(dirpath, f)).read()
                 assert not re.search(r"^\s*(from|import)\s+oracle|sste_oracle|libsste_oracle", src, flags=re.M), f
+
+
+def test_layer_scratch_size():
+    from paper_2409_09099_b200 import binding
+    text = open(os.path.join(ROOT, "include", "sste.h")).read()
+    assert f"#define SSTE_LAYER_SCRATCH_BYTES {binding.LAYER_SCRATCH_BYTES}\n" in text
+    assert ctypes.sizeof(binding.LayerBuffers) == 7 * 4 + 4 + 8 + 14 * 8      # as before the scratch had a size

@@ -29,10 +29,10 @@ def _bits(t):
     return t.contiguous().view(torch.uint8)
 
 
-def _slots_empty(ctx):
-    """the context's counters and slots, in front of the partial tiles, are zero again"""
+def _slots_empty(ctx, *layers):
+    """the context's counters, in front of the partial tiles, and the layers' scratch are zero again"""
     torch.cuda.synchronize()
-    return not ctx.workspace[17408:17408 + 4 * 8192].any()
+    return not ctx.workspace[17408:17408 + 4 * 8192].any() and not any(lin._scratch.view(torch.int32).any() for lin in layers)
 
 
 def _check_x(ctx, X, Xq, amax):
@@ -55,7 +55,7 @@ def test_quantised_input(ctx, T, I):
     for scale in (1.0, 0.0, 0.25):
         lin.forward(X * scale)
         _check_x(ctx, X * scale, lin.Xq, lin.amax[0:1])
-        assert _slots_empty(ctx)
+        assert _slots_empty(ctx, lin)
 
 
 # O x I: one tile of 32 x 128 per block up to 592 of them, two up to 1184, four up to 1776, then two launches
@@ -74,7 +74,7 @@ def test_projected_weight(ctx, O, I, dense_copy):
         assert torch.equal(a.amax[1:2], b.amax[1:2])
         for name in ("vals", "meta") + (("w_dense",) if dense_copy else ()):
             assert torch.equal(_bits(getattr(a, name)), _bits(getattr(b, name))), name
-        assert _slots_empty(ctx)
+        assert _slots_empty(ctx, *layers)
         W.mul_(factor * 0.5)
 
 
@@ -108,7 +108,7 @@ def test_blocks_that_cannot_run_are_not_waited_for(ctx):
         lin.prune()
         torch.cuda.synchronize()
         assert torch.equal(_bits(wide.Xq), _bits(codes)) and torch.equal(_bits(lin.vals), _bits(vals))
-        assert _slots_empty(ctx)
+        assert _slots_empty(ctx, lin, wide)
     assert other.poll_device_status() == 0
 
 
@@ -135,8 +135,61 @@ def test_chunks_that_others_work_out(ctx, O, I, T):
             pruned = taken.clone()
             lin.forward(X)
             assert int(pruned) >= chunks // 2 and int(taken) - int(pruned) >= chunks_x // 2
-            assert _slots_empty(ctx)
+            assert _slots_empty(ctx, lin)
             for a, b in zip((lin.amax, lin.vals, lin.meta, lin.w_dense, lin.Xq, lin.Y), want):
                 assert torch.equal(_bits(a), _bits(b))
     finally:
         ctx.debug_withhold_maxima(None)
+
+
+def test_layers_of_one_context_side_by_side(ctx):
+    """Prunes need no context of their own (a product does): two at once leave what one after the other leaves."""
+    own = B.Context(0)
+    a, b, c = (SsteLinear(k, _randn(O, I, O) * s, 2048, seed=1, fp8=True)
+               for k, O, I, s in ((ctx, 3072, 768, 0.02), (ctx, 768, 3072, 0.7), (own, 1280, 1280, 3.0)))
+    X = _randn(2048, 1280, 5)
+    for lin in (a, b, c):
+        lin.init_beta()
+        lin.prune()
+    Y = c.forward(X).clone()
+    watched = [t for lin in (a, b) for t in (lin.amax[1:2], lin.vals, lin.meta, lin.w_dense)]
+    want = [t.clone() for t in watched]
+    side = torch.cuda.Stream()
+    for _ in range(50):
+        for t in watched:
+            t.zero_()
+        c.Y.zero_()
+        torch.cuda.synchronize()
+        a.prune()
+        with torch.cuda.stream(side):
+            b.prune()
+        c.forward(X)
+        with torch.cuda.stream(side):
+            b.prune()
+        assert _slots_empty(ctx, a, b, c)
+        assert all(torch.equal(_bits(t), _bits(w)) for t, w in zip(watched, want)) and torch.equal(_bits(c.Y), _bits(Y))
+    assert own.poll_device_status() == 0
+    own.close()
+
+
+@pytest.mark.parametrize("minimal", [False, True])
+def test_launches(minimal):
+    """One launch in front of the product where the scratch has room, whatever the workspace; two with the former 8 bytes."""
+    ctx = B.Context(0, minimal_workspace=minimal)
+    try:
+        lin = SsteLinear(ctx, _randn(256, 1024, 1) * 0.02, 1024, fp8=True)
+        X = _randn(1024, 1024, 2)
+        got = []
+        for scratch in (lin._scratch, torch.zeros(2, dtype=torch.float32, device="cuda")):
+            lin._scratch = scratch
+            lin.init_beta()
+            before = B.launch_count()
+            lin.prune()
+            pruned = B.launch_count()
+            lin.forward(X)
+            got.append((pruned - before, B.launch_count() - pruned, lin.Y.clone(), lin.vals.clone(), lin.amax.clone()))
+            assert _slots_empty(ctx, lin)
+        assert got[0][:2] == (1, 2) and got[1][:2] == (2, 3)
+        assert all(torch.equal(_bits(p), _bits(q)) for p, q in zip(got[0][2:], got[1][2:]))
+    finally:
+        ctx.close()
