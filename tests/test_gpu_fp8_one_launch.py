@@ -142,6 +142,59 @@ def test_chunks_that_others_work_out(ctx, O, I, T):
         ctx.debug_withhold_maxima(None)
 
 
+_UNUSUAL = [float("inf"), -float("inf"), float("nan"), 3.3e38, -3.3e38, 2.0 ** 127, 2.0 ** -133, -0.0]
+
+
+def _with_unusual(t, at):
+    """`t` with two unusual values in each of the groups of four `at`, every pair of them in turn"""
+    flat, pick, k = t.clone().view(-1, 4), torch.tensor(_UNUSUAL, dtype=t.dtype, device=t.device), torch.arange(len(at), device=t.device)
+    flat[list(at), 0], flat[list(at), 1] = pick[k % 8], pick[k // 8 % 8]
+    return flat.view_as(t)
+
+
+# one tile of W per block, two, four (of which the last block has fewer than four)
+@pytest.mark.parametrize("O,I", [(4736, 512), (2432, 1024), (4864, 1024), (6912, 1024)])
+@pytest.mark.parametrize("where", ["first", "last", "everywhere"])
+def test_projection_of_any_values(ctx, O, I, where):
+    groups = O * I // 4
+    at = {"first": range(64), "last": range(groups - 64, groups), "everywhere": range(5, groups, groups // 300)}[where]
+    W = _with_unusual(_randn(O, I, O) * 0.02, at)
+    layers = [SsteLinear(ctx, W, 128, fp8=True) for _ in range(2)]
+    layers[1].mark = lambda label: None               # the single calls
+    for beta in (1.5, 0.0, float("inf"), float("nan")):
+        for lin in layers:
+            lin.beta.fill_(beta)
+            lin.beta_ready = True
+            lin.prune()
+        a, b = layers
+        assert torch.equal(_bits(a.amax[1:2]), _bits(b.amax[1:2])), beta
+        for name in ("vals", "meta", "w_dense"):
+            assert torch.equal(_bits(getattr(a, name)), _bits(getattr(b, name))), (beta, name)
+        assert _slots_empty(ctx, *layers)
+
+
+# one vector of X per thread, two, four, eight
+@pytest.mark.parametrize("T,I", [(1024, 1024), (2176, 1024), (4608, 1024), (9216, 1024)])
+def test_quantisation_of_any_values(ctx, T, I):
+    lin = SsteLinear(ctx, _randn(128, I, 1) * 0.02, T, fp8=True)
+    lin.init_beta()
+    lin.prune()
+    X = _randn(T, I, T)
+    last = T * I // 4 - 1
+    for at in (range(0), range(64), range(last - 63, last + 1), range(3, last, last // 500)):
+        for values in ((0, 1, 2, 3, 4, 5, 6, 7), (3, 4, 5), (0, 3), (2, 6)):
+            Z = X.clone().view(-1, 4)
+            k = torch.arange(len(at), device="cuda")
+            Z[list(at), k % 4] = torch.tensor([_UNUSUAL[v] for v in values], dtype=X.dtype, device="cuda")[k % len(values)]
+            Z = Z.view_as(X)
+            lin.forward(Z)
+            ref_amax, ref_q = torch.empty_like(lin.amax[0:1]), torch.empty_like(lin.Xq)
+            ctx.amax(Z, ref_amax)
+            ctx.quantize_fp8(Z, ref_amax, ref_q)
+            assert torch.equal(_bits(lin.amax[0:1]), _bits(ref_amax)) and torch.equal(_bits(lin.Xq), _bits(ref_q))
+            assert _slots_empty(ctx, lin)
+
+
 def test_layers_of_one_context_side_by_side(ctx):
     """Prunes need no context of their own (a product does): two at once leave what one after the other leaves."""
     own = B.Context(0)
