@@ -335,15 +335,29 @@ __host__ __device__ constexpr uint32_t instr_desc(bool sparse, uint32_t afmt, ui
 // fastest.  The 74 tiles in flight at any time therefore cover group_m tile rows x 74 / group_m tile columns,
 // and the A rows of a band stay in L2 while the band sweeps over all of B.  group_m = m_tiles is plain
 // column-major order (all of A resident, B streamed once).
+// Without integer divisions (450 clk of dependent instructions for each tile of each role): a quotient by an approximate reciprocal,
+// put right by its remainder, whatever the numbers (FP8 forward of 3072 x 768, 8192 tokens: 20.0 -> 18.8 us, bf16 24.1 -> 24.0).
+__host__ __device__ __forceinline__ int divide(int a, int b, int &rem)
+{
+#ifdef __CUDA_ARCH__
+    int q = static_cast<int>(__fdividef(static_cast<float>(a), static_cast<float>(b)));
+#else
+    int q = static_cast<int>(static_cast<float>(a) / static_cast<float>(b));
+#endif
+    rem = a - q * b;
+    while (rem < 0) { --q; rem += b; }
+    while (rem >= b) { ++q; rem -= b; }
+    return q;
+}
 __host__ __device__ __forceinline__ void tile_coords(int tile, int m_tiles, int n_tiles, int group_m, int &mt, int &nt)
 {
-    const int per_band = group_m * n_tiles;
-    const int band = tile / per_band;
-    const int first = band * group_m;
-    const int rows = (m_tiles - first < group_m) ? (m_tiles - first) : group_m;
-    const int within = tile - band * per_band;
-    mt = first + within % rows;
-    nt = within / rows;
+    int within = tile, first = 0, rows = group_m;
+    if (group_m < m_tiles) {
+        first = divide(tile, group_m * n_tiles, within) * group_m;
+        rows = (m_tiles - first < group_m) ? m_tiles - first : group_m;
+    }
+    nt = divide(within, rows, mt);
+    mt += first;
 }
 
 struct GemmParams {
@@ -468,25 +482,6 @@ product(const CUtensorMap &map_a, const CUtensorMap &map_b, const CUtensorMap &m
     // Work units: tiles [0, split_from) are whole; every later tile is cut into `splits` K ranges that differ by
     // at most one stage.  Whole tiles fill complete waves, the split ones spread the last, partial wave over all pairs.
     const int num_units = p.split_from + (num_tiles - p.split_from) * p.splits;
-    // tile_coords without its integer divisions (450 clk of dependent instructions for each tile of each role): the quotient by an
-    // approximate reciprocal, put right by its remainder, whatever the numbers (FP8 forward of 3072 x 768, 8192 tokens: 20.0 ->
-    // 18.8 us, bf16 24.1 -> 24.0)
-    auto divide = [](int a, int b, int &rem) {
-        int q = static_cast<int>(__fdividef(static_cast<float>(a), static_cast<float>(b)));
-        rem = a - q * b;
-        while (rem < 0) { --q; rem += b; }
-        while (rem >= b) { ++q; rem -= b; }
-        return q;
-    };
-    auto coords = [&](int tile, int &mt, int &nt) {
-        int within = tile, first = 0, rows = p.group_m;
-        if (p.group_m < m_tiles) {
-            first = divide(tile, p.group_m * n_tiles, within) * p.group_m;
-            rows = min(m_tiles - first, p.group_m);
-        }
-        nt = divide(within, rows, mt);
-        mt += first;
-    };
     struct Unit { int tile, split, kb0, kb1; };
     auto decode = [&](int unit) {
         Unit u;
@@ -510,7 +505,7 @@ product(const CUtensorMap &map_a, const CUtensorMap &map_b, const CUtensorMap &m
             for (int j = 0, unit = seq.first(); unit < num_units && ok; ++j, unit = seq.next(unit, j)) {
                 const Unit u = decode(unit);
                 int mt, nt;
-                coords(u.tile, mt, nt);
+                tile_coords(u.tile, m_tiles, n_tiles, p.group_m, mt, nt);
                 const int m0 = mt * 2 * BM + static_cast<int>(rank) * BM;      // this CTA's rows of A
                 const int n0 = nt * BN + static_cast<int>(rank) * (BN / 2);    // this CTA's half of B
                 // rows beyond M (zero-filled values) take the codes of the last row block: zero is not one of the six codes
@@ -673,7 +668,7 @@ product(const CUtensorMap &map_a, const CUtensorMap &map_b, const CUtensorMap &m
         for (int unit = seq.first(); unit < num_units; ++local_tile, unit = seq.next(unit, local_tile)) {
             const Unit u = decode(unit);
             int mt, nt;
-            coords(u.tile, mt, nt);
+            tile_coords(u.tile, m_tiles, n_tiles, p.group_m, mt, nt);
             const int m0 = mt * 2 * BM + static_cast<int>(rank) * BM;
             const int n0 = nt * BN;
             const uint32_t buf = local_tile % NB, use = local_tile / NB;
@@ -1032,7 +1027,7 @@ product(const CUtensorMap &map_a, const CUtensorMap &map_b, const CUtensorMap &m
             if (e_unit >= num_units) return;
             const Unit u = decode(e_unit);
             int mt, nt;
-            coords(u.tile, mt, nt);
+            tile_coords(u.tile, m_tiles, n_tiles, p.group_m, mt, nt);
             const int n0 = nt * BN + static_cast<int>(rank) * (BN / 2);
             e_cols = n0 < p.N;
             e_vals = p.b_vals + (static_cast<size_t>(n0 / 2) + seg * (EPU / 2)) * ELT + r0 * row_bytes;

@@ -36,6 +36,19 @@ def test_tile_order_is_a_bijection(lib, m_tiles, n_tiles, group_m):
     assert lib.sste_debug_tile_coords(m_tiles * n_tiles, m_tiles, n_tiles, group_m, ctypes.byref(mt), ctypes.byref(nt)) == B.ERR_INVALID_ARG
 
 
+@pytest.mark.parametrize("m_tiles,n_tiles,group_m", [(43, 64, 43), (43, 64, 6), (4000, 3000, 7), (40000, 41000, 4001), (1, 1 << 30, 1)])
+def test_tile_coordinates_of_any_number(lib, m_tiles, n_tiles, group_m):
+    """The kernels' own division (by an approximate quotient, put right): numbers that a float holds and ones that it does not."""
+    mt, nt = ctypes.c_int(), ctypes.c_int()
+    tiles, per_band = m_tiles * n_tiles, group_m * n_tiles
+    for base in {0, per_band, per_band * (m_tiles // group_m), tiles // 3, tiles // 2, tiles - 1, (1 << 24) % tiles, ((1 << 24) + 1) % tiles}:
+        for tile in range(max(0, base - 40), min(tiles, base + 40)):
+            assert lib.sste_debug_tile_coords(tile, m_tiles, n_tiles, group_m, ctypes.byref(mt), ctypes.byref(nt)) == B.OK
+            band, within = divmod(tile, per_band)
+            rows = min(group_m, m_tiles - band * group_m)
+            assert (mt.value, nt.value) == (band * group_m + within % rows, within // rows), tile
+
+
 def test_column_major_order_when_the_band_is_everything(lib):
     mt, nt = ctypes.c_int(), ctypes.c_int()
     for tile in range(35):
