@@ -289,9 +289,11 @@ sste_status sste_layer_backward(sste_ctx *ctx, const sste_layer *layer, const vo
  * grad_W's tiles leave idle start on grad_X's.  (The split of grad_W's reduction may then differ from the single call's: same
  * sums, other rounding.)  Otherwise one product follows the other. */
 sste_status sste_layer_grads(sste_ctx *ctx, const sste_layer *layer, const void *X, const void *dY, void *stream);
-/* 1 if sste_layer_grads takes one launch for this layer and that also beats two side by side, 0 otherwise: a caller with a second
- * stream and context of its own may then put sste_linear_bwd_weight there beside sste_linear_bwd_input here.  Host only. */
+/* 1 if sste_layer_grads takes one launch for this layer, 0 if two.  Host only. */
 int sste_layer_grads_joint(const sste_ctx *ctx, const sste_layer *layer);
+/* For a caller with a second stream and a context of its own: 1 if sste_linear_bwd_weight goes there beside sste_linear_bwd_input
+ * here, 0 if sste_layer_grads takes one launch that is clearly ahead of the two side by side.  Host only. */
+int sste_layer_grads_beside(const sste_ctx *ctx, const sste_layer *layer);
 
 /*
  * A layer of ANY shape (see sste_pad_2d): `inner` is the layer of the padded sizes, O, I, T the real ones.  Xp [inner.T,

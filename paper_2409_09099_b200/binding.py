@@ -33,7 +33,7 @@ EXPORTS = [
     "sste_decompress", "sste_padded_dim", "sste_pad_2d", "sste_crop_2d", "sste_debug_inject_stall",
     "sste_debug_force_tile_order", "sste_debug_plan", "sste_debug_tile_coords",
     "sste_debug_mvue_groups", "sste_debug_selftest_device_once", "sste_layer_prune", "sste_layer_forward",
-    "sste_layer_backward", "sste_layer_grads", "sste_layer_grads_joint", "sste_debug_joint_plan",
+    "sste_layer_backward", "sste_layer_grads", "sste_layer_grads_joint", "sste_layer_grads_beside", "sste_debug_joint_plan",
     "sste_debug_plan_searches", "sste_debug_withhold_maxima",
     "sste_padded_forward", "sste_padded_backward",
 ]
@@ -59,6 +59,7 @@ _ARGTYPES = {
     "sste_layer_backward": [_P, _P, _P, _P, _U32, _U64, _P],
     "sste_layer_grads": [_P, _P, _P, _P, _P],
     "sste_layer_grads_joint": [_P, _P],
+    "sste_layer_grads_beside": [_P, _P],
     "sste_padded_forward": [_P, _P, _P, _P],
     "sste_padded_backward": [_P, _P, _P, _U32, _U64, _P],
 }

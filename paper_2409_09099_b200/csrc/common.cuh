@@ -181,8 +181,9 @@ sste_status sste_bwd_products(sste_ctx *ctx, const void *gvals, const void *gmet
                               int T, sste_dtype gdt, sste_dtype wdt, const void *w_dense, const void *vals, const void *meta,
                               const float *g_amax, const float *x_amax, const float *w_amax, void *dW, void *dX,
                               sste_dtype odt, void *stream);
-// Whether one launch also beats the two side by side on two streams, for these sizes (multiples of 128; elt: bytes of an operand's element).
-bool sste_bwd_in_one_launch(const sste_ctx *ctx, int elt, int O, int I, int T, bool dense_copy, sste_dtype odt);
+// Whether that is one launch for these sizes (multiples of 128; elt: bytes of an operand's element); beside: whether it also beats the
+// two side by side on two streams.
+bool sste_bwd_in_one_launch(const sste_ctx *ctx, int elt, int O, int I, int T, bool dense_copy, sste_dtype odt, bool beside);
 
 // two sste_crop_2d in one launch (arguments as checked by that call)
 sste_status sste_crop_two(sste_ctx *ctx, const void *src0, int rows_p0, int cols_p0, void *dst0, int rows0, int cols0,

@@ -1950,13 +1950,13 @@ extern "C" sste_status sste_linear_bwd_input(sste_ctx *ctx, const void *dY, int 
     return launch_out<GRAD_INPUT, 1>(ctx, dY, Wt_dense, nullptr, p, xdt, s);
 }
 
-bool sste_bwd_in_one_launch(const sste_ctx *ctx, int elt, int O, int I, int T, bool dense_copy, sste_dtype odt)
+bool sste_bwd_in_one_launch(const sste_ctx *ctx, int elt, int O, int I, int T, bool dense_copy, sste_dtype odt, bool beside)
 {
     size_t partial_bytes = ctx->splitk_partials ? ctx->splitk_partial_bytes : 0;
     if (odt != SSTE_BF16 || test_hook_set()) return false;
     if (!dense_copy && !dense_copy_in_workspace(ctx, O, I, elt, &partial_bytes)) return false;
     JointPlan plan;
-    return joint_wins(ctx, elt, partial_bytes, O, I, T, true, &plan);
+    return joint_wins(ctx, elt, partial_bytes, O, I, T, beside, &plan);
 }
 
 sste_status sste_bwd_products(sste_ctx *ctx, const void *gvals, const void *gmeta, const void *X, const void *dY, int O, int I,

@@ -151,12 +151,17 @@ extern "C" sste_status sste_layer_grads(sste_ctx *ctx, const sste_layer *l, cons
                              static_cast<sste_dtype>(l->out_dtype), stream);
 }
 
-extern "C" int sste_layer_grads_joint(const sste_ctx *ctx, const sste_layer *l)
+namespace {
+bool one_launch(const sste_ctx *ctx, const sste_layer *l, bool beside)
 {
-    if (!ctx || !layer_ok(l) || !sste_mult128(l->O) || !sste_mult128(l->I) || !sste_mult128(l->T)) return 0;
+    if (!ctx || !layer_ok(l) || !sste_mult128(l->O) || !sste_mult128(l->I) || !sste_mult128(l->T)) return false;
     return sste_bwd_in_one_launch(ctx, fp8_of(l) ? 1 : 2, l->O, l->I, l->T, l->w_dense != nullptr,
-                                  static_cast<sste_dtype>(l->out_dtype));
+                                  static_cast<sste_dtype>(l->out_dtype), beside);
 }
+}  // namespace
+
+extern "C" int sste_layer_grads_joint(const sste_ctx *ctx, const sste_layer *l) { return one_launch(ctx, l, false); }
+extern "C" int sste_layer_grads_beside(const sste_ctx *ctx, const sste_layer *l) { return !one_launch(ctx, l, true); }
 
 namespace {
 

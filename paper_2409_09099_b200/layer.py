@@ -296,7 +296,7 @@ class SsteLinear:
                 desc = self._moved()
             X = None if self.fp8 else self.X
             if (desc.fits and _takes(dY, desc.g_shape) and (X is None or _takes(X, desc.x_shape))
-                    and self.ctx.lib.sste_layer_grads_joint(self.ctx.handle, desc.at)):
+                    and not self.ctx.lib.sste_layer_grads_beside(self.ctx.handle, desc.at)):
                 st = desc.grads(self.ctx.handle, desc.at, None if X is None else X.data_ptr(), dY.data_ptr(),
                                    _raw_stream(_device()))
                 if st:
