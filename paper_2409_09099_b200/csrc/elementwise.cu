@@ -834,11 +834,9 @@ struct RaggedRows {
 
 // One CTA: 4 G tokens x 64 output columns of dY.  A thread handles 4 tokens x 8 columns (8 groups, two Philox calls); results
 // are transposed through shared memory so that every output row (= column of dY) receives whole lines (G = 32, 256 threads) or halves
-// of them, the other half coming from the neighbouring CTA (G = 16, 128 threads).  Bound by instruction issue, not by HBM (15.6 us
-// is what the loads and stores of dY[8192, 3072] take alone): maxima by masks instead of chains of selections, bf16 terms of fp32
-// sums, 16-bit stores of the metadata and the draws in front of the loads' arrival took that size from 25.9 to 22.0 us in bf16, 31.6
-// to 26.2 in FP8, and dY[16384, 11008] from 166 to 142 and 201 to 168.  (Five blocks per SM: 23.4 us; tasks of 4 columns or two
-// tasks of 128, and persistent CTAs with cp.async prefetch, were slower too.)
+// of them, the other half coming from the neighbouring CTA (G = 16, 128 threads).  Bound by instruction issue, not by HBM: dY[8192,
+// 3072] takes 22.0 us in bf16 (25.9 with the rule by selections), of which the loads and stores alone take 15.6, and 26.2 in FP8 (31.6);
+// five blocks per SM 23.4.
 // ANY_COUNTER: counter_cols is not a multiple of 4 (a padded, odd column count), so a thread's eight
 // consecutive group indices do not start on a Philox block and span three blocks instead of two.
 // PADDED: dY is given as ragged rows; the kernel also writes the zero-padded copy that grad_X reads (a padding pass of its
@@ -1143,9 +1141,8 @@ quantize_kernel(const uint4 *__restrict__ x, size_t n_chunks, const AmaxIn amax,
 // Block b keeps chunk b of the tensor in registers and leaves the chunk's maximum (its bits with the lowest set: bf16
 // magnitudes end in zeros) in slot b of the layer's scratch.  Block 0 reads the slots until none is empty and leaves the tensor's maximum in
 // one more word, which the others wait for; then each goes on with its chunk.  A word is both value and flag, so reading it needs
-// no order: a store, and a load that finds it.  (All blocks reading all slots held the stores up: 13 us for the weight of 3072 x
-// 768, 8 us in two launches.  A maximum and a count by atomics, with a fence between: 7.5 us, and 9.5 us instead of 8.6 for a
-// forward of 256 x 256 with 512 tokens.)  A block that has waited for a while reads the slots itself and works out the missing
+// no order: a store, and a load that finds it.  (Weight of 3072 x 768: two launches 8 us, all blocks reading all slots 13, atomics with
+// a fence 7.5, this 6.)  A block that has waited for a while reads the slots itself and works out the missing
 // chunks (a maximum may be left twice, a code written twice), so no block depends on another one running: the launch needs no
 // guarantee that all its blocks run at the same time, which a collective beside it could hold up.  The last block empties the
 // words.  That does need an order: a slot may hold somebody else's value by then while its owner's store is still on its way, so a

@@ -71,9 +71,8 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t byt
 }
 // Arrive on a barrier that may live in the peer CTA (shared::cluster address).  CLUSTER: what this thread wrote to shared memory is
 // for the peer too.  Without it the arrival only says that something has been read (tensor memory, behind its own fence), and
-// need not wait until the thread's writes are visible in the cluster.  (With cluster scope on every arrival and wait, a forward of 3072 x
-// 768 with 8192 tokens took 26.8 us in bf16 and 23.5 in FP8, now 24.1 and 20.0; with 128 tokens 7.4 and 6.8; a shape whose
-// epilogue sets the pace gains most: 1024 x 50304 60 -> 55.)
+// need not wait until the thread's writes are visible in the cluster (cluster scope everywhere: forward of 3072 x 768, 8192 tokens,
+// bf16 26.8 us, so 24.1).
 template <bool CLUSTER>
 __device__ __forceinline__ void mbar_arrive_at(uint32_t cluster_addr)
 {
@@ -605,8 +604,8 @@ product(const CUtensorMap &map_a, const CUtensorMap &map_b, const CUtensorMap &m
     } else if (warp < 2 + C::EPI_WARPS) {
         // ------------------------------------------------------------ epilogue (warps 2.., both CTAs)
         // A warp owns 32 rows and a range of columns (half of them with eight warps) of the accumulator from tensor memory
-        // to the output.  Its part is pulled into registers (packed bf16) and the accumulator released before the first
-        // store, so that the next main loop waits for the tensor-memory reads only.
+        // to the output, two panels of 32 columns at a time: pulled into registers (packed bf16), staged and stored.  The
+        // accumulator is released when the last panels are in registers, before they are stored; the next main loop has the other one.
         // What leaves is whole 128-byte lines: a row-major output by boxes of 32 rows x 64 columns of one warp, a transposed
         // one by boxes of 64 rows x 32 columns of a pair of warps (a warp alone has 64 bytes of each output row).  Half
         // lines by TMA were 2-3 % slower (3840 x 1280, 16384 tokens, bf16 forward: 82 -> 80 us), by plain stores 25 %.
@@ -1340,9 +1339,10 @@ constexpr Widths widths_of(Product pr, int elt)
     return pr == FORWARD ? Widths{{256, 224, 192, 128}} : elt == 2 ? Widths{{256, 128, 0, 0}} : Widths{{256, 0, 0, 0}};
 }
 
-// Microseconds of one stage of the main loop and what a tile costs besides (tensor-memory reads that the next main loop
-// waits for, the output's share of the L2 traffic), all CTA pairs busy; fitted to timings of every width on B200 at
-// K = 768 ... 16384.  A narrower tile moves more operand bytes per flop, a wider one quantises worse into waves.
+// Microseconds of one stage of the main loop and what a tile costs besides (the part of the epilogue that is not hidden, the
+// output's share of the L2 traffic), all CTA pairs busy; fitted to timings of every width on B200 at K = 768 ... 16384.  (Fitted when a
+// 256-wide sparse tile had one accumulator, and before the epilogue's and the coordinates' share fell: tiles cost less than this by
+// now, most of all those; the choice between widths has not been fitted again.)  A narrower tile moves more operand bytes per flop, a wider one quantises worse into waves.
 struct TileCost { double stage_us, tile_us; };
 constexpr TileCost tile_cost(Product pr, int elt, int bn)
 {
@@ -1481,7 +1481,7 @@ struct JointPlan { LaunchPlan w, x; int pairs; GradsPlan g; double us; };
 // grad_W units go round the pairs; the last, partial round leaves `late` pairs busy for one unit more.  For every width,
 // split and number of early rounds the model gives the time at which the last pair ends; a pair that changes over from one
 // product to the other drains and refills its pipeline (SWITCH_US, about what a kernel boundary costs).
-constexpr double SWITCH_US = 2.5, SUM_WAIT_US = 1.5, LAUNCH_US = 3.0;      // (a second launch: what a product of one stage takes besides it)
+constexpr double SWITCH_US = 2.5, SUM_WAIT_US = 1.5;
 JointPlan find_joint_plan(int elt, int sm_count, size_t partial_bytes, int O, int I, int T)
 {
     const int max_pairs = sm_count / 2;
@@ -1744,18 +1744,17 @@ void *dense_copy_in_workspace(const sste_ctx *ctx, int O, int I, int elt, size_t
 bool test_hook_set() { return g_inject_stall || g_force_bn || g_force_splits || g_force_group_m; }
 
 // The plan of both gradient products in one launch; whether that beats two in a row, or (beside) two side by side on two streams.
-// Two win where the second launch and its own last wave cost less than what tiles lose beside the other product's, some 3 % (6016 x
-// 1152, 5504 tokens, bf16: 100 us apart, 104 together; 5248 x 768, 8832 tokens: 88 and 94; 3840 x 1280, 16384 tokens: 183 and 168; 1280 x
-// 5120, 16384: 237 and 227; 2560 x 1280, 640: 22 and 19).  The line was drawn over 146 shapes timed both ways; with 10 % in place of 3 %
-// and 2 us, 66 of them went the wrong way, by 9 % on the mean.  A caller that offers a second stream keeps it unless one launch is clearly
-// ahead (4 %, without the 2 us: 22 of the 146 go the other way than with 10 %, 10 % faster on the mean: 1280 x 5120, 8192 tokens 126 -> 119,
-// 512 x 7040, 1792 tokens 28.7 -> 21.6; the other line would be faster on most of the rest too, but such callers count on their stream).
+// Two win where the second launch and its own last wave, 5 us, cost less than what tiles lose beside the other product's, some 3 %
+// (bf16: 6016 x 1152, 5504 tokens 100 us apart, 104 together; 3840 x 1280, 16384 tokens 183 and 168); the line was drawn over 146
+// shapes timed both ways.  A caller that offers a second stream keeps it unless one launch is clearly ahead (512 x 7040, 1792 tokens
+// 28.7 us side by side, 21.6 together).  That line is not the fastest one: of the 61 shapes that stay side by side most take 8 % less in
+// one launch.
 bool joint_wins(const sste_ctx *ctx, int elt, size_t partial_bytes, int O, int I, int T, bool beside, JointPlan *plan)
 {
     *plan = make_joint_plan(elt, ctx->sm_count, partial_bytes, O, I, T);
     const double apart = make_plan(GRAD_WEIGHT, elt, 0, false, false, ctx->sm_count, partial_bytes, O, I, T).us +
-                         make_plan(GRAD_INPUT, elt, 0, false, false, ctx->sm_count, partial_bytes, T, I, O, true).us + LAUNCH_US;
-    return beside ? 1.04 * plan->us <= apart : 1.03 * plan->us <= apart + 2.0;
+                         make_plan(GRAD_INPUT, elt, 0, false, false, ctx->sm_count, partial_bytes, T, I, O, true).us;
+    return beside ? 1.04 * plan->us <= apart + 3.0 : 1.03 * plan->us <= apart + 5.0;
 }
 
 // FP8 operands come with the amax of the tensors they were quantised from (both or neither); bf16 with none.

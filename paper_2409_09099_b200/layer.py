@@ -285,10 +285,10 @@ class SsteLinear:
 
     def grad_weight_and_input(self, dY, side_ctx: B.Context, side_stream: torch.cuda.Stream):
         """grad_W and grad_X at the same time: they are independent once MVUE has run.  Where one launch for both is the
-        faster way (bf16 results, see sste_layer_grads), it runs on the current stream and shares the SMs between them;
+        clearly faster way (bf16 results, see sste_layer_grads_beside), it runs on the current stream and shares the SMs between them;
         otherwise grad_W runs on `side_stream` (through `side_ctx`: its own split-K workspace) beside grad_X, which takes about
-        as long as one after the other (10496 x 768, 4096 tokens, FP8: 54.0 against 56.7 us; 3584 x 1024, 7168 tokens, bf16: 73.1
-        against 73.7; 5632 x 1664, 1024 tokens: 40.0 against 40.8; 8064 x 384, 4352 tokens: 53.3 against 51.0).
+        as long as one after the other (10496 x 768, 4096 tokens, FP8: 54.0 against 56.7 us; 8064 x 384, 4352 tokens: 53.3 against
+        51.0).  `backward` alone is often faster by now: it takes one launch more often.
         Both are complete in current-stream order on return."""
         if self.mark is None:
             desc = self._desc or self._describe()
