@@ -131,7 +131,17 @@ __device__ __host__ __forceinline__ uint32_t sste_meta_atom_byte8(uint32_t m, ui
 // first thing, is what lets the NEXT kernel of the stream be scheduled early (it takes effect when every CTA
 // of this grid has issued it or exited, so the successor never competes with CTAs not yet started).
 __device__ __forceinline__ void sste_pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void sste_pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// The pointers that the kernel reads through are given to the wait and come out of it as new values: data behind `const T *__restrict__`
+// or __ldg counts as constant while the kernel runs, so the compiler may otherwise load it in front of any asm statement (it did
+// so in a kernel that had a branch before the wait).
+template <typename T>
+__device__ __forceinline__ void sste_fresh(T &pointer) { asm volatile("" : "+l"(pointer) : : "memory"); }
+template <typename... T>
+__device__ __forceinline__ void sste_pdl_wait(T &...read_after)
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    (sste_fresh(read_after), ...);
+}
 
 template <typename... KArgs, typename... Args>
 inline cudaError_t sste_launch(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,

@@ -367,7 +367,7 @@ project_compress_kernel(const uint4 *__restrict__ W, int I, const float *__restr
     const int kb = blockIdx.x, rb = blockIdx.y;
     if (MODE == 0 && tid < PROJECT_ENTRIES) lut[tid] = project_table_dev.e[tid];
     sste_pdl_trigger();
-    sste_pdl_wait();
+    sste_pdl_wait(W, beta_dev, w_amax_dev);
     const size_t row_chunks = static_cast<size_t>(I) / 8;
     const ProjectOut p{W, row_chunks, *beta_dev, FP8 ? sste_scale_from_amax(*w_amax_dev, 448.0f) : 1.0f, gamma, vals, meta, dense};
     uint4 in[PC_CHUNKS];
@@ -398,7 +398,7 @@ beta_kernel(const uint4 *__restrict__ W, size_t n_chunks, double *__restrict__ p
     __shared__ double red[2][EW_THREADS / 32];
     __shared__ bool is_last;
     sste_pdl_trigger();
-    sste_pdl_wait();
+    sste_pdl_wait(W);
     double num = 0.0, den = 0.0;
     for (size_t c = static_cast<size_t>(blockIdx.x) * EW_THREADS + threadIdx.x; c < n_chunks;
          c += static_cast<size_t>(gridDim.x) * EW_THREADS) {
@@ -735,7 +735,7 @@ mvue_groups_kernel(const uint2 *__restrict__ a, const uint32_t *__restrict__ k24
     if (threadIdx.x < MVUE_ENTRIES) lut[threadIdx.x] = mvue_table_bf16.e[threadIdx.x];
     __syncthreads();
     sste_pdl_trigger();
-    sste_pdl_wait();
+    sste_pdl_wait(a, k24);
     for (size_t i = static_cast<size_t>(blockIdx.x) * EW_THREADS + threadIdx.x; i < n;
          i += static_cast<size_t>(gridDim.x) * EW_THREADS) {
         const uint2 g = a[i];
@@ -846,7 +846,7 @@ __global__ void __launch_bounds__(8 * G, G == 32 ? 4 : 8)
 mvue_kernel(const uint4 *__restrict__ dY, int O, int T, uint32_t key0, uint32_t key1, uint32_t tensor_id,
             uint32_t step, uint64_t tg_offset, uint32_t counter_cols, const AmaxIn g_amax,
             void *__restrict__ gvals,
-            uint8_t *__restrict__ gmeta, void *__restrict__ dense_q, const RaggedRows rag, uint4 *__restrict__ padded)
+            uint8_t *__restrict__ gmeta, void *__restrict__ dense_q, RaggedRows rag, uint4 *__restrict__ padded)
 {
     // 64 rows of G words (bf16) or halfwords (fp8)
     __shared__ __align__(16) uint32_t vals_s[64 * G / (FP8 ? 2 : 1)];
@@ -857,7 +857,7 @@ mvue_kernel(const uint4 *__restrict__ dY, int O, int T, uint32_t key0, uint32_t 
     const int jb = G == 32 ? blockIdx.x : blockIdx.x >> 1, tb = G == 32 ? blockIdx.y : 2 * blockIdx.y + (blockIdx.x & 1);
     if (tid < MVUE_ENTRIES) lut[tid] = FP8 ? mvue_table_fp8.e[tid] : mvue_table_bf16.e[tid];
     sste_pdl_trigger();
-    sste_pdl_wait();
+    sste_pdl_wait(dY, rag.src);
     const float gscale = FP8 ? sste_scale_from_amax(amax_take(g_amax, jb == 0 && tb == 0 && tid == 0), 57344.0f) : 1.0f;
     __syncthreads();                              // the table is in place
     const size_t row_chunks = static_cast<size_t>(O) / 8;
@@ -1028,7 +1028,7 @@ amax_kernel(const uint4 *__restrict__ x, size_t n_chunks, unsigned int *__restri
 {
     uint32_t best2 = 0;   // magnitude bits of bf16 compare like unsigned integers: running maximum in both halves
     sste_pdl_trigger();
-    sste_pdl_wait();
+    sste_pdl_wait(x);
     // four independent 16-byte loads per thread and iteration: a pure read needs the bytes in flight
     const size_t stride = static_cast<size_t>(gridDim.x) * EW_THREADS;
     for (size_t c = static_cast<size_t>(blockIdx.x) * EW_THREADS + threadIdx.x; c < n_chunks; c += 4 * stride) {
@@ -1066,7 +1066,7 @@ project_amax_kernel(const uint4 *__restrict__ W, size_t n_chunks, const float *_
                     float *__restrict__ amax_dev, unsigned int *__restrict__ scratch)
 {
     sste_pdl_trigger();
-    sste_pdl_wait();
+    sste_pdl_wait(W, beta_dev);
     const float beta = *beta_dev;
     float best = 0.0f;
     const size_t stride = static_cast<size_t>(gridDim.x) * EW_THREADS;
@@ -1093,7 +1093,7 @@ project_amax_kernel(const uint4 *__restrict__ W, size_t n_chunks, const float *_
 __global__ void fp8_scale_kernel(const float *amax_dev, float fp8_max, float *scale_dev, float *inv_scale_dev)
 {
     sste_pdl_trigger();
-    sste_pdl_wait();
+    sste_pdl_wait(amax_dev);
     const float a = *amax_dev;
     const float s = sste_scale_from_amax(a, fp8_max);
     *scale_dev = s;
@@ -1121,7 +1121,7 @@ quantize_kernel(const uint4 *__restrict__ x, size_t n_chunks, const AmaxIn amax,
                 uint2 *__restrict__ q)
 {
     sste_pdl_trigger();
-    sste_pdl_wait();
+    sste_pdl_wait(x);
     const float scale = sste_scale_from_amax(amax_take(amax, blockIdx.x == 0 && threadIdx.x == 0), E5M2 ? 57344.0f : 448.0f);
     const size_t stride = static_cast<size_t>(gridDim.x) * EW_THREADS;
     for (size_t c = static_cast<size_t>(blockIdx.x) * EW_THREADS + threadIdx.x; c < n_chunks; c += 4 * stride) {
@@ -1301,7 +1301,7 @@ amax_quantize_kernel(const uint4 *__restrict__ x, size_t n_vec, float *__restric
     __shared__ uint32_t word_s[2];
     const int tid = threadIdx.x;
     sste_pdl_trigger();
-    sste_pdl_wait();
+    sste_pdl_wait(x);
     GridMaximum gm{slots, status, taken_s, word_s, 0, 0, taken_test};
     uint4 v[V];
     auto load = [&](uint32_t chunk) {
@@ -1358,7 +1358,7 @@ project_fp8_kernel(const uint4 *__restrict__ W, int I, uint32_t tiles, const flo
     const uint32_t across = static_cast<uint32_t>(I) / 128;
     if (tid < PROJECT_ENTRIES) lut[tid] = project_table_dev.e[tid];
     sste_pdl_trigger();
-    sste_pdl_wait();
+    sste_pdl_wait(W, beta_dev);
     GridMaximum gm{slots, status, taken_s, word_s, 0, 0, taken_test};
     const float beta = *beta_dev;
     const size_t row_chunks = static_cast<size_t>(I) / 8;
@@ -1414,7 +1414,7 @@ __global__ void __launch_bounds__(EW_THREADS)
 meta_to_canonical_kernel(const uint8_t *__restrict__ meta, int rows, int k, uint16_t *__restrict__ out)
 {
     sste_pdl_trigger();
-    sste_pdl_wait();
+    sste_pdl_wait(meta);
     const size_t words = static_cast<size_t>(rows) * (k / 16);
     for (size_t w = static_cast<size_t>(blockIdx.x) * EW_THREADS + threadIdx.x; w < words;
          w += static_cast<size_t>(gridDim.x) * EW_THREADS) {
@@ -1438,7 +1438,7 @@ decompress_kernel(const uint4 *__restrict__ vals, const uint8_t *__restrict__ me
                   uint4 *__restrict__ dense)
 {
     sste_pdl_trigger();
-    sste_pdl_wait();
+    sste_pdl_wait(vals, meta);
     const uint32_t units_per_row = static_cast<uint32_t>(k) / (EIGHT_BIT ? 32 : 16);
     for (size_t un = static_cast<size_t>(blockIdx.x) * EW_THREADS + threadIdx.x; un < n_units;
          un += static_cast<size_t>(gridDim.x) * EW_THREADS) {
@@ -1484,10 +1484,10 @@ decompress_kernel(const uint4 *__restrict__ vals, const uint8_t *__restrict__ me
 // INDEX: unsigned type that holds the number of destination vectors (a 64-bit division costs more than the copy).
 template <typename INDEX>
 __global__ void __launch_bounds__(EW_THREADS)
-pad_2d_kernel(const RaggedRows src, uint4 *__restrict__ dst, uint32_t vec_per_row, INDEX n_vec)
+pad_2d_kernel(RaggedRows src, uint4 *__restrict__ dst, uint32_t vec_per_row, INDEX n_vec)
 {
     sste_pdl_trigger();
-    sste_pdl_wait();
+    sste_pdl_wait(src.src);
     for (INDEX v = static_cast<INDEX>(blockIdx.x) * EW_THREADS + threadIdx.x; v < n_vec;
          v += static_cast<INDEX>(gridDim.x) * EW_THREADS) {
         const uint32_t r = static_cast<uint32_t>(v / vec_per_row);
@@ -1513,7 +1513,8 @@ crop_2d_kernel(const CropJob job0, const CropJob job1)
     sste_pdl_wait();
     const bool second = blockIdx.x >= job0.blocks;
     const CropJob &job = second ? job1 : job0;
-    const uint16_t *__restrict__ src = job.src;
+    const uint16_t *src = job.src;
+    sste_fresh(src);
     uint16_t *__restrict__ dst = job.dst;
     const uint32_t cols = job.cols, cols_p = job.cols_p, block = blockIdx.x - (second ? job0.blocks : 0u);
     const INDEX n = static_cast<INDEX>(job.n), n_vec = static_cast<INDEX>(job.n_vec);
@@ -1566,7 +1567,7 @@ srste_decay_kernel(const uint4 *__restrict__ W, const uint8_t *__restrict__ meta
                    uint4 *__restrict__ dW)
 {
     sste_pdl_trigger();
-    sste_pdl_wait();
+    sste_pdl_wait(W, meta);
     const size_t row_chunks = static_cast<size_t>(I) / 8;
     for (size_t c = static_cast<size_t>(blockIdx.x) * EW_THREADS + threadIdx.x; c < n_chunks;
          c += static_cast<size_t>(gridDim.x) * EW_THREADS) {
@@ -1605,7 +1606,7 @@ flip_count_kernel(const uint4 *__restrict__ a, const uint4 *__restrict__ b, size
                   unsigned long long *__restrict__ count)
 {
     sste_pdl_trigger();
-    sste_pdl_wait();
+    sste_pdl_wait(a, b);
     unsigned int local = 0;
     for (size_t v = static_cast<size_t>(blockIdx.x) * EW_THREADS + threadIdx.x; v < n_vec;
          v += static_cast<size_t>(gridDim.x) * EW_THREADS) {

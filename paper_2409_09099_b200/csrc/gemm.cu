@@ -863,6 +863,7 @@ product(const CUtensorMap &map_a, const CUtensorMap &map_b, const CUtensorMap &m
                     if (p.splits == 2) {
                         // one other partial, and a sum of two has no order: the next panel is on its way while one is stored
                         const float4 *src = part0 + static_cast<size_t>(1 - u.split) * 4 * PART;
+                        sste_fresh(src);
                         float4 q[8];
 #pragma unroll
                         for (int i = 0; i < 8; ++i) q[i] = __ldcg(src + (8 * lo + i) * 32);
@@ -897,6 +898,7 @@ product(const CUtensorMap &map_a, const CUtensorMap &map_b, const CUtensorMap &m
 #pragma unroll
                         for (int b = 0; b < BOXP; ++b) {
                             const float4 *src = part0 + (pnl + b) * 8 * 32;
+                            sste_fresh(src);
 #pragma unroll
                             for (int h = 0; h < 2; ++h) {
                                 uint32_t v[16];
@@ -1058,7 +1060,7 @@ product(const CUtensorMap &map_a, const CUtensorMap &map_b, const CUtensorMap &m
             return true;
         };
         e_setup();
-        sste_pdl_wait();
+        sste_pdl_wait(e_vals, e_meta);
         // three stages of loads in flight in registers: a round trip to L2 is longer than two stages of MMAs
         uint4 v0[UNITS], v1[UNITS], v2[UNITS];
         uint32_t m0[UNITS], m1[UNITS], m2[UNITS];
@@ -1210,6 +1212,7 @@ __global__ void __launch_bounds__(128) splitk_sum_kernel(const __grid_constant__
         const size_t step = static_cast<size_t>(4) * groups * 32;       // float4 between two splits
         const float4 *src = reinterpret_cast<const float4 *>(p.partials) +
                             (static_cast<size_t>(slot) * p.splits * 4 + quarter) * (groups * 32) + c4 * 32 + row;
+        sste_fresh(src);
         float4 v = __ldcg(src);
         auto add = [&](const float4 &x) {
             v.x = __fadd_rn(v.x, x.x); v.y = __fadd_rn(v.y, x.y); v.z = __fadd_rn(v.z, x.z); v.w = __fadd_rn(v.w, x.w);
