@@ -365,15 +365,17 @@ project_compress_kernel(const uint4 *__restrict__ W, int I, const float *__restr
     __shared__ uint2 lut[PROJECT_ENTRIES];
     const int tid = threadIdx.x;
     const int kb = blockIdx.x, rb = blockIdx.y;
-    if (MODE == 0 && tid < PROJECT_ENTRIES) lut[tid] = project_table_dev.e[tid];
     sste_pdl_trigger();
+    if (MODE == 0) {
+        if (tid < PROJECT_ENTRIES) lut[tid] = project_table_dev.e[tid];
+        __syncthreads();                         // the table is in place
+    }
     sste_pdl_wait(W, beta_dev, w_amax_dev);
     const size_t row_chunks = static_cast<size_t>(I) / 8;
     const ProjectOut p{W, row_chunks, *beta_dev, FP8 ? sste_scale_from_amax(*w_amax_dev, 448.0f) : 1.0f, gamma, vals, meta, dense};
     uint4 in[PC_CHUNKS];
 #pragma unroll
-    for (int i = 0; i < PC_CHUNKS; ++i) in[i] = __ldg(project_src(W, row_chunks, kb, rb, i * EW_THREADS + tid));
-    if (MODE == 0) __syncthreads();              // the table is in place
+    for (int i = 0; i < PC_CHUNKS; ++i) in[i] = sste_ld_once(project_src(W, row_chunks, kb, rb, i * EW_THREADS + tid));
     project_tile<FP8, MODE>(in, kb, rb, p, meta_s, lut);
 }
 
@@ -402,7 +404,7 @@ beta_kernel(const uint4 *__restrict__ W, size_t n_chunks, double *__restrict__ p
     double num = 0.0, den = 0.0;
     for (size_t c = static_cast<size_t>(blockIdx.x) * EW_THREADS + threadIdx.x; c < n_chunks;
          c += static_cast<size_t>(gridDim.x) * EW_THREADS) {
-        const uint4 v = __ldg(W + c);
+        const uint4 v = sste_ld_once(W + c);
         const uint32_t raw[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
         for (int g = 0; g < 2; ++g) {
@@ -785,9 +787,9 @@ __device__ __forceinline__ uint4 shift8(const uint4 &a, const uint4 &b, uint32_t
 }
 __device__ __forceinline__ uint4 load8(const uint4 *__restrict__ base, size_t first)
 {
-    const uint4 a = __ldg(base + (first >> 3));
+    const uint4 a = sste_ld(base + (first >> 3));
     const uint32_t sh = static_cast<uint32_t>(first) & 7u;
-    return sh == 0 ? a : shift8(a, __ldg(base + (first >> 3) + 1), sh);
+    return sh == 0 ? a : shift8(a, sste_ld(base + (first >> 3) + 1), sh);
 }
 
 // A [rows, cols] array of 2-byte elements whose rows may start anywhere, seen as the top-left corner of a larger one of zeros.
@@ -803,7 +805,7 @@ struct RaggedRows {
         if (c0 + 8 <= cols && load8_fits(first, lead, end)) return load8(reinterpret_cast<const uint4 *>(src - lead), first);
         uint32_t e[8];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) e[i] = (c0 + i < cols) ? __ldg(src + static_cast<size_t>(r) * cols + c0 + i) : 0u;
+        for (int i = 0; i < 8; ++i) e[i] = (c0 + i < cols) ? sste_ld(src + static_cast<size_t>(r) * cols + c0 + i) : 0u;
         return make_uint4(e[0] | (e[1] << 16), e[2] | (e[3] << 16), e[4] | (e[5] << 16), e[6] | (e[7] << 16));
     }
     // the same of four consecutive rows; all their loads are under way before the first is used
@@ -818,8 +820,8 @@ struct RaggedRows {
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const uint4 *v = base + ((first + static_cast<size_t>(i) * cols) >> 3);
-                a[i] = __ldg(v);
-                b[i] = __ldg(v + 1);
+                a[i] = sste_ld(v);
+                b[i] = sste_ld(v + 1);
             }
 #pragma unroll
             for (int i = 0; i < 4; ++i) out[i] = shift8(a[i], b[i], static_cast<uint32_t>(first + static_cast<size_t>(i) * cols) & 7u);
@@ -846,7 +848,7 @@ __global__ void __launch_bounds__(8 * G, G == 32 ? 4 : 8)
 mvue_kernel(const uint4 *__restrict__ dY, int O, int T, uint32_t key0, uint32_t key1, uint32_t tensor_id,
             uint32_t step, uint64_t tg_offset, uint32_t counter_cols, const AmaxIn g_amax,
             void *__restrict__ gvals,
-            uint8_t *__restrict__ gmeta, void *__restrict__ dense_q, RaggedRows rag, uint4 *__restrict__ padded)
+            uint8_t *__restrict__ gmeta, void *__restrict__ dense_q, const RaggedRows rag_in, uint4 *__restrict__ padded)
 {
     // 64 rows of G words (bf16) or halfwords (fp8)
     __shared__ __align__(16) uint32_t vals_s[64 * G / (FP8 ? 2 : 1)];
@@ -855,14 +857,14 @@ mvue_kernel(const uint4 *__restrict__ dY, int O, int T, uint32_t key0, uint32_t 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // column block (64), token block (4 G)
     const int jb = G == 32 ? blockIdx.x : blockIdx.x >> 1, tb = G == 32 ? blockIdx.y : 2 * blockIdx.y + (blockIdx.x & 1);
-    if (tid < MVUE_ENTRIES) lut[tid] = FP8 ? mvue_table_fp8.e[tid] : mvue_table_bf16.e[tid];
     sste_pdl_trigger();
-    sste_pdl_wait(dY, rag.src);
-    const float gscale = FP8 ? sste_scale_from_amax(amax_take(g_amax, jb == 0 && tb == 0 && tid == 0), 57344.0f) : 1.0f;
+    if (tid < MVUE_ENTRIES) lut[tid] = FP8 ? mvue_table_fp8.e[tid] : mvue_table_bf16.e[tid];
     __syncthreads();                              // the table is in place
+    RaggedRows rag = rag_in;
+    sste_pdl_wait(dY, rag.src);
     const size_t row_chunks = static_cast<size_t>(O) / 8;
-    bool plain = !FP8 || gscale < INFINITY;              // no infinity, NaN or sum that may overflow
-
+    bool plain = true;                                   // no infinity, NaN or sum that may overflow
+    float gscale = 1.0f;
     {
         const int jc = lane & 7;                         // column chunk 0..7
         const int tgl = warp * 4 + (lane >> 3);          // token group 0..31 inside the tile
@@ -870,11 +872,16 @@ mvue_kernel(const uint4 *__restrict__ dY, int O, int T, uint32_t key0, uint32_t 
         uint4 in[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i)
-            if (!PADDED) in[i] = __ldg(dY + (tok0 + i) * row_chunks + jb * 8 + jc);
+            if (!PADDED) in[i] = sste_ld_once(dY + (tok0 + i) * row_chunks + jb * 8 + jc);
         if (PADDED) {
             rag.load4(static_cast<uint32_t>(tok0), jb * 64u + jc * 8u, in);
 #pragma unroll
             for (int i = 0; i < 4; ++i) padded[(tok0 + i) * row_chunks + jb * 8 + jc] = in[i];
+        }
+        // (behind the loads: nothing moves them in front of the store of the maximum)
+        if (FP8) {
+            gscale = sste_scale_from_amax(amax_take(g_amax, jb == 0 && tb == 0 && tid == 0), 57344.0f);
+            plain = gscale < INFINITY;
         }
 
         const uint64_t g0 = (tg_offset + static_cast<uint64_t>(tb) * G + tgl) * static_cast<uint64_t>(counter_cols) +
@@ -1034,7 +1041,7 @@ amax_kernel(const uint4 *__restrict__ x, size_t n_chunks, unsigned int *__restri
     for (size_t c = static_cast<size_t>(blockIdx.x) * EW_THREADS + threadIdx.x; c < n_chunks; c += 4 * stride) {
         uint4 v[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) v[j] = (c + j * stride < n_chunks) ? __ldg(x + c + j * stride) : make_uint4(0, 0, 0, 0);
+        for (int j = 0; j < 4; ++j) v[j] = (c + j * stride < n_chunks) ? sste_ld_once(x + c + j * stride) : make_uint4(0, 0, 0, 0);
 #pragma unroll
         for (int j = 0; j < 4; ++j) best2 = max_magnitudes(best2, v[j]);
     }
@@ -1073,7 +1080,7 @@ project_amax_kernel(const uint4 *__restrict__ W, size_t n_chunks, const float *_
     for (size_t c = static_cast<size_t>(blockIdx.x) * EW_THREADS + threadIdx.x; c < n_chunks; c += 4 * stride) {
         uint4 v[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) v[j] = (c + j * stride < n_chunks) ? __ldg(W + c + j * stride) : make_uint4(0, 0, 0, 0);
+        for (int j = 0; j < 4; ++j) v[j] = (c + j * stride < n_chunks) ? sste_ld_once(W + c + j * stride) : make_uint4(0, 0, 0, 0);
 #pragma unroll
         for (int j = 0; j < 4; ++j) best = fmaxf(best, max_projected(v[j], beta));
     }
@@ -1127,7 +1134,7 @@ quantize_kernel(const uint4 *__restrict__ x, size_t n_chunks, const AmaxIn amax,
     for (size_t c = static_cast<size_t>(blockIdx.x) * EW_THREADS + threadIdx.x; c < n_chunks; c += 4 * stride) {
         uint4 v[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) v[j] = (c + j * stride < n_chunks) ? __ldg(x + c + j * stride) : make_uint4(0, 0, 0, 0);
+        for (int j = 0; j < 4; ++j) v[j] = (c + j * stride < n_chunks) ? sste_ld_once(x + c + j * stride) : make_uint4(0, 0, 0, 0);
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             if (c + j * stride >= n_chunks) break;
@@ -1308,7 +1315,7 @@ amax_quantize_kernel(const uint4 *__restrict__ x, size_t n_vec, float *__restric
 #pragma unroll
         for (int i = 0; i < V; ++i) {
             const size_t c = (static_cast<size_t>(chunk) * V + i) * AQ_THREADS + tid;
-            v[i] = c < n_vec ? __ldg(x + c) : make_uint4(0, 0, 0, 0);
+            v[i] = c < n_vec ? sste_ld_once(x + c) : make_uint4(0, 0, 0, 0);
         }
     };
     auto put_max = [&](uint32_t chunk) {
@@ -1369,7 +1376,7 @@ project_fp8_kernel(const uint4 *__restrict__ W, int I, uint32_t tiles, const flo
             const uint32_t tile = chunk * R + t, rb = tile / across;
 #pragma unroll
             for (int i = 0; i < PC_CHUNKS; ++i)
-                v[t][i] = tile < tiles ? __ldg(project_src(W, row_chunks, tile - rb * across, rb, i * EW_THREADS + tid)) : make_uint4(0, 0, 0, 0);
+                v[t][i] = tile < tiles ? sste_ld_once(project_src(W, row_chunks, tile - rb * across, rb, i * EW_THREADS + tid)) : make_uint4(0, 0, 0, 0);
         }
     };
     auto put_max = [&](uint32_t chunk) {
@@ -1446,7 +1453,7 @@ decompress_kernel(const uint4 *__restrict__ vals, const uint8_t *__restrict__ me
         const uint32_t row = (un >> 32) ? static_cast<uint32_t>(un / units_per_row) : static_cast<uint32_t>(un) / units_per_row;
         const uint32_t kk = static_cast<uint32_t>(un - static_cast<size_t>(row) * units_per_row) * (EIGHT_BIT ? 32u : 16u);
         const uint8_t *atom = meta + (static_cast<size_t>(row >> 7) * (k / 128) + (kk >> 7)) * 2048;
-        const uint4 v = __ldg(vals + un);
+        const uint4 v = sste_ld_once(vals + un);
         const uint32_t w[4] = {v.x, v.y, v.z, v.w};
         uint32_t o[8];
         if (EIGHT_BIT) {
@@ -1484,8 +1491,9 @@ decompress_kernel(const uint4 *__restrict__ vals, const uint8_t *__restrict__ me
 // INDEX: unsigned type that holds the number of destination vectors (a 64-bit division costs more than the copy).
 template <typename INDEX>
 __global__ void __launch_bounds__(EW_THREADS)
-pad_2d_kernel(RaggedRows src, uint4 *__restrict__ dst, uint32_t vec_per_row, INDEX n_vec)
+pad_2d_kernel(const RaggedRows src_in, uint4 *__restrict__ dst, uint32_t vec_per_row, INDEX n_vec)
 {
+    RaggedRows src = src_in;
     sste_pdl_trigger();
     sste_pdl_wait(src.src);
     for (INDEX v = static_cast<INDEX>(blockIdx.x) * EW_THREADS + threadIdx.x; v < n_vec;
@@ -1532,7 +1540,7 @@ crop_2d_kernel(const CropJob job0, const CropJob job1)
             *reinterpret_cast<uint4 *>(dst + e0) = load8(base, first);
         } else {
             for (INDEX e = e0; e < e1; ++e) {
-                dst[e] = __ldg(src + static_cast<size_t>(r) * cols_p + c);
+                dst[e] = sste_ld(src + static_cast<size_t>(r) * cols_p + c);
                 if (++c == cols) { c = 0; ++r; }
             }
         }
@@ -1573,9 +1581,9 @@ srste_decay_kernel(const uint4 *__restrict__ W, const uint8_t *__restrict__ meta
          c += static_cast<size_t>(gridDim.x) * EW_THREADS) {
         const uint32_t row = static_cast<uint32_t>(c / row_chunks), k = static_cast<uint32_t>(c % row_chunks) * 8u;
         const size_t atom = static_cast<size_t>(row >> 7) * (I / 128) + (k >> 7);
-        const uint32_t byte = __ldg(meta + atom * 2048 + (EIGHT_BIT ? sste_meta_atom_byte8(row & 127u, k & 127u)
+        const uint32_t byte = sste_ld(meta + atom * 2048 + (EIGHT_BIT ? sste_meta_atom_byte8(row & 127u, k & 127u)
                                                                      : sste_meta_atom_byte16(row & 127u, k & 127u)));
-        const uint4 w = __ldg(W + c);
+        const uint4 w = sste_ld_once(W + c);
         uint4 g = dW[c];
         const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
         uint32_t gw[4] = {g.x, g.y, g.z, g.w};
@@ -1610,7 +1618,7 @@ flip_count_kernel(const uint4 *__restrict__ a, const uint4 *__restrict__ b, size
     unsigned int local = 0;
     for (size_t v = static_cast<size_t>(blockIdx.x) * EW_THREADS + threadIdx.x; v < n_vec;
          v += static_cast<size_t>(gridDim.x) * EW_THREADS) {
-        const uint4 x = __ldg(a + v), y = __ldg(b + v);
+        const uint4 x = sste_ld_once(a + v), y = sste_ld_once(b + v);
         const uint32_t wx[4] = {x.x, x.y, x.z, x.w}, wy[4] = {y.x, y.y, y.z, y.w};
 #pragma unroll
         for (int w = 0; w < 4; ++w) {

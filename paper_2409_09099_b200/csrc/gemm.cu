@@ -1044,9 +1044,9 @@ product(const CUtensorMap &map_a, const CUtensorMap &map_b, const CUtensorMap &m
 #pragma unroll
             for (int j = 0; j < UNITS; ++j) {
                 if (e_cols) {
-                    v[j] = __ldg(reinterpret_cast<const uint4 *>(vp + static_cast<size_t>(j) * ROWS_STEP * row_bytes));
-                    if (F8) m[j] = __ldg(reinterpret_cast<const uint32_t *>(mp + moff[j]));
-                    else m[j] = __ldg(reinterpret_cast<const uint16_t *>(mp + moff[j]));
+                    v[j] = sste_ld(reinterpret_cast<const uint4 *>(vp + static_cast<size_t>(j) * ROWS_STEP * row_bytes));
+                    if (F8) m[j] = sste_ld(reinterpret_cast<const uint32_t *>(mp + moff[j]));
+                    else m[j] = sste_ld(reinterpret_cast<const uint16_t *>(mp + moff[j]));
                 } else {
                     v[j] = make_uint4(0, 0, 0, 0);         // columns beyond N: zeros (any valid code will do)
                     m[j] = 0x44444444u;
