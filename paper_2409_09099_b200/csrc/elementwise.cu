@@ -1189,6 +1189,13 @@ struct GridMaximum {
     unsigned int left;             // (thread 0) blocks that were done before this one
     unsigned int *taken_test;      // test hook: null, or where the chunks are counted that blocks work out besides their own
 
+    // The words are the layer's, so they are usually not in L2 any more: fetched while the previous kernel drains (a prefetch
+    // into L2 needs no order with anybody's writes).
+    __device__ __forceinline__ void fetch() const
+    {
+        if (blockIdx.x == 0 && threadIdx.x <= SSTE_MAX_SLOTS / 32)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(slots + min(threadIdx.x * 32u, SSTE_MAX_SLOTS - 1u)));
+    }
     // thread 0 (test hook: every other block's own chunk is left to the others)
     __device__ __forceinline__ void put(uint32_t chunk, uint32_t bits)
     {
@@ -1308,8 +1315,9 @@ amax_quantize_kernel(const uint4 *__restrict__ x, size_t n_vec, float *__restric
     __shared__ uint32_t word_s[2];
     const int tid = threadIdx.x;
     sste_pdl_trigger();
-    sste_pdl_wait(x);
     GridMaximum gm{slots, status, taken_s, word_s, 0, 0, taken_test};
+    gm.fetch();
+    sste_pdl_wait(x);
     uint4 v[V];
     auto load = [&](uint32_t chunk) {
 #pragma unroll
@@ -1365,8 +1373,9 @@ project_fp8_kernel(const uint4 *__restrict__ W, int I, uint32_t tiles, const flo
     const uint32_t across = static_cast<uint32_t>(I) / 128;
     if (tid < PROJECT_ENTRIES) lut[tid] = project_table_dev.e[tid];
     sste_pdl_trigger();
-    sste_pdl_wait(W, beta_dev);
     GridMaximum gm{slots, status, taken_s, word_s, 0, 0, taken_test};
+    gm.fetch();
+    sste_pdl_wait(W, beta_dev);
     const float beta = *beta_dev;
     const size_t row_chunks = static_cast<size_t>(I) / 8;
     uint4 v[R][PC_CHUNKS];
