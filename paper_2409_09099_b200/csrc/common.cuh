@@ -127,7 +127,7 @@ __device__ __host__ __forceinline__ uint32_t sste_meta_atom_byte8(uint32_t m, ui
 // Every kernel of the path is launched with programmatic stream serialisation: its CTAs may be scheduled,
 // and run their prologue (barrier and tensor-memory set-up, descriptor prefetch, index arithmetic), while the
 // previous kernel of the stream is still draining.  sste_pdl_wait() returns once that previous kernel has
-// finished and its writes are visible; no kernel touches global memory before it.  sste_pdl_trigger(), issued
+// finished and its writes are visible; before it a kernel reads tables only.  sste_pdl_trigger(), issued
 // first thing, is what lets the NEXT kernel of the stream be scheduled early (it takes effect when every CTA
 // of this grid has issued it or exited, so the successor never competes with CTAs not yet started).
 __device__ __forceinline__ void sste_pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
