@@ -79,7 +79,8 @@ def test_projected_weight(ctx, O, I, dense_copy):
 
 
 def test_blocks_that_cannot_run_are_not_waited_for(ctx):
-    """A product on 80 SMs of another stream (its context cannot split it) leaves room for half of the blocks."""
+    """A product on 80 SMs of another stream (its context cannot split it) leaves room for half of the blocks: the results are the same.
+    (Whether blocks are overtaken here is a matter of time; test_chunks_that_others_work_out makes it so.)"""
     other, side = B.Context(0, minimal_workspace=True), torch.cuda.Stream()
     M, K = 10240, 16384
     busy = SsteLinear(other, _randn(M, 256, 3) * 0.02, K)          # grad_W: 40 tiles of the whole reduction
